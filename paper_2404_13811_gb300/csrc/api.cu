@@ -33,9 +33,9 @@ cudaError_t launch_assemble2d(const DevPtrs& P, const double* X, int nitems, int
                               cudaStream_t s);
 cudaError_t launch_faces(const MemberDev* dmem, int nmem, long long maxcells, const double* K, double* Tf,
                          double* hk, double* wh, cudaStream_t s);
-cudaError_t launch_output(const MemberDev* dmem, int nmem, int member, const double* p, const double* u,
-                          long long off, long long nc, int nside, double* dmean, double* pout,
-                          double* uout, cudaStream_t s);
+int output_scratch();
+cudaError_t launch_output(const double* p, const double* u, long long nc, int nside, bool gauge, double* part,
+                          double* pout, double* uout, cudaStream_t s);
 
 cudaError_t if_assemble(const DevPtrs& P, const MethodDev& M, const IfPtrs& I, int nitems, int nrows,
                         cudaStream_t s);
@@ -562,7 +562,7 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
     if ((e = dalloc(h, &h->d_ubg, (size_t)nitems * MRCM_MAXSIDE * h->side_max))) return e;
     if ((e = dalloc(h, &h->d_mom, (size_t)nitems * (h->nbasis_max + 1) * MRCM_MAXSIDE * h->npsi * 2))) return e;
     if ((e = dalloc(h, &h->d_status, MRCM_STATUS_WORDS))) return e;
-    if ((e = dalloc(h, &h->d_mean, nmem))) return e;
+    if ((e = dalloc(h, &h->d_mean, output_scratch()))) return e;
     cudaStream_t st = h->stream;
     CUDA_TRY(h, cudaMemcpyAsync(h->d_mem, h->mem.data(), sizeof(MemberDev) * nmem, cudaMemcpyHostToDevice, st));
     CUDA_TRY(h, cudaMemcpyAsync(h->d_sub, h->sub.data(), sizeof(SubDev) * nitems, cudaMemcpyHostToDevice, st));
@@ -1647,7 +1647,7 @@ int mrcm_fluxes(mrcm_handle* h, int member, double* u_cellfaces, double* p_cells
         pd = tp;
         ud = tu;
     }
-    CUDA_TRY(h, launch_output(h->d_mem, (int)h->mem.size(), member, h->d_p, h->d_u, md.cell_off, nc, nside,
+    CUDA_TRY(h, launch_output(h->d_p + md.cell_off, h->d_u + md.cell_off * nside, nc, nside, md.pure_neumann != 0,
                               h->d_mean, pd, ud, st));
     if (!device_ptrs) {
         if (p_cells) CUDA_TRY(h, cudaMemcpyAsync(p_cells, tp, sizeof(double) * nc, cudaMemcpyDeviceToHost, st));

@@ -69,29 +69,57 @@ __global__ void k_assemble2d(DevPtrs P, const double* __restrict__ X) {
     }
 }
 
-// Deterministic per-member mean of the pressure (one CTA per member).
-__global__ void k_member_mean(const MemberDev* mem, const double* p, double* mean) {
-    __shared__ double red[256];
-    const MemberDev& md = mem[blockIdx.x];
-    long long nc = (long long)md.n[0] * md.n[1] * (md.dim == 3 ? md.n[2] : 1);
+// Partial sums of a member's pressure in a fixed order (pure-Neumann members
+// are reported with zero mean): block b sums cells [b * per, (b + 1) * per).
+// One block per member took 179 us for 262,144 cells (one SM's loads, each
+// waited for); with a block per 2048 cells (256 blocks at most) the sum is a
+// few microseconds, and members with a Dirichlet side skip it.
+constexpr int GAUGE_BLOCKS = 256;   // most partial sums (the handle's scratch)
+constexpr int GAUGE_CELLS = 2048;   // cells per block below that
+
+__global__ void __launch_bounds__(256) k_gauge_partials(const double* __restrict__ p, long long nc, long long per,
+                                                        double* part) {
+    __shared__ double red[8];
+    const long long c0 = blockIdx.x * per, c1 = min(nc, c0 + per);
     double s = 0.0;
-    for (long long c = threadIdx.x; c < nc; c += blockDim.x) s += p[md.cell_off + c];
-    red[threadIdx.x] = s;
+#pragma unroll 4
+    for (long long c = c0 + threadIdx.x; c < c1; c += 256) s += p[c];
+    for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
     __syncthreads();
-    for (int o = blockDim.x / 2; o; o >>= 1) {
-        if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-        __syncthreads();
+    if (threadIdx.x == 0) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        part[blockIdx.x] = t;
     }
-    if (threadIdx.x == 0) mean[blockIdx.x] = md.pure_neumann ? red[0] / (double)nc : 0.0;
 }
 
-__global__ void k_output(const double* p, const double* u, long long off, long long nc, int nside,
-                         const double* mean, double* pout, double* uout) {
-    const long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (c >= nc) return;
-    if (pout) pout[c] = p[off + c] - mean[0];
-    if (uout)
-        for (int s = 0; s < nside; ++s) uout[c * nside + s] = u[(off + c) * nside + s];
+// Copies a member's pressure (less the mean given by npart partial sums, 0: no
+// gauge) and velocities, both as flat arrays: consecutive threads, consecutive
+// values.
+__global__ void __launch_bounds__(256) k_output(const double* __restrict__ p, const double* __restrict__ u,
+                                                long long nc, int nside, const double* __restrict__ part, int npart,
+                                                double* __restrict__ pout, double* __restrict__ uout) {
+    double mean = 0.0;
+    if (npart > 0) {
+        __shared__ double sm;
+        if (threadIdx.x < 32) {
+            double s = 0.0;
+            for (int b = threadIdx.x; b < npart; b += 32) s += part[b];
+            for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+            if (threadIdx.x == 0) sm = s / (double)nc;
+        }
+        __syncthreads();
+        mean = sm;
+    }
+    const long long t0 = blockIdx.x * 256LL + threadIdx.x, step = gridDim.x * 256LL;
+    if (pout)
+        for (long long c = t0; c < nc; c += step) pout[c] = p[c] - mean;
+    if (uout) {
+        const long long n = nc * nside;
+#pragma unroll 4
+        for (long long c = t0; c < n; c += step) uout[c] = u[c];
+    }
 }
 
 cudaError_t launch_assemble2d(const DevPtrs& P, const double* X, int nitems, int ncell_i_max,
@@ -100,11 +128,19 @@ cudaError_t launch_assemble2d(const DevPtrs& P, const double* X, int nitems, int
     return cudaGetLastError();
 }
 
-cudaError_t launch_output(const MemberDev* dmem, int nmem, int member, const double* p, const double* u,
-                          long long off, long long nc, int nside, double* dmean, double* pout,
-                          double* uout, cudaStream_t s) {
-    k_member_mean<<<nmem, 256, 0, s>>>(dmem, p, dmean);
-    k_output<<<(unsigned)((nc + 255) / 256), 256, 0, s>>>(p, u, off, nc, nside, dmean + member, pout, uout);
+// part: scratch of at least output_scratch() doubles; gauge: report zero mean.
+int output_scratch() { return GAUGE_BLOCKS; }
+
+cudaError_t launch_output(const double* p, const double* u, long long nc, int nside, bool gauge, double* part,
+                          double* pout, double* uout, cudaStream_t s) {
+    int npart = 0;
+    if (gauge && pout) {
+        const long long per = std::max<long long>(GAUGE_CELLS, (nc + GAUGE_BLOCKS - 1) / GAUGE_BLOCKS);
+        npart = (int)((nc + per - 1) / per);
+        k_gauge_partials<<<npart, 256, 0, s>>>(p, nc, per, part);
+    }
+    const int blocks = (int)std::min<long long>((nc + 255) / 256, 152 * 8);
+    k_output<<<blocks, 256, 0, s>>>(p, u, nc, nside, part, npart, pout, uout);
     return cudaGetLastError();
 }
 
