@@ -1,38 +1,39 @@
 // 3D local Robin/Darcy solves of MRCM-OS on sm_103a.
 //
-// One CTA (256 threads) per job (a subdomain box).  The cell-centred RT0
+// One CTA (17 warps) per job (a subdomain box).  The cell-centred RT0
 // operator of the box (Sec. 2.2; the face laws of Eq. (genRobin)) is block
 // tridiagonal over the planes normal to the box's longest axis a2; a plane
 // has b = n_a0 n_a1 cells (a0 fastest) and planes couple through diagonal
 // blocks D_j (the a2-face transmissibilities).  The factorisation
 // (Algorithm 1, Steps 1 and 6) keeps the inverses of the plane Schur
-// complements S_j = A_jj - D_{j-1} S_{j-1}^{-1} D_{j-1}: each S_j is formed
-// in shared memory from S_{j-1}^{-1} in place (D is diagonal) and inverted
-// there by the whole CTA (Gauss-Jordan, SPD so no pivoting); the inverses go
-// to global memory (a box's factor, n_a2 b^2 entries, does not fit on chip).
+// complements S_j = A_jj - D_{j-1} S_{j-1}^{-1} D_{j-1}: S_j is formed in
+// registers from S_{j-1}^{-1} in place (D is diagonal) and inverted there by
+// the whole CTA (Gauss-Jordan, SPD so no pivoting); the inverses go to global
+// memory (a box's factor, n_a2 b^2 entries, does not fit on chip).
 // A solve is two sweeps of dense b x b products, all right-hand sides of a
 // round at once, so each plane inverse is read once per sweep.
 //
 // Precision: T = double is the FP64 form.  T = float is the mixed form:
-// Jacobi-scaled operator, Schur diagonals and pivot reciprocals from FP64,
-// FP32 sweeps, FP64 residual refinement to ir_tol (as in 2D).
+// Jacobi-scaled operator, Schur diagonals from FP64, FP32 sweeps, FP64
+// residual refinement to ir_tol in the scaled variables (as in 2D).
 #include "box2d.cuh"
 
 namespace {
 
-constexpr int T3 = 256;   // threads per CTA
-constexpr int NR3 = 4;    // right-hand sides per round
-constexpr int CR3 = 16;   // rows of a plane inverse per streamed chunk
+constexpr int NW3 = 16;             // warps that compute in the sweeps
+constexpr int T3 = 32 * (NW3 + 1);  // threads per CTA: one more warp issues the sweeps' copies
+constexpr int NR3 = 4;              // right-hand sides per round, at most
+constexpr int GT3 = 4;              // side of a register tile of the plane inverses
+constexpr int GB3 = 128;            // widest plane inverted in registers
+constexpr int ST3 = 4;              // most stages of the sweeps' copies
 
-// plane stride of a kept factor: b^2 entries padded to 16 bytes
-__host__ __device__ __forceinline__ size_t plane_stride(int b) { return ((size_t)b * b + 3) & ~size_t(3); }
-// entries of one staging buffer for `rows` rows of a plane: a multiple of 4
-// entries, so that the second buffer starts on a 16-byte boundary (the bulk
-// copy needs 16-byte aligned destinations) and the copy size, rounded up to
-// 16 bytes, fits
-__host__ __device__ __forceinline__ size_t stage_cap(int rows, int b) {
-    return (((size_t)rows * b + 3) & ~size_t(3)) + 4;
-}
+// row stride of a plane inverse: b entries padded to 4 (16 bytes in FP32, 32 in FP64)
+__host__ __device__ constexpr int plane_ld(int b) { return (b + 3) & ~3; }
+__host__ __device__ __forceinline__ size_t plane_stride(int b) { return (size_t)b * plane_ld(b); }
+// rows of a plane inverse per copy (32 KB in FP32, 16 KB in FP64 for planes of
+// 128 cells): a wait and its bookkeeping cost a few hundred cycles, as much as
+// the products of 32 FP32 rows
+__host__ __device__ constexpr int stage_rows(int tsz) { return tsz == 4 ? 64 : 16; }
 
 struct Box3 {
     int lo[3], hi[3], n[3];
@@ -44,12 +45,7 @@ struct Box3 {
     double alpha;
     int ts[6], tt[6]; // tangential axes (ascending) of each side
     int soff[7];      // offsets of the sides in the boundary-face arrays
-    int crows;        // rows of a plane inverse per streamed copy
 };
-
-// rows per streamed copy: whole planes in the mixed form (two plane buffers
-// keep ~64 KB in flight per SM), 16-row chunks in the FP64 form
-__host__ __device__ __forceinline__ int stream_rows(int b, bool mixed) { return mixed ? b : (b < CR3 ? b : CR3); }
 
 __device__ void setup_box3(Box3& B, const MemberDev& md, const int* lo, const int* hi, double alpha) {
     for (int a = 0; a < 3; ++a) {
@@ -116,59 +112,66 @@ struct Ops3 {
     unsigned char* nb;                 // neighbour bits: 1 -a0, 2 +a0, 4 -a1, 8 +a1, 16 -a2, 32 +a2
 };
 
+// side of face f of the boundary-face arrays
+__device__ __forceinline__ int side_of(const Box3& B, int f) {
+    int sid = 0;
+#pragma unroll
+    for (int s = 1; s < 6; ++s) sid += f >= B.soff[s];
+    return sid;
+}
+// cell at face f of the boundary-face arrays (side sid)
+__device__ __forceinline__ void face_cell(const Box3& B, int sid, int f, int* c) {
+    const int e = f - B.soff[sid], ls = B.n[B.ts[sid]], q = e / ls;
+    c[sid >> 1] = (sid & 1) ? B.n[sid >> 1] - 1 : 0;
+    c[B.ts[sid]] = e - q * ls;
+    c[B.tt[sid]] = q;
+}
+
+// The box operator from the face coefficients.  The faces of all sides are
+// one list, so that their loads are in flight together.
 __device__ void build_ops3(const Box3& B, const MemberDev& md, const DevPtrs& P, Ops3& O, bool mixed) {
     const double* Tf = P.Tf + md.cell_off * 3;
     const double* hkg = P.hk + md.cell_off * 3;
     const double* wh = P.wh + md.cell_off * 3;
     const double vol = md.h[0] * md.h[1] * md.h[2];
-    for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
+    const int a0 = B.a0, a1 = B.a1, a2 = B.a2, e0 = B.n[a0], e1 = B.n[a1], e2 = B.np, b = B.b, nc = B.nc;
+    for (int t = threadIdx.x; t < nc; t += blockDim.x) {
         int c[3];
         bcoord(B, t, c);
-        const long long g = gidx(B, md, c);
-        O.c0[t] = c[B.a0] < B.n[B.a0] - 1 ? Tf[g * 3 + B.a0] : 0.0;
-        O.c1[t] = c[B.a1] < B.n[B.a1] - 1 ? Tf[g * 3 + B.a1] : 0.0;
-        O.c2[t] = c[B.a2] < B.n[B.a2] - 1 ? Tf[g * 3 + B.a2] : 0.0;
-        unsigned char m = 0;
-        if (c[B.a0] > 0) m |= 1;
-        if (c[B.a0] < B.n[B.a0] - 1) m |= 2;
-        if (c[B.a1] > 0) m |= 4;
-        if (c[B.a1] < B.n[B.a1] - 1) m |= 8;
-        if (c[B.a2] > 0) m |= 16;
-        if (c[B.a2] < B.n[B.a2] - 1) m |= 32;
-        O.nb[t] = m;
+        const double* T = Tf + gidx(B, md, c) * 3;
+        const double t0 = T[a0], t1 = T[a1], t2 = T[a2];
+        const int i = c[a0], j = c[a1], k = c[a2];
+        O.c0[t] = i < e0 - 1 ? t0 : 0.0;
+        O.c1[t] = j < e1 - 1 ? t1 : 0.0;
+        O.c2[t] = k < e2 - 1 ? t2 : 0.0;
+        O.nb[t] = (unsigned char)((i > 0) | (i < e0 - 1) << 1 | (j > 0) << 2 | (j < e1 - 1) << 3 | (k > 0) << 4 |
+                                  (k < e2 - 1) << 5);
     }
-    for (int sid = 0; sid < 6; ++sid) {
-        const int a = sid >> 1;
-        const int ls = B.n[B.ts[sid]];
-        const int faces = B.soff[sid + 1] - B.soff[sid];
+    for (int f = threadIdx.x; f < B.soff[6]; f += blockDim.x) {
+        const int sid = side_of(B, f), a = sid >> 1;
+        int c[3];
+        face_cell(B, sid, f, c);
+        const long long g = gidx(B, md, c);
         const double area = vol / md.h[a];
-        for (int e = threadIdx.x; e < faces; e += blockDim.x) {
-            int c[3];
-            c[a] = (sid & 1) ? B.n[a] - 1 : 0;
-            c[B.ts[sid]] = e % ls;
-            c[B.tt[sid]] = e / ls;
-            const long long g = gidx(B, md, c);
-            const double hin = hkg[g * 3 + a];
-            double T = 0.0, beta = 0.0;
-            if (B.kind[sid] == 2) {
-                const long long gf = (sid & 1) ? g : g - gstride(md, a);
-                beta = B.alpha * wh[gf * 3 + a];
-                T = area * rcp64(hin + beta);
-            } else if (B.kind[sid] == 1) {
-                T = area * rcp64(hin);
-            }
-            O.bT[B.soff[sid] + e] = T;
-            O.bB[B.soff[sid] + e] = beta;
+        const double hin = hkg[g * 3 + a];
+        double T = 0.0, beta = 0.0;
+        if (B.kind[sid] == 2) {
+            const long long gf = (sid & 1) ? g : g - gstride(md, a);
+            beta = B.alpha * wh[gf * 3 + a];
+            T = area * rcp64(hin + beta);
+        } else if (B.kind[sid] == 1) {
+            T = area * rcp64(hin);
         }
+        O.bT[f] = T;
+        O.bB[f] = beta;
     }
     __syncthreads();
-    const int s0 = 1, s1 = B.n[B.a0], s2 = B.b;
-    for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
+    for (int t = threadIdx.x; t < nc; t += blockDim.x) {
         const unsigned char m = O.nb[t];
         double d = O.c0[t] + O.c1[t] + O.c2[t];
-        if (m & 1) d += O.c0[t - s0];
-        if (m & 4) d += O.c1[t - s1];
-        if (m & 16) d += O.c2[t - s2];
+        if (m & 1) d += O.c0[t - 1];
+        if (m & 4) d += O.c1[t - e0];
+        if (m & 16) d += O.c2[t - b];
         if ((m & 63) != 63) {
             int c[3];
             bcoord(B, t, c);
@@ -183,27 +186,321 @@ __device__ void build_ops3(const Box3& B, const MemberDev& md, const DevPtrs& P,
     __syncthreads();
 }
 
-// (A x)_t of the unscaled FP64 operator with the couplings read from the
-// global face coefficients (the mixed form keeps no coupling arrays on chip
-// during the solves)
-__device__ __forceinline__ double applyA3g(const Box3& B, const MemberDev& md, const double* __restrict__ Tf,
-                                           const double* cd, const unsigned char* nbits, const double* x, int t) {
-    int c[3];
-    bcoord(B, t, c);
-    const long long g = gidx(B, md, c);
-    const unsigned char m = nbits[t];
+// Mixed form: the operator in scaled variables, D A D (as scale_ops in 2D).
+__device__ void scale_ops3(const Box3& B, Ops3& O) {
     const int s1 = B.n[B.a0], s2 = B.b;
-    double s = cd[t] * x[t];
-    if (m & 1) s -= Tf[(g - gstride(md, B.a0)) * 3 + B.a0] * x[t - 1];
-    if (m & 2) s -= Tf[g * 3 + B.a0] * x[t + 1];
-    if (m & 4) s -= Tf[(g - gstride(md, B.a1)) * 3 + B.a1] * x[t - s1];
-    if (m & 8) s -= Tf[g * 3 + B.a1] * x[t + s1];
-    if (m & 16) s -= Tf[(g - gstride(md, B.a2)) * 3 + B.a2] * x[t - s2];
-    if (m & 32) s -= Tf[g * 3 + B.a2] * x[t + s2];
+    for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
+        const unsigned char m = O.nb[t];
+        const double d = O.dsc[t];
+        O.cd[t] = O.cd[t] * d * d;
+        O.c0[t] = (m & 2) ? O.c0[t] * d * O.dsc[t + 1] : 0.0;
+        O.c1[t] = (m & 8) ? O.c1[t] * d * O.dsc[t + s1] : 0.0;
+        O.c2[t] = (m & 32) ? O.c2[t] * d * O.dsc[t + s2] : 0.0;
+    }
+    __syncthreads();
+}
+
+// b_t - (A x)_t in FP64 (both scaled in the mixed form)
+__device__ __forceinline__ double resid3(const Ops3& O, int s1, int s2, const double* x, double bt, int t) {
+    const unsigned char m = O.nb[t];
+    double s = fma(-O.cd[t], x[t], bt);
+    if (m & 1) s = fma(O.c0[t - 1], x[t - 1], s);
+    if (m & 2) s = fma(O.c0[t], x[t + 1], s);
+    if (m & 4) s = fma(O.c1[t - s1], x[t - s1], s);
+    if (m & 8) s = fma(O.c1[t], x[t + s1], s);
+    if (m & 16) s = fma(O.c2[t - s2], x[t - s2], s);
+    if (m & 32) s = fma(O.c2[t], x[t + s2], s);
     return s;
 }
 
-// 16-byte vectors of the shared-memory kernels (float4 / double2)
+// N consecutive values of shared memory, 16 bytes a load where N allows it
+template <typename T, int N>
+__device__ __forceinline__ void ldv(const T* __restrict__ p, T (&v)[N]) {
+    constexpr int W = 16 / (int)sizeof(T);
+    if constexpr (N % W == 0) {
+        using V = std::conditional_t<sizeof(T) == 4, float4, double2>;
+#pragma unroll
+        for (int q = 0; q < N / W; ++q) {
+            const V t = reinterpret_cast<const V*>(p)[q];
+            v[W * q] = t.x;
+            v[W * q + 1] = t.y;
+            if constexpr (W == 4) {
+                v[W * q + 2] = t.z;
+                v[W * q + 3] = t.w;
+            }
+        }
+    } else if constexpr (N == 2) {
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        v[0] = t.x;
+        v[1] = t.y;
+    } else {
+#pragma unroll
+        for (int q = 0; q < N; ++q) v[q] = p[q];
+    }
+}
+template <typename T>
+__device__ __forceinline__ void stv4(T* p, T a, T b, T c, T d) {
+    if constexpr (sizeof(T) == 4) {
+        *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+    } else {
+        reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
+        reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
+    }
+}
+
+// 1 / v for the pivots.  FP32: the hardware approximation and one
+// Newton-Raphson step.  FP64: from the FP32 seed r one third-order step,
+// r + r (e + e^2) with e = 1 - v r (e is about 2^-22, the error left e^3); the
+// conversions on the integer pipe.  Outside the FP32 normal range the division.
+__device__ __forceinline__ float rcp_piv(float v) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return fmaf(r, fmaf(-v, r, 1.f), r);
+}
+__device__ __forceinline__ double rcp_piv(double v) {
+    if (!in_f32_range(v)) return 1.0 / v;
+    const double r = f2d_bits(__frcp_rn(d2f_bits(v)));
+    const double e = fma(-v, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// Workspace of the register inverses (entries): two panels of GT3 rows, the
+// scaled panel, two inverse pivot blocks, two diagonal tiles, the diagonal of
+// the last inverse and of the next Schur block.
+constexpr int GLD3 = GB3 + 4;
+constexpr int GJW3 = 3 * GT3 * GLD3 + 4 * GT3 * GT3 + 2 * GLD3;
+
+// Block LDL^T over planes of at most GB3 cells, each plane's Schur block
+// inverted in registers: the block is symmetric, and the in-place
+// Gauss-Jordan elimination of a symmetric block keeps M_IJ = +-M_JI^T (minus
+// when exactly one of I, J has been eliminated), so only the GT3 x GT3 tiles
+// (I, J), I <= J, are held, one per thread (528 for 128 cells).  Pivots go by
+// blocks K of GT3 rows, two barriers per block:
+//   - the threads holding row or column block K have published the panel
+//     M_K., the last warp the inverse pivot block P = M_KK^-1; every thread
+//     forms one entry of P M_K.;
+//   - every thread updates its tile, M_IJ -= M_IK (P M_KJ), and publishes it
+//     if it belongs to the next panel.  Meanwhile the last warp updates the
+//     next pivot block by itself, from the copy its holder left in dt, and
+//     inverts it with one entry per lane, so that the pivots' reciprocals are
+//     off the chain.
+// Bound by the update's FP64 FMAs in the FP64 form, by the latency of the
+// per-block chain in the mixed form.  c0s, c1s: the in-plane couplings in T.
+template <typename T>
+__device__ void factor3_reg(const Box3& B, const Ops3& O, const T* c0s, const T* c1s, const T* c2s, T* F, T* ws,
+                            int* bad) {
+    constexpr int G = GT3;
+    const int b = B.b, ld = plane_ld(b), nb4 = ld / G, n0 = B.n[B.a0], np = B.np;
+    T* R = ws;                        // [2][G][GLD3]
+    T* Rn = R + 2 * G * GLD3;         // [G][GLD3]
+    T* pinv = Rn + G * GLD3;          // [2][G * G]
+    T* dt = pinv + 2 * G * G;         // [2][G * G] tile (k, k) before the update by block k - 1
+    T* dg = dt + 2 * G * G;           // [GLD3] diagonal of the last inverse
+    T* dn = dg + GLD3;                // [GLD3] diagonal of the Schur block
+    const int tid = threadIdx.x, lane = tid & 31;
+    const bool act = tid < nb4 * (nb4 + 1) / 2;
+    const bool pivot_warp = tid >= 32 * NW3;
+    int I = 0, J = tid;               // tile of this thread, row-major over I <= J
+    if (act) {
+        while (J >= nb4 - I) {
+            J -= nb4 - I;
+            ++I;
+        }
+        J += I;
+    } else {
+        I = J = -4;
+    }
+    const int dd = G * (J - I), o1 = n0 - dd;   // the plane's couplings of stride n0 are at x - y == o1
+    T V[G][G];
+#pragma unroll
+    for (int y = 0; y < G; ++y)
+#pragma unroll
+        for (int x = 0; x < G; ++x) V[y][x] = T(0);
+    // the panel of block k from the tiles that hold it, and the next pivot block
+    auto publish = [&](int k) {
+        T* Rk = R + (k & 1) * G * GLD3;
+        if (I == k) {
+#pragma unroll
+            for (int y = 0; y < G; ++y) stv4(Rk + y * GLD3 + G * J, V[y][0], V[y][1], V[y][2], V[y][3]);
+        } else if (J == k) {
+            // I < k has been eliminated: M_kI = -M_Ik^T
+#pragma unroll
+            for (int x = 0; x < G; ++x) stv4(Rk + x * GLD3 + G * I, -V[0][x], -V[1][x], -V[2][x], -V[3][x]);
+        }
+        if (I == k + 1 && J == k + 1) {
+            T* d = dt + ((k + 1) & 1) * G * G;
+#pragma unroll
+            for (int y = 0; y < G; ++y) stv4(d + G * y, V[y][0], V[y][1], V[y][2], V[y][3]);
+        }
+    };
+    // (last warp) inverse of the pivot block whose entry (lane / 4 mod 4, lane mod 4) is v
+    auto invert = [&](T v, int k) {
+        const int y = (lane >> 2) & 3, x = lane & 3;
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+            T piv = __shfl_sync(0xffffffffu, v, 5 * q);
+            if (!(piv > T(0))) {
+                if (lane == 0) *bad = 1;
+                piv = T(1);
+            }
+            const T ip = rcp_piv(piv);
+            const T r = __shfl_sync(0xffffffffu, v, G * q + x), c = __shfl_sync(0xffffffffu, v, G * y + q);
+            const T rp = x == q ? ip : r * ip;
+            v = y == q ? rp : (x == q ? T(0) : v) - c * rp;
+        }
+        if (lane < G * G) pinv[(k & 1) * G * G + lane] = v;
+    };
+    const int rc = tid & (GB3 - 1), ry = tid >> 7;   // the entry of P M_K. this thread forms
+    for (int j = 0; j < np; ++j) {
+        const int p0 = j * b;
+        // diagonal of S_j in FP64 (where the cancellation is)
+        if (tid < b) {
+            double s = O.cd[p0 + tid];
+            if (j > 0) {
+                const double cc = (double)c2s[p0 - b + tid];
+                s -= cc * (cc * (double)dg[tid]);   // not cc^2 (range at tiny couplings)
+            }
+            dn[tid] = (T)s;
+        }
+        __syncthreads();
+        if (act) {
+            T ci[G], ck[G];
+#pragma unroll
+            for (int y = 0; y < G; ++y) {
+                ci[y] = (j > 0 && G * I + y < b) ? c2s[p0 - b + G * I + y] : T(0);
+                ck[y] = (j > 0 && G * J + y < b) ? c2s[p0 - b + G * J + y] : T(0);
+            }
+#pragma unroll
+            for (int y = 0; y < G; ++y)
+#pragma unroll
+                for (int x = 0; x < G; ++x) V[y][x] = -(ci[y] * V[y][x] * ck[x]);
+            if (dd <= G) {
+                // couplings of stride 1, the diagonal; padding: the identity
+                T e[G];
+#pragma unroll
+                for (int y = 0; y < G; ++y) e[y] = G * I + y + 1 < b ? c0s[p0 + G * I + y] : T(0);
+                if (dd == G) {
+                    V[G - 1][0] -= e[G - 1];
+                } else {
+#pragma unroll
+                    for (int y = 0; y < G; ++y) {
+                        V[y][y] = G * I + y < b ? dn[G * I + y] : T(1);
+                        if (y + 1 < G) {
+                            V[y][y + 1] -= e[y];
+                            V[y + 1][y] -= e[y];
+                        }
+                    }
+                }
+            }
+            if (o1 > -G && o1 < G) {
+                T e[G];
+#pragma unroll
+                for (int y = 0; y < G; ++y) e[y] = G * I + y + n0 < b ? c1s[p0 + G * I + y] : T(0);
+#pragma unroll
+                for (int y = 0; y < G; ++y)
+#pragma unroll
+                    for (int x = 0; x < G; ++x) {
+                        if (x - y == o1) V[y][x] -= e[y];
+                        if (dd == 0 && y - x == o1) V[y][x] -= e[x];
+                    }
+            }
+        }
+        publish(0);
+        if (I == 0 && J == 0) {
+#pragma unroll
+            for (int y = 0; y < G; ++y) stv4(dt + G * y, V[y][0], V[y][1], V[y][2], V[y][3]);
+        }
+        __syncthreads();
+        if (pivot_warp) invert(dt[lane & (G * G - 1)], 0);
+        __syncthreads();
+        for (int k = 0; k < nb4; ++k) {
+            const T* Rk = R + (k & 1) * G * GLD3;
+            if (!pivot_warp && rc < ld) {
+                const bool own = (rc / G) == k;
+                T r[G], p[G];
+#pragma unroll
+                for (int m = 0; m < G; ++m) r[m] = Rk[m * GLD3 + rc];
+                ldv<T, G>(pinv + (k & 1) * G * G + G * ry, p);
+                const T v = (p[0] * r[0] + p[1] * r[1]) + (p[2] * r[2] + p[3] * r[3]);
+                Rn[ry * GLD3 + rc] = own ? pinv[(k & 1) * G * G + G * ry + (rc & (G - 1))] : v;
+            }
+            __syncthreads();
+            if (pivot_warp && k + 1 < nb4) {
+                const int y = (lane >> 2) & 3, x = lane & 3, c = G * (k + 1);
+                T v = dt[((k + 1) & 1) * G * G + (lane & (G * G - 1))];
+#pragma unroll
+                for (int m = 0; m < G; ++m) v -= Rk[m * GLD3 + c + y] * Rn[m * GLD3 + c + x];
+                invert(v, k + 1);
+            }
+            if (act) {
+                if (I == k) {
+#pragma unroll
+                    for (int y = 0; y < G; ++y) {
+                        T r[G];
+                        ldv<T, G>(Rn + y * GLD3 + G * J, r);
+#pragma unroll
+                        for (int x = 0; x < G; ++x) V[y][x] = r[x];
+                    }
+                } else if (J == k) {
+#pragma unroll
+                    for (int x = 0; x < G; ++x) {
+                        T r[G];
+                        ldv<T, G>(Rn + x * GLD3 + G * I, r);
+#pragma unroll
+                        for (int y = 0; y < G; ++y) V[y][x] = r[y];
+                    }
+                } else if (I > k) {
+                    // V -= M_IK (P M_KJ), M_IK = R^T where I is not eliminated yet, else -R^T
+#pragma unroll
+                    for (int m = 0; m < G; ++m) {
+                        T a[G], r[G];
+                        ldv<T, G>(Rk + m * GLD3 + G * I, a);
+                        ldv<T, G>(Rn + m * GLD3 + G * J, r);
+#pragma unroll
+                        for (int y = 0; y < G; ++y)
+#pragma unroll
+                            for (int x = 0; x < G; ++x) V[y][x] -= a[y] * r[x];
+                    }
+                } else {
+#pragma unroll
+                    for (int m = 0; m < G; ++m) {
+                        T a[G], r[G];
+                        ldv<T, G>(Rk + m * GLD3 + G * I, a);
+                        ldv<T, G>(Rn + m * GLD3 + G * J, r);
+#pragma unroll
+                        for (int y = 0; y < G; ++y)
+#pragma unroll
+                            for (int x = 0; x < G; ++x) V[y][x] += a[y] * r[x];
+                    }
+                }
+                if (k + 1 < nb4) publish(k + 1);
+            }
+            __syncthreads();
+        }
+        // the inverse to global memory (both triangles) and its diagonal to dg
+        if (act) {
+            T* Fj = F + (size_t)j * plane_stride(b);
+#pragma unroll
+            for (int y = 0; y < G; ++y)
+                if (G * I + y < b) stv4(Fj + (size_t)(G * I + y) * ld + G * J, V[y][0], V[y][1], V[y][2], V[y][3]);
+            if (I != J) {
+#pragma unroll
+                for (int x = 0; x < G; ++x)
+                    if (G * J + x < b) stv4(Fj + (size_t)(G * J + x) * ld + G * I, V[0][x], V[1][x], V[2][x], V[3][x]);
+            } else {
+#pragma unroll
+                for (int y = 0; y < G; ++y) dg[G * I + y] = V[y][y];
+            }
+        }
+        __syncthreads();
+    }
+    // the solves read the factor through the bulk-copy (async) proxy, into
+    // shared memory this phase used
+    asm volatile("fence.proxy.async;" ::: "memory");
+    __syncthreads();
+}
+
+// 16-byte vectors of the shared-memory path
 template <typename T> struct V16;
 template <> struct V16<float> {
     using V = float4;
@@ -219,13 +516,10 @@ union VU {
     T a[V16<T>::W];
 };
 
-// leading dimension of the shared plane block: b padded to 4 entries
-__host__ __device__ __forceinline__ int plane_ld(int b) { return (b + 3) & ~3; }
-
 // In-place Gauss-Jordan inverse of an SPD b x b matrix in shared memory by
 // the whole CTA (row-major, leading dimension ld = plane_ld(b), padding
-// columns zero).  Each thread updates 16-byte groups of a row.  Pivot
-// reciprocals from the FP64 pivot.
+// columns zero), for planes wider than GB3.  Each thread updates 16-byte
+// groups of a row.
 template <typename T>
 __device__ void gj_cta(T* S, int b, int ld, T* rowbuf, T* colbuf, T* ipb, int* bad) {
     constexpr int W = V16<T>::W;
@@ -277,250 +571,371 @@ __device__ void gj_cta(T* S, int b, int ld, T* rowbuf, T* colbuf, T* ipb, int* b
     }
 }
 
-// Block LDL^T over planes; inverses of the plane Schur complements to F
-// (row stride b, plane stride plane_stride(b)).  Sb: ld = plane_ld(b).
+// The same factorisation for planes wider than GB3, the Schur block in shared
+// memory.  Sb: b x plane_ld(b).
 template <typename T>
-__device__ void factor3(const Box3& B, const Ops3& O, const T* c2s, T* F, T* Sb, T* rowbuf, T* colbuf, T* ipb,
-                        int* bad, bool mixed) {
+__device__ void factor3_smem(const Box3& B, const Ops3& O, const T* c2s, T* F, T* Sb, T* rowbuf, T* colbuf, T* ipb,
+                             int* bad) {
     const int b = B.b, ld = plane_ld(b), bb = b * b;
     const int tid = threadIdx.x, nt = blockDim.x;
-    const int i0 = tid / b, k0 = tid - i0 * b;
-    const int di = nt / b, dk = nt - di * b;
     const int n0 = B.n[B.a0];
     for (int t = tid; t < b * ld; t += nt) Sb[t] = T(0);   // padding columns stay zero
     __syncthreads();
     for (int j = 0; j < B.np; ++j) {
-        int i = i0, k = k0;
         for (int t = tid; t < bb; t += nt) {
+            const int i = t / b, k = t - i * b;
             const int ci = j * b + i, ck = j * b + k;
             const int sidx = i * ld + k;
-            const double si = mixed ? O.dsc[ci] : 1.0;
             if (i == k) {
-                double s = O.cd[ci] * si * si;
+                double s = O.cd[ci];
                 if (j > 0) {
                     const double cc = (double)c2s[ci - b];
                     s -= cc * (cc * (double)Sb[sidx]);   // not cc^2 (range at tiny couplings)
                 }
                 Sb[sidx] = (T)s;
             } else {
-                const double sk = mixed ? O.dsc[ck] : 1.0;
                 T s = T(0);
-                if (k == i + 1 && (O.nb[ci] & 2)) s = (T)(-O.c0[ci] * si * sk);
-                else if (k == i - 1 && (O.nb[ci] & 1)) s = (T)(-O.c0[ck] * si * sk);
-                else if (k == i + n0) s = (T)(-O.c1[ci] * si * sk);
-                else if (k == i - n0) s = (T)(-O.c1[ck] * si * sk);
+                if (k == i + 1) s -= (T)O.c0[ci];
+                if (k == i - 1) s -= (T)O.c0[ck];
+                if (k == i + n0) s -= (T)O.c1[ci];
+                if (k == i - n0) s -= (T)O.c1[ck];
                 if (j > 0) s -= c2s[ci - b] * Sb[sidx] * c2s[ck - b];
                 Sb[sidx] = s;
-            }
-            k += dk;
-            i += di;
-            if (k >= b) {
-                k -= b;
-                ++i;
             }
         }
         __syncthreads();
         gj_cta<T>(Sb, b, ld, rowbuf, colbuf, ipb, bad);
         T* Fj = F + (size_t)j * plane_stride(b);
-        {
-            int ii = i0, kk = k0;
-            for (int t = tid; t < bb; t += nt) {
-                Fj[t] = Sb[ii * ld + kk];
-                kk += dk;
-                ii += di;
-                if (kk >= b) {
-                    kk -= b;
-                    ++ii;
-                }
-            }
-        }
-        // the solves read the factor through the bulk-copy (async) proxy
-        asm volatile("fence.proxy.async.global;" ::: "memory");
+        for (int t = tid; t < b * ld; t += nt) Fj[t] = Sb[t];
         __syncthreads();
     }
+    asm volatile("fence.proxy.async;" ::: "memory");
+    __syncthreads();
 }
 
-// Two sweeps over the planes for nr right-hand sides in W ([nr][nc], block
-// order): on entry the scaled right-hand sides, on exit the scaled
-// solutions.  The plane inverses (symmetric, row-major, plane stride padded
-// to 16 bytes) stream from global memory through the bulk-copy (TMA) engine
-// in chunks of B.crows rows into two shared buffers: chunk s + 1 is in flight
-// while chunk s is used.  The sweep input of a plane is kept interleaved
-// (vb[c][4], all right-hand sides of a column in one 16-byte load).  For
-// b <= T3/2 the two halves of the CTA take the two halves of each chunk and
-// meet in red (which reuses vb once a plane is done); otherwise one thread
-// per row.  Returns false when a copy did
-// not complete in time (the CTA then stops using the buffers).
+// The sweeps' copies: stages of `cap` entries filled by bulk copies (full) and
+// handed back by the computing warps (empty).  Every thread tracks its own
+// position; waits are bounded.
 template <typename T>
-__device__ bool sweeps3(const Box3& B, const T* __restrict__ F, const T* __restrict__ c2s, T* W, T* vb, T* cbuf,
-                        T* red, uint64_t* bar, uint32_t* par, int nr) {
-    const int b = B.b, nc = B.nc;
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const size_t ps = plane_stride(b);
-    const int CRr = B.crows;
-    const int nch = (b + CRr - 1) / CRr;
-    const int nplane = 2 * B.np - 1;                  // forward planes, then backward planes np-2 .. 0
-    const int total = nplane * nch;
-    const size_t cap = stage_cap(CRr, b);              // entries per buffer
-    const bool split = b <= nt / 2;
-    const int r = split ? tid % (nt / 2) : tid;        // row of this thread (active if r < b)
-    const int hf = split ? tid / (nt / 2) : 0;         // half of each chunk
-    auto plane_of = [&](int p) { return p < B.np ? p : 2 * B.np - 2 - p; };
-    auto issue = [&](int st) {
-        const int j = plane_of(st / nch), ci = st % nch;
-        const int c0 = ci * CRr, cr = min(CRr, b - c0);
-        const uint32_t bytes = (uint32_t)((sizeof(T) * (size_t)cr * b + 15) & ~size_t(15));
-        T* dst = cbuf + (size_t)(st & 1) * cap;
-        mbar_expect_tx(&bar[st & 1], bytes);
-        bulk_g2s(dst, F + (size_t)j * ps + (size_t)c0 * b, bytes, &bar[st & 1]);
-    };
-    if (tid == 0) issue(0);
-    T acc[NR3];
-    bool ok = true;
-    for (int st = 0; st < total; ++st) {
-        const int p = st / nch, ci = st % nch, j = plane_of(p);
-        const bool fwd = p < B.np;
-        if (ci == 0) {
-            for (int c = tid; c < b; c += nt) {
-#pragma unroll
-                for (int q = 0; q < NR3; ++q) {
-                    T v = T(0);
-                    if (q < nr) {
-                        if (fwd) {
-                            v = W[q * nc + j * b + c];
-                            if (j > 0) v += c2s[(j - 1) * b + c] * W[q * nc + (j - 1) * b + c];
-                        } else {
-                            v = c2s[j * b + c] * W[q * nc + (j + 1) * b + c];
-                        }
-                    }
-                    vb[c * NR3 + q] = v;
-                }
-            }
-#pragma unroll
-            for (int q = 0; q < NR3; ++q) acc[q] = T(0);
+struct Pipe3 {
+    uint64_t *full, *empty;
+    T* buf;
+    size_t cap;
+    int st;            // stages
+    int slot;          // position of this thread
+    uint32_t ph;
+    uint32_t issued;   // copies issued (the issuing thread)
+    bool ok;           // no wait of this thread ran out
+    __device__ __forceinline__ void next() {
+        if (++slot == st) {
+            slot = 0;
+            ph ^= 1u;
         }
-        const bool done = mbar_wait(&bar[st & 1], par[st & 1]);
-        par[st & 1] ^= 1u;
-        if (__syncthreads_or(!done)) {
-            // the copy of step st is late: wait once more (bounded) so that no
-            // copy targets the buffer after the CTA stops using it
-            ok = false;
-            if (tid == 0) mbar_wait(&bar[st & 1], par[st & 1] ^ 1u);
-            break;
-        }
-        if (tid == 0 && st + 1 < total) issue(st + 1);
-        const T* S = cbuf + (size_t)(st & 1) * cap;
-        const int c0 = ci * CRr, cr = min(CRr, b - c0);
-        if (r < b) {
-            int ca = 0, cb = cr;
-            if (split) {
-                const int hc = (cr + 1) / 2;
-                ca = hf * hc;
-                cb = min(cr, ca + hc);
-            }
-            for (int c = ca; c < cb; ++c) {
-                const T sv = S[c * b + r];
-                const T* vq = vb + (size_t)(c0 + c) * NR3;
-                if (NR3 == 4 && std::is_same<T, float>::value) {
-                    const float4 v4 = *reinterpret_cast<const float4*>(vq);
-                    acc[0] += sv * (T)v4.x;
-                    acc[1] += sv * (T)v4.y;
-                    acc[2] += sv * (T)v4.z;
-                    acc[3] += sv * (T)v4.w;
-                } else {
-#pragma unroll
-                    for (int q = 0; q < NR3; ++q) acc[q] += sv * vq[q];
-                }
-            }
-        }
-        if (ci == nch - 1) {
-            if (split) {
-                __syncthreads();   // red shares memory with vb: every thread is done reading vb
-                if (hf == 1 && r < b)
-#pragma unroll
-                    for (int q = 0; q < NR3; ++q) red[r * NR3 + q] = acc[q];
-                __syncthreads();
-            }
-            if (hf == 0 && r < b) {
-#pragma unroll
-                for (int q = 0; q < NR3; ++q) {
-                    if (q >= nr) continue;
-                    const T v = split ? acc[q] + red[r * NR3 + q] : acc[q];
-                    if (fwd) W[q * nc + j * b + r] = v;
-                    else W[q * nc + j * b + r] += v;
-                }
-            }
-        }
-        __syncthreads();
     }
-    return ok;
+};
+
+// One poll, then the bounded wait.
+__device__ __forceinline__ bool wait3(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok || mbar_wait(bar, parity);
+}
+__device__ __forceinline__ void bar_consumers() { asm volatile("bar.sync 1, %0;" ::"n"(32 * NW3) : "memory"); }
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
-__device__ __forceinline__ void atomic_max_f(unsigned int* a, float v) { atomicMax(a, __float_as_uint(v)); }
+// Two sweeps over the planes for NR right-hand sides in W ([NR][nc], block
+// order): on entry the scaled right-hand sides, on exit the scaled solutions.
+// The plane inverses (symmetric, rows padded to 16 bytes) stream from global
+// memory through the bulk-copy (TMA) engine in chunks of stage_rows rows;
+// the last warp issues the copies, up to Pipe3::st chunks ahead of their use
+// and across planes, so that only the dependence of a plane on the one
+// before it is waited for.  The other NW3 warps form S v: a lane takes RW
+// consecutive rows (read as columns: consecutive lanes, consecutive words),
+// nrw warps cover the rows of a plane, and G groups of them take every G-th
+// column; the groups' partial sums meet in red, and the thread that adds
+// them writes the plane's result and its part of the next plane's input
+// (vb[c][q]).  Two barriers of the computing warps per plane.
+// RW: 4, 2 or 1 in FP32, so that a plane of up to 128, 64 or 32 cells is one
+// warp wide (one row per lane took 18 instructions per column and 5400 cycles
+// per plane of 126 cells, four rows a quarter of the instructions); 1 in FP64,
+// where the FMAs bind.
+// GC: the groups, where they are known at compile time (planes of up to 32 RW
+// cells), else 0.
+template <typename T, int NR, int RW, int GC>
+__device__ __forceinline__ void sweeps3_rw(const Box3& B, const T* c2s, T* W, T* vb, T* red, Pipe3<T>& pref, int* bad) {
+    Pipe3<T> pp = pref;   // in registers
+    constexpr int VS = NR == 3 ? 4 : NR;   // stride of vb
+    const int b = B.b, nc = B.nc, ld = plane_ld(b), np = B.np;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    constexpr int CR = stage_rows(sizeof(T));
+    const int nplane = 2 * np - 1;                    // forward planes, then backward planes np-2 .. 0
+    const int nrw = GC > 0 ? NW3 / GC : (b + 32 * RW - 1) / (32 * RW), G = GC > 0 ? GC : NW3 / nrw;
+    const int RP = nrw * 32 * RW;
+    const int g = warp / nrw, r0 = ((warp - g * nrw) * 32 + lane) * RW;
+    const bool act = g < G && r0 < b;
+    // the thread's result rows: row rs of right-hand sides qs, qs + qd, ...
+    const int rs = tid % RP, qs = tid / RP, qd = (32 * NW3) / RP;
+    const bool sum = rs < b && qs < qd;
+    if (sum)
+        for (int q = qs; q < NR; q += qd) vb[rs * VS + q] = W[q * nc + rs];
+    bar_consumers();
+    for (int p = 0; p < nplane; ++p) {
+        const int j = p < np ? p : 2 * np - 2 - p;
+        T acc[NR][RW];
+#pragma unroll
+        for (int q = 0; q < NR; ++q)
+#pragma unroll
+            for (int e = 0; e < RW; ++e) acc[q][e] = T(0);
+        for (int c0 = 0; c0 < b; c0 += CR) {
+            if (pp.ok && !wait3(&pp.full[pp.slot], pp.ph)) {
+                pp.ok = false;
+                *bad = 1;
+            }
+            if (act) {
+                const int cr = min(CR, b - c0);
+                const T* S = pp.buf + pp.slot * pp.cap + g * ld + r0;
+                const T* v0 = vb + (c0 + g) * VS;
+                const int sS = G * ld;
+                if (GC > 0 && cr == CR) {
+#pragma unroll
+                    for (int i = 0; i < (GC > 0 ? CR / GC : 1); ++i) {
+                        T sr[RW], v[VS];
+                        ldv<T, RW>(S + i * sS, sr);
+                        ldv<T, VS>(v0 + i * GC * VS, v);
+#pragma unroll
+                        for (int q = 0; q < NR; ++q)
+#pragma unroll
+                            for (int e = 0; e < RW; ++e) acc[q][e] += sr[e] * v[q];
+                    }
+                } else {
+                    const int sv = G * VS;
+#pragma unroll 4
+                    for (int c = g; c < cr; c += G) {
+                        T sr[RW], v[VS];
+                        ldv<T, RW>(S, sr);
+                        ldv<T, VS>(v0, v);
+                        S += sS;
+                        v0 += sv;
+#pragma unroll
+                        for (int q = 0; q < NR; ++q)
+#pragma unroll
+                            for (int e = 0; e < RW; ++e) acc[q][e] += sr[e] * v[q];
+                    }
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&pp.empty[pp.slot]);
+            pp.next();
+        }
+        if (act) {
+#pragma unroll
+            for (int q = 0; q < NR; ++q) {
+                T* d = red + (q * G + g) * RP + r0;
+                if constexpr (RW == 4) stv4(d, acc[q][0], acc[q][1], acc[q][2], acc[q][3]);
+                else {
+#pragma unroll
+                    for (int e = 0; e < RW; ++e) d[e] = acc[q][e];
+                }
+            }
+        }
+        bar_consumers();
+        if (sum)
+            for (int q = qs; q < NR; q += qd) {
+                const T* d = red + q * G * RP + rs;
+                T y0 = T(0), y1 = T(0);
+                int k = 0;
+#pragma unroll 4
+                for (; k + 1 < G; k += 2) {
+                    y0 += d[k * RP];
+                    y1 += d[(k + 1) * RP];
+                }
+                if (k < G) y0 += d[k * RP];
+                T y = y0 + y1;
+                T* w = W + q * nc + j * b + rs;
+                T v = T(0);
+                if (p < np) {
+                    w[0] = y;
+                    if (p + 1 < np) v = w[b] + c2s[j * b + rs] * y;
+                } else {
+                    y += w[0];
+                    w[0] = y;
+                }
+                if (p + 1 >= np && j > 0) v = c2s[(j - 1) * b + rs] * y;
+                vb[rs * VS + q] = v;
+            }
+        bar_consumers();
+    }
+    pref.slot = pp.slot;
+    pref.ph = pp.ph;
+    pref.ok = pp.ok;
+}
 
-// Solves A x_q = rhs_q for nr right-hand sides with the whole CTA: sweeps
+// issues the sweeps' copies (one lane of the last warp)
+template <typename T>
+__device__ void sweeps3_copies(const Box3& B, const T* __restrict__ F, Pipe3<T>& pref, int* bad) {
+    Pipe3<T> pp = pref;   // in registers
+    const int b = B.b, ld = plane_ld(b), np = B.np;
+    constexpr int CR = stage_rows(sizeof(T));
+    const size_t ps = plane_stride(b);
+    for (int p = 0; p < 2 * np - 1 && pp.ok; ++p) {
+        const T* Fj = F + (size_t)(p < np ? p : 2 * np - 2 - p) * ps;
+        for (int c0 = 0; c0 < b; c0 += CR) {
+            if (!wait3(&pp.empty[pp.slot], pp.ph ^ 1u)) {
+                pp.ok = false;
+                *bad = 1;
+                break;
+            }
+            const uint32_t bytes = (uint32_t)(sizeof(T) * (size_t)min(CR, b - c0) * ld);
+            mbar_expect_tx(&pp.full[pp.slot], bytes);
+            bulk_g2s(pp.buf + pp.slot * pp.cap, Fj + (size_t)c0 * ld, bytes, &pp.full[pp.slot]);
+            ++pp.issued;
+            pp.next();
+        }
+    }
+    pref = pp;
+}
+
+template <typename T, int NR>
+__device__ void sweeps3(const Box3& B, const T* __restrict__ F, const T* c2s, T* W, T* vb, T* red, Pipe3<T>& pp,
+                        int* bad) {
+    if (threadIdx.x >= 32 * NW3) {
+        if (threadIdx.x == 32 * NW3) sweeps3_copies<T>(B, F, pp, bad);
+        __syncwarp();
+    } else if constexpr (sizeof(T) == 8) {
+        sweeps3_rw<T, NR, 1, 0>(B, c2s, W, vb, red, pp, bad);
+    } else {
+        if (B.b <= 32) sweeps3_rw<T, NR, 1, NW3>(B, c2s, W, vb, red, pp, bad);
+        else if (B.b <= 64) sweeps3_rw<T, NR, 2, NW3>(B, c2s, W, vb, red, pp, bad);
+        else if (B.b <= 128) sweeps3_rw<T, NR, 4, NW3>(B, c2s, W, vb, red, pp, bad);
+        else sweeps3_rw<T, NR, 4, NW3 / 2>(B, c2s, W, vb, red, pp, bad);
+    }
+}
+
+__device__ __forceinline__ void warp_max_to(unsigned int* a, float v) {
+    for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(a, __float_as_uint(v));
+}
+
+// Solves A x_q = rhs_q for NR right-hand sides with the whole CTA: sweeps
 // with the kept factor (FP32 in the mixed form, FP64 in the FP64 form) and
-// refinement with FP64 residuals of the unscaled operator, the iterate X in
-// FP64.  High-contrast boxes reach a residual floor above what a fixed
-// tolerance can ask for, so the refinement runs to that floor: it stops when
-// every right-hand side has |r| <= 1e-3 ir_tol |b| (scaled max norms), or has
-// |r| <= ir_tol |b| and no longer halves its residual per step.  The FP64 form
-// (a direct solve, then refinement with the same rule, at most 4 sweep
-// pairs) never reports non-convergence.  Returns the number of sweep pairs.
-template <typename T, typename Rhs>
-__device__ int solve3(const Box3& B, const MemberDev& md, const double* Tfm, const Ops3& O, const T* F, const T* c2s,
-                      double* X, T* W, T* vb, T* cbuf, T* red, uint64_t* bar, uint32_t* par, unsigned int* nrm, int nr,
-                      const Rhs& rhs, double tol, int max_ir, int* noconv, int* bad) {
+// refinement with FP64 residuals, the iterate X in FP64 (mixed form: the
+// scaled x~ = D^-1 x until the end, rhs scaled).  warm (mixed form): X holds
+// a starting x~.  High-contrast boxes reach a residual floor above what a
+// fixed tolerance can ask for, so the refinement runs to that floor: it stops
+// when every right-hand side has |r| <= 1e-3 ir_tol |b| (scaled max norms),
+// or has |r| <= ir_tol |b| and no longer halves its residual per step.  The
+// FP64 form (a direct solve, then refinement with the same rule, at most 4
+// sweep pairs) never reports non-convergence.  Returns the number of sweep
+// pairs.
+template <typename T, int NR, typename Rhs>
+__device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, double* X, T* W, T* vb, T* red,
+                        Pipe3<T>& pp, unsigned int* nrm, const Rhs& rhs, double tol, int max_ir, int* noconv, int* bad,
+                        bool warm) {
     constexpr bool mixed = std::is_same<T, float>::value;
     const int nc = B.nc, tid = threadIdx.x, nt = blockDim.x;
-    if (*bad) return 0;   // a staged copy failed earlier: the buffers are not usable
+    const int s1 = B.n[B.a0], s2 = B.b;
     const int mit = mixed ? max_ir : 4;
-    if (tid < 3 * NR3) nrm[tid] = tid < NR3 ? 0u : 0x7f800000u;   // |b|, then |r| of the previous step (inf)
+    if (*bad) return 0;   // a staged copy failed earlier: the buffers are not usable
+    if (tid < 3 * NR3) nrm[tid] = tid < 2 * NR3 ? 0u : 0x7f800000u;   // |b|, |r|, |r| of the previous step (inf)
     __syncthreads();
-    for (int q = 0; q < nr; ++q)
+#pragma unroll
+    for (int q = 0; q < NR; ++q) {
+        float bn = 0.f, rn = 0.f;
         for (int t = tid; t < nc; t += nt) {
-            const double v = (mixed ? O.dsc[t] : 1.0) * rhs(q, t);
-            X[q * nc + t] = 0.0;
-            W[q * nc + t] = (T)v;
-            atomic_max_f(&nrm[q], fabsf((float)v));
+            const double v = rhs(q, t);
+            double r = v;
+            if (warm) r = resid3(O, s1, s2, X + q * nc, v, t);
+            else X[q * nc + t] = 0.0;
+            if constexpr (mixed) W[q * nc + t] = d2f_bits(r);
+            else W[q * nc + t] = r;
+            bn = fmaxf(bn, fabsf((float)v));
+            rn = fmaxf(rn, fabsf((float)r));
         }
+        warp_max_to(&nrm[q], bn);
+        warp_max_to(&nrm[NR3 + q], rn);
+    }
     __syncthreads();
-    int it = 0;
-    for (; it < mit; ++it) {
-        if (!sweeps3<T>(B, F, c2s, W, vb, cbuf, red, bar, par, nr)) {
-            if (threadIdx.x == 0) *bad = 1;
-            __syncthreads();
-            break;
-        }
-        for (int q = 0; q < nr; ++q)
-            for (int t = tid; t < nc; t += nt) X[q * nc + t] += (mixed ? O.dsc[t] : 1.0) * (double)W[q * nc + t];
-        if (tid < NR3) nrm[NR3 + tid] = 0u;
-        __syncthreads();
-        for (int q = 0; q < nr; ++q)
-            for (int t = tid; t < nc; t += nt) {
-                const double v = (mixed ? O.dsc[t] : 1.0) * (rhs(q, t) - applyA3g(B, md, Tfm, O.cd, O.nb, X + q * nc, t));
-                W[q * nc + t] = (T)v;
-                atomic_max_f(&nrm[NR3 + q], fabsf((float)v));
-            }
-        __syncthreads();
-        bool done = true, reached = true;
-        for (int q = 0; q < nr; ++q) {
+    // done: every residual at its floor; reached: every residual within tol
+    auto test = [&](bool& reached) {
+        bool done = true;
+        reached = true;
+        for (int q = 0; q < NR; ++q) {
             const double bn = (double)__uint_as_float(nrm[q]), rn = (double)__uint_as_float(nrm[NR3 + q]);
             const double rp = (double)__uint_as_float(nrm[2 * NR3 + q]);
-            const bool ok = bn == 0.0 || rn <= 1e-3 * tol * bn || (rn <= tol * bn && rn > 0.5 * rp);
-            if (!ok) done = false;
+            if (!(bn == 0.0 || rn <= 1e-3 * tol * bn || (rn <= tol * bn && rn > 0.5 * rp))) done = false;
             if (!(bn == 0.0 || rn <= tol * bn)) reached = false;
         }
+        return done;
+    };
+    bool reached = false;
+    int it = 0;
+    bool done = warm && test(reached);
+    if (warm) {
+        // a zero right-hand side has the zero solution, whatever the start
+        for (int q = 0; q < NR; ++q)
+            if (nrm[q] == 0u)
+                for (int t = tid; t < nc; t += nt) X[q * nc + t] = 0.0;
+    }
+    for (; !done && it < mit; ++it) {
+        sweeps3<T, NR>(B, F, c2s, W, vb, red, pp, bad);
         __syncthreads();
-        if (tid < NR3) nrm[2 * NR3 + tid] = nrm[NR3 + tid];
-        if (done) {
-            ++it;
-            break;
+        if (*bad) break;
+#pragma unroll
+        for (int q = 0; q < NR; ++q)
+            for (int t = tid; t < nc; t += nt) {
+                if constexpr (mixed) X[q * nc + t] += f2d_bits(W[q * nc + t]);
+                else X[q * nc + t] += W[q * nc + t];
+            }
+        if (tid < NR3) {
+            nrm[2 * NR3 + tid] = it == 0 && !warm ? 0x7f800000u : nrm[NR3 + tid];
+            nrm[NR3 + tid] = 0u;
         }
-        if (it == mit - 1 && !reached && tid == 0 && mixed) *noconv = 1;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < NR; ++q) {
+            float rn = 0.f;
+            for (int t = tid; t < nc; t += nt) {
+                const double v = resid3(O, s1, s2, X + q * nc, rhs(q, t), t);
+                if constexpr (mixed) {
+                    const float w = d2f_bits(v);
+                    W[q * nc + t] = w;
+                    rn = fmaxf(rn, fabsf(w));
+                } else {
+                    W[q * nc + t] = v;
+                    rn = fmaxf(rn, fabsf((float)v));
+                }
+            }
+            warp_max_to(&nrm[NR3 + q], rn);
+        }
+        __syncthreads();
+        done = test(reached);
+        if (!done && it == mit - 1 && !reached && tid == 0 && mixed) *noconv = 1;
+        __syncthreads();
+    }
+    if constexpr (mixed) {
+        // back from the scaled iterate
+        for (int q = 0; q < NR; ++q)
+            for (int t = tid; t < nc; t += nt) X[q * nc + t] *= O.dsc[t];
     }
     __syncthreads();
     return it;
+}
+
+template <typename T, typename Rhs>
+__device__ int solve3(int nr, const Box3& B, const Ops3& O, const T* F, const T* c2s, double* X, T* W, T* vb, T* red,
+                      Pipe3<T>& pp, unsigned int* nrm, const Rhs& rhs, double tol, int max_ir, int* noconv, int* bad) {
+    switch (nr) {   // the sweeps' work is that of the right-hand sides there are
+        case 1: return solve3_n<T, 1>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad, false);
+        case 2: return solve3_n<T, 2>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad, false);
+        case 3: return solve3_n<T, 3>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad, false);
+        default: return solve3_n<T, 4>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad, false);
+    }
 }
 
 // f |c| + Dirichlet / Neumann data + Robin data lam (may be null) of cell t
@@ -547,17 +962,18 @@ __device__ double source_rhs3(const Box3& B, const Ops3& O, const MemberDev& md,
 // problem on hat-Omega_i (a variant of Step 4), whose vector bs is stored.
 struct RhsBasis3 {
     const Box3* B;
-    const double* bT;
-    const double* bs;
-    int sk[NR3], mk[NR3];
+    const Ops3* O;
+    const double* bs;   // scaled in the mixed form
+    int sk[NR3], mk[NR3], bit[NR3];   // side, function, and the neighbour bit that cells of the side lack
     __device__ double operator()(int q, int t) const {
         if (sk[q] < 0) return bs[t];
-        const int sid = sk[q], a = sid >> 1;
+        if (O->nb[t] & bit[q]) return 0.0;
+        const int sid = sk[q];
         int c[3];
         bcoord(*B, t, c);
-        if (c[a] != ((sid & 1) ? B->n[a] - 1 : 0)) return 0.0;
         const int ts = B->ts[sid], tt = B->tt[sid];
-        return bT[B->soff[sid] + side_e(*B, sid, c)] * psi3(mk[q], c[ts], B->n[ts], c[tt], B->n[tt]);
+        const double v = O->bT[B->soff[sid] + side_e(*B, sid, c)] * psi3(mk[q], c[ts], B->n[ts], c[tt], B->n[tt]);
+        return O->dsc ? O->dsc[t] * v : v;
     }
 };
 
@@ -566,14 +982,13 @@ struct RhsStored3 {
     __device__ double operator()(int, int t) const { return b[t]; }
 };
 
-// Shared-memory layout.  Persistent: diagonal, neighbour bits, scaled plane
-// coupling, boundary faces, Robin data, stored right-hand side and (mixed
-// form) the FP32 work vectors W and the sweep input vb.  Overlaid: the
-// factor phase (the plane Schur block and, in the mixed form, the in-plane
-// couplings) and the solve phase (the streamed plane buffers; in the FP64
-// form also W and vb).  The FP64 iterates live in global scratch (one slot
-// per CTA).  The mixed form streams whole planes, the FP64 form 16-row
-// chunks.
+// Shared-memory layout.  Persistent: the operator, neighbour bits, scaled
+// plane coupling, boundary faces, and (smoothing) Robin data and (one right-
+// hand side) the stored right-hand side.  Overlaid: the factor phase (the
+// panels of the register inverses, or the plane Schur block where it is too
+// wide for them) and the solve phase (work vectors, sweep input, partial
+// sums and the stages of the streamed plane inverses, as many as fit, two at
+// least).  The FP64 iterates live in global scratch (one slot per CTA).
 __host__ __device__ inline void box3_dims(int nx, int ny, int nz, int* b, int* npl) {
     int n[3] = {nx, ny, nz};
     int a2 = 2;
@@ -583,28 +998,44 @@ __host__ __device__ inline void box3_dims(int nx, int ny, int nz, int* b, int* n
     *npl = n[a2];
 }
 
-__host__ __device__ inline size_t carve3_bytes(int tsz, int nx, int ny, int nz, bool stored_rhs) {
+// partial sums of the sweeps per right-hand side: G RP of sweeps3_rw
+__host__ __device__ inline size_t red3(int tsz, int b) {
+    const int rw = tsz == 8 || b <= 32 ? 1 : b <= 64 ? 2 : 4;
+    return (size_t)32 * NW3 * rw;
+}
+
+struct Lay3 {
+    size_t fixed;    // persistent bytes
+    size_t fac;      // factor phase
+    size_t work;     // solve phase without the stages
+    size_t stage;    // bytes of one stage
+    int st;          // stages
+    size_t total;
+};
+
+__host__ __device__ inline Lay3 lay3(int tsz, int nx, int ny, int nz, int nr, bool stored_rhs, bool robin) {
     int b, npl;
     box3_dims(nx, ny, nz, &b, &npl);
     const bool mixed = tsz == 4;
-    const size_t nc = (size_t)nx * ny * nz;
+    const size_t nc = (size_t)nx * ny * nz, ld = (size_t)plane_ld(b);
     const size_t per = 2 * ((size_t)nx * ny + (size_t)ny * nz + (size_t)nx * nz);
-    const size_t crw = (size_t)stream_rows(b, mixed);
-    size_t s = align16(sizeof(double) * nc);                                  // cd
-    if (mixed) s += align16(sizeof(double) * nc) + align16(tsz * nc);         // dsc c2s
-    else s += align16(sizeof(double) * nc) * 3;                               // c0 c1 c2
-    s += align16(nc);                                                          // nb
-    s += align16(sizeof(double) * per) * 3;                                    // bT bB lam
-    s += stored_rhs ? align16(sizeof(double) * nc) : 0;                       // bsrc
-    const size_t ld = (size_t)plane_ld(b);
-    size_t fac = (mixed ? align16(sizeof(double) * nc) * 3 : 0) + align16(tsz * (size_t)b * ld) +
-                 align16(tsz * ld) + align16(tsz * (size_t)b) + 16;
-    size_t sol = align16(tsz * 2 * stage_cap((int)crw, b));
-    if (mixed) s += align16(tsz * NR3 * nc) + align16(tsz * NR3 * (size_t)b);  // W vb persistent
-    else sol += align16(tsz * NR3 * nc) + align16(tsz * NR3 * (size_t)b);      // W vb in the solve overlay
-    s += fac > sol ? fac : sol;
-    s += align16(sizeof(double) * NR3 * 6 * 3 * 2) + 32 + 64 + 16;
-    return s + 64;
+    Lay3 L;
+    L.fixed = align16(sizeof(double) * nc) * 4;                               // cd c0 c1 c2
+    if (mixed) L.fixed += align16(sizeof(double) * nc) + align16(tsz * nc);   // dsc c2s
+    L.fixed += align16(nc);                                                    // nb
+    L.fixed += align16(sizeof(double) * per) * (robin ? 3 : 2);                // bT bB (lam)
+    if (stored_rhs) L.fixed += align16(sizeof(double) * nc);                   // bsrc
+    L.fac = b <= GB3 ? align16((size_t)tsz * (GJW3 + (mixed ? 2 * nc : 0)))
+                     : align16(tsz * b * ld) + align16(tsz * ld) + align16((size_t)tsz * b) + 16;
+    L.work = align16(tsz * nr * nc) + align16((size_t)tsz * NR3 * b) + align16((size_t)tsz * nr * red3(tsz, b));
+    const int rows = b < stage_rows(tsz) ? b : stage_rows(tsz);
+    L.stage = tsz * rows * ld;
+    const size_t tail = 64 + 32 + 2 * sizeof(uint64_t) * ST3;
+    L.st = ST3;
+    while (L.st > 2 && L.fixed + L.work + L.st * L.stage + tail > 227 * 1024) --L.st;
+    const size_t sol = L.work + L.st * L.stage;
+    L.total = L.fixed + (L.fac > sol ? L.fac : sol) + tail;
+    return L;
 }
 
 template <typename T>
@@ -613,72 +1044,82 @@ struct Carve3 {
     T* c2s;
     double* lam;
     double* bsrc;
-    T *Sb, *rowbuf, *colbuf, *ipb;   // factor phase
-    double* X;                       // solve phase (mixed: global scratch)
-    T *W, *vb, *cbuf, *red;
-    uint64_t* bar;
-    double* macc;
+    T* fac;                          // factor phase
+    double* X;                       // solve phase (global scratch)
+    T *W, *vb, *red;
+    Pipe3<T> pp;
     int* flags;
     unsigned int* nrm;
     size_t end;   // bytes of shared memory the layout takes
 };
 
 template <typename T>
-__device__ Carve3<T> carve3(unsigned char* base, const Box3& B, bool stored_rhs, double* xglobal) {
+__device__ Carve3<T> carve3(unsigned char* base, const Box3& B, int nr, bool stored_rhs, bool robin, double* xglobal) {
     constexpr bool mixed = std::is_same<T, float>::value;
     Carve3<T> C;
     const size_t nc = B.nc, b = B.b;
     const size_t per = B.soff[6];
+    const Lay3 L = lay3((int)sizeof(T), B.n[0], B.n[1], B.n[2], nr, stored_rhs, robin);
     size_t o = 0;
     auto take = [&](size_t bytes) { unsigned char* p = base + o; o += align16(bytes); return p; };
     C.O.cd = (double*)take(sizeof(double) * nc);
+    C.O.c0 = (double*)take(sizeof(double) * nc);
+    C.O.c1 = (double*)take(sizeof(double) * nc);
+    C.O.c2 = (double*)take(sizeof(double) * nc);
     if (mixed) {
         C.O.dsc = (double*)take(sizeof(double) * nc);
         C.c2s = (T*)take(sizeof(T) * nc);
     } else {
         C.O.dsc = nullptr;
-        C.O.c0 = (double*)take(sizeof(double) * nc);
-        C.O.c1 = (double*)take(sizeof(double) * nc);
-        C.O.c2 = (double*)take(sizeof(double) * nc);
         C.c2s = (T*)C.O.c2;
     }
     C.O.nb = (unsigned char*)take(nc);
     C.O.bT = (double*)take(sizeof(double) * per);
     C.O.bB = (double*)take(sizeof(double) * per);
-    C.lam = (double*)take(sizeof(double) * per);
+    C.lam = robin ? (double*)take(sizeof(double) * per) : nullptr;
     C.bsrc = stored_rhs ? (double*)take(sizeof(double) * nc) : nullptr;
-    if (mixed) {
-        C.W = (T*)take(sizeof(T) * NR3 * nc);
-        C.vb = (T*)take(sizeof(T) * NR3 * b);
-        C.X = xglobal;
-    }
+    C.X = xglobal;
     const size_t u0 = o;
-    if (mixed) {
-        C.O.c0 = (double*)take(sizeof(double) * nc);
-        C.O.c1 = (double*)take(sizeof(double) * nc);
-        C.O.c2 = (double*)take(sizeof(double) * nc);
-    }
-    const size_t ld = (size_t)plane_ld((int)b);
-    C.Sb = (T*)take(sizeof(T) * b * ld);
-    C.rowbuf = (T*)take(sizeof(T) * ld);
-    C.colbuf = (T*)take(sizeof(T) * b);
-    C.ipb = (T*)take(16);
-    const size_t u1 = o;
-    o = u0;
-    C.cbuf = (T*)take(sizeof(T) * 2 * stage_cap(B.crows, (int)b));
-    if (!mixed) {
-        C.W = (T*)take(sizeof(T) * NR3 * nc);
-        C.X = xglobal;
-        C.vb = (T*)take(sizeof(T) * NR3 * b);
-    }
-    if (o < u1) o = u1;
-    C.red = C.vb;   // the sweeps' partial sums reuse the sweep input (NR3 * b >= NR3 * rows)
-    C.macc = (double*)take(sizeof(double) * NR3 * 6 * 3 * 2);
+    C.fac = (T*)(base + u0);
+    C.W = (T*)take(sizeof(T) * nr * nc);
+    C.vb = (T*)take(sizeof(T) * NR3 * b);
+    C.red = (T*)take(sizeof(T) * nr * red3((int)sizeof(T), (int)b));
+    C.pp.buf = (T*)(base + o);
+    C.pp.cap = L.stage / sizeof(T);
+    C.pp.st = L.st;
+    C.pp.slot = 0;
+    C.pp.ph = 0u;
+    C.pp.issued = 0u;
+    C.pp.ok = true;
+    o += L.st * L.stage;
+    if (o < u0 + L.fac) o = u0 + L.fac;
     C.flags = (int*)take(32);
     C.nrm = (unsigned int*)take(64);
-    C.bar = (uint64_t*)take(16);
+    C.pp.full = (uint64_t*)take(sizeof(uint64_t) * ST3);
+    C.pp.empty = (uint64_t*)take(sizeof(uint64_t) * ST3);
     C.end = o;
+    if (threadIdx.x == 0) {
+        C.flags[0] = 0;
+        C.flags[1] = 0;
+        C.flags[2] = 0;
+        for (int s = 0; s < ST3; ++s) {
+            mbar_init(&C.pp.full[s], 1);
+            mbar_init(&C.pp.empty[s], NW3);
+        }
+    }
     return C;
+}
+
+// After a wait that ran out: no copy may target the shared memory of a CTA
+// that has left, so the issuing thread waits (bounded) for its last copy into
+// each stage.
+template <typename T>
+__device__ void drain3(Pipe3<T>& pp) {
+    if (threadIdx.x != 32 * NW3) return;
+    for (int s = 0; s < pp.st && s < (int)pp.issued; ++s) {
+        const uint32_t k = (pp.issued - 1 - s) / pp.st;   // rounds before the stage's last copy
+        mbar_wait(&pp.full[s], k & 1u);
+    }
 }
 
 }  // namespace
@@ -689,7 +1130,7 @@ __device__ Carve3<T> carve3(unsigned char* base, const Box3& B, bool stored_rhs,
 // with alpha_basis == alpha_smooth, or the Step 6 job), or scratch.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(T3) k_local3d(DevPtrs P, MethodDev Mth, const Job* jobs) {
+__global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, const Job* jobs) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool mixed = std::is_same<T, float>::value;
     const Job job = jobs[blockIdx.x];
@@ -700,32 +1141,45 @@ __global__ void __launch_bounds__(T3) k_local3d(DevPtrs P, MethodDev Mth, const 
         if (job.type == JOB_PART) setup_box3(B, md, sd.lo, sd.hi, Mth.alpha_b);
         else setup_box3(B, md, sd.loh, sd.hih, job.type == JOB_SFACT ? Mth.alpha_s : Mth.alpha_b);
     }
-    if (threadIdx.x == 0) B.crows = stream_rows(B.b, mixed);
     __syncthreads();
     const bool part = job.type == JOB_PART;
-    Carve3<T> C = carve3<T>(smem, B, part, P.xs + (size_t)blockIdx.x * P.xs_stride);
-    if (!mrcm_check(P.status, C.end <= mrcm_dyn_smem_bytes(), 6, (long long)C.end)) return;   // uniform
-    uint32_t par[2] = {0u, 0u};
-    if (threadIdx.x == 0) {
-        C.flags[0] = 0;
-        C.flags[1] = 0;
-        C.flags[2] = 0;
-        mbar_init(&C.bar[0], 1);
-        mbar_init(&C.bar[1], 1);
-    }
+    if (!mrcm_check(P.status,
+                    lay3((int)sizeof(T), B.n[0], B.n[1], B.n[2], part ? 1 : NR3, part, false).total <= mrcm_dyn_smem_bytes(),
+                    6, 0))
+        return;   // uniform
+    Carve3<T> C = carve3<T>(smem, B, part ? 1 : NR3, part, false, P.xs + (size_t)blockIdx.x * P.xs_stride);
     build_ops3(B, md, P, C.O, mixed);
-    if (mixed)
-        for (int t = threadIdx.x; t < B.nc; t += blockDim.x)
-            C.c2s[t] = (T)(C.O.c2[t] * C.O.dsc[t] * ((C.O.nb[t] & 32) ? C.O.dsc[t + B.b] : 0.0));
-    __syncthreads();
+    if constexpr (mixed) {
+        scale_ops3(B, C.O);
+        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.c2s[t] = (T)C.O.c2[t];
+        __syncthreads();
+    }
     T* F;
     if (part) F = (T*)P.fac_part + (size_t)job.item * P.part_stride;
     else if (job.type == JOB_SFACT || Mth.same_alpha) F = (T*)P.fac + (size_t)job.item * P.fac_stride;
     else F = (T*)P.fac_aux + (size_t)job.item * P.fac_stride;
-    factor3<T>(B, C.O, C.c2s, F, C.Sb, C.rowbuf, C.colbuf, C.ipb, &C.flags[0], mixed);
-    if (!part && (job.type == JOB_SFACT || Mth.same_alpha)) {
-        double* dd = P.dsc + (size_t)job.item * P.dsc_stride;
-        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) dd[t] = mixed ? C.O.dsc[t] : 1.0;
+    if (B.b <= GB3) {
+        const T *c0s, *c1s;
+        if constexpr (mixed) {
+            T* cs = C.fac + GJW3;   // in-plane couplings in T, in the factor phase's overlay
+            for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
+                cs[t] = d2f_bits(C.O.c0[t]);
+                cs[B.nc + t] = d2f_bits(C.O.c1[t]);
+            }
+            c0s = cs;
+            c1s = cs + B.nc;
+        } else {
+            c0s = C.O.c0;
+            c1s = C.O.c1;
+        }
+        factor3_reg<T>(B, C.O, c0s, c1s, C.c2s, F, C.fac, &C.flags[0]);
+    } else {
+        const size_t ld = plane_ld(B.b);
+        T* Sb = C.fac;
+        T* rowbuf = (T*)((unsigned char*)Sb + align16(sizeof(T) * B.b * ld));
+        T* colbuf = (T*)((unsigned char*)rowbuf + align16(sizeof(T) * ld));
+        T* ipb = (T*)((unsigned char*)colbuf + align16(sizeof(T) * B.b));
+        factor3_smem<T>(B, C.O, C.c2s, F, Sb, rowbuf, colbuf, ipb, &C.flags[0]);
     }
     if (C.flags[0] && threadIdx.x == 0) {
         atomicOr(&P.status[0], ST_NOT_SPD);
@@ -743,7 +1197,8 @@ __global__ void __launch_bounds__(T3) k_local3d(DevPtrs P, MethodDev Mth, const 
     double* bsg = hat_part ? P.bsrc + (size_t)job.item * P.dsc_stride : nullptr;
     if (part || hat_part) {
         double* bs = part ? C.bsrc : bsg;
-        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) bs[t] = source_rhs3(B, C.O, md, fm, nullptr, t);
+        for (int t = threadIdx.x; t < B.nc; t += blockDim.x)
+            bs[t] = (mixed ? C.O.dsc[t] : 1.0) * source_rhs3(B, C.O, md, fm, nullptr, t);
         __syncthreads();
     }
     int nI[3], off[3];
@@ -758,33 +1213,35 @@ __global__ void __launch_bounds__(T3) k_local3d(DevPtrs P, MethodDev Mth, const 
         int it;
         RhsBasis3 rb;
         rb.B = &B;
-        rb.bT = C.O.bT;
+        rb.O = &C.O;
         rb.bs = bsg;
         if (!part) {
-            for (int q = 0; q < nr; ++q) {
+#pragma unroll
+            for (int q = 0; q < NR3; ++q) {
                 const int k = k0 + q;
                 int qq = k / npsi;
                 rb.mk[q] = k % npsi;
                 rb.sk[q] = k >= sd.nbasis ? -1 : 0;
-                if (k >= sd.nbasis) continue;
-                for (int sid = 0; sid < 6; ++sid)
-                    if (sd.side_mask & (1 << sid)) {
-                        if (qq == 0) { rb.sk[q] = sid; break; }
-                        --qq;
-                    }
+                if (k < sd.nbasis)
+                    for (int sid = 0; sid < 6; ++sid)
+                        if (sd.side_mask & (1 << sid)) {
+                            if (qq == 0) { rb.sk[q] = sid; break; }
+                            --qq;
+                        }
+                const int a = rb.sk[q] >> 1;
+                rb.bit[q] = 1 << (2 * (a == B.a0 ? 0 : a == B.a1 ? 1 : 2) + (rb.sk[q] & 1));
             }
-            it = solve3<T>(B, md, P.Tf + md.cell_off * 3, C.O, F, C.c2s, C.X, C.W, C.vb, C.cbuf, C.red, C.bar, par, C.nrm, nr, rb, Mth.ir_tol,
-                           Mth.max_ir, &C.flags[1], &C.flags[2]);
+            it = solve3<T>(nr, B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rb, Mth.ir_tol, Mth.max_ir,
+                           &C.flags[1], &C.flags[2]);
         } else {
             RhsStored3 rs{C.bsrc};
-            it = solve3<T>(B, md, P.Tf + md.cell_off * 3, C.O, F, C.c2s, C.X, C.W, C.vb, C.cbuf, C.red, C.bar, par, C.nrm, nr, rs, Mth.ir_tol,
-                           Mth.max_ir, &C.flags[1], &C.flags[2]);
+            it = solve3_n<T, 1>(B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rs, Mth.ir_tol, Mth.max_ir,
+                                &C.flags[1], &C.flags[2], false);
         }
         maxit = max(maxit, it);
         nsolve += it * nr;
         __syncthreads();
         // ---- outputs: restriction to Omega_i, Gamma_i velocities and moments ----
-        for (int t = threadIdx.x; t < NR3 * 6 * 3 * 2; t += blockDim.x) C.macc[t] = 0.0;
         for (int q = 0; q < nr; ++q) {
             const double* x = C.X + (size_t)q * B.nc;
             const bool pq = part || k0 + q >= sd.nbasis;   // the particular problem
@@ -799,65 +1256,81 @@ __global__ void __launch_bounds__(T3) k_local3d(DevPtrs P, MethodDev Mth, const 
             }
         }
         __syncthreads();
-        for (int q = 0; q < nr; ++q) {
+        // one warp per right-hand side and side: velocities, and their moments by a warp reduction
+        for (int w = threadIdx.x >> 5; w < nr * 6; w += T3 / 32) {
+            const int q = w / 6, sid = w - 6 * (w / 6), lane = threadIdx.x & 31;
+            if (!(sd.side_mask & (1 << sid))) continue;
             const double* x = C.X + (size_t)q * B.nc;
             const int k = k0 + q;
             const bool pq = part || k >= sd.nbasis;
-            for (int sid = 0; sid < 6; ++sid) {
-                if (!(sd.side_mask & (1 << sid))) continue;
-                const int a = sid >> 1;
-                const int ts = B.ts[sid], tt = B.tt[sid];
-                const int ls = nI[ts], lt = nI[tt];
-                const double area = vol / md.h[a];
-                const double rarea = 1.0 / area;
-                double* ug = pq ? P.ubg + ((size_t)job.item * MRCM_MAXSIDE + sid) * P.side_max
-                                : P.Ug + (((size_t)job.item * P.nbasis_max + k) * MRCM_MAXSIDE + sid) * P.side_max;
-                for (int e = threadIdx.x; e < ls * lt; e += blockDim.x) {
-                    int c[3];
-                    c[a] = (sid & 1) ? off[a] + nI[a] - 1 : off[a];
-                    c[ts] = off[ts] + e % ls;
-                    c[tt] = off[tt] + e / ls;
-                    const int tL = bidx(B, c);
-                    const double pL = x[tL];
-                    const long long gL = gidx(B, md, c);
-                    const double hkL = P.hk[(md.cell_off + gL) * 3 + a];
-                    int cn[3] = {c[0], c[1], c[2]};
-                    cn[a] += (sid & 1) ? 1 : -1;
-                    const bool inner = cn[a] >= 0 && cn[a] < B.n[a];
-                    double uo, pi;
-                    if (inner) {
-                        const long long gf = (sid & 1) ? gL : gL - gstride(md, a);
-                        const double Tf = P.Tf[(md.cell_off + gf) * 3 + a];
-                        uo = Tf * (pL - x[bidx(B, cn)]) * rarea;
-                        pi = pL - uo * hkL;
-                    } else {
-                        const int eb = B.soff[sid] + side_e(B, sid, c);
-                        double lam = 0.0;
-                        if (!pq && sid == rb.sk[q])
-                            lam = psi3(rb.mk[q], c[ts], B.n[ts], c[tt], B.n[tt]);
-                        uo = C.O.bT[eb] * (pL - lam) * rarea;
-                        pi = part ? C.O.bB[eb] * uo : pL - uo * hkL;
+            int skq = -1, mkq = 0;
+            if (!pq) {
+#pragma unroll
+                for (int e = 0; e < NR3; ++e)
+                    if (e == q) {
+                        skq = rb.sk[e];
+                        mkq = rb.mk[e];
                     }
-                    ug[e] = uo;
-                    const int cs = e % ls, ct = e / ls;
-                    for (int m = 0; m < npsi; ++m) {
+            }
+            const int a = sid >> 1;
+            const int ts = B.ts[sid], tt = B.tt[sid];
+            const int ls = nI[ts], lt = nI[tt];
+            const double area = vol / md.h[a];
+            const double rarea = 1.0 / area;
+            double* ug = pq ? P.ubg + ((size_t)job.item * MRCM_MAXSIDE + sid) * P.side_max
+                            : P.Ug + (((size_t)job.item * P.nbasis_max + k) * MRCM_MAXSIDE + sid) * P.side_max;
+            double fmv[3] = {0.0, 0.0, 0.0}, pmv[3] = {0.0, 0.0, 0.0};
+            for (int e = lane; e < ls * lt; e += 32) {
+                const int cs = e % ls, ct = e / ls;
+                int c[3];
+                c[a] = (sid & 1) ? off[a] + nI[a] - 1 : off[a];
+                c[ts] = off[ts] + cs;
+                c[tt] = off[tt] + ct;
+                const double pL = x[bidx(B, c)];
+                const long long gL = gidx(B, md, c);
+                const double hkL = P.hk[(md.cell_off + gL) * 3 + a];
+                int cn[3] = {c[0], c[1], c[2]};
+                cn[a] += (sid & 1) ? 1 : -1;
+                const bool inner = cn[a] >= 0 && cn[a] < B.n[a];
+                double uo, pi;
+                if (inner) {
+                    const long long gf = (sid & 1) ? gL : gL - gstride(md, a);
+                    const double Tf = P.Tf[(md.cell_off + gf) * 3 + a];
+                    uo = Tf * (pL - x[bidx(B, cn)]) * rarea;
+                    pi = pL - uo * hkL;
+                } else {
+                    const int eb = B.soff[sid] + side_e(B, sid, c);
+                    const double lam = sid == skq ? psi3(mkq, c[ts], B.n[ts], c[tt], B.n[tt]) : 0.0;
+                    uo = C.O.bT[eb] * (pL - lam) * rarea;
+                    pi = part ? C.O.bB[eb] * uo : pL - uo * hkL;
+                }
+                ug[e] = uo;
+#pragma unroll
+                for (int m = 0; m < 3; ++m)
+                    if (m < npsi) {
                         const double ps = psi3(m, cs, ls, ct, lt);
-                        atomicAdd(&C.macc[((q * 6 + sid) * 3 + m) * 2 + 0], ps * uo * area);
-                        atomicAdd(&C.macc[((q * 6 + sid) * 3 + m) * 2 + 1], area * ps * pi);
+                        fmv[m] += ps * uo * area;
+                        pmv[m] += area * ps * pi;
+                    }
+            }
+            const int slot = pq ? P.nbasis_max : k;
+            double* mom = P.mom + (((size_t)job.item * (P.nbasis_max + 1) + slot) * MRCM_MAXSIDE + sid) * npsi * 2;
+#pragma unroll
+            for (int m = 0; m < 3; ++m)
+                if (m < npsi) {
+                    for (int o = 16; o; o >>= 1) {
+                        fmv[m] += __shfl_xor_sync(0xffffffffu, fmv[m], o);
+                        pmv[m] += __shfl_xor_sync(0xffffffffu, pmv[m], o);
+                    }
+                    if (lane == 0) {
+                        mom[m * 2] = fmv[m];
+                        mom[m * 2 + 1] = pmv[m];
                     }
                 }
-            }
-        }
-        __syncthreads();
-        for (int t = threadIdx.x; t < nr * 6 * npsi * 2; t += blockDim.x) {
-            const int w = t & 1, m = (t >> 1) % npsi, sid = ((t >> 1) / npsi) % 6, q = (t >> 1) / (npsi * 6);
-            if (!(sd.side_mask & (1 << sid))) continue;
-            const int slot = (part || k0 + q >= sd.nbasis) ? P.nbasis_max : k0 + q;
-            P.mom[((((size_t)job.item * (P.nbasis_max + 1) + slot) * MRCM_MAXSIDE + sid) * npsi + m) * 2 + w] =
-                C.macc[((q * 6 + sid) * 3 + m) * 2 + w];
         }
         __syncthreads();
     }
+    if (C.flags[2]) drain3(C.pp);
     if (threadIdx.x == 0) {
         atomicMax(&P.status[1], maxit);
         atomicAdd(&P.status[3], nsolve);
@@ -872,63 +1345,54 @@ __global__ void __launch_bounds__(T3) k_local3d(DevPtrs P, MethodDev Mth, const 
 // global memory.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(T3) k_smooth3d(DevPtrs P, MethodDev Mth, const int* items) {
+__global__ void __launch_bounds__(T3, 1) k_smooth3d(DevPtrs P, MethodDev Mth, const int* items) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool mixed = std::is_same<T, float>::value;
     const int item = items[blockIdx.x];
     const SubDev sd = P.sub[item];
     const MemberDev& md = P.mem[sd.member];
     __shared__ Box3 B;
-    if (threadIdx.x == 0) {
-        setup_box3(B, md, sd.loh, sd.hih, Mth.alpha_s);
-        B.crows = stream_rows(B.b, mixed);
-    }
+    if (threadIdx.x == 0) setup_box3(B, md, sd.loh, sd.hih, Mth.alpha_s);
     __syncthreads();
-    Carve3<T> C = carve3<T>(smem, B, true, P.xs + (size_t)blockIdx.x * P.xs_stride);
-    if (!mrcm_check(P.status, C.end <= mrcm_dyn_smem_bytes(), 6, (long long)C.end)) return;   // uniform
-    uint32_t par[2] = {0u, 0u};
-    if (threadIdx.x == 0) {
-        C.flags[0] = 0;
-        C.flags[1] = 0;
-        C.flags[2] = 0;
-        mbar_init(&C.bar[0], 1);
-        mbar_init(&C.bar[1], 1);
-    }
-    build_ops3(B, md, P, C.O, false);
-    const double* dd = P.dsc + (size_t)item * P.dsc_stride;
-    if (mixed) {
-        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.O.dsc[t] = dd[t];
-        __syncthreads();
-        for (int t = threadIdx.x; t < B.nc; t += blockDim.x)
-            C.c2s[t] = (T)(C.O.c2[t] * C.O.dsc[t] * ((C.O.nb[t] & 32) ? C.O.dsc[t + B.b] : 0.0));
+    if (!mrcm_check(P.status,
+                    lay3((int)sizeof(T), B.n[0], B.n[1], B.n[2], 1, true, true).total <= mrcm_dyn_smem_bytes(), 6, 0))
+        return;   // uniform
+    Carve3<T> C = carve3<T>(smem, B, 1, true, true, P.xs + (size_t)blockIdx.x * P.xs_stride);
+    // (the Jacobi scale comes out as in the factorisation: the same faces, the same arithmetic)
+    build_ops3(B, md, P, C.O, mixed);
+    if constexpr (mixed) {
+        scale_ops3(B, C.O);
+        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.c2s[t] = (T)C.O.c2[t];
     }
     // Robin data from the current solution: lambda = -beta u.n + pi (n outward of hat-Omega_i)
     const double* pst = P.p + md.cell_off;
     const double* ust = P.u + md.cell_off * 6;
-    for (int sid = 0; sid < 6; ++sid) {
+    for (int f = threadIdx.x; f < B.soff[6]; f += blockDim.x) {
+        const int sid = side_of(B, f), a = sid >> 1;
         if (B.kind[sid] != 2) continue;
-        const int a = sid >> 1;
-        const int ls = B.n[B.ts[sid]];
-        const int faces = B.soff[sid + 1] - B.soff[sid];
-        for (int e = threadIdx.x; e < faces; e += blockDim.x) {
-            int c[3];
-            c[a] = (sid & 1) ? B.n[a] - 1 : 0;
-            c[B.ts[sid]] = e % ls;
-            c[B.tt[sid]] = e / ls;
-            const long long g = gidx(B, md, c);
-            const double un = ust[g * 6 + sid];
-            const double pi = pst[g] - un * P.hk[(md.cell_off + g) * 3 + a];
-            C.lam[B.soff[sid] + e] = -C.O.bB[B.soff[sid] + e] * un + pi;
-        }
+        int c[3];
+        face_cell(B, sid, f, c);
+        const long long g = gidx(B, md, c);
+        const double un = ust[g * 6 + sid];
+        C.lam[f] = -C.O.bB[f] * un + (pst[g] - un * P.hk[(md.cell_off + g) * 3 + a]);
     }
     __syncthreads();
     const double* fm = P.f + md.cell_off;
-    for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.bsrc[t] = source_rhs3(B, C.O, md, fm, C.lam, t);
+    for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
+        C.bsrc[t] = (mixed ? C.O.dsc[t] : 1.0) * source_rhs3(B, C.O, md, fm, C.lam, t);
+        if constexpr (mixed) {
+            // the refinement starts from the current pressure, scaled (a start only: an FP32 reciprocal)
+            int c[3];
+            bcoord(B, t, c);
+            C.X[t] = pst[gidx(B, md, c)] * f2d_bits(__frcp_rn(d2f_bits(C.O.dsc[t])));
+        }
+    }
     __syncthreads();
     const T* F = (const T*)P.fac + (size_t)item * P.fac_stride;
     RhsStored3 rs{C.bsrc};
-    const int it = solve3<T>(B, md, P.Tf + md.cell_off * 3, C.O, F, C.c2s, C.X, C.W, C.vb, C.cbuf, C.red, C.bar, par, C.nrm, 1, rs, Mth.ir_tol,
-                             Mth.max_ir, &C.flags[0], &C.flags[2]);
+    const int it = solve3_n<T, 1>(B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rs, Mth.ir_tol, Mth.max_ir,
+                                  &C.flags[0], &C.flags[2], mixed);
+    if (C.flags[2]) drain3(C.pp);
     __syncthreads();
     // overwrite (u, p) on Omega_i with the restriction
     int nI[3], off[3];
@@ -1046,28 +1510,12 @@ __global__ void k_assemble3d(DevPtrs P, const double* __restrict__ X) {
 // host-side launch helpers
 // ---------------------------------------------------------------------------
 size_t local3d_smem(int prec, int nx, int ny, int nz, bool part) {
-    return carve3_bytes(prec == 0 ? 8 : 4, nx, ny, nz, part);
+    return lay3(prec == 0 ? 8 : 4, nx, ny, nz, part ? 1 : NR3, part, false).total;
 }
 
-size_t smooth3d_smem(int prec, int nx, int ny, int nz) { return carve3_bytes(prec == 0 ? 8 : 4, nx, ny, nz, true); }
+size_t smooth3d_smem(int prec, int nx, int ny, int nz) { return lay3(prec == 0 ? 8 : 4, nx, ny, nz, 1, true, true).total; }
 
-// entries of one box factor (n_a2 planes of b x b)
-// The bulk copies of the sweeps need 16-byte aligned sources, destinations
-// and sizes: plane strides, chunk offsets and staging capacities of a box.
-bool stage3_aligned(int prec, int nx, int ny, int nz) {
-    int b, npl;
-    box3_dims(nx, ny, nz, &b, &npl);
-    const size_t tsz = prec == 0 ? sizeof(double) : sizeof(float);
-    const int rows = stream_rows(b, prec != 0);
-    const size_t cap = stage_cap(rows, b);
-    const int nch = (b + rows - 1) / rows;
-    if ((plane_stride(b) * tsz) % 16 || (cap * tsz) % 16) return false;
-    if (nch > 1 && ((size_t)rows * b * tsz) % 16) return false;          // chunk starts
-    const size_t c0 = (size_t)(nch - 1) * rows;                            // last chunk
-    const size_t last = (((size_t)b - c0) * b * tsz + 15) & ~size_t(15);   // its rounded size
-    return last <= cap * tsz && c0 * b * tsz + last <= plane_stride(b) * tsz;
-}
-
+// entries of one box factor (n_a2 planes of b rows)
 size_t factor3_entries(int nx, int ny, int nz) {
     int b, npl;
     box3_dims(nx, ny, nz, &b, &npl);
