@@ -76,7 +76,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     const int per = 2 * (B.nx + B.ny);
     size_t o = 0;
     auto take = [&](size_t bytes) { unsigned char* p = smem + o; o += align16(bytes); return p; };
-    T* Sinv = (T*)take(sizeof(T) * sinv_len(B.nx, B.ny, sizeof(T)));
+    T* Sinv = (T*)take(sizeof(T) * sinv_len(B.nx, B.ny, sizeof(T), Mth.pad));
     Ops O;
     O.cd = (double*)take(sizeof(double) * n);
     O.cx = (double*)take(sizeof(double) * n);
@@ -87,7 +87,8 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     O.bB = (double*)take(sizeof(double) * per);
     double* lam = (double*)take(sizeof(double) * per);
     double* rt = (double*)take(sizeof(double) * n);
-    T* cys = (T*)take(sizeof(T) * n);
+    const int bp = line_width(B.nx, sizeof(T), Mth.pad);   // line stride of cys
+    T* cys = (T*)take(sizeof(T) * bp * B.ny);
     T* zbuf = (T*)take(sizeof(T) * 64);   // two line inputs of the twisted sweeps
     double* x = (double*)take(sizeof(double) * n);
     double* mu = (double*)take(sizeof(double) * n);
@@ -96,14 +97,14 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     int* flags = (int*)take(64);
 
     const T* Sg = (const T*)P.fac + (size_t)item * P.fac_stride;
-    for (size_t t = threadIdx.x; t < sinv_len(B.nx, B.ny, sizeof(T)); t += blockDim.x) Sinv[t] = Sg[t];
+    for (size_t t = threadIdx.x; t < sinv_len(B.nx, B.ny, sizeof(T), Mth.pad); t += blockDim.x) Sinv[t] = Sg[t];
     if (threadIdx.x == 0) flags[0] = 0;
     build_ops(B, md, P, O);
     const double* dd = P.dsc + (size_t)item * P.dsc_stride;
     for (int c = threadIdx.x; c < B.n; c += blockDim.x) O.dsc[c] = dd[c];
     __syncthreads();
     for (int c = threadIdx.x; c < B.n; c += blockDim.x)
-        cys[c] = (T)(O.cy[c] * O.dsc[c] * ((c + B.nx < B.n) ? O.dsc[c + B.nx] : 0.0));
+        cys[(c / B.nx) * bp + c % B.nx] = (T)(O.cy[c] * O.dsc[c] * ((c + B.nx < B.n) ? O.dsc[c + B.nx] : 0.0));
     const int nxg = md.n[0];
     const double* pst = A.ps + md.cell_off;
     const double* ust = A.us + md.cell_off * 4;
@@ -129,7 +130,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     __syncthreads();
     if (threadIdx.x < 32) {
         RhsStored rs{rt};
-        warp_solve<T>(B, O, Sinv, cys, x, mixed ? w : (T*)x, zbuf, rs, Mth.ir_tol, Mth.max_ir, &flags[0]);
+        warp_solve<T>(B, O, Sinv, cys, x, mixed ? w : (T*)x, zbuf, rs, Mth.ir_tol, Mth.max_ir, &flags[0], bp);
     }
     __syncthreads();
 
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     __syncthreads();
     if (threadIdx.x < 32) {
         RhsStored rs{rt};
-        warp_solve<T>(B, O, Sinv, cys, mu, mixed ? w : (T*)mu, zbuf, rs, Mth.ir_tol, Mth.max_ir, &flags[0]);
+        warp_solve<T>(B, O, Sinv, cys, mu, mixed ? w : (T*)mu, zbuf, rs, Mth.ir_tol, Mth.max_ir, &flags[0], bp);
     }
     __syncthreads();
 
@@ -364,7 +365,7 @@ __host__ __device__ inline size_t adj_carve_bytes(int nx, int ny, int nw, bool p
     const size_t per = 2 * (size_t)(nx + ny);
     size_t s = align16(sizeof(double) * n) * 4 + align16(sizeof(double) * 2 * n);   // cd cx cy dsc hk
     s += align16(sizeof(double) * per) * 3;                                           // bT bB gbT
-    s += align16(sizeof(T) * sinv_len(nx, ny, sizeof(T))) + align16(sizeof(T) * n) * 2;
+    s += align16(sizeof(T) * sinv_len(nx, ny, sizeof(T), 0)) + align16(sizeof(T) * n) * 2;
     s += align16(sizeof(T) * 64 * nw);
     s += part ? align16(sizeof(double) * n) : 0;
     s += align16(sizeof(double) * n) * 2;                                             // gcx gcy
@@ -400,7 +401,8 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
     O.bT = (double*)take(sizeof(double) * per);
     O.bB = (double*)take(sizeof(double) * per);
     double* gbT = (double*)take(sizeof(double) * per);
-    T* Sinv = (T*)take(sizeof(T) * sinv_len(B.nx, B.ny, sizeof(T)));
+    T* Sinv = (T*)take(sizeof(T) * sinv_len(B.nx, B.ny, sizeof(T), 0));
+    const int bp = B.nx;   // lines not widened (the factor is this kernel's own)
     T* cys = (T*)take(sizeof(T) * n);
     T* cxs = (T*)take(sizeof(T) * n);
     T* zall = (T*)take(sizeof(T) * 64 * nw);
@@ -455,14 +457,14 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
                     --q;
                 }
             RhsBasis rb{sk, mk};
-            warp_solve<T>(B, O, Sinv, cys, x, mixed ? wv : (T*)x, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1]);
+            warp_solve<T>(B, O, Sinv, cys, x, mixed ? wv : (T*)x, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1], bp);
         } else {
             double* bs = basis ? P.bsrc + (size_t)job.item * P.dsc_stride : bsrc;
             for (int c = lane; c < B.n; c += 32)
                 bs[c] = source_rhs(B, O, fm, nxg, vol, ax, ay, nullptr, c % B.nx, c / B.nx);
             __syncwarp();
             RhsStored rs{bs};
-            warp_solve<T>(B, O, Sinv, cys, x, mixed ? wv : (T*)x, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1]);
+            warp_solve<T>(B, O, Sinv, cys, x, mixed ? wv : (T*)x, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1], bp);
         }
         __syncwarp();
         // adjoint right-hand side
@@ -539,7 +541,7 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
             __syncwarp();
         }
         RhsStored rs{rt};
-        warp_solve<T>(B, O, Sinv, cys, mu, mixed ? wv : (T*)mu, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1]);
+        warp_solve<T>(B, O, Sinv, cys, mu, mixed ? wv : (T*)mu, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1], bp);
         __syncwarp();
         // -mu^T (dA/dc) x
         for (int c = lane; c < B.n; c += 32) {
@@ -644,14 +646,14 @@ __global__ void k_set_K(const double* src, double* K, long long n, int is_log, i
 // ---------------------------------------------------------------------------
 // host launchers
 // ---------------------------------------------------------------------------
-size_t adj_smooth2d_smem(int prec, int nx, int ny) {
+size_t adj_smooth2d_smem(int prec, int nx, int ny, int pad) {
     const size_t n = (size_t)nx * ny;
     const size_t per = 2 * (size_t)(nx + ny);
     const size_t tsz = prec == 0 ? sizeof(double) : sizeof(float);
-    size_t s = align16(tsz * sinv_len(nx, ny, (int)tsz));
+    size_t s = align16(tsz * sinv_len(nx, ny, (int)tsz, pad));
     s += align16(sizeof(double) * n) * 4 + align16(sizeof(double) * 2 * n);
     s += align16(sizeof(double) * per) * 3 + align16(sizeof(double) * n);
-    s += align16(tsz * n) + align16(tsz * 64) + align16(sizeof(double) * n) * 2;
+    s += align16(tsz * (size_t)line_width(nx, (int)tsz, pad) * ny) + align16(tsz * 64) + align16(sizeof(double) * n) * 2;
     if (prec != 0) s += align16(tsz * n);
     s += align16(sizeof(double) * 4 * n);
     return s + 64;

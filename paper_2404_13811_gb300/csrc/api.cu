@@ -21,10 +21,10 @@
 #include "mrcm_internal.cuh"
 
 // launchers defined in the other translation units
-size_t local2d_smem(int prec, int nx, int ny, int nrhs, bool part);
-size_t smooth2d_smem(int prec, int nx, int ny);
-size_t spack_bytes(int prec, int nx, int ny);
-int local2d_class(int prec, int nx);
+size_t local2d_smem(int prec, int nx, int ny, int nrhs, bool part, int pad);
+size_t smooth2d_smem(int prec, int nx, int ny, int pad);
+size_t spack_bytes(int prec, int nx, int ny, int pad);
+int local2d_class(int prec, int nx, int pad);
 cudaError_t launch_local2d(const DevPtrs& P, const MethodDev& M, const Job* jobs, int njobs, int bw,
                            size_t smem, cudaStream_t s);
 cudaError_t launch_smooth2d(const DevPtrs& P, const MethodDev& M, const int* items, int nitems,
@@ -70,7 +70,7 @@ cudaError_t if_residualT(const IfPtrs& I, const SubDev* sub, const int* col_item
 cudaError_t bcr_bwdT(const IfPtrs& I, const ElimDev* el, int nel, int nmax, int up, cudaStream_t s);
 cudaError_t bcr_fwdT(const IfPtrs& I, const ElimDev* el, int nel, int nmax, cudaStream_t s);
 cudaError_t if_updateT(const IfPtrs& I, double* y, int n, cudaStream_t s);
-size_t adj_smooth2d_smem(int prec, int nx, int ny);
+size_t adj_smooth2d_smem(int prec, int nx, int ny, int pad);
 size_t adj_local2d_smem(int prec, int nx, int ny, int nw, bool part);
 cudaError_t launch_adj_smooth2d(const DevPtrs& P, const MethodDev& M, const AdjPtrs& A, const int* items,
                                 int nitems, size_t smem, cudaStream_t s);
@@ -469,6 +469,22 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
     std::map<int, size_t> smem_w;
     size_t fac_stride = 0, dsc_stride = 0, part_stride = 0;
     const int nitems = (int)h->sub.size();
+    // 2D FP32 lines widened to a multiple of 4, unless some box then does not
+    // fit shared memory (tall boxes of a width that is no multiple of 4), be
+    // it in the forward kernels or in the adjoint's
+    h->mth.pad = prec != MRCM_FP64;
+    for (int s = 0; s < nitems && d == 2 && h->mth.pad; ++s) {
+        const SubDev& sd = h->sub[s];
+        const size_t lim = 227 * 1024;
+        const int bx = sd.hih[0] - sd.loh[0], by = sd.hih[1] - sd.loh[1];
+        const int ix = sd.hi[0] - sd.lo[0], iy = sd.hi[1] - sd.lo[1];
+        if (bx > 32) break;   // refused below
+        const int nb = std::max(std::min(sd.nbasis + (h->mth.part_hat ? 1 : 0), 4), 1);
+        if (local2d_smem(prec, bx, by, nb, false, 1) > lim || local2d_smem(prec, ix, iy, 1, true, 1) > lim ||
+            smooth2d_smem(prec, bx, by, 1) > lim || adj_smooth2d_smem(prec, bx, by, 1) > lim)
+            h->mth.pad = 0;
+    }
+    const int pad = h->mth.pad;
     for (int s = 0; s < nitems; ++s) {
         const SubDev& sd = h->sub[s];
         int bx = sd.hih[0] - sd.loh[0], by = sd.hih[1] - sd.loh[1], bz = sd.hih[2] - sd.loh[2];
@@ -494,21 +510,21 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
         }
         if (bx > 32 || ix > 32)
             return fail(h, MRCM_ERR_UNSUPPORTED, "2D boxes wider than 32 cells along x are not supported");
-        fac_stride = std::max(fac_stride, spack_bytes(prec, bx, by) / tsz);   // smoothing packs, 16-byte multiples
+        fac_stride = std::max(fac_stride, spack_bytes(prec, bx, by, pad) / tsz);   // smoothing packs, 16-byte multiples
         dsc_stride = std::max(dsc_stride, (size_t)bx * by);
         // with the particular problem on hat-Omega_i it is one more
         // right-hand side of the basis job (kept in global memory, so the
         // basis box needs no more shared memory)
         const bool hat = h->mth.part_hat;
         auto add = [&](int type, int nx, int ny, int nrhs, bool staged) {
-            const int bw = local2d_class(prec, nx);
+            const int bw = local2d_class(prec, nx, pad);
             byw[bw].push_back(Job{s, type});
-            smem_w[bw] = std::max(smem_w[bw], local2d_smem(prec, nx, ny, std::max(std::min(nrhs, 4), 1), staged));
+            smem_w[bw] = std::max(smem_w[bw], local2d_smem(prec, nx, ny, std::max(std::min(nrhs, 4), 1), staged, pad));
         };
         add(JOB_BASIS, bx, by, sd.nbasis + (hat ? 1 : 0), false);
         if (!hat) add(JOB_PART, ix, iy, 1, true);
         if (!h->mth.same_alpha) add(JOB_SFACT, bx, by, 0, false);
-        h->smooth_smem = std::max(h->smooth_smem, smooth2d_smem(prec, bx, by));
+        h->smooth_smem = std::max(h->smooth_smem, smooth2d_smem(prec, bx, by, pad));
     }
     if (h->smooth_smem > 227 * 1024) return fail(h, MRCM_ERR_UNSUPPORTED, "subdomain box too large for shared memory");
     std::vector<Job> jobs;
@@ -957,7 +973,7 @@ static int prepare_adjoint(mrcm_handle* h) {
             by[{bw, nw}].push_back(Job{s, type});
             smem[{bw, nw}] = std::max(smem[{bw, nw}], b);
         }
-        W.smooth_smem = std::max(W.smooth_smem, adj_smooth2d_smem(prec, sd.hih[0] - sd.loh[0], sd.hih[1] - sd.loh[1]));
+        W.smooth_smem = std::max(W.smooth_smem, adj_smooth2d_smem(prec, sd.hih[0] - sd.loh[0], sd.hih[1] - sd.loh[1], h->mth.pad));
     }
     if (W.smooth_smem > lim) return fail(h, MRCM_ERR_UNSUPPORTED, "subdomain box too large for the adjoint kernels");
     std::vector<Job> jobs;

@@ -210,25 +210,35 @@ __device__ __forceinline__ double resid_sc(const Box& B, const Ops& O, const dou
 // chain instead of nb).
 //
 // Storage: block j of lines of b cells at j b ld, row-major with row stride
-// ld = sld(b).  FP32 rows are read as float4 by one lane each; rows of b
-// floats with b / 4 even would put the rows of lanes i and i + 4 (or closer)
-// of an 8-lane phase in one bank group, so they are padded by four floats
-// (then ld / 4 is odd and the eight rows start in distinct groups).  FP64
-// blocks are read by column (no padding).
+// ld = sld(bp), bp the line width.  FP32 lines are widened to bp, the next
+// multiple of 4 (entries beyond b are zero, and so are the entries of a line's
+// input there), so that every row is read as float4 by one lane, at any b;
+// rows of bp floats with bp / 4 even would put the rows of lanes i and i + 4
+// (or closer) of an 8-lane phase in one bank group, so they are padded by four
+// floats (then ld / 4 is odd and the eight rows start in distinct groups).
+// The line couplings cys are kept with bp entries a line.  FP64 blocks are
+// read by column (no widening, no padding), as are FP32 ones of a handle whose
+// boxes would not fit shared memory with widened lines (pad = 0): one warp by
+// column takes about twice as long per sweep as two by row.
 // ---------------------------------------------------------------------------
-__host__ __device__ constexpr int sld_of(int b, int tsz) {
-    return (tsz == 4 && b % 4 == 0 && (b / 4) % 2 == 0) ? b + 4 : b;
+__host__ __device__ constexpr int sld_of(int bp, int tsz) {
+    return (tsz == 4 && bp % 4 == 0 && (bp / 4) % 2 == 0) ? bp + 4 : bp;
 }
 template <typename T>
-__host__ __device__ constexpr int sld(int b) { return sld_of(b, (int)sizeof(T)); }
-__host__ __device__ inline size_t sinv_len(int nx, int ny, int tsz) { return (size_t)ny * nx * sld_of(nx, tsz); }
+__host__ __device__ constexpr int sld(int bp) { return sld_of(bp, (int)sizeof(T)); }
+// line width of lines of b cells
+__host__ __device__ constexpr int line_width(int b, int tsz, int pad) { return tsz == 4 && pad ? (b + 3) & ~3 : b; }
+__host__ __device__ inline size_t sinv_len(int nx, int ny, int tsz, int pad) {
+    return (size_t)ny * nx * sld_of(line_width(nx, tsz, pad), tsz);
+}
 
 // In-register Gauss-Jordan inverse of an SPD b x b block (row i in lane i),
 // SPD so no pivoting.  The pivot row reaches every lane by shuffles from lane
 // k; the pivot lane and the other lanes update with selects (no divergent
 // paths), so a step is one chain of b shuffles and b FMAs.  Pivot
 // reciprocals: the correctly rounded FP32 reciprocal in the FP32 form, FP64
-// otherwise.  EX: b == BW (the width known at compile time).
+// otherwise.  EX: BW is the line width (lanes and entries beyond b hold the
+// identity); else b <= BW.
 template <typename T, int BW, bool EX>
 __device__ __forceinline__ void gj_regs(T (&a)[BW], int b, int* bad) {
     const int lane = threadIdx.x & 31;
@@ -282,16 +292,14 @@ __device__ __forceinline__ void gj_regs(T (&a)[BW], int b, int* bad) {
 template <typename T, int BW, bool EX, bool SC>
 __device__ __forceinline__ void form_line(T (&a)[BW], const Ops& O, const T* cys, const T* cxs, int b, int ld,
                                           int j, const T* up, const T* dn) {
-    if constexpr (EX) {
-        b = BW;
-        ld = sld<T>(BW);
-    }
+    if constexpr (EX) ld = sld<T>(BW);
+    const int cs = EX ? BW : b;   // line stride of cys
     const int i = threadIdx.x & 31;
     const bool act = i < b;
     const int ii = act ? i : 0;
     const int ci = j * b + ii;
-    const T cu = up ? cys[ci - b] : T(0);
-    const T cn = dn ? cys[ci] : T(0);
+    const T cu = up ? cys[(j - 1) * cs + ii] : T(0);
+    const T cn = dn ? cys[j * cs + ii] : T(0);
     // in-line couplings of cell i: to i + 1 and to i - 1
     const T xr = (act && ii < b - 1) ? cxs[ci] : T(0);
     const T xl = (act && ii > 0) ? cxs[ci - 1] : T(0);
@@ -316,13 +324,13 @@ __device__ __forceinline__ void form_line(T (&a)[BW], const Ops& O, const T* cys
         float4 ru[NQ], rd[NQ], ku[NQ], kd[NQ];
         if (up) {
             const float4* r = reinterpret_cast<const float4*>(up + ii * ld);
-            const float4* k = reinterpret_cast<const float4*>(cys + (j - 1) * b);
+            const float4* k = reinterpret_cast<const float4*>(cys + (j - 1) * BW);
 #pragma unroll
             for (int q = 0; q < NQ; ++q) { ru[q] = r[q]; ku[q] = k[q]; }
         }
         if (dn) {
             const float4* r = reinterpret_cast<const float4*>(dn + ii * ld);
-            const float4* k = reinterpret_cast<const float4*>(cys + j * b);
+            const float4* k = reinterpret_cast<const float4*>(cys + j * BW);
 #pragma unroll
             for (int q = 0; q < NQ; ++q) { rd[q] = r[q]; kd[q] = k[q]; }
         }
@@ -351,8 +359,8 @@ __device__ __forceinline__ void form_line(T (&a)[BW], const Ops& O, const T* cys
             if (act && (EX || c < b)) {
                 s = c == i + 1 ? xr : c == i - 1 ? xl : T(0);
                 // by column (consecutive lanes, consecutive words) where rows are not read as float4
-                if (up) s -= cu * up[c * ld + ii] * cys[(j - 1) * b + c];
-                if (dn) s -= cn * dn[c * ld + ii] * cys[j * b + c];
+                if (up) s -= cu * up[c * ld + ii] * cys[(j - 1) * cs + c];
+                if (dn) s -= cn * dn[c * ld + ii] * cys[j * cs + c];
             }
             a[c] = (act && (EX || c < b)) ? (c == i ? dT : s) : T(i == c ? 1 : 0);
         }
@@ -364,37 +372,38 @@ __device__ __forceinline__ void form_line(T (&a)[BW], const Ops& O, const T* cys
 // an SPD block is symmetric, so this is the block up to rounding.
 template <typename T, int BW, bool EX>
 __device__ __forceinline__ void store_line(const T (&a)[BW], T* S, int b, int ld) {
-    if constexpr (EX) {
-        b = BW;
-        ld = sld<T>(BW);
-    }
+    if constexpr (EX) ld = sld<T>(BW);
     const int i = threadIdx.x & 31;
-    if (i < b) {
+    if (i < (EX ? BW : b)) {   // (the identity's lanes store the zeros beyond b)
 #pragma unroll
         for (int c = 0; c < BW; ++c)
-            if (EX || c < b) S[c * ld + i] = a[c];
+            if (c < b) S[c * ld + i] = a[c];
     }
 }
 
 // Twisted block LDL^T factorisation: Sinv[j] as above.  cys / cxs: the scaled
 // line / in-line couplings (type T, formed once by all threads).  Warp 0
 // runs the top chain and then the middle line, warp 1 the bottom chain.
-// EX: the line width b equals BW.
+// EX: the line width is BW.
 template <typename T, int BW, bool EX, bool SC = false>
 __device__ void factor_box(const Box& B, const Ops& O, T* Sinv, T* cys, T* cxs, int* bad) {
-    const int b = EX ? BW : B.nx, nb = B.ny;
-    const int ld = sld<T>(b);
+    const int b = B.nx, nb = B.ny;
+    const int ld = sld<T>(EX ? BW : b);
     const size_t bl = (size_t)b * ld;
     const int tid = threadIdx.x, nt = blockDim.x;
+    const int cs = EX ? BW : b;   // line stride of cys
     for (int c = tid; c < B.n; c += nt) {
+        const int cj = c / b, ci = c - cj * b;
         if (SC) {   // the operator is scaled already (scale_ops)
-            cys[c] = (T)O.cy[c];
+            cys[cj * cs + ci] = (T)O.cy[c];
             cxs[c] = (T)(-O.cx[c]);
         } else {
-            cys[c] = (T)(O.cy[c] * O.dsc[c] * ((c + b < B.n) ? O.dsc[c + b] : 0.0));
-            cxs[c] = (T)(-O.cx[c] * O.dsc[c] * ((c % b) < b - 1 ? O.dsc[c + 1] : 0.0));
+            cys[cj * cs + ci] = (T)(O.cy[c] * O.dsc[c] * ((c + b < B.n) ? O.dsc[c + b] : 0.0));
+            cxs[c] = (T)(-O.cx[c] * O.dsc[c] * (ci < b - 1 ? O.dsc[c + 1] : 0.0));
         }
     }
+    if (EX && b < BW)
+        for (int t = tid; t < nb * (BW - b); t += nt) cys[(t / (BW - b)) * BW + b + t % (BW - b)] = T(0);
     __syncthreads();
     const int warp = tid >> 5;
     const int m = nb >> 1;
@@ -469,13 +478,13 @@ __device__ __forceinline__ T dot_col(const T* __restrict__ S, const T* z, int b,
 // Both twisted sweeps by one warp, the two chains interleaved step by step.
 // w: the scaled right-hand side in, the scaled solution out (line-major, b
 // per line); z: 64 entries (two line inputs), 16-byte aligned.  BB > 0: the
-// FP32 row path for lines of BB cells; BB = 0: the column path for any b.
+// FP32 row path for lines of width BB; BB = 0: the column path for any b.
 // Steps where both chains have a line run as one unit (both products in one
 // loop, so the loads and FMAs of the two chains overlap); the top chain has
 // at most one line more than the bottom one, run alone at the end.
 template <typename T, int BB>
 __device__ void tw_warp(const T* __restrict__ Sinv, const T* __restrict__ cys, T* w, T* z, int b, int nb) {
-    if constexpr (BB > 0) b = BB;
+    const int cs = BB > 0 ? BB : b;   // line stride of cys
     using Row = RowF<(BB > 0 ? BB : 4)>;
     const int ld = BB > 0 ? Row::LD : sld<T>(b);
     const int lane = threadIdx.x & 31;
@@ -519,10 +528,8 @@ __device__ void tw_warp(const T* __restrict__ Sinv, const T* __restrict__ cys, T
     Row Nt, Nb;
     auto fwd = [&](int s, Row& Ct, Row& Cb, Row& Xt, Row& Xb) {
         const int jt = s, jb = nb - 1 - s;
-        if (act) {
-            zt[lane] = w[jt * b + lane] + (jt > 0 ? cys[(jt - 1) * b + lane] * ct : T(0));
-            zb[lane] = w[jb * b + lane] + (s > 0 ? cys[jb * b + lane] * cb : T(0));
-        }
+        zt[lane] = act ? w[jt * b + lane] + (jt > 0 ? cys[(jt - 1) * cs + lane] * ct : T(0)) : T(0);
+        zb[lane] = act ? w[jb * b + lane] + (s > 0 ? cys[jb * cs + lane] * cb : T(0)) : T(0);
         __syncwarp();
         prod2(Ct, Cb, Sinv + jt * bl, Sinv + jb * bl, ct, cb, true);
         if constexpr (BB > 0) {
@@ -555,7 +562,7 @@ __device__ void tw_warp(const T* __restrict__ Sinv, const T* __restrict__ cys, T
     if (ntop > nbot) {   // the last top line, j = ntop - 1
         const int jt = ntop - 1;
         if constexpr (BB > 0) Lt.load((const float*)(Sinv + jt * bl), lane);
-        if (act) zt[lane] = w[jt * b + lane] + (jt > 0 ? cys[(jt - 1) * b + lane] * ct : T(0));
+        zt[lane] = act ? w[jt * b + lane] + (jt > 0 ? cys[(jt - 1) * cs + lane] * ct : T(0)) : T(0);
         __syncwarp();
         T dummy = T(0);
         prod2(Lt, Lb, Sinv + jt * bl, Sinv, ct, dummy, false);
@@ -565,12 +572,13 @@ __device__ void tw_warp(const T* __restrict__ Sinv, const T* __restrict__ cys, T
     // middle line
     {
         if constexpr (BB > 0) Lt.load((const float*)(Sinv + m * bl), lane);
+        T zm = T(0);
         if (act) {
-            T zm = w[m * b + lane];
-            if (m > 0) zm += cys[(m - 1) * b + lane] * ct;
-            if (m < nb - 1) zm += cys[m * b + lane] * cb;
-            zt[lane] = zm;
+            zm = w[m * b + lane];
+            if (m > 0) zm += cys[(m - 1) * cs + lane] * ct;
+            if (m < nb - 1) zm += cys[m * cs + lane] * cb;
         }
+        zt[lane] = zm;
         __syncwarp();
         T dummy = T(0);
         prod2(Lt, Lb, Sinv + m * bl, Sinv, ct, dummy, false);
@@ -583,9 +591,9 @@ __device__ void tw_warp(const T* __restrict__ Sinv, const T* __restrict__ cys, T
     auto bwd = [&](int s, Row& Ct, Row& Cb, Row& Xt, Row& Xb) {
         const int jt = m - 1 - s, jb = m + 1 + s;
         T wt = T(0), wb = T(0);
+        zt[lane] = act ? cys[jt * cs + lane] * ct : T(0);
+        zb[lane] = act ? cys[(jb - 1) * cs + lane] * cb : T(0);
         if (act) {
-            zt[lane] = cys[jt * b + lane] * ct;
-            zb[lane] = cys[(jb - 1) * b + lane] * cb;
             wt = w[jt * b + lane];
             wb = w[jb * b + lane];
         }
@@ -624,10 +632,8 @@ __device__ void tw_warp(const T* __restrict__ Sinv, const T* __restrict__ cys, T
     if (ntop > nbot) {   // the last top line, j = 0
         if constexpr (BB > 0) Lt.load((const float*)Sinv, lane);
         T wt = T(0);
-        if (act) {
-            zt[lane] = cys[lane] * ct;
-            wt = w[lane];
-        }
+        zt[lane] = act ? cys[lane] * ct : T(0);
+        if (act) wt = w[lane];
         __syncwarp();
         T pt, dummy = T(0);
         prod2(Lt, Lb, Sinv, Sinv, pt, dummy, false);
@@ -643,11 +649,11 @@ __device__ void tw_warp(const T* __restrict__ Sinv, const T* __restrict__ cys, T
 // refinement step.
 template <int BB>
 __device__ __noinline__ void tw_warp_f32(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w,
-                                         float* z, int nb) {
-    tw_warp<float, BB>(Sinv, cys, w, z, BB, nb);
+                                         float* z, int b, int nb) {
+    tw_warp<float, BB>(Sinv, cys, w, z, b, nb);
 }
 
-// Both twisted sweeps on two warps (FP32 row path, lines of BB cells): warp
+// Both twisted sweeps on two warps (FP32 row path, lines of width BB): warp
 // 0 runs the top chain (lines 0 .. m - 1) and warp 1 the bottom chain (lines
 // nb - 1 .. m + 1), each with its rows prefetched a line ahead; after a
 // barrier of the two warps (named barrier 1) warp 0 solves the middle line m
@@ -658,9 +664,9 @@ __device__ __noinline__ void tw_warp_f32(const float* __restrict__ Sinv, const f
 // differently).  Called by threads 0 .. 63; z: 64 entries (one line input per
 // warp).
 template <int BB>
-__device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w, float* z, int nb) {
+__device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w, float* z, int b,
+                         int nb) {
     using Row = RowF<BB>;
-    constexpr int b = BB;
     const int lane = threadIdx.x & 31, h = (threadIdx.x >> 5) & 1;
     const bool act = lane < b;
     const size_t bl = (size_t)b * Row::LD;
@@ -672,7 +678,7 @@ __device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict
     auto jf = [&](int s) { return h == 0 ? s : nb - 1 - s; };
     auto fwd = [&](int s, Row& C, Row& X) {
         const int j = jf(s);
-        if (act) zz[lane] = w[j * b + lane] + (s > 0 ? cys[(h == 0 ? j - 1 : j) * b + lane] * c : 0.f);
+        zz[lane] = act ? w[j * b + lane] + (s > 0 ? cys[(h == 0 ? j - 1 : j) * BB + lane] * c : 0.f) : 0.f;
         __syncwarp();
         if (s + 1 < cnt) X.load(Sinv + (size_t)jf(s + 1) * bl, lane);
         c = C.dot(zz);
@@ -692,12 +698,13 @@ __device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict
     if (h == 0) {
         Row L;
         L.load(Sinv + (size_t)m * bl, lane);
+        float zm = 0.f;
         if (act) {
-            float zm = w[m * b + lane];
-            if (m > 0) zm += cys[(m - 1) * b + lane] * w[(m - 1) * b + lane];
-            if (m < nb - 1) zm += cys[m * b + lane] * w[(m + 1) * b + lane];
-            zz[lane] = zm;
+            zm = w[m * b + lane];
+            if (m > 0) zm += cys[(m - 1) * BB + lane] * w[(m - 1) * b + lane];
+            if (m < nb - 1) zm += cys[m * BB + lane] * w[(m + 1) * b + lane];
         }
+        zz[lane] = zm;
         __syncwarp();
         const float r = L.dot(zz);
         if (act) w[m * b + lane] = r;
@@ -708,10 +715,8 @@ __device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict
     auto bwd = [&](int s, Row& C, Row& X) {
         const int j = jb(s);
         float wj = 0.f;
-        if (act) {
-            zz[lane] = cys[(h == 0 ? j : j - 1) * b + lane] * c;
-            wj = w[j * b + lane];
-        }
+        zz[lane] = act ? cys[(h == 0 ? j : j - 1) * BB + lane] * c : 0.f;
+        if (act) wj = w[j * b + lane];
         __syncwarp();
         if (s + 1 < cnt) X.load(Sinv + (size_t)jb(s + 1) * bl, lane);
         c = wj + C.dot(zz);
@@ -731,42 +736,45 @@ __device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict
 
 template <int BB>
 __device__ __noinline__ void tw_2warp_f32(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w,
-                                          float* z, int nb) {
-    tw_2warp<BB>(Sinv, cys, w, z, nb);
+                                          float* z, int b, int nb) {
+    tw_2warp<BB>(Sinv, cys, w, z, b, nb);
 }
 
 // The FP32 sweeps of one right-hand side by threads 0 .. 63: two warps on the
-// row path of the box's line width where there is one, else warp 0 alone by
+// row path of the line width bp where there is one, else warp 0 alone by
 // column.  zbuf: 64 entries.  The caller synchronises the block afterwards.
 __device__ void warp2_sweeps(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w, float* zbuf,
-                             int b, int nb) {
-    switch (b) {
-        case 8: tw_2warp_f32<8>(Sinv, cys, w, zbuf, nb); return;
-        case 12: tw_2warp_f32<12>(Sinv, cys, w, zbuf, nb); return;
-        case 16: tw_2warp_f32<16>(Sinv, cys, w, zbuf, nb); return;
-        case 20: tw_2warp_f32<20>(Sinv, cys, w, zbuf, nb); return;
-        case 24: tw_2warp_f32<24>(Sinv, cys, w, zbuf, nb); return;
-        case 28: tw_2warp_f32<28>(Sinv, cys, w, zbuf, nb); return;
-        case 32: tw_2warp_f32<32>(Sinv, cys, w, zbuf, nb); return;
+                             int b, int nb, int bp) {
+    switch (bp) {
+        case 4: tw_2warp_f32<4>(Sinv, cys, w, zbuf, b, nb); return;
+        case 8: tw_2warp_f32<8>(Sinv, cys, w, zbuf, b, nb); return;
+        case 12: tw_2warp_f32<12>(Sinv, cys, w, zbuf, b, nb); return;
+        case 16: tw_2warp_f32<16>(Sinv, cys, w, zbuf, b, nb); return;
+        case 20: tw_2warp_f32<20>(Sinv, cys, w, zbuf, b, nb); return;
+        case 24: tw_2warp_f32<24>(Sinv, cys, w, zbuf, b, nb); return;
+        case 28: tw_2warp_f32<28>(Sinv, cys, w, zbuf, b, nb); return;
+        case 32: tw_2warp_f32<32>(Sinv, cys, w, zbuf, b, nb); return;
         default: break;
     }
     if (threadIdx.x < 32) tw_warp<float, 0>(Sinv, cys, w, zbuf, b, nb);
 }
 
 // One warp solves in place (one right-hand side): the twisted sweeps, on the
-// FP32 row path of the box's line width where there is one, else by column.
+// FP32 row path of the line width bp where there is one, else by column.
 // zbuf: 64 entries of this warp.
 template <typename T>
-__device__ void warp_sweeps(const T* __restrict__ Sinv, const T* __restrict__ cys, T* w, T* zbuf, int b, int nb) {
+__device__ void warp_sweeps(const T* __restrict__ Sinv, const T* __restrict__ cys, T* w, T* zbuf, int b, int nb,
+                            int bp) {
     if constexpr (std::is_same<T, float>::value) {
-        switch (b) {
-            case 8: tw_warp_f32<8>(Sinv, cys, w, zbuf, nb); return;
-            case 12: tw_warp_f32<12>(Sinv, cys, w, zbuf, nb); return;
-            case 16: tw_warp_f32<16>(Sinv, cys, w, zbuf, nb); return;
-            case 20: tw_warp_f32<20>(Sinv, cys, w, zbuf, nb); return;
-            case 24: tw_warp_f32<24>(Sinv, cys, w, zbuf, nb); return;
-            case 28: tw_warp_f32<28>(Sinv, cys, w, zbuf, nb); return;
-            case 32: tw_warp_f32<32>(Sinv, cys, w, zbuf, nb); return;
+        switch (bp) {
+            case 4: tw_warp_f32<4>(Sinv, cys, w, zbuf, b, nb); return;
+            case 8: tw_warp_f32<8>(Sinv, cys, w, zbuf, b, nb); return;
+            case 12: tw_warp_f32<12>(Sinv, cys, w, zbuf, b, nb); return;
+            case 16: tw_warp_f32<16>(Sinv, cys, w, zbuf, b, nb); return;
+            case 20: tw_warp_f32<20>(Sinv, cys, w, zbuf, b, nb); return;
+            case 24: tw_warp_f32<24>(Sinv, cys, w, zbuf, b, nb); return;
+            case 28: tw_warp_f32<28>(Sinv, cys, w, zbuf, b, nb); return;
+            case 32: tw_warp_f32<32>(Sinv, cys, w, zbuf, b, nb); return;
             default: break;
         }
     }
@@ -816,16 +824,16 @@ __device__ double source_rhs(const Box& B, const Ops& O, const double* fm, int n
 // Solves A x = b for one right-hand side with one warp.  FP64 form: one
 // solve.  Mixed form: FP32 sweeps + FP64 residual refinement.  Returns the
 // number of sweeps (solves) performed.
-template <typename T, typename Rhs, int SW = 0>
+template <typename T, typename Rhs>
 __device__ int warp_solve(const Box& B, const Ops& O, const T* Sinv, const T* cys, double* x, T* w,
-                          T* zbuf, const Rhs& rhs, double tol, int max_ir, int* noconv) {
+                          T* zbuf, const Rhs& rhs, double tol, int max_ir, int* noconv, int bp) {
     const int lane = threadIdx.x & 31;
     const int b = B.nx, nb = B.ny;
     if (std::is_same<T, double>::value) {
         for (int j = 0; j < nb; ++j)
             for (int i = lane; i < b; i += 32) w[j * b + i] = (T)rhs(B, O, i, j);
         __syncwarp();
-        warp_sweeps<T>(Sinv, cys, w, zbuf, b, nb);
+        warp_sweeps<T>(Sinv, cys, w, zbuf, b, nb, bp);
         return 1;
     } else {
         float bn = 0.f;
@@ -841,8 +849,7 @@ __device__ int warp_solve(const Box& B, const Ops& O, const T* Sinv, const T* cy
         __syncwarp();
         int it = 0;
         for (; it < max_ir; ++it) {
-            if constexpr (SW > 0) tw_warp<float, SW>(Sinv, cys, w, zbuf, b, nb);
-            else warp_sweeps<T>(Sinv, cys, w, zbuf, b, nb);
+            warp_sweeps<T>(Sinv, cys, w, zbuf, b, nb, bp);
             for (int c = lane; c < B.n; c += 32) x[c] += O.dsc[c] * (double)w[c];
             __syncwarp();
             // FP64 residual of the unscaled operator; the (scaled) norms are taken in FP32
@@ -899,7 +906,7 @@ template <typename T>
 __device__ void cta_sweeps(const T* __restrict__ Sinv, const T* __restrict__ cys, T* w, T* zw, T* red, int b,
                            int nb) {
     if constexpr (std::is_same<T, float>::value) {
-        if (threadIdx.x < 32) warp_sweeps<float>(Sinv, cys, w, zw, b, nb);
+        if (threadIdx.x < 32) warp_sweeps<float>(Sinv, cys, w, zw, b, nb, b);
         __syncthreads();
         return;
     } else {
@@ -1037,16 +1044,11 @@ struct RhsScStored {
     __device__ double operator()(const Box& B, int i, int j) const { return b[j * B.nx + i]; }
 };
 
-// (i, j) of cell c; the line width is a compile-time constant when SW > 0.
-template <int SW>
-__device__ __forceinline__ void cell_ij(int c, int b, int& i, int& j) {
-    if constexpr (SW > 0) {
-        i = c % SW;
-        j = c / SW;
-    } else {
-        i = c % b;
-        j = c / b;
-    }
+// (i, j) of cell c of lines of b <= 32 cells, rb = 1.f / b: (c + 0.5) / b is
+// at least 1 / 64 away from an integer, far above the FP32 error for c < 2^16.
+__device__ __forceinline__ void cell_ij(int c, int b, float rb, int& i, int& j) {
+    j = (int)(((float)c + 0.5f) * rb);
+    i = c - j * b;
 }
 
 // One right-hand side by one warp in the mixed form: FP32 twisted sweeps of
@@ -1059,13 +1061,14 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
                              float* zbuf, const Rhs& rhs, double tol, int max_ir, int* noconv) {
     const int lane = threadIdx.x & 31;
     const int b = B.nx, nb = B.ny;
+    const float rb = 1.f / (float)b;
     const int nit = (B.n + 31) >> 5;
     float bn = 0.f;
     for (int k = 0; k < nit; ++k) {
         const int c = k * 32 + lane;
         const bool ok = c < B.n;
         int i, j;
-        cell_ij<SW>(ok ? c : 0, b, i, j);
+        cell_ij(ok ? c : 0, b, rb, i, j);
         const double bt = rhs(B, i, j);
         if (ok) {
             const float wc = d2f_bits(bt);
@@ -1079,7 +1082,7 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
     int it = 0;
     for (; it < max_ir; ++it) {
         if constexpr (SW > 0) tw_warp<float, SW>(Sinv, cys, w, zbuf, b, nb);
-        else warp_sweeps<float>(Sinv, cys, w, zbuf, b, nb);
+        else tw_warp<float, 0>(Sinv, cys, w, zbuf, b, nb);
         for (int c = lane; c < B.n; c += 32) x[c] += f2d_bits(w[c]);
         __syncwarp();
         float rn = 0.f;
@@ -1087,7 +1090,7 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
             const int c = k * 32 + lane;
             const bool ok = c < B.n;
             int i, j;
-            cell_ij<SW>(ok ? c : 0, b, i, j);
+            cell_ij(ok ? c : 0, b, rb, i, j);
             const double bt = rhs(B, i, j);
             if (ok) {
                 const float wc = d2f_bits(resid_sc(B, O, x, bt, c, i, j));
@@ -1109,14 +1112,16 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
 // still relative to b~; no sweep when the start meets it).  b~ is stored.
 __device__ int cta_solve_sc(const Box& B, const Ops& O, const float* Sinv, const float* cys, double* x, float* w,
                             float* zw, unsigned int* nrm, const double* bt, double tol, int max_ir, int* noconv,
-                            bool warm) {
+                            bool warm, int bp) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int b = B.nx, nb = B.ny;
+    const float rb = 1.f / (float)b;
     if (tid < 2) nrm[tid] = 0u;
     __syncthreads();
     float bn = 0.f, r0 = 0.f;
     for (int c = tid; c < B.n; c += nt) {
-        const int i = c % b, j = c / b;
+        int i, j;
+        cell_ij(c, b, rb, i, j);
         const float wb = d2f_bits(bt[c]);
         const float wc = warm ? d2f_bits(resid_sc(B, O, x, bt[c], c, i, j)) : wb;
         w[c] = wc;
@@ -1140,14 +1145,15 @@ __device__ int cta_solve_sc(const Box& B, const Ops& O, const float* Sinv, const
     int it = 0;
     if (warm && ((double)r0 <= tol * (double)bn || bn == 0.f)) return 0;
     for (; it < max_ir; ++it) {
-        if (tid < 64) warp2_sweeps(Sinv, cys, w, zw, b, nb);
+        if (tid < 64) warp2_sweeps(Sinv, cys, w, zw, b, nb, bp);
         __syncthreads();
         for (int c = tid; c < B.n; c += nt) x[c] += f2d_bits(w[c]);
         if (tid == 0) nrm[1] = 0u;
         __syncthreads();
         float rn = 0.f;
         for (int c = tid; c < B.n; c += nt) {
-            const int i = c % b, j = c / b;
+            int i, j;
+            cell_ij(c, b, rb, i, j);
             const float wc = d2f_bits(resid_sc(B, O, x, bt[c], c, i, j));
             w[c] = wc;
             rn = fmaxf(rn, fabsf(wc));
@@ -1179,10 +1185,10 @@ struct SPack {
     size_t cd, cx, cy, dsc, bT, bB, bst, cys, bytes;
 };
 
-__host__ __device__ inline SPack spack_layout(int nx, int ny, size_t tsz) {
+__host__ __device__ inline SPack spack_layout(int nx, int ny, size_t tsz, int pad) {
     SPack L;
     const size_t n = (size_t)nx * ny, m = 2 * (size_t)(nx + ny);
-    size_t o = align16(tsz * sinv_len(nx, ny, (int)tsz));
+    size_t o = align16(tsz * sinv_len(nx, ny, (int)tsz, pad));
     L.cd = o;  o += align16(sizeof(double) * n);
     L.cx = o;  o += align16(sizeof(double) * n);
     L.cy = o;  o += align16(sizeof(double) * n);
@@ -1190,7 +1196,7 @@ __host__ __device__ inline SPack spack_layout(int nx, int ny, size_t tsz) {
     L.bT = o;  o += align16(sizeof(double) * m);
     L.bB = o;  o += align16(sizeof(double) * m);
     L.bst = o; o += align16(sizeof(double) * n);
-    L.cys = o; o += align16(tsz * n);
+    L.cys = o; o += align16(tsz * (size_t)line_width(nx, (int)tsz, pad) * ny);
     L.bytes = o;
     return L;
 }
@@ -1215,11 +1221,12 @@ template <typename T>
 // values it needs at the Gamma faces from global memory -- and a stored
 // right-hand side only for the particular problem, so that two CTAs of the
 // 24 x 24 basis boxes fit on one SM)
-__host__ __device__ inline size_t carve_bytes(int nx, int ny, int nrhs, bool part) {
+__host__ __device__ inline size_t carve_bytes(int nx, int ny, int nrhs, bool part, int pad) {
     const size_t n = (size_t)nx * ny;
     size_t s = align16(sizeof(double) * n) * 4;                                      // cd cx cy dsc
     s += align16(sizeof(double) * 2 * (nx + ny)) * 2;                                 // bT bB
-    s += align16(sizeof(T) * sinv_len(nx, ny, sizeof(T))) + align16(sizeof(T) * n);   // Sinv, cys (cxs lives in W)
+    s += align16(sizeof(T) * sinv_len(nx, ny, sizeof(T), pad)) +
+         align16(sizeof(T) * line_width(nx, sizeof(T), pad) * ny);                     // Sinv, cys (cxs lives in W)
     s += align16(sizeof(T) * 64 * NWARP) + (part ? align16(sizeof(double) * n) : 0);
     if (std::is_same<T, float>::value) s += align16(sizeof(double) * n * nrhs);
     s += align16(sizeof(T) * n * nrhs);
@@ -1227,7 +1234,7 @@ __host__ __device__ inline size_t carve_bytes(int nx, int ny, int nrhs, bool par
 }
 
 template <typename T>
-__device__ Carve<T> carve(unsigned char* base, int nx, int ny, int nrhs, bool part) {
+__device__ Carve<T> carve(unsigned char* base, int nx, int ny, int nrhs, bool part, int pad) {
     Carve<T> C;
     const size_t n = (size_t)nx * ny;
     size_t o = 0;
@@ -1239,8 +1246,8 @@ __device__ Carve<T> carve(unsigned char* base, int nx, int ny, int nrhs, bool pa
     C.O.hk = nullptr;
     C.O.bT = (double*)take(sizeof(double) * 2 * (nx + ny));
     C.O.bB = (double*)take(sizeof(double) * 2 * (nx + ny));
-    C.Sinv = (T*)take(sizeof(T) * sinv_len(nx, ny, sizeof(T)));
-    C.cys = (T*)take(sizeof(T) * n);
+    C.Sinv = (T*)take(sizeof(T) * sinv_len(nx, ny, sizeof(T), pad));
+    C.cys = (T*)take(sizeof(T) * line_width(nx, sizeof(T), pad) * ny);
     C.zbuf = (T*)take(sizeof(T) * 64 * NWARP);
     C.bsrc = part ? (double*)take(sizeof(double) * n) : nullptr;
     if (std::is_same<T, float>::value) C.X = (double*)take(sizeof(double) * n * nrhs);

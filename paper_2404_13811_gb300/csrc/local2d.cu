@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
     // global memory (the basis box has no shared memory left for it)
     const bool hat_part = job.type == JOB_BASIS && Mth.part_hat;
     const int nrhs = job.type == JOB_BASIS ? sd.nbasis + (hat_part ? 1 : 0) : (job.type == JOB_PART ? 1 : 0);
-    Carve<T> C = carve<T>(smem, B.nx, B.ny, nrhs > 0 ? min(nrhs, NWARP) : 1, job.type == JOB_PART);
+    Carve<T> C = carve<T>(smem, B.nx, B.ny, nrhs > 0 ? min(nrhs, NWARP) : 1, job.type == JOB_PART, Mth.pad);
     if (!mrcm_check(P.status, C.end <= mrcm_dyn_smem_bytes(), 1, (long long)C.end)) return;   // uniform
     if (threadIdx.x == 0) { C.flags[0] = 0; C.flags[1] = 0; }
     build_ops(B, md, P, C.O);
@@ -58,9 +58,9 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
     const bool keep = (job.type == JOB_SFACT) || (job.type == JOB_BASIS && Mth.same_alpha);
     if (keep) {
         unsigned char* pk = (unsigned char*)((T*)P.fac + (size_t)job.item * P.fac_stride);
-        const SPack L = spack_layout(B.nx, B.ny, sizeof(T));
+        const SPack L = spack_layout(B.nx, B.ny, sizeof(T), Mth.pad);
         T* dst = (T*)pk;
-        const size_t nS = sinv_len(B.nx, B.ny, sizeof(T));
+        const size_t nS = sinv_len(B.nx, B.ny, sizeof(T), Mth.pad);
         for (size_t t = threadIdx.x; t < nS; t += blockDim.x) dst[t] = C.Sinv[t];
         double* dd = P.dsc + (size_t)job.item * P.dsc_stride;
         const double* fk = P.f + md.cell_off;
@@ -73,8 +73,9 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
             ((double*)(pk + L.dsc))[c] = C.O.dsc[c];
             ((double*)(pk + L.bst))[c] =
                 C.O.dsc[c] * source_rhs(B, C.O, fk, md.n[0], vk, md.h[1], md.h[0], nullptr, c % B.nx, c / B.nx);
-            ((T*)(pk + L.cys))[c] = C.cys[c];
         }
+        for (int t = threadIdx.x; t < line_width(B.nx, sizeof(T), Mth.pad) * B.ny; t += blockDim.x)
+            ((T*)(pk + L.cys))[t] = C.cys[t];
         for (int t = threadIdx.x; t < 2 * (B.nx + B.ny); t += blockDim.x) {
             ((double*)(pk + L.bT))[t] = C.O.bT[t];
             ((double*)(pk + L.bB))[t] = C.O.bB[t];
@@ -126,7 +127,7 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
             } else {
                 RhsBasis rb{sk, mk};
                 it = warp_solve<T, RhsBasis>(B, C.O, C.Sinv, C.cys, x, w, zb, rb, Mth.ir_tol, Mth.max_ir,
-                                             &C.flags[1]);
+                                             &C.flags[1], B.nx);
             }
         } else {
             // the particular problem: fixed right-hand side staged once (b~ in the mixed form)
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
             } else {
                 RhsStored rs{bs};
                 it = warp_solve<T, RhsStored>(B, C.O, C.Sinv, C.cys, x, w, zb, rs, Mth.ir_tol, Mth.max_ir,
-                                              &C.flags[1]);
+                                              &C.flags[1], B.nx);
             }
         }
         if constexpr (mixed) {
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
     __syncthreads();
     const size_t n = (size_t)B.n;
     // the smoothing pack (factor, operator, fixed right-hand side) first, by one bulk copy
-    const SPack L = spack_layout(B.nx, B.ny, sizeof(T));
+    const SPack L = spack_layout(B.nx, B.ny, sizeof(T), Mth.pad);
     T* Sinv = (T*)smem;
     Ops O;
     O.cd = (double*)(smem + L.cd);
@@ -369,7 +370,7 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
                 x[c] *= f2d_bits(__frcp_rn(d2f_bits(O.dsc[c])));
             __syncthreads();
             it = cta_solve_sc(B, O, (const float*)Sinv, (const float*)cys, x, (float*)w, (float*)zbuf, nrm, bsrc,
-                              Mth.ir_tol, Mth.max_ir, &flags[0], true);
+                              Mth.ir_tol, Mth.max_ir, &flags[0], true, line_width(B.nx, sizeof(T), Mth.pad));
             for (int c = threadIdx.x; c < B.n; c += blockDim.x) x[c] *= O.dsc[c];
             __syncthreads();
         } else {
@@ -441,18 +442,18 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
 // ---------------------------------------------------------------------------
 // host-side launch helpers
 // ---------------------------------------------------------------------------
-size_t local2d_smem(int prec, int nx, int ny, int nrhs, bool part) {
-    return prec == 0 ? carve_bytes<double>(nx, ny, nrhs, part) : carve_bytes<float>(nx, ny, nrhs, part);
+size_t local2d_smem(int prec, int nx, int ny, int nrhs, bool part, int pad) {
+    return prec == 0 ? carve_bytes<double>(nx, ny, nrhs, part, pad) : carve_bytes<float>(nx, ny, nrhs, part, pad);
 }
 
-size_t spack_bytes(int prec, int nx, int ny) {
-    return spack_layout(nx, ny, prec == 0 ? sizeof(double) : sizeof(float)).bytes;
+size_t spack_bytes(int prec, int nx, int ny, int pad) {
+    return spack_layout(nx, ny, prec == 0 ? sizeof(double) : sizeof(float), pad).bytes;
 }
 
-size_t smooth2d_smem(int prec, int nx, int ny) {
+size_t smooth2d_smem(int prec, int nx, int ny, int pad) {
     const size_t n = (size_t)nx * ny;
     const size_t tsz = prec == 0 ? sizeof(double) : sizeof(float);
-    size_t s = spack_bytes(prec, nx, ny);
+    size_t s = spack_bytes(prec, nx, ny, pad);
     s += align16(sizeof(double) * 2 * (nx + ny)) * 2;
     s += align16(tsz * 32 * SM_WARPS) + align16(tsz * 2 * 32 * SM_WARPS) + 16;
     s += align16(sizeof(double) * n);
@@ -477,12 +478,13 @@ static cudaError_t launch_local_t(const DevPtrs& P, const MethodDev& M, const Jo
     return cudaGetLastError();
 }
 
-// Job classes: local2d_class(prec, nx).  The FP32 form has one kernel per line
-// width that is a multiple of 4 (width known at compile time: its line
-// inversions and sweeps run without width guards); other widths, and the
-// FP64 form, run a kernel for widths up to 8, 16, 24 or 32.
-int local2d_class(int prec, int nx) {
-    if (prec != 0 && nx % 4 == 0 && nx <= 32) return nx;
+// Job classes: local2d_class(prec, nx, pad).  The FP32 form has one kernel per
+// line width (known at compile time: its line inversions and sweeps run
+// without width guards); the FP64 form, and FP32 handles without widened
+// lines, run a kernel for widths up to 8, 16, 24 or 32 (there a box line of 22
+// cells took 1.5 times a line of 24 of the other path).
+int local2d_class(int prec, int nx, int pad) {
+    if (prec != 0 && (pad || nx % 4 == 0) && nx <= 32) return (nx + 3) & ~3;
     return 100 + (nx <= 8 ? 8 : nx <= 16 ? 16 : nx <= 24 ? 24 : 32);
 }
 

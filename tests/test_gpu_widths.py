@@ -1,0 +1,58 @@
+"""2D boxes of every line width modulo 4 (FP32 lines are widened to the next
+multiple of 4): widths 1 to 32 through the basis, particular, smoothing and
+reverse kernels -- against the oracle at the bars of the
+parity and gradient tests (1e-10 FP64, 1e-8 mixed)."""
+import numpy as np
+import pytest
+
+from oracle import mrcm_adjoint as OA
+from oracle import mrcm_oracle as O
+from paper_2404_13811_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp64": 1e-10, "mixed": 1e-8}
+
+
+def _problem(n, seed):
+    prob = I.lognormal_problem(n, sigma2=2.0, corr_len=0.15, seed=seed)
+    prob.f = np.random.default_rng(seed + 11).standard_normal(prob.f.shape)
+    return prob
+
+
+# sub (x, y), overlap: three blocks along x, two along y; widths of boxes at the ends sub + l, inside sub + 2 l
+CASES = [((1, 4), 0), ((2, 5), 0), ((3, 4), 1), ((5, 7), 2), ((7, 6), 1), ((9, 8), 3), ((10, 9), 4), ((13, 9), 2),
+         ((15, 12), 3), ((17, 7), 3), ((19, 9), 4), ((23, 11), 4), ((27, 6), 2)]
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("case", range(len(CASES)))
+def test_widths_match_oracle(case, precision):
+    from paper_2404_13811_gb300.solver import MRCM
+    sub, ov = CASES[case]
+    n = (3 * sub[0], 2 * sub[1])
+    prob = _problem(n, 90 + case)
+    ns = 2 if ov else 0
+    space = 1 if min(sub) > 1 else 0   # a side of one cell carries no linear function
+    ref = O.mrcm_os(prob, sub, ov, space, 1.0, 1.0, ns)
+    s = MRCM(prob, I.Partition(sub, ov), space=space, alpha_basis=1.0, alpha_smooth=1.0, precision=precision)
+    s.run(ns)
+    p, u = s.fluxes()
+    s.close()
+    ep, eu = O.rel_errors(prob, p, u, ref.p, ref.u)
+    assert ep <= TOL[precision] and eu <= TOL[precision], (ep, eu)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("sub,ov", [((9, 8), 3), ((10, 9), 4), ((15, 12), 3)])
+def test_gradient_at_odd_widths(sub, ov, precision):
+    from paper_2404_13811_gb300.solver import MRCM
+    prob = _problem((3 * sub[0], 2 * sub[1]), 7)
+    rng = np.random.default_rng(3)
+    gp, gu = rng.standard_normal(prob.ncells), rng.standard_normal((prob.ncells, 4))
+    _, ref = OA.mrcm_os_adjoint(prob, sub, ov, 1, 1.0, 1.0, 2, gp, gu)
+    s = MRCM(prob, I.Partition(sub, ov), space=1, alpha_basis=1.0, alpha_smooth=1.0, precision=precision)
+    s.run(2)
+    g = s.adjoint(gp, gu)
+    s.close()
+    assert np.abs(g - np.asarray(ref).reshape(-1)).max() <= 1e-8 * np.abs(ref).max()
