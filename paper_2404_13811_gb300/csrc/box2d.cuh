@@ -1027,15 +1027,25 @@ __device__ int cta_solve(const Box& B, const Ops& O, const T* Sinv, const T* cys
 // --- the mixed form's refinement in scaled variables -------------------------
 // Right-hand sides b~ for the scaled solves.  Basis problem: nonzero only on
 // the Robin side sk, where lane pos holds b~ of the side's face pos (a
-// register, fetched by shuffle: every lane of the warp calls it); stored:
-// an array of b~.
+// register, fetched by shuffle: every lane of the warp calls it); the faces
+// beyond the 32 lanes (x sides of boxes higher than 32 cells) are formed anew
+// at each use; stored: an array of b~.
 struct RhsScSide {
-    int sk;
-    double mine;   // b~ of face `lane` of side sk (0 beyond the side)
+    int sk, m;
+    const double *dsc, *bT;   // of Ops
+    double mine;              // b~ of face `lane` of side sk (0 beyond the side)
+    __device__ static double face(const Box& B, const double* dsc, const double* bT, int sk, int m, int pos) {
+        const int len = (sk >> 1) == 0 ? B.ny : B.nx;
+        const int ci = (sk >> 1) == 0 ? pos * B.nx + (sk == 0 ? 0 : B.nx - 1)
+                                      : (sk == 2 ? 0 : (B.ny - 1) * B.nx) + pos;
+        return dsc[ci] * bT[side_off(B, sk) + pos] * psi_val(m, pos, len, B.rlen[sk]);
+    }
     __device__ double operator()(const Box& B, int i, int j) const {
         const bool on = (sk == 0 && i == 0) || (sk == 1 && i == B.nx - 1) || (sk == 2 && j == 0) ||
                         (sk == 3 && j == B.ny - 1);
-        const double v = __shfl_sync(0xffffffffu, mine, (sk >> 1) == 0 ? j : i);
+        const int pos = (sk >> 1) == 0 ? j : i;
+        const double v = __shfl_sync(0xffffffffu, mine, pos & 31);
+        if (on && pos >= 32) return face(B, dsc, bT, sk, m, pos);
         return on ? v : 0.0;
     }
 };

@@ -115,13 +115,8 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
             if constexpr (mixed) {
                 // b~ on the Robin side: lane pos holds that of face pos
                 const int len = (sk >> 1) == 0 ? B.ny : B.nx;
-                double mine = 0.0;
-                if (lane < len) {
-                    const int ci = (sk >> 1) == 0 ? lane * B.nx + (sk == 0 ? 0 : B.nx - 1)
-                                                  : (sk == 2 ? 0 : (B.ny - 1) * B.nx) + lane;
-                    mine = C.O.dsc[ci] * C.O.bT[side_off(B, sk) + lane] * psi_val(mk, lane, len, B.rlen[sk]);
-                }
-                RhsScSide rb{sk, mine};
+                const double mine = lane < len ? RhsScSide::face(B, C.O.dsc, C.O.bT, sk, mk, lane) : 0.0;
+                RhsScSide rb{sk, mk, C.O.dsc, C.O.bT, mine};
                 it = warp_solve_sc<RhsScSide, EX ? BW : 0>(B, C.O, C.Sinv, C.cys, x, w, zb, rb, Mth.ir_tol,
                                                             Mth.max_ir, &C.flags[1]);
             } else {
