@@ -252,10 +252,10 @@ int mrcm_set_permeability(mrcm_handle* h, const double* values, int is_log, int 
  *   g_logK [total cells] output dL/dlog K.
  *   device_ptrs 0: host arrays (the call synchronises); 1: device arrays.
  * The kept factors serve the transposed local solves (the operators are
- * symmetric); the local forward solutions are recomputed, not stored; the
- * smoothing steps are replayed once to record the state before each colour
- * pass (n_steps x 2^dim states of (p, u), allocated by the handle on first
- * use); the interface system is solved transposed with its FP32 slab factors
+ * symmetric); the basis solutions are recomputed, not stored; the smoothing
+ * steps are replayed once to record the solution of every box (n_steps x
+ * subdomains boxes of pressures and side data, allocated by the handle on
+ * first use); the interface system is solved transposed with its FP32 slab factors
  * and FP64 refinement.  Leaves the current solution unchanged.
  * MRCM_ERR_UNSUPPORTED for a member with no Dirichlet side (its pressure is
  * fixed only up to a constant) and for 3D problems.  Needs a solution

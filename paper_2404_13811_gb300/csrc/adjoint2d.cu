@@ -10,8 +10,8 @@
 // For one box solve A p = b(lambda), u = V(p, lambda) with seeds (gp, gu) the
 // adjoint is mu = A^{-1} (gp + dV/dp^T gu) -- the same factor, A is SPD -- and
 // dL/dc = -mu^T (dA/dc) p + mu^T db/dc + gu . dV/dc per face coefficient c.
-// The forward solution p is recomputed from the kept factor instead of
-// being stored.
+// The forward solution p of a basis or particular problem is recomputed, that
+// of a smoothing solve is recorded by a replay of the smoothing steps.
 //
 // Kernels, in the order the host issues them:
 //   k_adj_smooth2d    one colour pass of a smoothing step backwards
@@ -26,7 +26,7 @@
 
 namespace {
 
-constexpr int AS_WARPS = 4;   // k_adj_smooth2d: warp 0 solves, all warps form data
+constexpr int AS_WARPS = 4;   // k_adj_smooth2d
 
 // row of test function m on side `sid` of its owner (flux rows of the high
 // sides first, then pressure rows of the low sides; same order as
@@ -54,12 +54,17 @@ __device__ int row_pos(const SubDev& o, int d, int npsi, int kind, int sid, int 
 
 // ---------------------------------------------------------------------------
 // One colour pass of a smoothing step, backwards.  One CTA per subdomain of
-// the colour.  Forward: lambda from the recorded state on d hat-Omega_i \ d
-// Omega, a solve on hat-Omega_i with the sources, overwrite of (p, u) on
-// Omega_i.  Backward: the seeds on Omega_i are taken (and cleared), the
-// forward solution is recomputed, one adjoint solve, and dL/dlambda is
-// passed on to the recorded state.  Subdomains of one colour have disjoint
-// oversampled boxes (2 l < H), so their writes never meet.
+// the colour.  Forward: lambda from the state on d hat-Omega_i \ d Omega, a
+// solve on hat-Omega_i with the sources, overwrite of (p, u) on Omega_i.
+// Backward: the seeds on Omega_i are taken (and cleared), one adjoint solve,
+// and dL/dlambda is passed on to the state before the pass.  The forward
+// solution on the box and lambda were recorded by the replay; the smoothing
+// pack is staged by one bulk copy and the solve runs as the forward one does
+// (two-warp sweeps, residuals over the CTA).  Subdomains of one colour have
+// disjoint oversampled boxes (2 l < H), so their writes never meet.
+// A pass of 64 boxes of 24 x 24 cells takes 51 us (184 us when it solved twice
+// from zero on one warp, on a factor read by loads); bound by the latency of
+// the box's line sweeps.
 // ---------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, MethodDev Mth, AdjPtrs A,
@@ -70,113 +75,110 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     const SubDev sd = P.sub[item];
     const MemberDev& md = P.mem[sd.member];
     __shared__ Box B;
+    __shared__ __align__(8) uint64_t bar;
     if (threadIdx.x == 0) setup_box(B, md, sd.loh, sd.hih, Mth.alpha_s);
     __syncthreads();
     const size_t n = (size_t)B.n;
     const int per = 2 * (B.nx + B.ny);
-    size_t o = 0;
+    const SPack L = spack_layout(B.nx, B.ny, sizeof(T), Mth.pad);
+    T* Sinv = (T*)smem;
+    Ops O;   // scaled in the mixed form
+    O.cd = (double*)(smem + L.cd);
+    O.cx = (double*)(smem + L.cx);
+    O.cy = (double*)(smem + L.cy);
+    O.dsc = (double*)(smem + L.dsc);
+    O.hk = nullptr;
+    O.bT = (double*)(smem + L.bT);
+    O.bB = (double*)(smem + L.bB);
+    double* rt = (double*)(smem + L.bst);   // the adjoint right-hand side, in the place of the forward one
+    T* cys = (T*)(smem + L.cys);
+    size_t o = L.bytes;
     auto take = [&](size_t bytes) { unsigned char* p = smem + o; o += align16(bytes); return p; };
-    T* Sinv = (T*)take(sizeof(T) * sinv_len(B.nx, B.ny, sizeof(T), Mth.pad));
-    Ops O;
-    O.cd = (double*)take(sizeof(double) * n);
-    O.cx = (double*)take(sizeof(double) * n);
-    O.cy = (double*)take(sizeof(double) * n);
-    O.dsc = (double*)take(sizeof(double) * n);
-    O.hk = (double*)take(sizeof(double) * 2 * n);
-    O.bT = (double*)take(sizeof(double) * per);
-    O.bB = (double*)take(sizeof(double) * per);
-    double* lam = (double*)take(sizeof(double) * per);
-    double* rt = (double*)take(sizeof(double) * n);
-    const int bp = line_width(B.nx, sizeof(T), Mth.pad);   // line stride of cys
-    T* cys = (T*)take(sizeof(T) * bp * B.ny);
-    T* zbuf = (T*)take(sizeof(T) * 64);   // two line inputs of the twisted sweeps
     double* x = (double*)take(sizeof(double) * n);
     double* mu = (double*)take(sizeof(double) * n);
-    T* w = mixed ? (T*)take(sizeof(T) * n) : nullptr;
     double* su = (double*)take(sizeof(double) * 4 * n);
+    T* w = mixed ? (T*)take(sizeof(T) * n) : (T*)mu;
+    T* zbuf = (T*)take(sizeof(T) * 32 * AS_WARPS);
+    T* red = (T*)take(sizeof(T) * 2 * 32 * AS_WARPS);
+    unsigned int* nrm = (unsigned int*)take(16);
     int* flags = (int*)take(64);
-
-    const T* Sg = (const T*)P.fac + (size_t)item * P.fac_stride;
-    for (size_t t = threadIdx.x; t < sinv_len(B.nx, B.ny, sizeof(T), Mth.pad); t += blockDim.x) Sinv[t] = Sg[t];
-    if (threadIdx.x == 0) flags[0] = 0;
-    build_ops(B, md, P, O);
-    const double* dd = P.dsc + (size_t)item * P.dsc_stride;
-    for (int c = threadIdx.x; c < B.n; c += blockDim.x) O.dsc[c] = dd[c];
-    __syncthreads();
-    for (int c = threadIdx.x; c < B.n; c += blockDim.x)
-        cys[(c / B.nx) * bp + c % B.nx] = (T)(O.cy[c] * O.dsc[c] * ((c + B.nx < B.n) ? O.dsc[c + B.nx] : 0.0));
+    const uint32_t pbytes = (uint32_t)L.bytes;
+    const unsigned char* Pg = (const unsigned char*)((const T*)P.fac + (size_t)item * P.fac_stride);
+    if (threadIdx.x == 0) {
+        flags[0] = 0;
+        mbar_init(&bar, 1);
+        mbar_expect_tx(&bar, pbytes);
+        bulk_g2s(smem, Pg, pbytes, &bar);
+    }
+    const double* rec = A.rec + (size_t)item * A.rec_stride;
+    const double* lam = rec + n;
+    const double* lun = lam + per;
     const int nxg = md.n[0];
-    const double* pst = A.ps + md.cell_off;
-    const double* ust = A.us + md.cell_off * 4;
-    for (int sid = 0; sid < 4; ++sid) {
-        if (B.kind[sid] != 2) continue;
-        const int a = sid >> 1;
-        const int len = a == 0 ? B.ny : B.nx;
-        for (int pos = threadIdx.x; pos < len; pos += blockDim.x) {
-            int i, j;
-            if (a == 0) { j = pos; i = (sid == 0) ? 0 : B.nx - 1; }
-            else        { i = pos; j = (sid == 2) ? 0 : B.ny - 1; }
-            const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
-            const double un = ust[g * 4 + sid];
-            const double pi = pst[g] - un * O.hk[2 * (j * B.nx + i) + a];
-            lam[side_off(B, sid) + pos] = -O.bB[side_off(B, sid) + pos] * un + pi;
-        }
-    }
-    __syncthreads();
-    const double vol = md.h[0] * md.h[1];
-    const double* fm = P.f + md.cell_off;
-    for (int c = threadIdx.x; c < B.n; c += blockDim.x)
-        rt[c] = source_rhs(B, O, fm, nxg, vol, md.h[1], md.h[0], lam, c % B.nx, c / B.nx);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        RhsStored rs{rt};
-        warp_solve<T>(B, O, Sinv, cys, x, mixed ? w : (T*)x, zbuf, rs, Mth.ir_tol, Mth.max_ir, &flags[0], bp);
-    }
-    __syncthreads();
-
-    // seeds on Omega_i, taken and cleared (the forward overwrote them)
-    for (size_t c = threadIdx.x; c < n; c += blockDim.x) {
-        rt[c] = 0.0;
-        su[4 * c] = su[4 * c + 1] = su[4 * c + 2] = su[4 * c + 3] = 0.0;
-    }
-    __syncthreads();
-    const int nIx = sd.hi[0] - sd.lo[0], nIy = sd.hi[1] - sd.lo[1];
-    const int offx = sd.lo[0] - B.lo[0], offy = sd.lo[1] - B.lo[1];
+    const double* Tfg = P.Tf + md.cell_off * 3;
+    const double* hkg = P.hk + md.cell_off * 3;
     double* gpg = A.gp + md.cell_off;
     double* gug = A.gu + md.cell_off * 4;
-    for (int c = threadIdx.x; c < nIx * nIy; c += blockDim.x) {
-        const int i = c % nIx + offx, j = c / nIx + offy;
-        const int cl = j * B.nx + i;
-        const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
-        rt[cl] = gpg[g];
-        gpg[g] = 0.0;
-        for (int s = 0; s < 4; ++s) {
-            su[4 * cl + s] = gug[g * 4 + s];
-            gug[g * 4 + s] = 0.0;
+    const int ilo = sd.lo[0] - B.lo[0], ihi = sd.hi[0] - B.lo[0];
+    const int jlo = sd.lo[1] - B.lo[1], jhi = sd.hi[1] - B.lo[1];
+    // the forward solution; the seeds on Omega_i, taken and cleared (the
+    // forward overwrote them); mu starts as the pressure seed
+    for (int c = threadIdx.x; c < B.n; c += blockDim.x) {
+        const int i = c % B.nx, j = c / B.nx;
+        x[c] = rec[c];
+        double g0 = 0.0, s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+        if (i >= ilo && i < ihi && j >= jlo && j < jhi) {
+            const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
+            g0 = gpg[g];
+            s0 = gug[g * 4];
+            s1 = gug[g * 4 + 1];
+            s2 = gug[g * 4 + 2];
+            s3 = gug[g * 4 + 3];
+            gpg[g] = 0.0;
+            gug[g * 4] = gug[g * 4 + 1] = gug[g * 4 + 2] = gug[g * 4 + 3] = 0.0;
         }
+        mu[c] = g0;
+        su[4 * c] = s0;
+        su[4 * c + 1] = s1;
+        su[4 * c + 2] = s2;
+        su[4 * c + 3] = s3;
     }
-    __syncthreads();
-    // adjoint right-hand side gp + (du/dp)^T gu
+    const bool arrived = mbar_wait(&bar, 0);
+    if (__syncthreads_or(!arrived)) {
+        // the staged pack never arrived: report, wait once more for the copy
+        // in flight (bounded) so that no copy targets a finished CTA, and stop
+        if (threadIdx.x == 0) {
+            atomicOr(&P.status[0], ST_BAD);
+            mbar_wait(&bar, 0);
+        }
+        __syncthreads();
+        return;
+    }
+    // adjoint right-hand side gp + (du/dp)^T gu (scaled in the mixed form)
     const double rax = 1.0 / md.h[1], ray = 1.0 / md.h[0];
     for (int c = threadIdx.x; c < B.n; c += blockDim.x) {
         const int i = c % B.nx, j = c / B.nx;
-        double r = rt[c];
-        if (i < B.nx - 1) r += O.cx[c] * (su[4 * c + 1] - su[4 * (c + 1)]) * rax;
-        if (i > 0) r -= O.cx[c - 1] * (su[4 * (c - 1) + 1] - su[4 * c]) * rax;
-        if (j < B.ny - 1) r += O.cy[c] * (su[4 * c + 3] - su[4 * (c + B.nx) + 2]) * ray;
-        if (j > 0) r -= O.cy[c - B.nx] * (su[4 * (c - B.nx) + 3] - su[4 * c + 2]) * ray;
+        const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
+        double r = mu[c];
+        if (i < B.nx - 1) r += Tfg[g * 3] * (su[4 * c + 1] - su[4 * (c + 1)]) * rax;
+        if (i > 0) r -= Tfg[(g - 1) * 3] * (su[4 * (c - 1) + 1] - su[4 * c]) * rax;
+        if (j < B.ny - 1) r += Tfg[g * 3 + 1] * (su[4 * c + 3] - su[4 * (c + B.nx) + 2]) * ray;
+        if (j > 0) r -= Tfg[(g - nxg) * 3 + 1] * (su[4 * (c - B.nx) + 3] - su[4 * c + 2]) * ray;
         if (i == 0 && B.kind[0]) r += O.bT[side_off(B, 0) + j] * su[4 * c] * rax;
         if (i == B.nx - 1 && B.kind[1]) r += O.bT[side_off(B, 1) + j] * su[4 * c + 1] * rax;
         if (j == 0 && B.kind[2]) r += O.bT[side_off(B, 2) + i] * su[4 * c + 2] * ray;
         if (j == B.ny - 1 && B.kind[3]) r += O.bT[side_off(B, 3) + i] * su[4 * c + 3] * ray;
-        rt[c] = r;
+        rt[c] = mixed ? O.dsc[c] * r : r;
     }
     __syncthreads();
-    if (threadIdx.x < 32) {
+    if constexpr (mixed) {
+        cta_solve_sc(B, O, (const float*)Sinv, (const float*)cys, mu, (float*)w, (float*)zbuf, nrm, rt, Mth.ir_tol,
+                     Mth.max_ir, &flags[0], false, line_width(B.nx, sizeof(T), Mth.pad));
+        for (int c = threadIdx.x; c < B.n; c += blockDim.x) mu[c] *= O.dsc[c];
+        __syncthreads();
+    } else {
         RhsStored rs{rt};
-        warp_solve<T>(B, O, Sinv, cys, mu, mixed ? w : (T*)mu, zbuf, rs, Mth.ir_tol, Mth.max_ir, &flags[0], bp);
+        cta_solve<T>(B, O, Sinv, cys, mu, w, zbuf, red, nrm, rs, Mth.ir_tol, Mth.max_ir, &flags[0], false);
     }
-    __syncthreads();
 
     // interior faces: dL/dTf = (gu_L - gu_R) dp / a - (mu_L - mu_R) dp
     double* gTf = A.gTf + md.cell_off * 3;
@@ -213,13 +215,13 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
                     const double lv = lam[side_off(B, sid) + pos];
                     const double gT = (x[c] - lv) * (sc - mu[c]);
                     const double gl = Tb * (mu[c] - sc);
-                    const double un = ust[g * 4 + sid];
+                    const double un = lun[side_off(B, sid) + pos];
                     const long long gf = (sid & 1) ? g : g - (a == 0 ? 1 : nxg);
                     // lambda = -alpha wh u.n + p - u.n hk
                     ghk[g * 3 + a] += gT * q - gl * un;
                     gwh[gf * 3 + a] += B.alpha * (gT * q - gl * un);
                     gpg[g] += gl;
-                    gug[g * 4 + sid] += gl * (-O.bB[side_off(B, sid) + pos] - O.hk[2 * c + a]);
+                    gug[g * 4 + sid] += gl * (-O.bB[side_off(B, sid) + pos] - hkg[g * 3 + a]);
                 } else {
                     const double gT = (x[c] - B.val[sid]) * (sc - mu[c]);
                     ghk[g * 3 + a] += gT * q;
@@ -648,14 +650,11 @@ __global__ void k_set_K(const double* src, double* K, long long n, int is_log, i
 // ---------------------------------------------------------------------------
 size_t adj_smooth2d_smem(int prec, int nx, int ny, int pad) {
     const size_t n = (size_t)nx * ny;
-    const size_t per = 2 * (size_t)(nx + ny);
     const size_t tsz = prec == 0 ? sizeof(double) : sizeof(float);
-    size_t s = align16(tsz * sinv_len(nx, ny, (int)tsz, pad));
-    s += align16(sizeof(double) * n) * 4 + align16(sizeof(double) * 2 * n);
-    s += align16(sizeof(double) * per) * 3 + align16(sizeof(double) * n);
-    s += align16(tsz * (size_t)line_width(nx, (int)tsz, pad) * ny) + align16(tsz * 64) + align16(sizeof(double) * n) * 2;
+    size_t s = spack_layout(nx, ny, tsz, pad).bytes;
+    s += align16(sizeof(double) * n) * 2 + align16(sizeof(double) * 4 * n);   // x, mu, su
     if (prec != 0) s += align16(tsz * n);
-    s += align16(sizeof(double) * 4 * n);
+    s += align16(tsz * 32 * AS_WARPS) + align16(tsz * 2 * 32 * AS_WARPS) + 16;
     return s + 64;
 }
 

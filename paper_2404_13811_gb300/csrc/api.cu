@@ -27,8 +27,8 @@ size_t spack_bytes(int prec, int nx, int ny, int pad);
 int local2d_class(int prec, int nx, int pad);
 cudaError_t launch_local2d(const DevPtrs& P, const MethodDev& M, const Job* jobs, int njobs, int bw,
                            size_t smem, cudaStream_t s);
-cudaError_t launch_smooth2d(const DevPtrs& P, const MethodDev& M, const int* items, int nitems,
-                            size_t smem, cudaStream_t s);
+cudaError_t launch_smooth2d(const DevPtrs& P, const MethodDev& M, const int* items, int nitems, size_t smem,
+                            double* rec, long long rec_stride, cudaStream_t s);
 cudaError_t launch_assemble2d(const DevPtrs& P, const double* X, int nitems, int ncell_i_max,
                               cudaStream_t s);
 cudaError_t launch_faces(const MemberDev* dmem, int nmem, long long maxcells, const double* K, double* Tf,
@@ -112,8 +112,9 @@ struct AdjWork {
     Job* jobs = nullptr;
     std::vector<AdjClass> classes;
     size_t smooth_smem = 0;
-    double* snap = nullptr;
-    size_t snap_len = 0;      // doubles
+    double* rec = nullptr;    // forward solutions of the replay, [step][item][rec_stride]
+    size_t rec_len = 0;       // doubles
+    long long rec_stride = 0;
     double* gout = nullptr;   // device result when the caller passes host memory
 };
 
@@ -936,7 +937,8 @@ static int issue_smooth(mrcm_handle* h, int n_steps) {
             const int off = h->colour_off[c], cnt = h->colour_off[c + 1] - off;
             cudaError_t e = h->dim == 3
                                 ? launch_smooth3d(h->P, h->mth, h->d_colour_items + off, cnt, h->smooth_smem, h->stream)
-                                : launch_smooth2d(h->P, h->mth, h->d_colour_items + off, cnt, h->smooth_smem, h->stream);
+                                : launch_smooth2d(h->P, h->mth, h->d_colour_items + off, cnt, h->smooth_smem, nullptr, 0,
+                                                  h->stream);
             if (e != cudaSuccess) return fail(h, MRCM_ERR_CUDA, std::string("smoothing kernel: ") + cudaGetErrorString(e));
             h->launches[4] += 1;
         }
@@ -973,7 +975,9 @@ static int prepare_adjoint(mrcm_handle* h) {
             by[{bw, nw}].push_back(Job{s, type});
             smem[{bw, nw}] = std::max(smem[{bw, nw}], b);
         }
-        W.smooth_smem = std::max(W.smooth_smem, adj_smooth2d_smem(prec, sd.hih[0] - sd.loh[0], sd.hih[1] - sd.loh[1], h->mth.pad));
+        const int bx = sd.hih[0] - sd.loh[0], by = sd.hih[1] - sd.loh[1];
+        W.smooth_smem = std::max(W.smooth_smem, adj_smooth2d_smem(prec, bx, by, h->mth.pad));
+        W.rec_stride = std::max(W.rec_stride, (long long)bx * by + 4 * (bx + by));
     }
     if (W.smooth_smem > lim) return fail(h, MRCM_ERR_UNSUPPORTED, "subdomain box too large for the adjoint kernels");
     std::vector<Job> jobs;
@@ -1759,27 +1763,24 @@ static int adjoint_body(mrcm_handle* h, const double* gp, const double* gu, doub
     const int d = h->dim, nside = 2 * d, ncol = 1 << d;
     const int ns = h->smooth_steps;
     const size_t cells = (size_t)h->ncells;
-    const size_t per_snap = cells * (1 + nside);
-    const size_t need = per_snap * (size_t)ns * ncol;
-    if (need > W.snap_len) {
-        int e = dalloc(h, &W.snap, need);
+    const size_t per_step = (size_t)W.rec_stride * h->sub.size();
+    const size_t need = per_step * (size_t)ns;
+    if (need > W.rec_len) {
+        int e = dalloc(h, &W.rec, need);
         if (e) return e;
-        W.snap_len = need;
+        W.rec_len = need;
     }
     const int nitems = (int)h->sub.size();
     CUDA_TRY(h, cudaMemsetAsync(h->d_status, 0, sizeof(int) * MRCM_STATUS_WORDS, st));
     // replay: the MRCM-O state again, then the smoothing steps, recording the
-    // state before every colour pass (forward solves with the kept factors)
+    // solution of every box (forward solves with the kept factors)
     if ((rc = issue_assemble(h))) return rc;
     for (int s = 0; s < ns; ++s)
         for (int c = 0; c < ncol; ++c) {
-            double* sp = W.snap + per_snap * ((size_t)s * ncol + c);
-            CUDA_TRY(h, cudaMemcpyAsync(sp, h->d_p, sizeof(double) * cells, cudaMemcpyDeviceToDevice, st));
-            CUDA_TRY(h, cudaMemcpyAsync(sp + cells, h->d_u, sizeof(double) * cells * nside, cudaMemcpyDeviceToDevice,
-                                        st));
             Phase ph(h, 4);
             const int off = h->colour_off[c], cnt = h->colour_off[c + 1] - off;
-            CUDA_TRY(h, launch_smooth2d(h->P, h->mth, h->d_colour_items + off, cnt, h->smooth_smem, st));
+            CUDA_TRY(h, launch_smooth2d(h->P, h->mth, h->d_colour_items + off, cnt, h->smooth_smem,
+                                        W.rec + per_step * s, W.rec_stride, st));
             h->launches[4] += 1;
         }
     // seeds
@@ -1796,15 +1797,14 @@ static int adjoint_body(mrcm_handle* h, const double* gp, const double* gu, doub
     // smoothing backwards: steps and colours in reverse order
     for (int s = ns - 1; s >= 0; --s)
         for (int c = ncol - 1; c >= 0; --c) {
-            const double* sp = W.snap + per_snap * ((size_t)s * ncol + c);
-            A.ps = sp;
-            A.us = sp + cells;
+            A.rec = W.rec + per_step * s;
+            A.rec_stride = W.rec_stride;
             Phase ph(h, 4);
             const int off = h->colour_off[c], cnt = h->colour_off[c + 1] - off;
             CUDA_TRY(h, launch_adj_smooth2d(h->P, h->mth, A, h->d_colour_items + off, cnt, W.smooth_smem, st));
             h->launches[4] += 1;
         }
-    A.ps = A.us = nullptr;
+    A.rec = nullptr;
     // superposition backwards, interface transposed, moments
     {
         Phase ph(h, 3);

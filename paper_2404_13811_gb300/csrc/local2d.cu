@@ -237,7 +237,8 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
 constexpr int SM_WARPS = 4;
 
 template <typename T>
-__global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev Mth, const int* items) {
+__global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev Mth, const int* items, double* rec,
+                                                            long long rec_stride) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool mixed = std::is_same<T, float>::value;
     const int item = items[blockIdx.x];
@@ -386,6 +387,16 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
         __syncthreads();
         return;
     }
+    if (rec) {
+        // the reverse pass's replay: the box solution and its Robin data
+        double* r = rec + (size_t)item * rec_stride;
+        for (int c = threadIdx.x; c < B.n; c += blockDim.x) r[c] = x[c];
+        const int per = 2 * (B.nx + B.ny);
+        for (int t = threadIdx.x; t < per; t += blockDim.x) {
+            r[B.n + t] = lam[t];
+            r[B.n + per + t] = lun[t];
+        }
+    }
     // overwrite (u, p) on Omega_i with the restriction
     double* pw = P.p + md.cell_off;
     double* uw = P.u + md.cell_off * 4;
@@ -511,7 +522,7 @@ cudaError_t launch_local2d(const DevPtrs& P, const MethodDev& M, const Job* jobs
 
 template <typename T>
 static cudaError_t launch_smooth2d_t(const DevPtrs& P, const MethodDev& M, const int* items, int nitems, size_t smem,
-                                     cudaStream_t s) {
+                                     double* rec, long long rec_stride, cudaStream_t s) {
     auto kern = k_smooth2d<T>;
     static size_t set_smem = 0;
     if (smem > set_smem) {
@@ -533,13 +544,15 @@ static cudaError_t launch_smooth2d_t(const DevPtrs& P, const MethodDev& M, const
     cfg.numAttrs = 1;
     DevPtrs Pc = P;
     MethodDev Mc = M;
-    void* args[] = {&Pc, &Mc, (void*)&items};
+    void* args[] = {&Pc, &Mc, (void*)&items, (void*)&rec, (void*)&rec_stride};
     return cudaLaunchKernelExC(&cfg, (const void*)kern, args);
 }
 
+// rec (null in the forward pass): where the replay of the reverse pass records
+// each box's solution, [item][rec_stride].
 cudaError_t launch_smooth2d(const DevPtrs& P, const MethodDev& M, const int* items, int nitems, size_t smem,
-                            cudaStream_t s) {
+                            double* rec, long long rec_stride, cudaStream_t s) {
     if (nitems == 0) return cudaSuccess;
-    return M.prec == 0 ? launch_smooth2d_t<double>(P, M, items, nitems, smem, s)
-                       : launch_smooth2d_t<float>(P, M, items, nitems, smem, s);
+    return M.prec == 0 ? launch_smooth2d_t<double>(P, M, items, nitems, smem, rec, rec_stride, s)
+                       : launch_smooth2d_t<float>(P, M, items, nitems, smem, rec, rec_stride, s);
 }

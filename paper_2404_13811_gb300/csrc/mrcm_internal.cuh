@@ -147,8 +147,8 @@ struct AdjPtrs {
     double* gTf;         // [ncells][3]    dL/dTf
     double* ghk;         // [ncells][3]    dL/d(h / 2K)
     double* gwh;         // [ncells][3]    dL/d(H / K_H)
-    const double* ps;    // state recorded before the colour pass being reversed
-    const double* us;
+    const double* rec;   // forward solutions of the step being reversed, [item][rec_stride]: the box pressure, then
+    long long rec_stride;  // lambda and u.n of the box-side faces (written by the replay's k_smooth2d)
     double* gps;         // [item][ncell_i_max]        dL/d(assembled Omega_i pressure)
     double* gug;         // [item][6][side_max]        dL/d(Gamma_i face velocity)
     double* gX;          // [nif]                      dL/dX
