@@ -53,6 +53,7 @@ int kry_blocks();
 cudaError_t kry_mdot(const double* V, const double* w, int n, int nv, double* part, cudaStream_t s);
 cudaError_t kry_msub(double* w, const double* V, const double* coef, int nv, int n, cudaStream_t s);
 cudaError_t lu_inverse(const IfPtrs& I, const ElimDev* el, int nel, int* status, int variant, cudaStream_t s);
+cudaError_t interface_load(int npad);
 int slab_inverse_gj_ok(int npad);
 int slab_inverse_gjr_npad(int npad);
 size_t elim_smem_bytes(int nmv, int cw);
@@ -1479,6 +1480,7 @@ static int solve_interface_body(mrcm_handle* h) {
             h->tune_choice = cached;
             h->tune_source = 1;
         } else {
+            CUDA_TRY(h, interface_load(h->npad));
             RefineOut run[3];
             bool ok[3] = {false, false, false};
             int steps[3] = {0, 0, 0};

@@ -518,3 +518,19 @@ cudaError_t gjr_inverse(const IfPtrs& I, const ElimDev* el, int nel, int* status
         default: return cudaErrorInvalidValue;
     }
 }
+
+// Loads the kernels of a padded slab size.
+cudaError_t gjr_load(int npad) {
+    cudaFuncAttributes a;
+    auto load = [&](const void* k1, const void* k2) {
+        cudaError_t e = cudaFuncGetAttributes(&a, k1);
+        return e != cudaSuccess ? e : cudaFuncGetAttributes(&a, k2);
+    };
+    switch (slab_inverse_gjr_npad(npad)) {
+        case 128: return load((const void*)k_gjr_inverse<128, 4, 8>, (const void*)k_gjr_inverse<128, 2, 16>);
+        case 256: return load((const void*)k_gjr_inverse<256, 8, 8>, (const void*)k_gjr_inverse<256, 4, 16>);
+        case 512: return load((const void*)k_gjr_inverse<512, 16, 8>, (const void*)k_gjr_inverse<512, 8, 16>);
+        case 768: return load((const void*)k_gjr_inverse<768, 16, 12>, (const void*)k_gjr_inverse<768, 16, 12>);
+        default: return cudaSuccess;
+    }
+}
