@@ -474,17 +474,20 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
     // 2D FP32 lines widened to a multiple of 4, unless some box then does not
     // fit shared memory (tall boxes of a width that is no multiple of 4), be
     // it in the forward kernels or in the adjoint's
-    h->mth.pad = prec != MRCM_FP64;
-    for (int s = 0; s < nitems && d == 2 && h->mth.pad; ++s) {
+    h->mth.pad = 0;
+    for (int s = 0; s < nitems && d == 2 && prec != MRCM_FP64; ++s) {
         const SubDev& sd = h->sub[s];
         const size_t lim = 227 * 1024;
         const int bx = sd.hih[0] - sd.loh[0], by = sd.hih[1] - sd.loh[1];
         const int ix = sd.hi[0] - sd.lo[0], iy = sd.hi[1] - sd.lo[1];
+        h->mth.pad = std::max(h->mth.pad, (bx + 3) & ~3);
         if (bx > 32) break;   // refused below
         const int nb = std::max(std::min(sd.nbasis + (h->mth.part_hat ? 1 : 0), 4), 1);
         if (local2d_smem(prec, bx, by, nb, false, 1) > lim || local2d_smem(prec, ix, iy, 1, true, 1) > lim ||
-            smooth2d_smem(prec, bx, by, 1) > lim || adj_smooth2d_smem(prec, bx, by, 1) > lim)
+            smooth2d_smem(prec, bx, by, 1) > lim || adj_smooth2d_smem(prec, bx, by, 1) > lim) {
             h->mth.pad = 0;
+            break;
+        }
     }
     const int pad = h->mth.pad;
     for (int s = 0; s < nitems; ++s) {

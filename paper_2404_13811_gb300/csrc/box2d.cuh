@@ -439,21 +439,26 @@ template <int BB>
 struct RowF {
     static constexpr int LD = sld<float>(BB), NQ = BB / 4;
     float4 s[NQ];
+    // a row of a narrower line width (nq < NQ groups of 4, row stride ld)
+    __device__ __forceinline__ void load(const float* __restrict__ S, int lane, int nq, int ld) {
+        const float4* r = reinterpret_cast<const float4*>(S + lane * ld);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) s[q] = q < nq ? r[q] : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
     __device__ __forceinline__ void load(const float* __restrict__ S, int lane) {
         const float4* r = reinterpret_cast<const float4*>(S + (lane < BB ? lane : 0) * LD);
 #pragma unroll
         for (int q = 0; q < NQ; ++q) s[q] = r[q];
     }
-    __device__ __forceinline__ float dot(const float* z) const {
-        const float4* z4 = reinterpret_cast<const float4*>(z);
+    // row . z, entry k of z in lane k
+    __device__ __forceinline__ float dot(float z) const {
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
 #pragma unroll
         for (int q = 0; q < NQ; ++q) {
-            const float4 zz = z4[q];
-            a0 += s[q].x * zz.x;
-            a1 += s[q].y * zz.y;
-            a2 += s[q].z * zz.z;
-            a3 += s[q].w * zz.w;
+            a0 += s[q].x * __shfl_sync(0xffffffffu, z, 4 * q);
+            a1 += s[q].y * __shfl_sync(0xffffffffu, z, 4 * q + 1);
+            a2 += s[q].z * __shfl_sync(0xffffffffu, z, 4 * q + 2);
+            a3 += s[q].w * __shfl_sync(0xffffffffu, z, 4 * q + 3);
         }
         return (a0 + a1) + (a2 + a3);
     }
@@ -653,41 +658,50 @@ __device__ __noinline__ void tw_warp_f32(const float* __restrict__ Sinv, const f
     tw_warp<float, BB>(Sinv, cys, w, z, b, nb);
 }
 
-// Both twisted sweeps on two warps (FP32 row path, lines of width BB): warp
+// Both twisted sweeps on two warps (FP32 row path, lines of width bp <= BB): warp
 // 0 runs the top chain (lines 0 .. m - 1) and warp 1 the bottom chain (lines
-// nb - 1 .. m + 1), each with its rows prefetched a line ahead; after a
-// barrier of the two warps (named barrier 1) warp 0 solves the middle line m
-// from both chains' last lines, and after another the two chains run back out
-// from it.  The line products of tw_warp in the same order, each chain's
-// dependent steps on its own warp; the results agree with tw_warp's to
-// rounding (the compiler may fuse the line inputs' multiply-adds
-// differently).  Called by threads 0 .. 63; z: 64 entries (one line input per
-// warp).
+// nb - 1 .. m + 1); after a barrier of the two warps (named barrier 1) warp 0
+// solves the middle line m from both chains' last lines, and after another
+// the two chains run back out from it.  A line's input stays in registers, an
+// entry a lane, and reaches the others by shuffles; the next line's row and
+// entries are loaded a line ahead: a step is the chain of its BB shuffles and
+// multiply-adds.  (Through shared memory, with the line products of tw_warp,
+// a step took 370 cycles for 24 cells.)  Called by threads 0 .. 63.
 template <int BB>
-__device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w, float* z, int b,
-                         int nb) {
+__device__ __forceinline__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w, int b,
+                                         int nb, int bp) {
     using Row = RowF<BB>;
     const int lane = threadIdx.x & 31, h = (threadIdx.x >> 5) & 1;
     const bool act = lane < b;
-    const size_t bl = (size_t)b * Row::LD;
+    const int row = act ? lane : 0, nq = bp >> 2, ld = sld<float>(bp);
+    const int bl = b * ld;
     const int m = nb >> 1;
     const int cnt = h == 0 ? m : nb - 1 - m;   // lines of this warp's chain
-    float* zz = z + 32 * h;
+    const int d = h == 0 ? 1 : -1;             // the next line, towards the middle
+    const int j0 = h == 0 ? 0 : nb - 1;
+    // the couplings of step s of a chain: between its lines j - d and j, line min(j - d, j)
+    const float* cyl = cys + (h == 0 ? -bp : 0) + lane;
     float c = 0.f;   // this lane's entry of the chain's last finished line
     Row N, P;
-    auto jf = [&](int s) { return h == 0 ? s : nb - 1 - s; };
-    auto fwd = [&](int s, Row& C, Row& X) {
-        const int j = jf(s);
-        zz[lane] = act ? w[j * b + lane] + (s > 0 ? cys[(h == 0 ? j - 1 : j) * BB + lane] * c : 0.f) : 0.f;
-        __syncwarp();
-        if (s + 1 < cnt) X.load(Sinv + (size_t)jf(s + 1) * bl, lane);
-        c = C.dot(zz);
-        if (act) w[j * b + lane] = c;
-        __syncwarp();
+    float wn = 0.f, cn = 0.f;   // w and coupling of the next line
+    auto pre_f = [&](int s, Row& X) {
+        const int j = j0 + d * s;
+        X.load(Sinv + j * bl, row, nq, ld);
+        if (act) {
+            wn = w[j * b + lane];
+            cn = s > 0 ? cyl[j * bp] : 0.f;
+        }
     };
-    if (cnt > 0) N.load(Sinv + (size_t)jf(0) * bl, lane);
+    auto fwd = [&](int s, Row& C, Row& X) {
+        const float z = act ? fmaf(cn, c, wn) : 0.f;
+        if (s + 1 < cnt) pre_f(s + 1, X);
+        c = C.dot(z);
+        if (act) w[(j0 + d * s) * b + lane] = c;
+    };
+    if (cnt > 0) pre_f(0, N);
     {
         int s = 0;
+#pragma unroll 1
         for (; s + 1 < cnt; s += 2) {
             fwd(s, N, P);
             fwd(s + 1, P, N);
@@ -696,36 +710,38 @@ __device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict
     }
     asm volatile("bar.sync 1, 64;" ::: "memory");
     if (h == 0) {
-        Row L;
-        L.load(Sinv + (size_t)m * bl, lane);
-        float zm = 0.f;
+        N.load(Sinv + m * bl, row, nq, ld);
+        float z = 0.f;
         if (act) {
-            zm = w[m * b + lane];
-            if (m > 0) zm += cys[(m - 1) * BB + lane] * w[(m - 1) * b + lane];
-            if (m < nb - 1) zm += cys[m * BB + lane] * w[(m + 1) * b + lane];
+            z = w[m * b + lane];
+            if (m > 0) z += cys[(m - 1) * bp + lane] * w[(m - 1) * b + lane];
+            if (m < nb - 1) z += cys[m * bp + lane] * w[(m + 1) * b + lane];
         }
-        zz[lane] = zm;
-        __syncwarp();
-        const float r = L.dot(zz);
+        const float r = N.dot(z);
         if (act) w[m * b + lane] = r;
     }
     asm volatile("bar.sync 1, 64;" ::: "memory");
     c = act ? w[m * b + lane] : 0.f;
-    auto jb = [&](int s) { return h == 0 ? m - 1 - s : m + 1 + s; };
-    auto bwd = [&](int s, Row& C, Row& X) {
-        const int j = jb(s);
-        float wj = 0.f;
-        zz[lane] = act ? cys[(h == 0 ? j : j - 1) * BB + lane] * c : 0.f;
-        if (act) wj = w[j * b + lane];
-        __syncwarp();
-        if (s + 1 < cnt) X.load(Sinv + (size_t)jb(s + 1) * bl, lane);
-        c = wj + C.dot(zz);
-        if (act) w[j * b + lane] = c;
-        __syncwarp();
+    // back: lines m - d (s = 0) .. j0, coupled to the line finished before
+    auto pre_b = [&](int s, Row& X) {
+        const int j = m - d * (s + 1);
+        X.load(Sinv + j * bl, row, nq, ld);
+        if (act) {
+            wn = w[j * b + lane];
+            cn = cyl[(j + d) * bp];
+        }
     };
-    if (cnt > 0) N.load(Sinv + (size_t)jb(0) * bl, lane);
+    auto bwd = [&](int s, Row& C, Row& X) {
+        const float z = act ? cn * c : 0.f, wj = wn;
+        if (s + 1 < cnt) pre_b(s + 1, X);
+        c = wj + C.dot(z);
+        if (act) w[(m - d * (s + 1)) * b + lane] = c;
+    };
+    wn = cn = 0.f;
+    if (cnt > 0) pre_b(0, N);
     {
         int s = 0;
+#pragma unroll 1
         for (; s + 1 < cnt; s += 2) {
             bwd(s, N, P);
             bwd(s + 1, P, N);
@@ -736,24 +752,24 @@ __device__ void tw_2warp(const float* __restrict__ Sinv, const float* __restrict
 
 template <int BB>
 __device__ __noinline__ void tw_2warp_f32(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w,
-                                          float* z, int b, int nb) {
-    tw_2warp<BB>(Sinv, cys, w, z, b, nb);
+                                          int b, int nb) {
+    tw_2warp<BB>(Sinv, cys, w, b, nb, BB);
 }
 
 // The FP32 sweeps of one right-hand side by threads 0 .. 63: two warps on the
 // row path of the line width bp where there is one, else warp 0 alone by
-// column.  zbuf: 64 entries.  The caller synchronises the block afterwards.
+// column (zbuf: 64 entries, for that).  The caller synchronises the block afterwards.
 __device__ void warp2_sweeps(const float* __restrict__ Sinv, const float* __restrict__ cys, float* w, float* zbuf,
                              int b, int nb, int bp) {
     switch (bp) {
-        case 4: tw_2warp_f32<4>(Sinv, cys, w, zbuf, b, nb); return;
-        case 8: tw_2warp_f32<8>(Sinv, cys, w, zbuf, b, nb); return;
-        case 12: tw_2warp_f32<12>(Sinv, cys, w, zbuf, b, nb); return;
-        case 16: tw_2warp_f32<16>(Sinv, cys, w, zbuf, b, nb); return;
-        case 20: tw_2warp_f32<20>(Sinv, cys, w, zbuf, b, nb); return;
-        case 24: tw_2warp_f32<24>(Sinv, cys, w, zbuf, b, nb); return;
-        case 28: tw_2warp_f32<28>(Sinv, cys, w, zbuf, b, nb); return;
-        case 32: tw_2warp_f32<32>(Sinv, cys, w, zbuf, b, nb); return;
+        case 4: tw_2warp_f32<4>(Sinv, cys, w, b, nb); return;
+        case 8: tw_2warp_f32<8>(Sinv, cys, w, b, nb); return;
+        case 12: tw_2warp_f32<12>(Sinv, cys, w, b, nb); return;
+        case 16: tw_2warp_f32<16>(Sinv, cys, w, b, nb); return;
+        case 20: tw_2warp_f32<20>(Sinv, cys, w, b, nb); return;
+        case 24: tw_2warp_f32<24>(Sinv, cys, w, b, nb); return;
+        case 28: tw_2warp_f32<28>(Sinv, cys, w, b, nb); return;
+        case 32: tw_2warp_f32<32>(Sinv, cys, w, b, nb); return;
         default: break;
     }
     if (threadIdx.x < 32) tw_warp<float, 0>(Sinv, cys, w, zbuf, b, nb);
@@ -1120,6 +1136,8 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
 // chains), FP64 updates and residuals over all threads.  warm: x holds a
 // starting x~ and the refinement starts from its residual (stopping rule
 // still relative to b~; no sweep when the start meets it).  b~ is stored.
+// BB > 0: lines of width at most BB; BB = 0: any width by a switch (bp).
+template <int BB = 0>
 __device__ int cta_solve_sc(const Box& B, const Ops& O, const float* Sinv, const float* cys, double* x, float* w,
                             float* zw, unsigned int* nrm, const double* bt, double tol, int max_ir, int* noconv,
                             bool warm, int bp) {
@@ -1155,7 +1173,11 @@ __device__ int cta_solve_sc(const Box& B, const Ops& O, const float* Sinv, const
     int it = 0;
     if (warm && ((double)r0 <= tol * (double)bn || bn == 0.f)) return 0;
     for (; it < max_ir; ++it) {
-        if (tid < 64) warp2_sweeps(Sinv, cys, w, zw, b, nb, bp);
+        if constexpr (BB > 0) {
+            if (tid < 64) tw_2warp<BB>(Sinv, cys, w, b, nb, bp);
+        } else {
+            if (tid < 64) warp2_sweeps(Sinv, cys, w, zw, b, nb, bp);
+        }
         __syncthreads();
         for (int c = tid; c < B.n; c += nt) x[c] += f2d_bits(w[c]);
         if (tid == 0) nrm[1] = 0u;

@@ -229,18 +229,28 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
 
 // ---------------------------------------------------------------------------
 // Step 7: one colour phase of a smoothing step (Sec. 3, Eqs. (sm_1)-(sm_2)).
-// One CTA (SM_WARPS warps) per subdomain of the colour; the kept factor is
-// staged into shared memory by the bulk-copy (TMA) engine while the
-// coefficients and Robin data are formed; the whole CTA runs the sweeps
-// (each line's product split over the warps) and the FP64 residuals.
+// One CTA per subdomain of the colour; the kept factor is staged into shared
+// memory by the bulk-copy (TMA) engine while the coefficients and Robin data
+// are formed.  Mixed form: FP32 sweeps on two warps, FP64 residuals over the
+// CTA; FP64 form: each line's product split over the warps.
+// One wave of CTAs whose length is one box's chain: state and coefficient
+// loads, sweeps (two warps), residuals, output.  The loads that do not depend
+// on the state are issued before the wait for the previous colour and the
+// state's in one batch (one latency instead of one per side).  8 warps in the
+// mixed form: two CTAs of 24 x 24 boxes still fit an SM (128 registers), and the
+// loads, residuals and output take half the rounds of 4; 4 in the FP64 form,
+// where every warp adds up all warps' partial sums of a line.
 // ---------------------------------------------------------------------------
-constexpr int SM_WARPS = 4;
-
 template <typename T>
-__global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev Mth, const int* items, double* rec,
+constexpr int SMW = sizeof(T) == 4 ? 8 : 4;
+
+// BB: the widest line of the handle's boxes (FP32 with widened lines), else 0.
+template <typename T, int BB>
+__global__ void __launch_bounds__(SMW<T> * 32, 2) k_smooth2d(DevPtrs P, MethodDev Mth, const int* items, double* rec,
                                                             long long rec_stride) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool mixed = std::is_same<T, float>::value;
+    constexpr int NT = SMW<T> * 32;
     const int item = items[blockIdx.x];
     const SubDev sd = P.sub[item];
     const MemberDev& md = P.mem[sd.member];
@@ -267,8 +277,8 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
     auto take = [&](size_t bytes) { unsigned char* p = smem + o; o += align16(bytes); return p; };
     double* lam = (double*)take(sizeof(double) * 2 * (B.nx + B.ny));
     double* lun = (double*)take(sizeof(double) * 2 * (B.nx + B.ny));
-    T* zbuf = (T*)take(sizeof(T) * 32 * SM_WARPS);       // line input of the sweeps
-    T* red = (T*)take(sizeof(T) * 2 * 32 * SM_WARPS);    // partial sums of the warps (FP64 sweeps), two line parities
+    T* zbuf = (T*)take(sizeof(T) * (mixed ? 64 : NT));            // line input of the sweeps
+    T* red = mixed ? nullptr : (T*)take(sizeof(T) * 2 * NT);    // partial sums of the warps (FP64 sweeps), two line parities
     unsigned int* nrm = (unsigned int*)take(16);
     double* x = (double*)take(sizeof(double) * n);
     T* w = mixed ? (T*)take(sizeof(T) * n) : (T*)x;
@@ -287,6 +297,38 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
                        (long long)pbytes))
             bulk_g2s(smem, Pg, pbytes, &bar);
     }
+    // the unscaled face transmissibilities of this thread's first cell of Omega_i (faces x-, x+, y-, y+; shared
+    // memory will hold D A D), and the position of its first box face
+    const int nIx = sd.hi[0] - sd.lo[0], nIy = sd.hi[1] - sd.lo[1];
+    const int offx = sd.lo[0] - B.lo[0], offy = sd.lo[1] - B.lo[1];
+    const double* Tfg = P.Tf + md.cell_off * 3;
+    const int nxg = md.n[0];
+    const long long g00 = B.lo[0] + (long long)nxg * B.lo[1];   // the box's first cell
+    auto face_T = [&](int c, double* tf) {
+        const int i = c % nIx + offx, j = c / nIx + offy;
+        const long long g = g00 + i + (long long)nxg * j;
+        const bool ok = c < nIx * nIy;
+        tf[0] = (ok && i > 0) ? Tfg[(g - 1) * 3 + 0] : 0.0;
+        tf[1] = (ok && i < B.nx - 1) ? Tfg[g * 3 + 0] : 0.0;
+        tf[2] = (ok && j > 0) ? Tfg[(g - nxg) * 3 + 1] : 0.0;
+        tf[3] = (ok && j < B.ny - 1) ? Tfg[g * 3 + 1] : 0.0;
+    };
+    double tfo[4];
+    face_T(threadIdx.x, tfo);
+    const int per = 2 * (B.nx + B.ny);
+    // face f of the box's sides -> side, cell (i, j)
+    auto face_at = [&](int f, int& sid, int& i, int& j) {
+        if (f < 2 * B.ny) {
+            sid = f >= B.ny;
+            i = sid ? B.nx - 1 : 0;
+            j = f - sid * B.ny;
+        } else {
+            const int q = f - 2 * B.ny;
+            sid = 2 + (q >= B.nx);
+            i = q - (sid - 2) * B.nx;
+            j = sid == 3 ? B.ny - 1 : 0;
+        }
+    };
     // launched as a programmatic dependent of the previous colour: the pack
     // (written by the basis kernel, two or more launches earlier) is in flight
     // already; the state is read only once the previous launch is complete
@@ -294,45 +336,48 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // Robin data from the current solution, while the pack is in flight:
     // lambda = -beta u.n + pi with n the outward normal of hat-Omega_i and
-    // pi = p - u.n h / (2K) of the cell inside
+    // pi = p - u.n h / (2K) of the cell inside.  Mixed form: the refinement
+    // starts from the current pressure on the box (scaled once the pack, with
+    // D, has arrived)
     const double* pst = P.p + md.cell_off;
     const double* ust = P.u + md.cell_off * 4;
     const double* hkg = P.hk + md.cell_off * 3;
-    for (int sid = 0; sid < 4; ++sid) {
-        if (B.kind[sid] != 2) continue;
-        const int a = sid >> 1;
-        const int len = a == 0 ? B.ny : B.nx;
-        for (int pos = threadIdx.x; pos < len; pos += blockDim.x) {
-            int i, j;
-            if (a == 0) { j = pos; i = (sid == 0) ? 0 : B.nx - 1; }
-            else        { i = pos; j = (sid == 2) ? 0 : B.ny - 1; }
-            const long long g = (B.lo[0] + i) + (long long)md.n[0] * (B.lo[1] + j);
-            const double un = ust[g * 4 + sid];
-            lun[side_off(B, sid) + pos] = un;
-            lam[side_off(B, sid) + pos] = pst[g] - un * hkg[g * 3 + a];
-        }
-    }
-    // mixed form: the refinement starts from the current pressure on the box
-    // (read now; scaled once the pack, with D, has arrived)
-    if (mixed)
-        for (int c = threadIdx.x; c < B.n; c += blockDim.x)
-            x[c] = pst[(B.lo[0] + c % B.nx) + (long long)md.n[0] * (B.lo[1] + c / B.nx)];
-    // the unscaled face transmissibilities the output needs (shared memory holds D A D), read while the pack
-    // is in flight: this thread's cells of Omega_i, faces x-, x+, y-, y+ (two cells per thread at most)
-    const int nIx = sd.hi[0] - sd.lo[0], nIy = sd.hi[1] - sd.lo[1];
-    const int offx = sd.lo[0] - B.lo[0], offy = sd.lo[1] - B.lo[1];
-    const double* Tfg = P.Tf + md.cell_off * 3;
-    double tfo[2][4];
+    auto load_face = [&](int f, double& un, double& pi) {
+        int sid, i, j;
+        face_at(f, sid, i, j);
+        const long long g = g00 + i + (long long)nxg * j;
+        un = ust[g * 4 + sid];
+        pi = fma(-un, hkg[g * 3 + (sid >> 1)], pst[g]);
+    };
+    {
+        constexpr int NB = 3;   // cells of a thread in the batch
+        double xr[NB], un = 0.0, pi = 0.0;
+        if constexpr (mixed) {
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int c = threadIdx.x + q * blockDim.x;
-        const int i = c % nIx + offx, j = c / nIx + offy;
-        const long long g = (B.lo[0] + i) + (long long)md.n[0] * (B.lo[1] + j);
-        const bool ok = c < nIx * nIy;
-        tfo[q][0] = (ok && i > 0) ? Tfg[(g - 1) * 3 + 0] : 0.0;
-        tfo[q][1] = (ok && i < B.nx - 1) ? Tfg[g * 3 + 0] : 0.0;
-        tfo[q][2] = (ok && j > 0) ? Tfg[(g - md.n[0]) * 3 + 1] : 0.0;
-        tfo[q][3] = (ok && j < B.ny - 1) ? Tfg[g * 3 + 1] : 0.0;
+            for (int k = 0; k < NB; ++k) {
+                const int c = threadIdx.x + k * NT, j = c / B.nx;
+                xr[k] = c < B.n ? pst[g00 + (c - j * B.nx) + (long long)nxg * j] : 0.0;
+            }
+        }
+        if (threadIdx.x < per) load_face(threadIdx.x, un, pi);
+        if constexpr (mixed) {
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
+                const int c = threadIdx.x + k * NT;
+                if (c < B.n) x[c] = xr[k];
+            }
+            for (int c = threadIdx.x + NB * NT; c < B.n; c += NT)
+                x[c] = pst[g00 + c % B.nx + (long long)nxg * (c / B.nx)];
+        }
+        if (threadIdx.x < per) {
+            lun[threadIdx.x] = un;
+            lam[threadIdx.x] = pi;
+        }
+        for (int f = threadIdx.x + NT; f < per; f += NT) {
+            load_face(f, un, pi);
+            lun[f] = un;
+            lam[f] = pi;
+        }
     }
     int it = 0;
     // every thread reads the staged pack: all wait for the copy, and agree on a late one
@@ -340,23 +385,17 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
     // barrier nothing arrives at, for that many cycles: it runs out)
     const bool arrived = Mth.wait0 > 0 ? mbar_wait(&never, 0, Mth.wait0) : mbar_wait(&bar, 0);
     if (!__syncthreads_or(!arrived)) {
-        for (int sid = 0; sid < 4; ++sid) {
-            if (B.kind[sid] != 2) continue;
-            const int len = (sid >> 1) == 0 ? B.ny : B.nx;
-            for (int pos = threadIdx.x; pos < len; pos += blockDim.x)
-                lam[side_off(B, sid) + pos] -= O.bB[side_off(B, sid) + pos] * lun[side_off(B, sid) + pos];
-        }
-        __syncthreads();
-        // Robin terms of the right-hand side, one side at a time (corner cells lie on two)
-        for (int sid = 0; sid < 4; ++sid) {
-            if (B.kind[sid] != 2) continue;
-            const int a = sid >> 1;
-            const int len = a == 0 ? B.ny : B.nx;
-            for (int pos = threadIdx.x; pos < len; pos += blockDim.x) {
-                const int i = a == 0 ? ((sid == 0) ? 0 : B.nx - 1) : pos;
-                const int j = a == 0 ? pos : ((sid == 2) ? 0 : B.ny - 1);
+        // lambda (each face by the thread that loaded it) and the Robin terms of
+        // the right-hand side, one side at a time (a cell may lie on several)
+        for (int side = 0; side < 4; ++side) {
+            for (int f = threadIdx.x; f < per; f += NT) {
+                int sid, i, j;
+                face_at(f, sid, i, j);
+                if (sid != side || B.kind[sid] != 2) continue;
+                const double lv = lam[f] - O.bB[f] * lun[f];
+                lam[f] = lv;
                 const int c = j * B.nx + i;
-                bsrc[c] += O.dsc[c] * (O.bT[side_off(B, sid) + pos] * lam[side_off(B, sid) + pos]);
+                bsrc[c] += O.dsc[c] * (O.bT[f] * lv);
             }
             __syncthreads();
         }
@@ -365,7 +404,7 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
             for (int c = threadIdx.x; c < B.n; c += blockDim.x)
                 x[c] *= f2d_bits(__frcp_rn(d2f_bits(O.dsc[c])));
             __syncthreads();
-            it = cta_solve_sc(B, O, (const float*)Sinv, (const float*)cys, x, (float*)w, (float*)zbuf, nrm, bsrc,
+            it = cta_solve_sc<BB>(B, O, (const float*)Sinv, (const float*)cys, x, (float*)w, (float*)zbuf, nrm, bsrc,
                               Mth.ir_tol, Mth.max_ir, &flags[0], true, line_width(B.nx, sizeof(T), Mth.pad));
             for (int c = threadIdx.x; c < B.n; c += blockDim.x) x[c] *= O.dsc[c];
             __syncthreads();
@@ -391,7 +430,6 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
         // the reverse pass's replay: the box solution and its Robin data
         double* r = rec + (size_t)item * rec_stride;
         for (int c = threadIdx.x; c < B.n; c += blockDim.x) r[c] = x[c];
-        const int per = 2 * (B.nx + B.ny);
         for (int t = threadIdx.x; t < per; t += blockDim.x) {
             r[B.n + t] = lam[t];
             r[B.n + per + t] = lun[t];
@@ -408,16 +446,13 @@ __global__ void __launch_bounds__(SM_WARPS * 32) k_smooth2d(DevPtrs P, MethodDev
         if (!mrcm_check(P.status, g >= 0 && g < (long long)md.n[0] * md.n[1], 4, g)) continue;
         const double pc = x[cl];
         pw[g] = pc;
-        // transmissibilities: prefetched for a thread's first two cells, else read here
+        // transmissibilities: prefetched for a thread's first cell, else read here
         double tf[4];
-        if (q < 2) {
+        if (q == 0) {
 #pragma unroll
-            for (int sid = 0; sid < 4; ++sid) tf[sid] = q == 0 ? tfo[0][sid] : tfo[1][sid];
+            for (int sid = 0; sid < 4; ++sid) tf[sid] = tfo[sid];
         } else {
-            tf[0] = i > 0 ? Tfg[(g - 1) * 3 + 0] : 0.0;
-            tf[1] = i < B.nx - 1 ? Tfg[g * 3 + 0] : 0.0;
-            tf[2] = j > 0 ? Tfg[(g - md.n[0]) * 3 + 1] : 0.0;
-            tf[3] = j < B.ny - 1 ? Tfg[g * 3 + 1] : 0.0;
+            face_T(c, tf);
         }
         double uo[4];
         for (int sid = 0; sid < 4; ++sid) {
@@ -461,7 +496,8 @@ size_t smooth2d_smem(int prec, int nx, int ny, int pad) {
     const size_t tsz = prec == 0 ? sizeof(double) : sizeof(float);
     size_t s = spack_bytes(prec, nx, ny, pad);
     s += align16(sizeof(double) * 2 * (nx + ny)) * 2;
-    s += align16(tsz * 32 * SM_WARPS) + align16(tsz * 2 * 32 * SM_WARPS) + 16;
+    const int nt = 32 * SMW<double>;
+    s += prec == 0 ? align16(tsz * nt) + align16(tsz * 2 * nt) + 16 : align16(tsz * 64) + 16;
     s += align16(sizeof(double) * n);
     if (prec != 0) s += align16(tsz * n);
     return s + 64;
@@ -520,10 +556,10 @@ cudaError_t launch_local2d(const DevPtrs& P, const MethodDev& M, const Job* jobs
     return launch_local_t<float, 32, false>(P, M, jobs, njobs, smem, s);
 }
 
-template <typename T>
+template <typename T, int BB>
 static cudaError_t launch_smooth2d_t(const DevPtrs& P, const MethodDev& M, const int* items, int nitems, size_t smem,
                                      double* rec, long long rec_stride, cudaStream_t s) {
-    auto kern = k_smooth2d<T>;
+    auto kern = k_smooth2d<T, BB>;
     static size_t set_smem = 0;
     if (smem > set_smem) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -534,7 +570,7 @@ static cudaError_t launch_smooth2d_t(const DevPtrs& P, const MethodDev& M, const
     // previous kernel drains
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nitems);
-    cfg.blockDim = dim3(SM_WARPS * 32);
+    cfg.blockDim = dim3(SMW<T> * 32);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -553,6 +589,16 @@ static cudaError_t launch_smooth2d_t(const DevPtrs& P, const MethodDev& M, const
 cudaError_t launch_smooth2d(const DevPtrs& P, const MethodDev& M, const int* items, int nitems, size_t smem,
                             double* rec, long long rec_stride, cudaStream_t s) {
     if (nitems == 0) return cudaSuccess;
-    return M.prec == 0 ? launch_smooth2d_t<double>(P, M, items, nitems, smem, rec, rec_stride, s)
-                       : launch_smooth2d_t<float>(P, M, items, nitems, smem, rec, rec_stride, s);
+    if (M.prec == 0) return launch_smooth2d_t<double, 0>(P, M, items, nitems, smem, rec, rec_stride, s);
+    switch (M.pad) {
+        case 4: return launch_smooth2d_t<float, 4>(P, M, items, nitems, smem, rec, rec_stride, s);
+        case 8: return launch_smooth2d_t<float, 8>(P, M, items, nitems, smem, rec, rec_stride, s);
+        case 12: return launch_smooth2d_t<float, 12>(P, M, items, nitems, smem, rec, rec_stride, s);
+        case 16: return launch_smooth2d_t<float, 16>(P, M, items, nitems, smem, rec, rec_stride, s);
+        case 20: return launch_smooth2d_t<float, 20>(P, M, items, nitems, smem, rec, rec_stride, s);
+        case 24: return launch_smooth2d_t<float, 24>(P, M, items, nitems, smem, rec, rec_stride, s);
+        case 28: return launch_smooth2d_t<float, 28>(P, M, items, nitems, smem, rec, rec_stride, s);
+        case 32: return launch_smooth2d_t<float, 32>(P, M, items, nitems, smem, rec, rec_stride, s);
+        default: return launch_smooth2d_t<float, 0>(P, M, items, nitems, smem, rec, rec_stride, s);
+    }
 }

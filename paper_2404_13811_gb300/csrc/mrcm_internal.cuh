@@ -105,7 +105,8 @@ struct MethodDev {
     double ir_tol;
     int max_ir;
     int same_alpha;
-    int pad;           // 2D FP32 forms: lines widened to a multiple of 4 (0 where the boxes would not fit)
+    int pad;           // 2D FP32 forms: lines widened to a multiple of 4, the widest of the handle's boxes (0: not
+                       // widened, where the boxes would not fit)
     int part_hat;      // the particular problem on hat-Omega_i (one more right-hand side of the basis job)
     long long wait0;   // cycle limit of the first wait for a staged copy in the 2D smoothing kernel
 };
