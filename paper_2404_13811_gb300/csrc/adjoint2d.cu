@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
         __syncthreads();
     } else {
         RhsStored rs{rt};
-        cta_solve<T>(B, O, Sinv, cys, mu, w, zbuf, red, nrm, rs, Mth.ir_tol, Mth.max_ir, &flags[0], false);
+        cta_solve64(B, O, Sinv, cys, mu, red, rs);
     }
 
     // interior faces: dL/dTf = (gu_L - gu_R) dp / a - (mu_L - mu_R) dp

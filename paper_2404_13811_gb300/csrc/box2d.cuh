@@ -381,6 +381,211 @@ __device__ __forceinline__ void store_line(const T (&a)[BW], T* S, int b, int ld
     }
 }
 
+// 1 / v for the pivots.  FP32: the hardware approximation and one
+// Newton-Raphson step.  FP64: from the FP32 seed r one third-order step,
+// r + r (e + e^2) with e = 1 - v r (e is about 2^-22, the error left e^3); the
+// conversions on the integer pipe.  Outside the FP32 normal range the division.
+__device__ __forceinline__ float rcp_piv(float v) {
+    float r;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return fmaf(r, fmaf(-v, r, 1.f), r);
+}
+__device__ __forceinline__ double rcp_piv(double v) {
+    if (!in_f32_range(v)) return 1.0 / v;
+    const double r = f2d_bits(__frcp_rn(d2f_bits(v)));
+    const double e = fma(-v, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+
+// The FP64 form of the twisted factorisation for lines of 12 to 28 cells
+// (four warps).  Two warps run each chain: a line block is held as the 4 x 4
+// tiles (I, J), I <= J, of its upper triangle -- in-place Gauss-Jordan keeps
+// M_IJ = +-M_JI^T, minus when exactly one of I, J has been eliminated -- tile t
+// in lane t, rows 0-1 of it in the chain's first warp and rows 2-3 in the
+// second.  Pivots go by blocks K of 4: the panel M_K. and its product with the
+// inverse pivot block P = M_KK^-1 pass through shared memory (in the block's
+// own storage, which is written only once the line is done), each warp
+// inverts the next pivot block with an entry per lane while its tiles are
+// updated.  The inverse of the last line stays in the registers, where the
+// next one is formed from it.
+// Bound by the FP64 pipe (a warp instruction takes 64 cycles of its quarter of
+// the SM).  With one warp per chain, whole rows, a shuffle per entry and the
+// full square a line of 24 cells took 70k cycles.
+constexpr int F64_MIN = 12, F64_MAX = 28;
+
+__device__ __forceinline__ void bar_pair(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+
+__device__ void factor_box64(const Box& B, const Ops& O, double* Sinv, const double* cys, const double* cxs, int* bad) {
+    const int b = B.nx, nb = B.ny, nb4 = (b + 3) >> 2, bp = 4 * nb4, m = nb >> 1;
+    const int bl = b * b;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int h = warp >> 1, y0 = 2 * (warp & 1);   // chain; first tile row of this warp
+    const bool act = lane < nb4 * (nb4 + 1) / 2;
+    int I = 0, J = lane;
+    if (act) {
+        while (J >= nb4 - I) {
+            J -= nb4 - I;
+            ++I;
+        }
+        J += I;
+    } else {
+        I = J = -4;
+    }
+    const int py = (lane >> 2) & 3, px = lane & 3;   // entry of a pivot block held by this lane
+    double V[2][4];
+#pragma unroll
+    for (int y = 0; y < 2; ++y)
+#pragma unroll
+        for (int x = 0; x < 4; ++x) V[y][x] = 0.0;
+    auto invert = [&](double v) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            double piv = __shfl_sync(0xffffffffu, v, 5 * q);
+            if (!(piv > 0.0)) {
+                if (lane == 0) *bad = 1;
+                piv = 1.0;
+            }
+            const double ip = rcp_piv(piv);
+            const double r = __shfl_sync(0xffffffffu, v, 4 * q + px), c = __shfl_sync(0xffffffffu, v, 4 * py + q);
+            const double rp = px == q ? ip : r * ip;
+            v = py == q ? rp : (px == q ? 0.0 : v) - c * rp;
+        }
+        return v;
+    };
+    // line block j in V (from the last inverse in V when up, minus the kept inverse dn of line j + 1 for the middle
+    // line), its inverse in V and in Sinv
+    auto line = [&](int j, bool chained, int jc, const double* dn) {
+        double* S = Sinv + (size_t)j * bl;
+        double* R = S;             // [4][bp]
+        double* Rn = S + 4 * bp;   // [4][bp]
+        double* D = S + 8 * bp;    // [16] the next pivot block before this block's update
+        if (act) {
+#pragma unroll
+            for (int y = 0; y < 2; ++y) {
+                const int i = 4 * I + y0 + y;
+                const double ci = (chained && i < b) ? cys[jc * b + i] : 0.0;
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int k = 4 * J + x;
+                    double s;
+                    if (i >= b || k >= b) {
+                        s = i == k ? 1.0 : 0.0;   // padding: the identity
+                    } else {
+                        const double vs = V[y][x];
+                        if (i == k) {
+                            // c (c S_ii), not c^2 S_ii (range at tiny couplings)
+                            s = O.cd[j * b + i] * O.dsc[j * b + i] * O.dsc[j * b + i];
+                            if (chained) s -= ci * (ci * vs);
+                        } else {
+                            s = chained ? -(ci * vs * cys[jc * b + k]) : 0.0;
+                            if (k == i + 1) s += cxs[j * b + i];
+                            if (k == i - 1) s += cxs[j * b + k];
+                        }
+                        if (dn) s -= cys[j * b + i] * dn[i * b + k] * cys[j * b + k];
+                    }
+                    V[y][x] = s;
+                }
+            }
+        }
+        double p = 0.0;
+#pragma unroll 1
+        for (int k = 0; k < nb4; ++k) {
+            if (I == k) {
+#pragma unroll
+                for (int y = 0; y < 2; ++y)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) R[(y0 + y) * bp + 4 * J + x] = V[y][x];
+            } else if (J == k) {
+                // I < k has been eliminated: M_kI = -M_Ik^T
+#pragma unroll
+                for (int y = 0; y < 2; ++y)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) R[x * bp + 4 * I + y0 + y] = -V[y][x];
+            }
+            if (I == k + 1 && J == k + 1) {
+#pragma unroll
+                for (int y = 0; y < 2; ++y)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) D[4 * (y0 + y) + x] = V[y][x];
+            }
+            bar_pair(2 + h);
+            if (k == 0) p = invert(R[py * bp + px]);
+            {
+                // rows y0, y0 + 1 of P M_k., column `lane`
+                const int c = lane < bp ? lane : 0;
+                const double r0 = R[c], r1 = R[bp + c], r2 = R[2 * bp + c], r3 = R[3 * bp + c];
+#pragma unroll
+                for (int y = 0; y < 2; ++y) {
+                    const int s = 4 * (y0 + y);
+                    const double q0 = __shfl_sync(0xffffffffu, p, s), q1 = __shfl_sync(0xffffffffu, p, s + 1);
+                    const double q2 = __shfl_sync(0xffffffffu, p, s + 2), q3 = __shfl_sync(0xffffffffu, p, s + 3);
+                    const double own = __shfl_sync(0xffffffffu, p, s + (c & 3));
+                    const double v = (q0 * r0 + q1 * r1) + (q2 * r2 + q3 * r3);
+                    if (lane < bp) Rn[(y0 + y) * bp + c] = (c >> 2) == k ? own : v;
+                }
+            }
+            bar_pair(2 + h);
+            if (k + 1 < nb4) {
+                // the next pivot block, updated here and inverted
+                const int c = 4 * (k + 1);
+                double v = D[lane & 15];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) v -= R[q * bp + c + py] * Rn[q * bp + c + px];
+                p = invert(v);
+            }
+            if (I == k) {
+#pragma unroll
+                for (int y = 0; y < 2; ++y)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) V[y][x] = Rn[(y0 + y) * bp + 4 * J + x];
+            } else if (J == k) {
+#pragma unroll
+                for (int y = 0; y < 2; ++y)
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) V[y][x] = Rn[x * bp + 4 * I + y0 + y];
+            } else if (act) {
+                // V -= M_IK (P M_KJ), M_IK = R^T where I is not eliminated yet, else -R^T
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    double a[2];
+#pragma unroll
+                    for (int y = 0; y < 2; ++y) {
+                        a[y] = R[q * bp + 4 * I + y0 + y];
+                        a[y] = I > k ? -a[y] : a[y];
+                    }
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        const double r = Rn[q * bp + 4 * J + x];
+#pragma unroll
+                        for (int y = 0; y < 2; ++y) V[y][x] = fma(a[y], r, V[y][x]);
+                    }
+                }
+            }
+            bar_pair(2 + h);
+        }
+        if (act) {
+#pragma unroll
+            for (int y = 0; y < 2; ++y)
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int i = 4 * I + y0 + y, k = 4 * J + x;
+                    if (i < b && k < b) {
+                        S[i * b + k] = V[y][x];
+                        if (I != J) S[k * b + i] = V[y][x];
+                    }
+                }
+        }
+    };
+    const int cnt = h == 0 ? m : nb - 1 - m;
+    for (int s = 0; s < cnt; ++s) {
+        const int j = h == 0 ? s : nb - 1 - s;
+        line(j, s > 0, h == 0 ? j - 1 : j, nullptr);
+    }
+    __syncthreads();
+    if (h == 0) line(m, m > 0, m - 1, m < nb - 1 ? Sinv + (size_t)(m + 1) * bl : nullptr);
+    __syncthreads();
+}
+
 // Twisted block LDL^T factorisation: Sinv[j] as above.  cys / cxs: the scaled
 // line / in-line couplings (type T, formed once by all threads).  Warp 0
 // runs the top chain and then the middle line, warp 1 the bottom chain.
@@ -405,6 +610,12 @@ __device__ void factor_box(const Box& B, const Ops& O, T* Sinv, T* cys, T* cxs, 
     if (EX && b < BW)
         for (int t = tid; t < nb * (BW - b); t += nt) cys[(t / (BW - b)) * BW + b + t % (BW - b)] = T(0);
     __syncthreads();
+    if constexpr (std::is_same<T, double>::value && BW >= 16) {
+        if (b >= F64_MIN && b <= F64_MAX && blockDim.x == 128) {
+            factor_box64(B, O, Sinv, cys, cxs, bad);
+            return;
+        }
+    }
     const int warp = tid >> 5;
     const int m = nb >> 1;
     if (warp < 2) {
@@ -886,158 +1097,82 @@ __device__ int warp_solve(const Box& B, const Ops& O, const T* Sinv, const T* cy
     }
 }
 
-// One line product of an FP64 CTA-wide sweep: lane's entry of S zin with the
-// columns split over the warps (warp q reduces columns [q kq, (q + 1) kq)),
-// partial sums met in red (double-buffered by line parity: one block
-// barrier per line).  Every warp forms the line input in its own 32 entries
-// of zw and returns the full sum.
-template <typename T>
-__device__ __forceinline__ T cta_line(const T* __restrict__ S, T zin, T* zw, T* red, int& par, int b, int ld) {
-    const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5, nq = blockDim.x >> 5;
-    const int kq = (b + nq - 1) / nq, ka = wq * kq, kb = min(b, ka + kq);
-    T* z = zw + wq * 32;
-    if (lane < b) z[lane] = zin;
-    __syncwarp();
-    if (lane < b) {
-        T acc = T(0);
-        for (int k = ka; k < kb; ++k) acc += S[k * ld + lane] * z[k];
-        red[(par * nq + wq) * 32 + lane] = acc;
+// The twisted sweeps of an FP64 solve by four warps: two per chain, each with
+// half of a line product's columns (the narrow FP64 pipe is fed by all four
+// quarters of the SM), the line input passed by shuffles, the halves' sums met
+// in red (double-buffered by line parity: one barrier of the pair per line).
+// w: the right-hand side in, the solution out; red: 8 x 32 entries.  (The four
+// warps on one chain after the other took 1.7k cycles a line of 24 cells: twice
+// as many steps, and a chain of six multiply-adds and four sums in each.)
+__device__ void tw_4warp64(const double* __restrict__ Sinv, const double* __restrict__ cys, double* w, double* red,
+                           int b, int nb) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int h = warp >> 1, q = warp & 1;
+    const bool act = lane < b;
+    const int row = act ? lane : 0;
+    const size_t bl = (size_t)b * b;
+    const int m = nb >> 1, cnt = h == 0 ? m : nb - 1 - m, d = h == 0 ? 1 : -1, j0 = h == 0 ? 0 : nb - 1;
+    const int kq = (b + 1) >> 1, ka = q * kq, kb = min(b, ka + kq);
+    const double* cyl = cys + (h == 0 ? -b : 0) + row;   // coupling towards the line before, as in tw_2warp
+    int par = 0;
+    auto prod = [&](const double* S, double z) {
+        double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+        const double* s = S + (size_t)ka * b + row;
+        int k = ka;
+        for (; k + 3 < kb; k += 4, s += 4 * b) {
+            a0 = fma(s[0], __shfl_sync(0xffffffffu, z, k), a0);
+            a1 = fma(s[b], __shfl_sync(0xffffffffu, z, k + 1), a1);
+            a2 = fma(s[2 * b], __shfl_sync(0xffffffffu, z, k + 2), a2);
+            a3 = fma(s[3 * b], __shfl_sync(0xffffffffu, z, k + 3), a3);
+        }
+        for (; k < kb; ++k, s += b) a0 = fma(s[0], __shfl_sync(0xffffffffu, z, k), a0);
+        const double mine = (a0 + a1) + (a2 + a3);
+        red[(par * 4 + warp) * 32 + lane] = mine;
+        bar_pair(2 + h);
+        const double other = red[(par * 4 + (warp ^ 1)) * 32 + lane];
+        par ^= 1;
+        return mine + other;
+    };
+    double c = 0.0;
+    for (int s = 0; s < cnt; ++s) {
+        const int j = j0 + d * s;
+        double z = 0.0;
+        if (act) z = s > 0 ? fma(cyl[j * b], c, w[j * b + lane]) : w[j * b + lane];
+        c = prod(Sinv + j * bl, z);
+        if (q == 0 && act) w[j * b + lane] = c;
     }
     __syncthreads();
-    T s = T(0);
-    if (lane < b)
-        for (int q = 0; q < nq; ++q) s += red[(par * nq + q) * 32 + lane];
-    par ^= 1;
-    __syncwarp();
-    return s;
-}
-
-// The twisted sweeps of a CTA-wide solve.  FP32: warp 0 runs both chains
-// interleaved (as in a warp solve); the other warps wait at the closing
-// barrier.  FP64 (bound by the narrow FP64 pipe, which every warp's share of
-// a line product feeds): one chain after the other with each line product
-// split over all warps.  w: the scaled right-hand side in, the solution out;
-// zw: 32 entries per warp (at least 64).
-template <typename T>
-__device__ void cta_sweeps(const T* __restrict__ Sinv, const T* __restrict__ cys, T* w, T* zw, T* red, int b,
-                           int nb) {
-    if constexpr (std::is_same<T, float>::value) {
-        if (threadIdx.x < 32) warp_sweeps<float>(Sinv, cys, w, zw, b, nb, b);
-        __syncthreads();
-        return;
-    } else {
-        const int lane = threadIdx.x & 31, wq = threadIdx.x >> 5;
-        const int ld = sld<T>(b);
-        const size_t bl = (size_t)b * ld;
-        const int m = nb >> 1;
-        int par = 0;
-        T cur = T(0);
-        for (int j = 0; j < m; ++j) {
-            const T zin = lane < b ? w[j * b + lane] + (j > 0 ? cys[(j - 1) * b + lane] * cur : T(0)) : T(0);
-            cur = cta_line<T>(Sinv + j * bl, zin, zw, red, par, b, ld);
-            if (wq == 0 && lane < b) w[j * b + lane] = cur;
+    if (h == 0) {
+        double z = 0.0;
+        if (act) {
+            z = w[m * b + lane];
+            if (m > 0) z += cys[(m - 1) * b + lane] * c;
+            if (m < nb - 1) z += cys[m * b + lane] * w[(m + 1) * b + lane];
         }
-        const T ct = cur;
-        cur = T(0);
-        for (int j = nb - 1; j > m; --j) {
-            const T zin = lane < b ? w[j * b + lane] + (j < nb - 1 ? cys[j * b + lane] * cur : T(0)) : T(0);
-            cur = cta_line<T>(Sinv + j * bl, zin, zw, red, par, b, ld);
-            if (wq == 0 && lane < b) w[j * b + lane] = cur;
-        }
-        const T cbt = cur;
-        T zm = T(0);
-        if (lane < b) {
-            zm = w[m * b + lane];
-            if (m > 0) zm += cys[(m - 1) * b + lane] * ct;
-            if (m < nb - 1) zm += cys[m * b + lane] * cbt;
-        }
-        const T xm = cta_line<T>(Sinv + m * bl, zm, zw, red, par, b, ld);
-        if (wq == 0 && lane < b) w[m * b + lane] = xm;
-        cur = xm;
-        for (int j = m - 1; j >= 0; --j) {
-            const T wf = lane < b ? w[j * b + lane] : T(0);
-            const T zin = lane < b ? cys[j * b + lane] * cur : T(0);
-            cur = wf + cta_line<T>(Sinv + j * bl, zin, zw, red, par, b, ld);
-            if (wq == 0 && lane < b) w[j * b + lane] = cur;
-        }
-        cur = xm;
-        for (int j = m + 1; j < nb; ++j) {
-            const T wf = lane < b ? w[j * b + lane] : T(0);
-            const T zin = lane < b ? cys[(j - 1) * b + lane] * cur : T(0);
-            cur = wf + cta_line<T>(Sinv + j * bl, zin, zw, red, par, b, ld);
-            if (wq == 0 && lane < b) w[j * b + lane] = cur;
-        }
-        __syncthreads();
+        const double r = prod(Sinv + m * bl, z);
+        if (q == 0 && act) w[m * b + lane] = r;
     }
+    __syncthreads();
+    c = act ? w[m * b + lane] : 0.0;
+    for (int s = 0; s < cnt; ++s) {
+        const int j = m - d * (s + 1);
+        const double z = act ? cyl[(j + d) * b] * c : 0.0;
+        const double wj = act ? w[j * b + lane] : 0.0;
+        c = wj + prod(Sinv + j * bl, z);
+        if (q == 0 && act) w[j * b + lane] = c;
+    }
+    __syncthreads();
 }
 
-// One right-hand side solved by the whole CTA (as warp_solve: FP64 form one
-// solve; mixed form FP32 sweeps + FP64 residual refinement, residual and
-// norms over all threads).  nrm: 2 unsigned ints of shared memory.  warm
-// (mixed form): x holds a starting iterate on entry and the refinement
-// starts from its residual; the stopping rule stays relative to the
-// right-hand side, so the result meets the same tolerance, and no sweep is
-// run when the start already does.
-template <typename T, typename Rhs>
-__device__ int cta_solve(const Box& B, const Ops& O, const T* Sinv, const T* cys, double* x, T* w, T* zw, T* red,
-                         unsigned int* nrm, const Rhs& rhs, double tol, int max_ir, int* noconv, bool warm = false) {
-    const int tid = threadIdx.x, nt = blockDim.x;
+// One right-hand side by the whole CTA in the FP64 form: one solve.
+template <typename Rhs>
+__device__ int cta_solve64(const Box& B, const Ops& O, const double* Sinv, const double* cys, double* w, double* red,
+                           const Rhs& rhs) {
     const int b = B.nx, nb = B.ny;
-    if (std::is_same<T, double>::value) {
-        for (int c = tid; c < B.n; c += nt) w[c] = (T)rhs(B, O, c % b, c / b);
-        __syncthreads();
-        cta_sweeps<T>(Sinv, cys, w, zw, red, b, nb);
-        return 1;
-    }
-    if (tid < 2) nrm[tid] = 0u;
+    for (int c = threadIdx.x; c < B.n; c += blockDim.x) w[c] = rhs(B, O, c % b, c / b);
     __syncthreads();
-    float bn = 0.f, r0 = 0.f;
-    for (int c = tid; c < B.n; c += nt) {
-        const int i = c % b, j = c / b;
-        const double bc = rhs(B, O, i, j);
-        const T wc = (T)(O.dsc[c] * (warm ? bc - apply_A(B, O, x, i, j) : bc));
-        w[c] = wc;
-        bn = fmaxf(bn, fabsf((float)(O.dsc[c] * bc)));
-        r0 = fmaxf(r0, fabsf((float)wc));
-    }
-    if (!warm)
-        for (int c = tid; c < B.n; c += nt) x[c] = 0.0;
-    for (int o = 16; o; o >>= 1) {
-        bn = fmaxf(bn, __shfl_xor_sync(0xffffffffu, bn, o));
-        r0 = fmaxf(r0, __shfl_xor_sync(0xffffffffu, r0, o));
-    }
-    if ((tid & 31) == 0) {
-        atomicMax(&nrm[0], __float_as_uint(bn));
-        atomicMax(&nrm[1], __float_as_uint(r0));
-    }
-    __syncthreads();
-    bn = __uint_as_float(nrm[0]);
-    r0 = __uint_as_float(nrm[1]);
-    __syncthreads();   // nrm[1] is reset at the top of the first step
-    int it = 0;
-    if (warm && ((double)r0 <= tol * (double)bn || bn == 0.f)) return 0;
-    for (; it < max_ir; ++it) {
-        cta_sweeps<T>(Sinv, cys, w, zw, red, b, nb);
-        for (int c = tid; c < B.n; c += nt) x[c] += O.dsc[c] * (double)w[c];
-        if (tid == 0) nrm[1] = 0u;
-        __syncthreads();
-        float rn = 0.f;
-        for (int c = tid; c < B.n; c += nt) {
-            const int i = c % b, j = c / b;
-            const T wc = (T)(O.dsc[c] * (rhs(B, O, i, j) - apply_A(B, O, x, i, j)));
-            w[c] = wc;
-            rn = fmaxf(rn, fabsf((float)wc));
-        }
-        for (int o = 16; o; o >>= 1) rn = fmaxf(rn, __shfl_xor_sync(0xffffffffu, rn, o));
-        if ((tid & 31) == 0) atomicMax(&nrm[1], __float_as_uint(rn));
-        __syncthreads();
-        rn = __uint_as_float(nrm[1]);
-        if ((double)rn <= tol * (double)bn || bn == 0.f) { ++it; break; }
-        if (it == max_ir - 1 && tid == 0) *noconv = 1;
-        __syncthreads();   // nrm[1] is reset at the top of the next step
-    }
-    __syncthreads();
-    return it;
+    tw_4warp64(Sinv, cys, w, red, b, nb);
+    return 1;
 }
 
 // --- the mixed form's refinement in scaled variables -------------------------

@@ -410,7 +410,7 @@ __global__ void __launch_bounds__(SMW<T> * 32, 2) k_smooth2d(DevPtrs P, MethodDe
             __syncthreads();
         } else {
             RhsStored rs{bsrc};
-            it = cta_solve<T>(B, O, Sinv, cys, x, w, zbuf, red, nrm, rs, Mth.ir_tol, Mth.max_ir, &flags[0], false);
+            it = cta_solve64(B, O, Sinv, cys, x, red, rs);
         }
     } else if (threadIdx.x == 0) {
         flags[1] = 1;

@@ -248,22 +248,6 @@ __device__ __forceinline__ void stv4(T* p, T a, T b, T c, T d) {
     }
 }
 
-// 1 / v for the pivots.  FP32: the hardware approximation and one
-// Newton-Raphson step.  FP64: from the FP32 seed r one third-order step,
-// r + r (e + e^2) with e = 1 - v r (e is about 2^-22, the error left e^3); the
-// conversions on the integer pipe.  Outside the FP32 normal range the division.
-__device__ __forceinline__ float rcp_piv(float v) {
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return fmaf(r, fmaf(-v, r, 1.f), r);
-}
-__device__ __forceinline__ double rcp_piv(double v) {
-    if (!in_f32_range(v)) return 1.0 / v;
-    const double r = f2d_bits(__frcp_rn(d2f_bits(v)));
-    const double e = fma(-v, r, 1.0);
-    return fma(r, fma(e, e, e), r);
-}
-
 // Workspace of the register inverses (entries): two panels of GT3 rows, the
 // scaled panel, two inverse pivot blocks, two diagonal tiles, the diagonal of
 // the last inverse and of the next Schur block.
@@ -825,8 +809,7 @@ __device__ __forceinline__ void warp_max_to(unsigned int* a, float v) {
 // Solves A x_q = rhs_q for NR right-hand sides with the whole CTA: sweeps
 // with the kept factor (FP32 in the mixed form, FP64 in the FP64 form) and
 // refinement with FP64 residuals, the iterate X in FP64 (mixed form: the
-// scaled x~ = D^-1 x until the end, rhs scaled).  warm (mixed form): X holds
-// a starting x~.  High-contrast boxes reach a residual floor above what a
+// scaled x~ = D^-1 x until the end, rhs scaled).  warm: X holds a starting x~.  High-contrast boxes reach a residual floor above what a
 // fixed tolerance can ask for, so the refinement runs to that floor: it stops
 // when every right-hand side has |r| <= 1e-3 ir_tol |b| (scaled max norms),
 // or has |r| <= ir_tol |b| and no longer halves its residual per step.  The
@@ -1380,18 +1363,17 @@ __global__ void __launch_bounds__(T3, 1) k_smooth3d(DevPtrs P, MethodDev Mth, co
     const double* fm = P.f + md.cell_off;
     for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
         C.bsrc[t] = (mixed ? C.O.dsc[t] : 1.0) * source_rhs3(B, C.O, md, fm, C.lam, t);
-        if constexpr (mixed) {
-            // the refinement starts from the current pressure, scaled (a start only: an FP32 reciprocal)
-            int c[3];
-            bcoord(B, t, c);
-            C.X[t] = pst[gidx(B, md, c)] * f2d_bits(__frcp_rn(d2f_bits(C.O.dsc[t])));
-        }
+        // the refinement starts from the current pressure (mixed form: scaled by an FP32 reciprocal, a start only)
+        int c[3];
+        bcoord(B, t, c);
+        const double pt = pst[gidx(B, md, c)];
+        C.X[t] = mixed ? pt * f2d_bits(__frcp_rn(d2f_bits(C.O.dsc[t]))) : pt;
     }
     __syncthreads();
     const T* F = (const T*)P.fac + (size_t)item * P.fac_stride;
     RhsStored3 rs{C.bsrc};
     const int it = solve3_n<T, 1>(B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rs, Mth.ir_tol, Mth.max_ir,
-                                  &C.flags[0], &C.flags[2], mixed);
+                                  &C.flags[0], &C.flags[2], true);
     if (C.flags[2]) drain3(C.pp);
     __syncthreads();
     // overwrite (u, p) on Omega_i with the restriction
