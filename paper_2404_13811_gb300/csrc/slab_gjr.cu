@@ -17,8 +17,9 @@
 //     column's values with the entry of row p zeroed (the multipliers), p
 //     and the pivot into the panel's record in its CTA's shared memory; the
 //     finished record goes to every other CTA of the cluster by one bulk
-//     copy each (completing an mbarrier there by its bytes) and is released
-//     in its own CTA by one arrival;
+//     copy each (completing an mbarrier there by its bytes), in clusters of
+//     more than 8 CTAs by one multicast copy out of global memory, and is
+//     released in its own CTA by one arrival;
 //   * every other warp waits for the record and applies the panel's CB
 //     rank-1 updates to its own columns in turn, each taking the pivot row's
 //     current values on its columns from the lane holding row p (selected
@@ -127,7 +128,8 @@ struct GrShape {
     static constexpr int REC = CB * NPAD + HDR;     // floats per record
     static_assert(RA % 4 == 0 && (RA < 8 || RA % 8 == 0) && RA <= 32 && CB % 4 == 0 && CB * NW * CL == NPAD,
                   "unsupported slab inverse shape");
-    static constexpr int G = NPAD >= 768 ? 2 : NPAD >= 512 ? 4 : 8;   // panels between cluster barriers
+    static constexpr int G = NPAD >= 768 ? 3 : NPAD >= 512 ? 4 : 8;   // panels between cluster barriers
+    static constexpr bool MC = CL > 8;              // records by multicast through global memory
     static constexpr int R = 2 * G;                  // record slots (one panel each)
     static constexpr size_t smem() { return sizeof(float) * ((size_t)R * REC + (size_t)NW * NPAD * CB); }
 };
@@ -144,8 +146,9 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
     __shared__ int colready[R];            // columns of a slot's record written so far (P CB + c + 1)
     __shared__ int pivrow[NPAD];           // pivot row of every step
     __shared__ float pivval[NPAD];         // its pivot
-    __shared__ int pinv[NPAD];             // step at which each row was the pivot
-    __shared__ float rsc[NPAD];            // 1 / c_i
+    // after the elimination, in the place of the panel-start copies
+    int* pinv = reinterpret_cast<int*>(tiles);   // step at which each row was the pivot
+    float* rsc = tiles + NPAD;                   // 1 / c_i
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const unsigned rank = gr_rank();
@@ -156,6 +159,10 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
     const int npan = (n + CB - 1) / CB;    // panels holding a column below n
     const float* A = I.D + S.offD;
     float* Ainv = I.Dinv + S.offD;
+    // (MC) where the records pass through: the slab's own block, read into
+    // registers before the first record and not needed after (n^2 entries
+    // against R records of 4 n)
+    float* grec = I.D + S.offD;
 
     // the transposed slab: entry (i, j) of D^T is A[i np + j] in D's
     // column-major storage, so a lane's CB consecutive columns of row i are
@@ -306,6 +313,15 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
                 for (int q = 0; q < RA / 4; ++q)
                     *reinterpret_cast<float4*>(rc + c * NPAD + lane * RA + 4 * q) =
                         make_float4(col[4 * q], col[4 * q + 1], col[4 * q + 2], col[4 * q + 3]);
+                if constexpr (Sh::MC) {
+#pragma unroll
+                    for (int q = 0; q < RA / 4; ++q)
+                        *reinterpret_cast<float4*>(grec + slot * REC + c * NPAD + lane * RA + 4 * q) =
+                            make_float4(col[4 * q], col[4 * q + 1], col[4 * q + 2], col[4 * q + 3]);
+                    if (lane == 0)
+                        *reinterpret_cast<float4*>(grec + slot * REC + CB * NPAD + 4 * c) =
+                            make_float4(__int_as_float(p), piv, ip, 0.f);
+                }
                 if (lane == 0) {
                     *reinterpret_cast<float4*>(rc + CB * NPAD + 4 * c) = make_float4(__int_as_float(p), piv, ip, 0.f);
                     pivrow[k] = p;
@@ -344,13 +360,30 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
                 for (int a = 0; a < RA; ++a) V[a][c] = (lane + 32 * a == p) ? 1.f : -col[a] * ip;
                 if (lane == (p & 31)) usedm |= 1u << (p >> 5);
             }
-            // the finished record: one bulk copy into every other CTA (the
-            // copy engine reads it after the proxy fence), one arrival here
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            // the finished record: one arrival here, and to the other CTAs one
+            // multicast bulk copy from global memory (clusters of more than 8:
+            // 15 copies of a 12 KB record through one SM's port took longer
+            // than the panel; slabs of 540 to 740 unknowns 986 -> 707 us and
+            // 1520 -> 1106 us a level) or one bulk copy each (the copy engine reads the
+            // record after the proxy fence)
+            if constexpr (Sh::MC) {
+                __threadfence();
+                asm volatile("fence.proxy.async;" ::: "memory");
+            } else {
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
             __syncwarp();
             if (lane == 0) {
                 gr_arrive(bar);   // this CTA's warps first: the next panel's owner is most often here
                 const unsigned src = rbase + 4u * (unsigned)(slot * REC);
+                if constexpr (Sh::MC) {
+                    const unsigned short mask = (unsigned short)(((1u << CL) - 1u) & ~(1u << rank));
+                    asm volatile(
+                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], "
+                        "%2, [%3], %4;" ::"r"(src),
+                        "l"(grec + slot * REC), "r"(BYTES), "r"(bar), "h"(mask)
+                        : "memory");
+                } else {
 #pragma unroll 1
                 for (int r = 0; r < CL; ++r) {
                     if (r == (int)rank) continue;
@@ -359,6 +392,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
                             gr_mapa(src, (unsigned)r)),
                         "r"(src), "r"(BYTES), "r"(gr_mapa(bar, (unsigned)r))
                         : "memory");
+                }
                 }
             }
         } else {
