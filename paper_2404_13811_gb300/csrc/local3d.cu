@@ -45,6 +45,13 @@ struct Box3 {
     double alpha;
     int ts[6], tt[6]; // tangential axes (ascending) of each side
     int soff[7];      // offsets of the sides in the boundary-face arrays
+    // index strides, so that no coordinate array is indexed at run time
+    long long g0;     // first cell of the box in the member's grid
+    int gs[3], gb[3]; // grid strides by natural axis and by block axis (a0, a1, a2)
+    int bs[3];        // block-order strides by natural axis
+    int es[6][3], eb[6][3];   // face-index strides of each side by natural and by block axis (0 along its normal)
+    int bit[6];       // the neighbour bit that cells on the side lack
+    float rb, r0;     // 1 / b, 1 / n[a0]
 };
 
 __device__ void setup_box3(Box3& B, const MemberDev& md, const int* lo, const int* hi, double alpha) {
@@ -78,27 +85,46 @@ __device__ void setup_box3(Box3& B, const MemberDev& md, const int* lo, const in
         B.tt[sid] = a == 2 ? 1 : 2;
         B.soff[sid + 1] = B.soff[sid] + B.n[B.ts[sid]] * B.n[B.tt[sid]];
     }
+    const int ax[3] = {B.a0, B.a1, B.a2};
+    B.gs[0] = 1;
+    B.gs[1] = md.n[0];
+    B.gs[2] = md.n[0] * md.n[1];
+    B.g0 = lo[0] + (long long)B.gs[1] * lo[1] + (long long)B.gs[2] * lo[2];
+    B.bs[B.a0] = 1;
+    B.bs[B.a1] = B.n[B.a0];
+    B.bs[B.a2] = B.b;
+    for (int sid = 0; sid < 6; ++sid)
+        for (int a = 0; a < 3; ++a) B.es[sid][a] = a == B.ts[sid] ? 1 : a == B.tt[sid] ? B.n[B.ts[sid]] : 0;
+    for (int p = 0; p < 3; ++p) {
+        B.gb[p] = B.gs[ax[p]];
+        for (int sid = 0; sid < 6; ++sid) B.eb[sid][p] = B.es[sid][ax[p]];
+        B.bit[2 * ax[p]] = 1 << (2 * p);
+        B.bit[2 * ax[p] + 1] = 2 << (2 * p);
+    }
+    B.rb = 1.f / (float)B.b;
+    B.r0 = 1.f / (float)B.n[B.a0];
 }
 
-// natural coordinates of the cell at block index t
-__device__ __forceinline__ void bcoord(const Box3& B, int t, int* c) {
-    const int j = t / B.b, pos = t - j * B.b;
-    c[B.a2] = j;
-    c[B.a1] = pos / B.n[B.a0];
-    c[B.a0] = pos - c[B.a1] * B.n[B.a0];
+// block coordinates (along a0, a1, a2) of the cell at block index t: by FP32
+// reciprocals, (t + 0.5) / b is at least 1 / 512 away from an integer, far above
+// the rounding for the t < 2^14 of a box
+struct Ijk {
+    int i, j, k;
+};
+__device__ __forceinline__ Ijk bcoord(const Box3& B, int t) {
+    Ijk c;
+    c.k = (int)(((float)t + 0.5f) * B.rb);
+    const int pos = t - c.k * B.b;
+    c.j = (int)(((float)pos + 0.5f) * B.r0);
+    c.i = pos - c.j * B.n[B.a0];
+    return c;
 }
-__device__ __forceinline__ int bidx(const Box3& B, const int* c) {
-    return c[B.a2] * B.b + c[B.a0] + B.n[B.a0] * c[B.a1];
-}
-__device__ __forceinline__ long long gidx(const Box3& B, const MemberDev& md, const int* c) {
-    return (B.lo[0] + c[0]) + (long long)md.n[0] * ((B.lo[1] + c[1]) + (long long)md.n[1] * (B.lo[2] + c[2]));
-}
-__device__ __forceinline__ long long gstride(const MemberDev& md, int a) {
-    return a == 0 ? 1LL : a == 1 ? (long long)md.n[0] : (long long)md.n[0] * md.n[1];
+__device__ __forceinline__ long long gidx(const Box3& B, const Ijk& c) {
+    return B.g0 + c.i * B.gb[0] + c.j * B.gb[1] + (long long)c.k * B.gb[2];
 }
 // face index of a cell on side sid (first tangential axis fastest)
-__device__ __forceinline__ int side_e(const Box3& B, int sid, const int* c) {
-    return c[B.ts[sid]] + B.n[B.ts[sid]] * c[B.tt[sid]];
+__device__ __forceinline__ int side_e(const Box3& B, int sid, const Ijk& c) {
+    return c.i * B.eb[sid][0] + c.j * B.eb[sid][1] + c.k * B.eb[sid][2];
 }
 // P0 / P1 function m on a side face with tangential coordinates (cs, ct)
 // relative to a side of extents (ls, lt): 1, s, t in [-1, 1]
@@ -119,12 +145,11 @@ __device__ __forceinline__ int side_of(const Box3& B, int f) {
     for (int s = 1; s < 6; ++s) sid += f >= B.soff[s];
     return sid;
 }
-// cell at face f of the boundary-face arrays (side sid)
-__device__ __forceinline__ void face_cell(const Box3& B, int sid, int f, int* c) {
-    const int e = f - B.soff[sid], ls = B.n[B.ts[sid]], q = e / ls;
-    c[sid >> 1] = (sid & 1) ? B.n[sid >> 1] - 1 : 0;
-    c[B.ts[sid]] = e - q * ls;
-    c[B.tt[sid]] = q;
+// grid index of the cell at face f of the boundary-face arrays (side sid)
+__device__ __forceinline__ long long face_cell(const Box3& B, int sid, int f) {
+    const int a = sid >> 1, e = f - B.soff[sid], ls = B.n[B.ts[sid]], q = e / ls;
+    return B.g0 + ((sid & 1) ? (long long)(B.n[a] - 1) * B.gs[a] : 0) + (e - q * ls) * B.gs[B.ts[sid]] +
+           (long long)q * B.gs[B.tt[sid]];
 }
 
 // The box operator from the face coefficients.  The faces of all sides are
@@ -136,11 +161,10 @@ __device__ void build_ops3(const Box3& B, const MemberDev& md, const DevPtrs& P,
     const double vol = md.h[0] * md.h[1] * md.h[2];
     const int a0 = B.a0, a1 = B.a1, a2 = B.a2, e0 = B.n[a0], e1 = B.n[a1], e2 = B.np, b = B.b, nc = B.nc;
     for (int t = threadIdx.x; t < nc; t += blockDim.x) {
-        int c[3];
-        bcoord(B, t, c);
-        const double* T = Tf + gidx(B, md, c) * 3;
+        const Ijk c = bcoord(B, t);
+        const double* T = Tf + gidx(B, c) * 3;
         const double t0 = T[a0], t1 = T[a1], t2 = T[a2];
-        const int i = c[a0], j = c[a1], k = c[a2];
+        const int i = c.i, j = c.j, k = c.k;
         O.c0[t] = i < e0 - 1 ? t0 : 0.0;
         O.c1[t] = j < e1 - 1 ? t1 : 0.0;
         O.c2[t] = k < e2 - 1 ? t2 : 0.0;
@@ -149,14 +173,12 @@ __device__ void build_ops3(const Box3& B, const MemberDev& md, const DevPtrs& P,
     }
     for (int f = threadIdx.x; f < B.soff[6]; f += blockDim.x) {
         const int sid = side_of(B, f), a = sid >> 1;
-        int c[3];
-        face_cell(B, sid, f, c);
-        const long long g = gidx(B, md, c);
+        const long long g = face_cell(B, sid, f);
         const double area = vol / md.h[a];
         const double hin = hkg[g * 3 + a];
         double T = 0.0, beta = 0.0;
         if (B.kind[sid] == 2) {
-            const long long gf = (sid & 1) ? g : g - gstride(md, a);
+            const long long gf = (sid & 1) ? g : g - B.gs[a];
             beta = B.alpha * wh[gf * 3 + a];
             T = area * rcp64(hin + beta);
         } else if (B.kind[sid] == 1) {
@@ -173,12 +195,9 @@ __device__ void build_ops3(const Box3& B, const MemberDev& md, const DevPtrs& P,
         if (m & 4) d += O.c1[t - e0];
         if (m & 16) d += O.c2[t - b];
         if ((m & 63) != 63) {
-            int c[3];
-            bcoord(B, t, c);
-            for (int sid = 0; sid < 6; ++sid) {
-                const int a = sid >> 1;
-                if (c[a] == ((sid & 1) ? B.n[a] - 1 : 0)) d += O.bT[B.soff[sid] + side_e(B, sid, c)];
-            }
+            const Ijk c = bcoord(B, t);
+            for (int sid = 0; sid < 6; ++sid)
+                if (!(m & B.bit[sid])) d += O.bT[B.soff[sid] + side_e(B, sid, c)];
         }
         O.cd[t] = d;
         if (mixed) O.dsc[t] = in_f32_range(d) ? (double)rsqrtf((float)d) : 1.0 / sqrt(d);
@@ -924,14 +943,14 @@ __device__ int solve3(int nr, const Box3& B, const Ops3& O, const T* F, const T*
 // f |c| + Dirichlet / Neumann data + Robin data lam (may be null) of cell t
 __device__ double source_rhs3(const Box3& B, const Ops3& O, const MemberDev& md, const double* fm, const double* lam,
                               int t) {
-    int c[3];
-    bcoord(B, t, c);
+    const Ijk c = bcoord(B, t);
     const double vol = md.h[0] * md.h[1] * md.h[2];
-    double r = fm[gidx(B, md, c) - 0] * vol;
-    if ((O.nb[t] & 63) != 63) {
+    double r = fm[gidx(B, c)] * vol;
+    const unsigned char m = O.nb[t];
+    if ((m & 63) != 63) {
         for (int sid = 0; sid < 6; ++sid) {
             const int a = sid >> 1;
-            if (c[a] != ((sid & 1) ? B.n[a] - 1 : 0)) continue;
+            if (m & B.bit[sid]) continue;
             const int e = B.soff[sid] + side_e(B, sid, c);
             if (B.kind[sid] == 1) r += O.bT[e] * B.val[sid];
             else if (B.kind[sid] == 0) r -= vol / md.h[a] * B.val[sid];
@@ -952,10 +971,9 @@ struct RhsBasis3 {
         if (sk[q] < 0) return bs[t];
         if (O->nb[t] & bit[q]) return 0.0;
         const int sid = sk[q];
-        int c[3];
-        bcoord(*B, t, c);
-        const int ts = B->ts[sid], tt = B->tt[sid];
-        const double v = O->bT[B->soff[sid] + side_e(*B, sid, c)] * psi3(mk[q], c[ts], B->n[ts], c[tt], B->n[tt]);
+        const int ls = B->n[B->ts[sid]], lt = B->n[B->tt[sid]];
+        const int e = side_e(*B, sid, bcoord(*B, t)), ct = e / ls;
+        const double v = O->bT[B->soff[sid] + e] * psi3(mk[q], e - ct * ls, ls, ct, lt);
         return O->dsc ? O->dsc[t] * v : v;
     }
 };
@@ -1015,7 +1033,7 @@ __host__ __device__ inline Lay3 lay3(int tsz, int nx, int ny, int nz, int nr, bo
     L.stage = tsz * rows * ld;
     const size_t tail = 64 + 32 + 2 * sizeof(uint64_t) * ST3;
     L.st = ST3;
-    while (L.st > 2 && L.fixed + L.work + L.st * L.stage + tail > 227 * 1024) --L.st;
+    while (L.st > 2 && L.fixed + L.work + L.st * L.stage + tail > 226 * 1024) --L.st;   // (1 KB for static shared memory)
     const size_t sol = L.work + L.st * L.stage;
     L.total = L.fixed + (L.fac > sol ? L.fac : sol) + tail;
     return L;
@@ -1184,12 +1202,18 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
             bs[t] = (mixed ? C.O.dsc[t] : 1.0) * source_rhs3(B, C.O, md, fm, nullptr, t);
         __syncthreads();
     }
-    int nI[3], off[3];
-    for (int a = 0; a < 3; ++a) {
-        nI[a] = sd.hi[a] - sd.lo[a];
-        off[a] = sd.lo[a] - B.lo[a];
-    }
-    const int nIc = nI[0] * nI[1] * nI[2];
+    // Omega_i in the box (in shared memory: indexed by the axis at run time)
+    __shared__ int nI[3], off[3];
+    if (threadIdx.x == 0)
+        for (int a = 0; a < 3; ++a) {
+            nI[a] = sd.hi[a] - sd.lo[a];
+            off[a] = sd.lo[a] - B.lo[a];
+        }
+    __syncthreads();
+    const int nI0 = nI[0], nI1 = nI[1], nIc = nI0 * nI1 * nI[2];
+    const float r0i = 1.f / (float)nI0, r01 = 1.f / (float)(nI0 * nI1);
+    const int tO = off[0] * B.bs[0] + off[1] * B.bs[1] + off[2] * B.bs[2];   // its first cell
+    const long long gO = B.g0 + off[0] * B.gs[0] + off[1] * (long long)B.gs[1] + off[2] * (long long)B.gs[2];
     int maxit = 0, nsolve = 0;
     for (int k0 = 0; k0 < nrhs; k0 += NR3) {
         const int nr = min(NR3, nrhs - k0);
@@ -1211,8 +1235,7 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
                             if (qq == 0) { rb.sk[q] = sid; break; }
                             --qq;
                         }
-                const int a = rb.sk[q] >> 1;
-                rb.bit[q] = 1 << (2 * (a == B.a0 ? 0 : a == B.a1 ? 1 : 2) + (rb.sk[q] & 1));
+                rb.bit[q] = rb.sk[q] >= 0 ? B.bit[rb.sk[q]] : 0;
             }
             it = solve3<T>(nr, B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rb, Mth.ir_tol, Mth.max_ir,
                            &C.flags[1], &C.flags[2]);
@@ -1231,11 +1254,9 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
             double* psi_out = pq ? P.pbar + (size_t)job.item * P.ncell_i_max
                                  : P.Psi + ((size_t)job.item * P.nbasis_max + k0 + q) * P.ncell_i_max;
             for (int ci = threadIdx.x; ci < nIc; ci += blockDim.x) {
-                int c[3];
-                c[0] = ci % nI[0] + off[0];
-                c[1] = (ci / nI[0]) % nI[1] + off[1];
-                c[2] = ci / (nI[0] * nI[1]) + off[2];
-                psi_out[ci] = x[bidx(B, c)];
+                const int z = (int)(((float)ci + 0.5f) * r01), xy = ci - z * nI0 * nI1;
+                const int y = (int)(((float)xy + 0.5f) * r0i);
+                psi_out[ci] = x[tO + (xy - y * nI0) * B.bs[0] + y * B.bs[1] + z * B.bs[2]];
             }
         }
         __syncthreads();
@@ -1263,27 +1284,26 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
             double* ug = pq ? P.ubg + ((size_t)job.item * MRCM_MAXSIDE + sid) * P.side_max
                             : P.Ug + (((size_t)job.item * P.nbasis_max + k) * MRCM_MAXSIDE + sid) * P.side_max;
             double fmv[3] = {0.0, 0.0, 0.0}, pmv[3] = {0.0, 0.0, 0.0};
+            const int cn = off[a] + ((sid & 1) ? nI[a] - 1 : 0);   // the side's cells along its normal
+            const bool inner = (sid & 1) ? cn + 1 < B.n[a] : cn > 0;
+            const int t0 = tO + (cn - off[a]) * B.bs[a];
+            const long long g0 = gO + (cn - off[a]) * (long long)B.gs[a];
             for (int e = lane; e < ls * lt; e += 32) {
-                const int cs = e % ls, ct = e / ls;
-                int c[3];
-                c[a] = (sid & 1) ? off[a] + nI[a] - 1 : off[a];
-                c[ts] = off[ts] + cs;
-                c[tt] = off[tt] + ct;
-                const double pL = x[bidx(B, c)];
-                const long long gL = gidx(B, md, c);
+                const int ct = e / ls, cs = e - ct * ls;
+                const int tL = t0 + cs * B.bs[ts] + ct * B.bs[tt];
+                const double pL = x[tL];
+                const long long gL = g0 + cs * (long long)B.gs[ts] + ct * (long long)B.gs[tt];
                 const double hkL = P.hk[(md.cell_off + gL) * 3 + a];
-                int cn[3] = {c[0], c[1], c[2]};
-                cn[a] += (sid & 1) ? 1 : -1;
-                const bool inner = cn[a] >= 0 && cn[a] < B.n[a];
                 double uo, pi;
                 if (inner) {
-                    const long long gf = (sid & 1) ? gL : gL - gstride(md, a);
+                    const long long gf = (sid & 1) ? gL : gL - B.gs[a];
                     const double Tf = P.Tf[(md.cell_off + gf) * 3 + a];
-                    uo = Tf * (pL - x[bidx(B, cn)]) * rarea;
+                    uo = Tf * (pL - x[(sid & 1) ? tL + B.bs[a] : tL - B.bs[a]]) * rarea;
                     pi = pL - uo * hkL;
                 } else {
-                    const int eb = B.soff[sid] + side_e(B, sid, c);
-                    const double lam = sid == skq ? psi3(mkq, c[ts], B.n[ts], c[tt], B.n[tt]) : 0.0;
+                    const int bcs = off[ts] + cs, bct = off[tt] + ct;
+                    const int eb = B.soff[sid] + bcs + B.n[ts] * bct;
+                    const double lam = sid == skq ? psi3(mkq, bcs, B.n[ts], bct, B.n[tt]) : 0.0;
                     uo = C.O.bT[eb] * (pL - lam) * rarea;
                     pi = part ? C.O.bB[eb] * uo : pL - uo * hkL;
                 }
@@ -1353,9 +1373,7 @@ __global__ void __launch_bounds__(T3, 1) k_smooth3d(DevPtrs P, MethodDev Mth, co
     for (int f = threadIdx.x; f < B.soff[6]; f += blockDim.x) {
         const int sid = side_of(B, f), a = sid >> 1;
         if (B.kind[sid] != 2) continue;
-        int c[3];
-        face_cell(B, sid, f, c);
-        const long long g = gidx(B, md, c);
+        const long long g = face_cell(B, sid, f);
         const double un = ust[g * 6 + sid];
         C.lam[f] = -C.O.bB[f] * un + (pst[g] - un * P.hk[(md.cell_off + g) * 3 + a]);
     }
@@ -1363,57 +1381,55 @@ __global__ void __launch_bounds__(T3, 1) k_smooth3d(DevPtrs P, MethodDev Mth, co
     const double* fm = P.f + md.cell_off;
     for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
         C.bsrc[t] = (mixed ? C.O.dsc[t] : 1.0) * source_rhs3(B, C.O, md, fm, C.lam, t);
-        // the refinement starts from the current pressure (mixed form: scaled by an FP32 reciprocal, a start only)
-        int c[3];
-        bcoord(B, t, c);
-        const double pt = pst[gidx(B, md, c)];
-        C.X[t] = mixed ? pt * f2d_bits(__frcp_rn(d2f_bits(C.O.dsc[t]))) : pt;
+        if constexpr (mixed) {
+            // the refinement starts from the current pressure, scaled (a start only: an FP32 reciprocal)
+            C.X[t] = pst[gidx(B, bcoord(B, t))] * f2d_bits(__frcp_rn(d2f_bits(C.O.dsc[t])));
+        }
     }
     __syncthreads();
     const T* F = (const T*)P.fac + (size_t)item * P.fac_stride;
     RhsStored3 rs{C.bsrc};
     const int it = solve3_n<T, 1>(B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rs, Mth.ir_tol, Mth.max_ir,
-                                  &C.flags[0], &C.flags[2], true);
+                                  &C.flags[0], &C.flags[2], mixed);
     if (C.flags[2]) drain3(C.pp);
     __syncthreads();
     // overwrite (u, p) on Omega_i with the restriction
-    int nI[3], off[3];
-    for (int a = 0; a < 3; ++a) {
-        nI[a] = sd.hi[a] - sd.lo[a];
-        off[a] = sd.lo[a] - B.lo[a];
-    }
-    const int nIc = nI[0] * nI[1] * nI[2];
+    const int nI0 = sd.hi[0] - sd.lo[0], nI1 = sd.hi[1] - sd.lo[1], nI2 = sd.hi[2] - sd.lo[2];
+    const int o0 = sd.lo[0] - B.lo[0], o1 = sd.lo[1] - B.lo[1], o2 = sd.lo[2] - B.lo[2];
+    const int nIc = nI0 * nI1 * nI2;
+    const float r0i = 1.f / (float)nI0, r01 = 1.f / (float)(nI0 * nI1);
     double* pw = P.p + md.cell_off;
     double* uw = P.u + md.cell_off * 6;
+    const double* Tfm = P.Tf + md.cell_off * 3;
     const double vol = md.h[0] * md.h[1] * md.h[2];
     const double* x = C.X;
     for (int ci = threadIdx.x; ci < nIc; ci += blockDim.x) {
-        int c[3];
-        c[0] = ci % nI[0] + off[0];
-        c[1] = (ci / nI[0]) % nI[1] + off[1];
-        c[2] = ci / (nI[0] * nI[1]) + off[2];
-        const int t = bidx(B, c);
-        const long long g = gidx(B, md, c);
+        const int z = (int)(((float)ci + 0.5f) * r01), xy = ci - z * nI0 * nI1;
+        const int y = (int)(((float)xy + 0.5f) * r0i);
+        const int c0 = xy - y * nI0 + o0, c1 = y + o1, c2 = z + o2;
+        const int t = c0 * B.bs[0] + c1 * B.bs[1] + c2 * B.bs[2];
+        const long long g = B.g0 + c0 + c1 * (long long)B.gs[1] + c2 * (long long)B.gs[2];
         if (!mrcm_check(P.status, g >= 0 && g < (long long)md.n[0] * md.n[1] * md.n[2], 7, g)) continue;
         const double pc = x[t];
+        const unsigned char m = C.O.nb[t];
         pw[g] = pc;
+        double uo[6];
+#pragma unroll
         for (int sid = 0; sid < 6; ++sid) {
             const int a = sid >> 1;
             const double rarea = md.h[a] / vol;
-            int cn[3] = {c[0], c[1], c[2]};
-            cn[a] += (sid & 1) ? 1 : -1;
-            double uo;
-            if (cn[a] >= 0 && cn[a] < B.n[a]) {
-                const long long gf = (sid & 1) ? g : g - gstride(md, a);
-                uo = P.Tf[(md.cell_off + gf) * 3 + a] * (pc - x[bidx(B, cn)]) * rarea;
+            if (m & B.bit[sid]) {
+                const long long gf = (sid & 1) ? g : g - B.gs[a];
+                uo[sid] = Tfm[gf * 3 + a] * (pc - x[(sid & 1) ? t + B.bs[a] : t - B.bs[a]]) * rarea;
             } else {
-                const int eb = B.soff[sid] + side_e(B, sid, c);
-                if (B.kind[sid] == 2) uo = C.O.bT[eb] * (pc - C.lam[eb]) * rarea;
-                else if (B.kind[sid] == 1) uo = C.O.bT[eb] * (pc - B.val[sid]) * rarea;
-                else uo = B.val[sid];
+                const int eb = B.soff[sid] + c0 * B.es[sid][0] + c1 * B.es[sid][1] + c2 * B.es[sid][2];
+                if (B.kind[sid] == 2) uo[sid] = C.O.bT[eb] * (pc - C.lam[eb]) * rarea;
+                else if (B.kind[sid] == 1) uo[sid] = C.O.bT[eb] * (pc - B.val[sid]) * rarea;
+                else uo[sid] = B.val[sid];
             }
-            uw[g * 6 + sid] = uo;
         }
+#pragma unroll
+        for (int sid = 0; sid < 6; ++sid) uw[g * 6 + sid] = uo[sid];
     }
     if (threadIdx.x == 0) {
         atomicMax(&P.status[1], it);
