@@ -179,27 +179,50 @@ __global__ void k_bcr_fill(IfPtrs I, int nslab) {
 // AT <- (L Q)^T with L (M x K, row-major in global memory) and Q the
 // columns cols[0..N) of Dinv (rows 0..K): AT[n * Mp + m], Mp / Np = M / N
 // rounded up to 4, zero beyond M / N.  K in chunks of 32 staged transposed
-// (stLT[k * (Mp + 4) + m], stQ[k * (Np + 4) + n]); every thread owns 4 x 4
-// output tiles, read as float4 pairs per k (16 FMAs per two loads).  The
-// sum over k runs in increasing k for every entry.
+// (stLT[k * (Mp + 4) + m], stQ[k * (Np + 4) + n]); the next chunk is loaded into
+// registers (up to EL_PF values of each per thread) while this one is used;
+// a chunk is otherwise a load round trip in sequence with its products (with
+// the coupling block staged during this product: 512x512 step 3324 -> 3285 us);
+// every thread owns 4 x 4 output tiles, read as float4 pairs per k (16 FMAs
+// per two loads).  The sum over k runs in increasing k for every entry.
+constexpr int EL_THREADS = 512;
+constexpr int EL_PF = 10;
+
 __device__ void rows_times_cols(const float* L, int M, int K, const float* Dinv, int np, const int* cols, int N,
                                 float* AT, float* stLT, float* stQ) {
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const int tid = threadIdx.x;
+    constexpr int nt = EL_THREADS;
     const int Mp = (M + 3) & ~3, Np = (N + 3) & ~3, ldl = Mp + 4, ldq = Np + 4;
     const int tm = Mp >> 2, tn = Np >> 2;
+    const int kk = tid & 31, r0 = tid >> 5;   // staged entry: k, first row / column (then every 16th)
+    float pl[EL_PF], pq[EL_PF];
+    auto fetch = [&](int k0) {
+        const bool in = k0 + kk < K;
+#pragma unroll
+        for (int u = 0; u < EL_PF; ++u) {
+            const int m = r0 + u * (nt / 32);
+            pl[u] = (in && m < M) ? __ldcg(&L[(size_t)m * K + k0 + kk]) : 0.f;
+            pq[u] = (in && m < N) ? Dinv[(size_t)cols[m] * np + k0 + kk] : 0.f;
+        }
+    };
     for (int t = tid; t < Np * Mp; t += nt) AT[t] = 0.f;
+    fetch(0);
     for (int k0 = 0; k0 < K; k0 += 32) {
         const int kb = min(32, K - k0);
         __syncthreads();
-        for (int t = tid; t < Mp * 32; t += nt) {
-            const int m = t >> 5, k = t & 31;
-            stLT[k * ldl + m] = (k < kb && m < M) ? __ldcg(&L[(size_t)m * K + k0 + k]) : 0.f;
+#pragma unroll
+        for (int u = 0; u < EL_PF; ++u) {
+            const int m = r0 + u * (nt / 32);
+            if (m < Mp) stLT[kk * ldl + m] = pl[u];
+            if (m < Np) stQ[kk * ldq + m] = pq[u];
         }
-        for (int t = tid; t < Np * 32; t += nt) {
-            const int n = t >> 5, k = t & 31;
-            stQ[k * ldq + n] = (k < kb && n < N) ? Dinv[(size_t)cols[n] * np + k0 + k] : 0.f;
-        }
+        // rows and columns beyond the prefetched ones (wide couplings)
+        for (int m = r0 + EL_PF * (nt / 32); m < Mp; m += nt / 32)
+            stLT[kk * ldl + m] = (kk < kb && m < M) ? __ldcg(&L[(size_t)m * K + k0 + kk]) : 0.f;
+        for (int m = r0 + EL_PF * (nt / 32); m < Np; m += nt / 32)
+            stQ[kk * ldq + m] = (kk < kb && m < N) ? Dinv[(size_t)cols[m] * np + k0 + kk] : 0.f;
         __syncthreads();
+        if (k0 + 32 < K) fetch(k0 + 32);
         for (int t = tid; t < tm * tn; t += nt) {
             const int i = t / tn, jn = t - (t / tn) * tn;
             float acc[4][4];
@@ -225,6 +248,24 @@ __device__ void rows_times_cols(const float* L, int M, int K, const float* Dinv,
     __syncthreads();
 }
 
+// Starts the copy of the first cw columns of a coupling block (M2 rows, ld
+// ldc) into Csm[q * cwp + c] (cp.async by entries: the rows need not be
+// 16-byte aligned), padding zeroed; complete after cp.async.wait_all and a
+// barrier.
+__device__ void stage_coupling(const float* Cg, int ldc, int M2, int cw, float* Csm) {
+    const int Np = (M2 + 3) & ~3, cwp = (cw + 3) & ~3, lane = threadIdx.x & 31;
+    for (int q = threadIdx.x >> 5; q < Np; q += EL_THREADS / 32)
+        for (int c = lane; c < cwp; c += 32) {
+            float* d = Csm + q * cwp + c;
+            if (q < M2 && c < cw)
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(d)),
+                             "l"(Cg + (size_t)q * ldc + c)
+                             : "memory");
+            else
+                *d = 0.f;
+        }
+}
+
 // Rows r < M of a target: tgt(r, c) op= sum_q A[r][q] C[q][c] for c < ncol,
 // with A given transposed (AT[q * Mp + r], q < Np = M2 rounded up to 4,
 // zero-padded) and C row-major (ld ldc) in global memory, staged in shared
@@ -234,14 +275,12 @@ template <bool ACCUM_INTO_D>
 __device__ void apply_coupling(const float* AT, int M, int M2, const float* Cg, int ldc, int ncol, float* Csm,
                                int cwmax, float* D, int np, const int* rows, float* Cout, int ldout, int nclear) {
     const int tid = threadIdx.x, nt = blockDim.x;
-    const int Mp = (M + 3) & ~3, Np = (M2 + 3) & ~3, tm = Mp >> 2;
+    const int Mp = (M + 3) & ~3, tm = Mp >> 2;
     for (int c0 = 0; c0 < ncol; c0 += cwmax) {
         const int cw = min(cwmax, ncol - c0), cwp = (cw + 3) & ~3, tc = cwp >> 2;
         __syncthreads();
-        for (int t = tid; t < Np * cwp; t += nt) {
-            const int q = t / cwp, c = t - (t / cwp) * cwp;
-            Csm[t] = (q < M2 && c < cw) ? Cg[(size_t)q * ldc + c0 + c] : 0.f;
-        }
+        if (c0 > 0) stage_coupling(Cg + c0, ldc, M2, cw, Csm);   // (the caller has staged the first)
+        asm volatile("cp.async.wait_all;" ::: "memory");
         __syncthreads();
         for (int t = tid; t < tm * tc; t += nt) {
             const int i = t / tc, jc = t - (t / tc) * tc;
@@ -303,8 +342,6 @@ __device__ void apply_coupling(const float* AT, int M, int M2, const float* Cg, 
 //   2: D_jp[vrows] -= (Rdn Qm) Cup_j      3: Cdn_jp <- -(Rdn Qv) Cdn_j
 // (every target row is written by one CTA only).
 // ---------------------------------------------------------------------------
-constexpr int EL_THREADS = 512;
-
 __global__ void __launch_bounds__(EL_THREADS) k_bcr_elim(IfPtrs I, const ElimDev* el, int nel) {
     cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
@@ -372,6 +409,11 @@ __global__ void __launch_bounds__(EL_THREADS) k_bcr_elim(IfPtrs I, const ElimDev
     float* stL = Asm + Np * Mp;         // 32 x (Mp + 4)
     float* stQ = stL + 32 * (Mp + 4);   // 32 x (Np + 4)
     float* Csm = stQ + 32 * (Np + 4);   // Np x (column chunk rounded up to 4)
+    // the coupling block that the product below needs, on its way meanwhile
+    {
+        const int ncol = (prod == 0 || prod == 3) ? Sm.n : Sp.n;
+        stage_coupling((prod == 0 || prod == 3) ? Cdn_j : Cup_j, Sj.ldc, N, min(I.elim_cw, ncol), Csm);
+    }
     __syncthreads();
     rows_times_cols(Lrows, M, Sj.n, Dinv, np, cols, N, Asm, stL, stQ);
     if (prod == 0) {
