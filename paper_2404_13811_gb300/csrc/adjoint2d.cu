@@ -403,8 +403,7 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
     O.bT = (double*)take(sizeof(double) * per);
     O.bB = (double*)take(sizeof(double) * per);
     double* gbT = (double*)take(sizeof(double) * per);
-    T* Sinv = (T*)take(sizeof(T) * sinv_len(B.nx, B.ny, sizeof(T), 0));
-    const int bp = B.nx;   // lines not widened (the factor is this kernel's own)
+    T* Sinv = (T*)take(sizeof(T) * sinv_len(B.nx, B.ny, sizeof(T), 0));   // lines not widened
     T* cys = (T*)take(sizeof(T) * n);
     T* cxs = (T*)take(sizeof(T) * n);
     T* zall = (T*)take(sizeof(T) * 64 * nw);
@@ -422,7 +421,8 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
     for (int t = threadIdx.x; t < per; t += blockDim.x) gbT[t] = 0.0;
     build_ops(B, md, P, O);
     fill_scale(B, O, mixed);
-    factor_box<T, BW, false>(B, O, Sinv, cys, cxs, &flags[0]);
+    if (mixed) scale_ops(B, O);   // as the forward kernel: factor and refinement in scaled variables
+    factor_box<T, BW, false, mixed>(B, O, Sinv, cys, cxs, &flags[0]);
     if (flags[0] && threadIdx.x == 0) {
         atomicOr(&P.status[0], ST_NOT_SPD);
         atomicExch(&P.status[2], job.item);
@@ -446,6 +446,16 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
     const double* gps = A.gps + (size_t)job.item * P.ncell_i_max;
     const double* gugi = A.gug + (size_t)job.item * MRCM_MAXSIDE * P.side_max;
     T* zb = zall + warp * 64;
+    // one solve by this warp with a stored right-hand side (scaled in the mixed form, as the solution)
+    auto stored = [&](double* xs, const double* b) {
+        if constexpr (mixed) {
+            RhsScStored rs{b};
+            warp_solve_sc<RhsScStored, -1>(B, O, Sinv, cys, xs, wv, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1]);
+        } else {
+            RhsStored rs{b};
+            warp_solve<T>(B, O, Sinv, cys, xs, (T*)xs, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1], B.nx);
+        }
+    };
     for (int k = warp; k < nrhs; k += nw) {
         // forward solution x_k
         int sk = -1, mk = 0;
@@ -458,15 +468,26 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
                     if (q == 0) { sk = sid; break; }
                     --q;
                 }
-            RhsBasis rb{sk, mk};
-            warp_solve<T>(B, O, Sinv, cys, x, mixed ? wv : (T*)x, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1], bp);
+            if constexpr (mixed) {
+                const int len = (sk >> 1) == 0 ? B.ny : B.nx;
+                const double mine = lane < len ? RhsScSide::face(B, O.dsc, O.bT, sk, mk, lane) : 0.0;
+                RhsScSide rb{sk, mk, O.dsc, O.bT, mine};
+                warp_solve_sc<RhsScSide, -1>(B, O, Sinv, cys, x, wv, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1]);
+            } else {
+                RhsBasis rb{sk, mk};
+                warp_solve<T>(B, O, Sinv, cys, x, (T*)x, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1], B.nx);
+            }
         } else {
             double* bs = basis ? P.bsrc + (size_t)job.item * P.dsc_stride : bsrc;
             for (int c = lane; c < B.n; c += 32)
-                bs[c] = source_rhs(B, O, fm, nxg, vol, ax, ay, nullptr, c % B.nx, c / B.nx);
+                bs[c] = (mixed ? O.dsc[c] : 1.0) * source_rhs(B, O, fm, nxg, vol, ax, ay, nullptr, c % B.nx, c / B.nx);
             __syncwarp();
-            RhsStored rs{bs};
-            warp_solve<T>(B, O, Sinv, cys, x, mixed ? wv : (T*)x, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1], bp);
+            stored(x, bs);
+        }
+        if constexpr (mixed) {
+            // back from the scaled iterate
+            __syncwarp();
+            for (int c = lane; c < B.n; c += 32) x[c] *= O.dsc[c];
         }
         __syncwarp();
         // adjoint right-hand side
@@ -500,7 +521,8 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
                 else if (sid == 1) { inner = i < B.nx - 1; cR = cL + 1;    fidx = cL;        gacc = gcx; }
                 else if (sid == 2) { inner = j > 0;        cR = cL - B.nx; fidx = cL - B.nx; gacc = gcy; }
                 else               { inner = j < B.ny - 1; cR = cL + B.nx; fidx = cL;        gacc = gcy; }
-                Tf = inner ? (a == 0 ? O.cx[fidx] : O.cy[fidx]) : 0.0;
+                // (unscaled, from the face coefficients: those of the box are scaled in the mixed form)
+                Tf = inner ? P.Tf[(md.cell_off + gL - ((sid & 1) ? 0 : a == 0 ? 1 : nxg)) * 3 + a] : 0.0;
                 double s0 = 0.0, s1 = 0.0;
                 for (int m = 0; m < npsi; ++m) {
                     const double psv = psi_val(m, e, len, rl);
@@ -542,9 +564,16 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
             }
             __syncwarp();
         }
-        RhsStored rs{rt};
-        warp_solve<T>(B, O, Sinv, cys, mu, mixed ? wv : (T*)mu, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1], bp);
+        if constexpr (mixed) {
+            for (int c = lane; c < B.n; c += 32) rt[c] *= O.dsc[c];
+            __syncwarp();
+        }
+        stored(mu, rt);
         __syncwarp();
+        if constexpr (mixed) {
+            for (int c = lane; c < B.n; c += 32) mu[c] *= O.dsc[c];
+            __syncwarp();
+        }
         // -mu^T (dA/dc) x
         for (int c = lane; c < B.n; c += 32) {
             const int i = c % B.nx, j = c / B.nx;

@@ -1217,6 +1217,8 @@ __device__ __forceinline__ void cell_ij(int c, int b, float rb, int& i, int& j) 
 // |r~|_inf <= tol |b~|_inf (the stopping rule of warp_solve, in the same
 // scaled norm).  Cells are visited 32 at a time by all lanes.  On exit x
 // holds x~ (the caller scales back with dsc).  Returns the number of sweeps.
+// SW: the line width where it is a template's (0: by column; -1: the row path
+// of the width b where there is one, chosen at run time).
 template <typename Rhs, int SW = 0>
 __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, const float* cys, double* x, float* w,
                              float* zbuf, const Rhs& rhs, double tol, int max_ir, int* noconv) {
@@ -1243,6 +1245,7 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
     int it = 0;
     for (; it < max_ir; ++it) {
         if constexpr (SW > 0) tw_warp<float, SW>(Sinv, cys, w, zbuf, b, nb);
+        else if constexpr (SW < 0) warp_sweeps<float>(Sinv, cys, w, zbuf, b, nb, b);
         else tw_warp<float, 0>(Sinv, cys, w, zbuf, b, nb);
         for (int c = lane; c < B.n; c += 32) x[c] += f2d_bits(w[c]);
         __syncwarp();
