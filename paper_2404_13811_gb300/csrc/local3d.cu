@@ -1039,6 +1039,15 @@ __host__ __device__ inline Lay3 lay3(int tsz, int nx, int ny, int nz, int nr, bo
     return L;
 }
 
+// Right-hand sides of a basis round: NR3, fewer where the work vectors of so
+// many do not fit (mixed form, boxes that nearly fill shared memory with their
+// operator: 3 x 22 x 34 cells take three).
+__host__ __device__ inline int round3(int tsz, int nx, int ny, int nz) {
+    int nr = NR3;
+    while (nr > 1 && lay3(tsz, nx, ny, nz, nr, false, false).total > 227 * 1024) --nr;
+    return nr;
+}
+
 template <typename T>
 struct Carve3 {
     Ops3 O;
@@ -1137,18 +1146,20 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
     const Job job = jobs[blockIdx.x];
     const SubDev sd = P.sub[job.item];
     const MemberDev& md = P.mem[sd.member];
+    const bool part = job.type == JOB_PART;
     __shared__ Box3 B;
+    __shared__ int round;   // right-hand sides per round
     if (threadIdx.x == 0) {
-        if (job.type == JOB_PART) setup_box3(B, md, sd.lo, sd.hi, Mth.alpha_b);
+        if (part) setup_box3(B, md, sd.lo, sd.hi, Mth.alpha_b);
         else setup_box3(B, md, sd.loh, sd.hih, job.type == JOB_SFACT ? Mth.alpha_s : Mth.alpha_b);
+        round = part ? 1 : round3((int)sizeof(T), B.n[0], B.n[1], B.n[2]);
     }
     __syncthreads();
-    const bool part = job.type == JOB_PART;
     if (!mrcm_check(P.status,
-                    lay3((int)sizeof(T), B.n[0], B.n[1], B.n[2], part ? 1 : NR3, part, false).total <= mrcm_dyn_smem_bytes(),
+                    lay3((int)sizeof(T), B.n[0], B.n[1], B.n[2], round, part, false).total <= mrcm_dyn_smem_bytes(),
                     6, 0))
         return;   // uniform
-    Carve3<T> C = carve3<T>(smem, B, part ? 1 : NR3, part, false, P.xs + (size_t)blockIdx.x * P.xs_stride);
+    Carve3<T> C = carve3<T>(smem, B, round, part, false, P.xs + (size_t)blockIdx.x * P.xs_stride);
     build_ops3(B, md, P, C.O, mixed);
     if constexpr (mixed) {
         scale_ops3(B, C.O);
@@ -1215,8 +1226,8 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
     const int tO = off[0] * B.bs[0] + off[1] * B.bs[1] + off[2] * B.bs[2];   // its first cell
     const long long gO = B.g0 + off[0] * B.gs[0] + off[1] * (long long)B.gs[1] + off[2] * (long long)B.gs[2];
     int maxit = 0, nsolve = 0;
-    for (int k0 = 0; k0 < nrhs; k0 += NR3) {
-        const int nr = min(NR3, nrhs - k0);
+    for (int k0 = 0; k0 < nrhs; k0 += round) {
+        const int nr = min(round, nrhs - k0);
         int it;
         RhsBasis3 rb;
         rb.B = &B;
@@ -1508,7 +1519,8 @@ __global__ void k_assemble3d(DevPtrs P, const double* __restrict__ X) {
 // host-side launch helpers
 // ---------------------------------------------------------------------------
 size_t local3d_smem(int prec, int nx, int ny, int nz, bool part) {
-    return lay3(prec == 0 ? 8 : 4, nx, ny, nz, part ? 1 : NR3, part, false).total;
+    const int tsz = prec == 0 ? 8 : 4;
+    return lay3(tsz, nx, ny, nz, part ? 1 : round3(tsz, nx, ny, nz), part, false).total;
 }
 
 size_t smooth3d_smem(int prec, int nx, int ny, int nz) { return lay3(prec == 0 ? 8 : 4, nx, ny, nz, 1, true, true).total; }

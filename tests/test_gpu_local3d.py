@@ -26,6 +26,7 @@ CASES = [
     ((16, 14, 14), (8, 14, 14), 1, 0),  # 9 x 14 x 14: planes of 126
     ((16, 32, 8), (8, 16, 8), 0, 0),    # 8 x 16 x 8: planes of 64
     ((24, 11, 12), (12, 11, 12), 0, 0),  # 12 x 11 x 12: planes of 132 (shared memory)
+    ((6, 44, 34), (3, 22, 34), 0, 1),   # 3 x 22 x 34: three right-hand sides a round fit (mixed), six are solved
 ]
 
 
