@@ -26,7 +26,8 @@
 
 namespace {
 
-constexpr int AS_WARPS = 4;   // k_adj_smooth2d
+constexpr int AS_WARPS = 4;   // k_adj_smooth2d: warps of the FP64 form, twice as many in the mixed form
+constexpr int AS_U = 3;       // cells per thread whose global loads are in flight together
 
 // row of test function m on side `sid` of its owner (flux rows of the high
 // sides first, then pressure rows of the low sides; same order as
@@ -62,12 +63,13 @@ __device__ int row_pos(const SubDev& o, int d, int npsi, int kind, int sid, int 
 // pack is staged by one bulk copy and the solve runs as the forward one does
 // (two-warp sweeps, residuals over the CTA).  Subdomains of one colour have
 // disjoint oversampled boxes (2 l < H), so their writes never meet.
-// A pass of 64 boxes of 24 x 24 cells takes 51 us (184 us when it solved twice
-// from zero on one warp, on a factor read by loads); bound by the latency of
-// the box's line sweeps.
+// A pass of 64 boxes of 24 x 24 cells takes 45 us (184 us when it solved twice
+// from zero on one warp, on a factor read by loads; 54 us with four warps in
+// the mixed form, a cell's loads at a time and the sides one after another);
+// bound by the latency of the box's line sweeps.
 // ---------------------------------------------------------------------------
 template <typename T>
-__global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, MethodDev Mth, AdjPtrs A,
+__global__ void __launch_bounds__((sizeof(T) == 4 ? 2 : 1) * AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, MethodDev Mth, AdjPtrs A,
                                                                 const int* items) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool mixed = std::is_same<T, float>::value;
@@ -122,25 +124,42 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     const int jlo = sd.lo[1] - B.lo[1], jhi = sd.hi[1] - B.lo[1];
     // the forward solution; the seeds on Omega_i, taken and cleared (the
     // forward overwrote them); mu starts as the pressure seed
-    for (int c = threadIdx.x; c < B.n; c += blockDim.x) {
-        const int i = c % B.nx, j = c / B.nx;
-        x[c] = rec[c];
-        double g0 = 0.0, s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-        if (i >= ilo && i < ihi && j >= jlo && j < jhi) {
-            const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
-            g0 = gpg[g];
-            s0 = gug[g * 4];
-            s1 = gug[g * 4 + 1];
-            s2 = gug[g * 4 + 2];
-            s3 = gug[g * 4 + 3];
-            gpg[g] = 0.0;
-            gug[g * 4] = gug[g * 4 + 1] = gug[g * 4 + 2] = gug[g * 4 + 3] = 0.0;
+    const int nt = blockDim.x;
+    const float rb = 1.f / (float)B.nx;
+    for (int c0 = threadIdx.x; c0 < B.n; c0 += AS_U * nt) {
+        double xr[AS_U], g0[AS_U], sv[AS_U][4];
+        long long gc[AS_U];
+#pragma unroll
+        for (int k = 0; k < AS_U; ++k) {
+            const int c = c0 + k * nt;
+            gc[k] = -1;
+            xr[k] = g0[k] = sv[k][0] = sv[k][1] = sv[k][2] = sv[k][3] = 0.0;
+            if (c >= B.n) continue;
+            int i, j;
+            cell_ij(c, B.nx, rb, i, j);
+            xr[k] = rec[c];
+            if (i >= ilo && i < ihi && j >= jlo && j < jhi) {
+                const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
+                gc[k] = g;
+                g0[k] = gpg[g];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) sv[k][q] = gug[g * 4 + q];
+            }
         }
-        mu[c] = g0;
-        su[4 * c] = s0;
-        su[4 * c + 1] = s1;
-        su[4 * c + 2] = s2;
-        su[4 * c + 3] = s3;
+#pragma unroll
+        for (int k = 0; k < AS_U; ++k) {
+            const int c = c0 + k * nt;
+            if (c >= B.n) continue;
+            x[c] = xr[k];
+            mu[c] = g0[k];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) su[4 * c + q] = sv[k][q];
+            if (gc[k] >= 0) {
+                gpg[gc[k]] = 0.0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) gug[gc[k] * 4 + q] = 0.0;
+            }
+        }
     }
     const bool arrived = mbar_wait(&bar, 0);
     if (__syncthreads_or(!arrived)) {
@@ -155,19 +174,38 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     }
     // adjoint right-hand side gp + (du/dp)^T gu (scaled in the mixed form)
     const double rax = 1.0 / md.h[1], ray = 1.0 / md.h[0];
-    for (int c = threadIdx.x; c < B.n; c += blockDim.x) {
-        const int i = c % B.nx, j = c / B.nx;
-        const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
-        double r = mu[c];
-        if (i < B.nx - 1) r += Tfg[g * 3] * (su[4 * c + 1] - su[4 * (c + 1)]) * rax;
-        if (i > 0) r -= Tfg[(g - 1) * 3] * (su[4 * (c - 1) + 1] - su[4 * c]) * rax;
-        if (j < B.ny - 1) r += Tfg[g * 3 + 1] * (su[4 * c + 3] - su[4 * (c + B.nx) + 2]) * ray;
-        if (j > 0) r -= Tfg[(g - nxg) * 3 + 1] * (su[4 * (c - B.nx) + 3] - su[4 * c + 2]) * ray;
-        if (i == 0 && B.kind[0]) r += O.bT[side_off(B, 0) + j] * su[4 * c] * rax;
-        if (i == B.nx - 1 && B.kind[1]) r += O.bT[side_off(B, 1) + j] * su[4 * c + 1] * rax;
-        if (j == 0 && B.kind[2]) r += O.bT[side_off(B, 2) + i] * su[4 * c + 2] * ray;
-        if (j == B.ny - 1 && B.kind[3]) r += O.bT[side_off(B, 3) + i] * su[4 * c + 3] * ray;
-        rt[c] = mixed ? O.dsc[c] * r : r;
+    for (int c0 = threadIdx.x; c0 < B.n; c0 += AS_U * nt) {
+        double tv[AS_U][4];   // transmissibilities of the cell's faces (0 on the box's sides)
+#pragma unroll
+        for (int k = 0; k < AS_U; ++k) {
+            const int c = c0 + k * nt;
+            tv[k][0] = tv[k][1] = tv[k][2] = tv[k][3] = 0.0;
+            if (c >= B.n) continue;
+            int i, j;
+            cell_ij(c, B.nx, rb, i, j);
+            const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
+            if (i < B.nx - 1) tv[k][0] = Tfg[g * 3];
+            if (i > 0) tv[k][1] = Tfg[(g - 1) * 3];
+            if (j < B.ny - 1) tv[k][2] = Tfg[g * 3 + 1];
+            if (j > 0) tv[k][3] = Tfg[(g - nxg) * 3 + 1];
+        }
+#pragma unroll
+        for (int k = 0; k < AS_U; ++k) {
+            const int c = c0 + k * nt;
+            if (c >= B.n) continue;
+            int i, j;
+            cell_ij(c, B.nx, rb, i, j);
+            double r = mu[c];
+            if (i < B.nx - 1) r += tv[k][0] * (su[4 * c + 1] - su[4 * (c + 1)]) * rax;
+            if (i > 0) r -= tv[k][1] * (su[4 * (c - 1) + 1] - su[4 * c]) * rax;
+            if (j < B.ny - 1) r += tv[k][2] * (su[4 * c + 3] - su[4 * (c + B.nx) + 2]) * ray;
+            if (j > 0) r -= tv[k][3] * (su[4 * (c - B.nx) + 3] - su[4 * c + 2]) * ray;
+            if (i == 0 && B.kind[0]) r += O.bT[side_off(B, 0) + j] * su[4 * c] * rax;
+            if (i == B.nx - 1 && B.kind[1]) r += O.bT[side_off(B, 1) + j] * su[4 * c + 1] * rax;
+            if (j == 0 && B.kind[2]) r += O.bT[side_off(B, 2) + i] * su[4 * c + 2] * ray;
+            if (j == B.ny - 1 && B.kind[3]) r += O.bT[side_off(B, 3) + i] * su[4 * c + 3] * ray;
+            rt[c] = mixed ? O.dsc[c] * r : r;
+        }
     }
     __syncthreads();
     if constexpr (mixed) {
@@ -184,51 +222,75 @@ __global__ void __launch_bounds__(AS_WARPS * 32) k_adj_smooth2d(DevPtrs P, Metho
     double* gTf = A.gTf + md.cell_off * 3;
     double* ghk = A.ghk + md.cell_off * 3;
     double* gwh = A.gwh + md.cell_off * 3;
-    for (int c = threadIdx.x; c < B.n; c += blockDim.x) {
-        const int i = c % B.nx, j = c / B.nx;
-        const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
-        if (i < B.nx - 1) {
-            const double dp = x[c] - x[c + 1];
-            gTf[g * 3] += ((su[4 * c + 1] - su[4 * (c + 1)]) * rax - (mu[c] - mu[c + 1])) * dp;
+    for (int c0 = threadIdx.x; c0 < B.n; c0 += AS_U * nt) {
+        double t0[AS_U], t1[AS_U];
+#pragma unroll
+        for (int k = 0; k < AS_U; ++k) {
+            const int c = c0 + k * nt;
+            t0[k] = t1[k] = 0.0;
+            if (c >= B.n) continue;
+            int i, j;
+            cell_ij(c, B.nx, rb, i, j);
+            const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
+            if (i < B.nx - 1) t0[k] = gTf[g * 3];
+            if (j < B.ny - 1) t1[k] = gTf[g * 3 + 1];
         }
-        if (j < B.ny - 1) {
-            const double dp = x[c] - x[c + B.nx];
-            gTf[g * 3 + 1] += ((su[4 * c + 3] - su[4 * (c + B.nx) + 2]) * ray - (mu[c] - mu[c + B.nx])) * dp;
-        }
-    }
-    // box sides one at a time (a corner cell lies on two sides)
-    for (int sid = 0; sid < 4; ++sid) {
-        if (B.kind[sid] != 0) {
-            const int a = sid >> 1;
-            const int len = a == 0 ? B.ny : B.nx;
-            const double rarea = a == 0 ? rax : ray;
-            for (int pos = threadIdx.x; pos < len; pos += blockDim.x) {
-                int i, j;
-                if (a == 0) { j = pos; i = (sid == 0) ? 0 : B.nx - 1; }
-                else        { i = pos; j = (sid == 2) ? 0 : B.ny - 1; }
-                const int c = j * B.nx + i;
-                const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
-                const double Tb = O.bT[side_off(B, sid) + pos];
-                const double sc = su[4 * c + sid] * rarea;
-                const double q = -Tb * Tb * rarea;   // dT/d(h/2K); alpha * q = dT/d(H/K_H)
-                if (B.kind[sid] == 2) {
-                    const double lv = lam[side_off(B, sid) + pos];
-                    const double gT = (x[c] - lv) * (sc - mu[c]);
-                    const double gl = Tb * (mu[c] - sc);
-                    const double un = lun[side_off(B, sid) + pos];
-                    const long long gf = (sid & 1) ? g : g - (a == 0 ? 1 : nxg);
-                    // lambda = -alpha wh u.n + p - u.n hk
-                    ghk[g * 3 + a] += gT * q - gl * un;
-                    gwh[gf * 3 + a] += B.alpha * (gT * q - gl * un);
-                    gpg[g] += gl;
-                    gug[g * 4 + sid] += gl * (-O.bB[side_off(B, sid) + pos] - hkg[g * 3 + a]);
-                } else {
-                    const double gT = (x[c] - B.val[sid]) * (sc - mu[c]);
-                    ghk[g * 3 + a] += gT * q;
-                }
+#pragma unroll
+        for (int k = 0; k < AS_U; ++k) {
+            const int c = c0 + k * nt;
+            if (c >= B.n) continue;
+            int i, j;
+            cell_ij(c, B.nx, rb, i, j);
+            const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
+            if (i < B.nx - 1) {
+                const double dp = x[c] - x[c + 1];
+                gTf[g * 3] = t0[k] + ((su[4 * c + 1] - su[4 * (c + 1)]) * rax - (mu[c] - mu[c + 1])) * dp;
+            }
+            if (j < B.ny - 1) {
+                const double dp = x[c] - x[c + B.nx];
+                gTf[g * 3 + 1] = t1[k] + ((su[4 * c + 3] - su[4 * (c + B.nx) + 2]) * ray - (mu[c] - mu[c + B.nx])) * dp;
             }
         }
-        __syncthreads();
+    }
+    // box sides, the two of an axis together (a corner cell lies on one side of
+    // each axis; a box one cell wide has both sides of that axis on its cells,
+    // which then go one at a time); a face's loads before its stores
+    for (int a = 0; a < 2; ++a) {
+        const int len = a == 0 ? B.ny : B.nx;
+        const double rarea = a == 0 ? rax : ray;
+        const bool thin = (a == 0 ? B.nx : B.ny) == 1;
+        for (int half = 0; half < (thin ? 2 : 1); ++half) {
+            for (int t = threadIdx.x; t < (thin ? len : 2 * len); t += nt) {
+                const int hi = thin ? half : (t >= len ? 1 : 0);
+                const int sid = 2 * a + hi, pos = t - (!thin && hi ? len : 0);
+                if (B.kind[sid] == 0) continue;
+                int i, j;
+                if (a == 0) { j = pos; i = hi ? B.nx - 1 : 0; }
+                else        { i = pos; j = hi ? B.ny - 1 : 0; }
+                const int c = j * B.nx + i, e = side_off(B, sid) + pos;
+                const long long g = (B.lo[0] + i) + (long long)nxg * (B.lo[1] + j);
+                const double Tb = O.bT[e];
+                const double sc = su[4 * c + sid] * rarea;
+                const double q = -Tb * Tb * rarea;   // dT/d(h/2K); alpha * q = dT/d(H/K_H)
+                const double ghk0 = ghk[g * 3 + a];
+                if (B.kind[sid] == 2) {
+                    const long long gf = hi ? g : g - (a == 0 ? 1 : nxg);
+                    const double lv = lam[e], un = lun[e], hk = hkg[g * 3 + a];
+                    const double gwh0 = gwh[gf * 3 + a], gp0 = gpg[g], gu0 = gug[g * 4 + sid];
+                    const double gT = (x[c] - lv) * (sc - mu[c]);
+                    const double gl = Tb * (mu[c] - sc);
+                    // lambda = -alpha wh u.n + p - u.n hk
+                    ghk[g * 3 + a] = ghk0 + (gT * q - gl * un);
+                    gwh[gf * 3 + a] = gwh0 + B.alpha * (gT * q - gl * un);
+                    gpg[g] = gp0 + gl;
+                    gug[g * 4 + sid] = gu0 + gl * (-O.bB[e] - hk);
+                } else {
+                    const double gT = (x[c] - B.val[sid]) * (sc - mu[c]);
+                    ghk[g * 3 + a] = ghk0 + gT * q;
+                }
+            }
+            __syncthreads();
+        }
     }
     if (threadIdx.x == 0 && flags[0]) atomicOr(&P.status[0], ST_NO_CONV);
 }
@@ -712,7 +774,7 @@ cudaError_t launch_adj_smooth2d(const DevPtrs& P, const MethodDev& M, const AdjP
     } else {
         static size_t cur = 0;
         if ((e = set_smem_attr(k_adj_smooth2d<float>, smem, &cur)) != cudaSuccess) return e;
-        k_adj_smooth2d<float><<<nitems, AS_WARPS * 32, smem, s>>>(P, M, A, items);
+        k_adj_smooth2d<float><<<nitems, 2 * AS_WARPS * 32, smem, s>>>(P, M, A, items);
     }
     return cudaGetLastError();
 }

@@ -62,3 +62,20 @@ def test_gradient_at_odd_widths(sub, ov, precision):
     g = s.adjoint(gp, gu)
     s.close()
     assert np.abs(g - np.asarray(ref).reshape(-1)).max() <= 1e-8 * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("sub", [(1, 4), (4, 1), (1, 1)])
+def test_gradient_of_boxes_one_cell_wide(sub, precision):
+    """Without overlap a box can be one cell wide: both sides of an axis lie on
+    the same cells in the reverse smoothing."""
+    from paper_2404_13811_gb300.solver import MRCM
+    prob = _problem((3 * sub[0], 3 * sub[1]), 8)
+    rng = np.random.default_rng(4)
+    gp, gu = rng.standard_normal(prob.ncells), rng.standard_normal((prob.ncells, 4))
+    _, ref = OA.mrcm_os_adjoint(prob, sub, 0, 0, 1.0, 1.0, 2, gp, gu)
+    s = MRCM(prob, I.Partition(sub, 0), space=0, alpha_basis=1.0, alpha_smooth=1.0, precision=precision)
+    s.run(2)
+    g = s.adjoint(gp, gu)
+    s.close()
+    assert np.abs(g - np.asarray(ref).reshape(-1)).max() <= 1e-8 * np.abs(ref).max()
