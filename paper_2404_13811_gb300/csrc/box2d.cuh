@@ -160,6 +160,13 @@ __device__ __forceinline__ float d2f_bits(double d) {
     return __uint_as_float(r);
 }
 
+// d2f_bits rounded to nearest (ties away from zero): for values that stay in the
+// factor, where truncation would shift every pivot the same way.
+__device__ __forceinline__ float d2f_near(double d) {
+    const float t = d2f_bits(d);
+    return in_f32_range(d) ? __uint_as_float(__float_as_uint(t) + (((unsigned)__double2loint(d) >> 28) & 1u)) : t;
+}
+
 // The mixed form refines in Jacobi-scaled variables: O holds D A D (D =
 // diag(dsc)) after scale_ops, the iterate is x~ = D^-1 x and the right-hand
 // side b~ = D b, so that a residual b~ - (D A D) x~ is five FP64 FMAs per cell
@@ -288,7 +295,8 @@ __device__ __forceinline__ void gj_regs(T (&a)[BW], int b, int* bad) {
 // the width known at compile time (EX, FP32) lane i reads row i of the
 // (symmetric) neighbour inverse and the coupling vector as float4 and the
 // FP64 diagonal converts on the integer pipe (FP32 -> FP64 exact, the FP64
-// result truncated to FP32 within one ulp); otherwise lane i reads column i.
+// result truncated to FP32 within one ulp, or rounded to nearest in widened
+// lines); otherwise lane i reads column i.
 template <typename T, int BW, bool EX, bool SC>
 __device__ __forceinline__ void form_line(T (&a)[BW], const Ops& O, const T* cys, const T* cxs, int b, int ld,
                                           int j, const T* up, const T* dn) {
@@ -317,7 +325,7 @@ __device__ __forceinline__ void form_line(T (&a)[BW], const Ops& O, const T* cys
         if (dn) d -= (double)cn * ((double)cn * (double)dn[ii * ld + ii]);
     }
     T dT;
-    if constexpr (VEC) dT = d2f_bits(d);
+    if constexpr (VEC) dT = b < BW ? d2f_near(d) : d2f_bits(d);
     else dT = (T)d;
     if constexpr (VEC) {
         constexpr int NQ = BW / 4;
@@ -369,12 +377,29 @@ __device__ __forceinline__ void form_line(T (&a)[BW], const Ops& O, const T* cys
 
 // Stores the inverse held in registers (lane i, entry c) as entry (c, i) of
 // the row-major block (consecutive lanes, consecutive words); the inverse of
-// an SPD block is symmetric, so this is the block up to rounding.
+// an SPD block is symmetric, so this is the block up to rounding.  Widened
+// FP32 lines (b < BW): by rows, as float4.  There the sweeps then apply the
+// inverse as computed, and the diagonal is rounded to nearest, as where lines
+// of such widths are read by column: transposed and truncated, the fluxes of a
+// 225 x 192 field in boxes of 18 and 21 cells came out two to four times
+// further from the exact ones at the same ir_tol (1.2e-11 and 2.8e-11 with
+// only the rows, 1.2e-11 with both).  Lines of full width keep theirs: with both
+// changed the 512x512 step took 3403 instead of 3374 us, at 6.8e-11 from the
+// exact fluxes instead of 4.0e-11.
 template <typename T, int BW, bool EX>
 __device__ __forceinline__ void store_line(const T (&a)[BW], T* S, int b, int ld) {
     if constexpr (EX) ld = sld<T>(BW);
     const int i = threadIdx.x & 31;
-    if (i < (EX ? BW : b)) {   // (the identity's lanes store the zeros beyond b)
+    if constexpr (EX && std::is_same<T, float>::value && BW % 4 == 0) {
+        if (b < BW) {
+            if (i >= b) return;
+            float4* r = reinterpret_cast<float4*>(S + i * ld);
+#pragma unroll
+            for (int q = 0; q < BW / 4; ++q) r[q] = make_float4(a[4 * q], a[4 * q + 1], a[4 * q + 2], a[4 * q + 3]);
+            return;
+        }
+    }
+    if (i < b) {
 #pragma unroll
         for (int c = 0; c < BW; ++c)
             if (c < b) S[c * ld + i] = a[c];
