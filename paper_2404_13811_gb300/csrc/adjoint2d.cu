@@ -78,7 +78,10 @@ __global__ void __launch_bounds__((sizeof(T) == 4 ? 2 : 1) * AS_WARPS * 32) k_ad
     const MemberDev& md = P.mem[sd.member];
     __shared__ Box B;
     __shared__ __align__(8) uint64_t bar;
-    if (threadIdx.x == 0) setup_box(B, md, sd.loh, sd.hih, Mth.alpha_s);
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);   // before the block barrier: every thread waits on it below
+        setup_box(B, md, sd.loh, sd.hih, Mth.alpha_s);
+    }
     __syncthreads();
     const size_t n = (size_t)B.n;
     const int per = 2 * (B.nx + B.ny);
@@ -108,7 +111,6 @@ __global__ void __launch_bounds__((sizeof(T) == 4 ? 2 : 1) * AS_WARPS * 32) k_ad
     const unsigned char* Pg = (const unsigned char*)((const T*)P.fac + (size_t)item * P.fac_stride);
     if (threadIdx.x == 0) {
         flags[0] = 0;
-        mbar_init(&bar, 1);
         mbar_expect_tx(&bar, pbytes);
         bulk_g2s(smem, Pg, pbytes, &bar);
     }
