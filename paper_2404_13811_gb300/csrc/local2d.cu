@@ -257,7 +257,11 @@ __global__ void __launch_bounds__(SMW<T> * 32, 2) k_smooth2d(DevPtrs P, MethodDe
     __shared__ Box B;
     __shared__ __align__(8) uint64_t bar;
     __shared__ __align__(8) uint64_t never;   // failure-detection test only: a barrier nothing arrives at
-    if (threadIdx.x == 0) setup_box(B, md, sd.loh, sd.hih, Mth.alpha_s);
+    if (threadIdx.x == 0) {
+        mbar_init(&bar, 1);   // before the block barrier: every thread waits on it below
+        if (Mth.wait0 > 0) mbar_init(&never, 1);
+        setup_box(B, md, sd.loh, sd.hih, Mth.alpha_s);
+    }
     __syncthreads();
     const size_t n = (size_t)B.n;
     // the smoothing pack (factor, operator, fixed right-hand side) first, by one bulk copy
@@ -289,8 +293,6 @@ __global__ void __launch_bounds__(SMW<T> * 32, 2) k_smooth2d(DevPtrs P, MethodDe
     if (threadIdx.x == 0) {
         flags[0] = 0;
         flags[1] = 0;
-        mbar_init(&bar, 1);
-        if (Mth.wait0 > 0) mbar_init(&never, 1);
         mbar_expect_tx(&bar, pbytes);
         // a bulk copy needs 16-byte aligned ends and a size that is a multiple of 16
         if (mrcm_check(P.status, ((uintptr_t)Pg & 15) == 0 && (pbytes & 15) == 0 && pbytes <= L.bytes, 3,

@@ -24,6 +24,7 @@ def _body(src, name):
 
 @pytest.mark.parametrize("path,kernel,init,wait", [
     ("adjoint2d.cu", "k_adj_smooth2d", r"mbar_init\(", r"mbar_wait\("),
+    ("local2d.cu", "k_smooth2d", r"mbar_init\(", r"mbar_wait\("),
 ])
 def test_block_barrier_between_init_and_wait(path, kernel, init, wait):
     with open(os.path.join(CSRC, path)) as f:
