@@ -16,10 +16,11 @@
 //     column k to -A_ik / A_pk (1 in row p, see below) and writes the
 //     column's values with the entry of row p zeroed (the multipliers), p
 //     and the pivot into the panel's record in its CTA's shared memory; the
-//     finished record goes to every other CTA of the cluster by one bulk
-//     copy each (completing an mbarrier there by its bytes), in clusters of
-//     more than 8 CTAs by one multicast copy out of global memory, and is
-//     released in its own CTA by one arrival;
+//     finished record is released in its own CTA by one arrival and goes to
+//     every other CTA of the cluster by one bulk copy each (completing an
+//     mbarrier there by its bytes); in clusters of more than 8 CTAs each
+//     other CTA fetches it by a bulk copy of its own from global memory,
+//     once the owner has arrived on a second mbarrier there;
 //   * every other warp waits for the record and applies the panel's CB
 //     rank-1 updates to its own columns in turn, each taking the pivot row's
 //     current values on its columns from the lane holding row p (selected
@@ -86,6 +87,13 @@ __device__ __forceinline__ bool gr_try(unsigned bar, unsigned parity) {
     return ok != 0;
 }
 
+// bulk copy of a record from global memory into this CTA's shared memory
+__device__ __forceinline__ void gr_fetch(unsigned dst, const float* src, unsigned bytes, unsigned bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+
 __device__ __forceinline__ void gr_arrive(unsigned bar) {
     asm volatile("mbarrier.arrive.release.cta.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -97,6 +105,11 @@ __device__ __forceinline__ float gr_rcp(float x) {
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(x));
     const float e = fmaf(-x, r, 1.f);
     return fmaf(r, e, r);
+}
+
+// arrival on an mbarrier of another CTA of the cluster (address from gr_mapa)
+__device__ __forceinline__ void gr_arrive_at(unsigned bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ void gr_release(int* flag, int v) {
@@ -129,7 +142,7 @@ struct GrShape {
     static_assert(RA % 4 == 0 && (RA < 8 || RA % 8 == 0) && RA <= 32 && CB % 4 == 0 && CB * NW * CL == NPAD,
                   "unsupported slab inverse shape");
     static constexpr int G = NPAD >= 768 ? 3 : NPAD >= 512 ? 4 : 8;   // panels between cluster barriers
-    static constexpr bool MC = CL > 8;              // records by multicast through global memory
+    static constexpr bool VIA = CL > 8;             // records through global memory, fetched by each CTA
     static constexpr int R = 2 * G;                  // record slots (one panel each)
     static constexpr size_t smem() { return sizeof(float) * ((size_t)R * REC + (size_t)NW * NPAD * CB); }
 };
@@ -144,6 +157,8 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
     float* tiles = recs + R * REC;         // [warp][NPAD][CB]
     __shared__ __align__(8) unsigned long long bars[R];
     __shared__ int colready[R];            // columns of a slot's record written so far (P CB + c + 1)
+    __shared__ __align__(8) unsigned long long ready[R];   // (VIA) the slot's record is in global memory
+    __shared__ int fetched[R];             // (VIA) panel + 1 of the last record fetched into the slot
     __shared__ int pivrow[NPAD];           // pivot row of every step
     __shared__ float pivval[NPAD];         // its pivot
     // after the elimination, in the place of the panel-start copies
@@ -159,7 +174,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
     const int npan = (n + CB - 1) / CB;    // panels holding a column below n
     const float* A = I.D + S.offD;
     float* Ainv = I.Dinv + S.offD;
-    // (MC) where the records pass through: the slab's own block, read into
+    // (VIA) where the records pass through: the slab's own block, read into
     // registers before the first record and not needed after (n^2 entries
     // against R records of 4 n)
     float* grec = I.D + S.offD;
@@ -192,21 +207,27 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
             }
         }
     }
-    const unsigned rbase = gr_smem(recs), bbase = gr_smem(bars);
+    const unsigned rbase = gr_smem(recs), bbase = gr_smem(bars), ybase = gr_smem(ready);
     if (tid == 0) {
-        for (int q = 0; q < R; ++q)
+        for (int q = 0; q < R; ++q) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bbase + 8u * (unsigned)q) : "memory");
+            if (Sh::VIA) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(ybase + 8u * (unsigned)q) : "memory");
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         // a record from another CTA completes the slot's phase by its bytes
-        // (armed here); a record of this CTA by its producer's arrival
-        for (int q = 0; q < R && q < npan; ++q)
+        // (armed here, with VIA by the warp that fetches it); a record of this
+        // CTA by its producer's arrival
+        for (int q = 0; q < R && q < npan && !Sh::VIA; ++q)
             if (q / NW != (int)rank) gr_arm(bbase + 8u * (unsigned)q, BYTES);
     }
     for (int i = tid; i < NPAD; i += Sh::NT) {
         pivrow[i] = i;
         pivval[i] = 1.f;
     }
-    if (tid < R) colready[tid] = 0;
+    if (tid < R) {
+        colready[tid] = 0;
+        fetched[tid] = 0;
+    }
     gr_cluster_sync();
 
     unsigned usedm = 0u;   // bit a: row lane + 32 a has been a pivot
@@ -233,8 +254,30 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
         // last column is then all that stands between the two panels)
         const bool follow = !mine && P / NW == (int)rank && (P + 1) / NW == (int)rank && (P + 1) % NW == warp;
         if (!mine && !follow && !timed_out) {
+            const unsigned par = (unsigned)(P / R) & 1u;
             long long it = 0;
-            while (!gr_try(bar, (unsigned)(P / R) & 1u))
+            if constexpr (Sh::VIA) {
+                // the first warp here fetches the record for its CTA (a warp
+                // idles here while the owner works; the slot is free: the owner
+                // passed the cluster barrier after every reader of its last use)
+                if (P / NW != (int)rank && lane == 0 && atomicExch(&fetched[slot], P + 1) != P + 1) {
+                    const unsigned rdy = ybase + 8u * (unsigned)slot;
+                    while (!gr_try(rdy, par))
+                        if (++it > GR_WAIT_LIMIT) {
+                            timed_out = true;
+                            break;
+                        }
+                    if (!timed_out) {
+                        asm volatile("fence.proxy.async;" ::: "memory");
+                        gr_arm(bar, BYTES);
+                        gr_fetch(rbase + 4u * (unsigned)(slot * REC), grec + slot * REC, BYTES, bar);
+                        it = -GR_WAIT_LIMIT;   // twice the limit for the copy it has in flight
+                    }
+                }
+                timed_out = __any_sync(GR_FULL, timed_out);
+                it = __shfl_sync(GR_FULL, it, 0);
+            }
+            while (!timed_out && !gr_try(bar, par))
                 if (++it > GR_WAIT_LIMIT) {
                     timed_out = true;
                     break;
@@ -313,7 +356,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
                 for (int q = 0; q < RA / 4; ++q)
                     *reinterpret_cast<float4*>(rc + c * NPAD + lane * RA + 4 * q) =
                         make_float4(col[4 * q], col[4 * q + 1], col[4 * q + 2], col[4 * q + 3]);
-                if constexpr (Sh::MC) {
+                if constexpr (Sh::VIA) {
 #pragma unroll
                     for (int q = 0; q < RA / 4; ++q)
                         *reinterpret_cast<float4*>(grec + slot * REC + c * NPAD + lane * RA + 4 * q) =
@@ -360,30 +403,25 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
                 for (int a = 0; a < RA; ++a) V[a][c] = (lane + 32 * a == p) ? 1.f : -col[a] * ip;
                 if (lane == (p & 31)) usedm |= 1u << (p >> 5);
             }
-            // the finished record: one arrival here, and to the other CTAs one
-            // multicast bulk copy from global memory (clusters of more than 8:
-            // 15 copies of a 12 KB record through one SM's port took longer
-            // than the panel; slabs of 540 to 740 unknowns 986 -> 707 us and
-            // 1520 -> 1106 us a level) or one bulk copy each (the copy engine reads the
-            // record after the proxy fence)
-            if constexpr (Sh::MC) {
+            // the finished record: one arrival here, and to the other CTAs either
+            // one bulk copy each (the copy engine reads the record after the proxy
+            // fence) or, in clusters of 16, an arrival that lets them fetch it: 15
+            // copies of a 12 KB record through one SM's port took longer than the
+            // panel (slabs of 540 and 740 unknowns, a level: 965 -> 722 us and
+            // 1519 -> 1143 us)
+            if constexpr (Sh::VIA) {
                 __threadfence();
                 asm volatile("fence.proxy.async;" ::: "memory");
             } else {
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             }
             __syncwarp();
-            if (lane == 0) {
-                gr_arrive(bar);   // this CTA's warps first: the next panel's owner is most often here
+            if (lane == 0) gr_arrive(bar);   // this CTA's warps first: the next panel's owner is most often here
+            if constexpr (Sh::VIA) {
+                // one arrival a panel in every CTA, this one too (the phases count panels)
+                if (lane < CL) gr_arrive_at(gr_mapa(ybase + 8u * (unsigned)slot, (unsigned)lane));
+            } else if (lane == 0) {
                 const unsigned src = rbase + 4u * (unsigned)(slot * REC);
-                if constexpr (Sh::MC) {
-                    const unsigned short mask = (unsigned short)(((1u << CL) - 1u) & ~(1u << rank));
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], [%1], "
-                        "%2, [%3], %4;" ::"r"(src),
-                        "l"(grec + slot * REC), "r"(BYTES), "r"(bar), "h"(mask)
-                        : "memory");
-                } else {
 #pragma unroll 1
                 for (int r = 0; r < CL; ++r) {
                     if (r == (int)rank) continue;
@@ -392,7 +430,6 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
                             gr_mapa(src, (unsigned)r)),
                         "r"(src), "r"(BYTES), "r"(gr_mapa(bar, (unsigned)r))
                         : "memory");
-                }
                 }
             }
         } else {
@@ -459,7 +496,7 @@ __global__ void __launch_bounds__(32 * NW, 1) k_gjr_inverse(IfPtrs I, const Elim
         }
         __syncwarp();   // the copy is rewritten at the next panel
         // re-arm the slot for the record R panels on, once its phase is complete here
-        if (tid == 0 && !timed_out && P + R < npan && (P + R) / NW != (int)rank) gr_arm(bar, BYTES);
+        if (!Sh::VIA && tid == 0 && !timed_out && P + R < npan && (P + R) / NW != (int)rank) gr_arm(bar, BYTES);
     }
 
     __syncthreads();
