@@ -1456,6 +1456,8 @@ static int solve_interface_body(mrcm_handle* h) {
         h->slab_variant = 1;
     if (h->slab_variant < 0 && cands.size() == 1) h->slab_variant = 1;
     double lu_measured = -1.0;   // the LU's final residual when this call's tuning ran it
+    int missed = -1;             // the kept choice when it missed ir_tol in this call, and its run
+    RefineOut missed_run;
     if (h->tune_kept) {
         // the choice made for an earlier permeability (the shapes are the
         // same): used if it reaches ir_tol, else made again below
@@ -1464,6 +1466,9 @@ static int solve_interface_body(mrcm_handle* h) {
         if (rc && rc != MRCM_ERR_SINGULAR) return rc;
         if (rc || !(o.worst <= if_target(h))) {
             h->err.clear();
+            missed = h->slab_variant;
+            missed_run = o;
+            if (rc) missed_run.worst = INFINITY;
             rc = 0;
             o = RefineOut();
             hist += " (tuned again)";
@@ -1472,13 +1477,14 @@ static int solve_interface_body(mrcm_handle* h) {
         }
     }
     if (h->slab_variant < 0) {
-        // autotuner: the cached choice for this shape class, else every
-        // admissible slab inverse timed on this solve (device time of the
-        // factorisation and the refinement steps) and the fastest one that
-        // converges kept (the LU when none does)
+        // autotuner: the cached choice for this shape class (unless it is the
+        // one that has just missed ir_tol), else every admissible slab inverse
+        // timed on this solve (device time of the factorisation and the
+        // refinement steps) and the fastest one that converges kept (the LU
+        // when none does)
         const std::string key = tune_key(h);
         const int cached = tune_cache_lookup(key);
-        if (cached >= 0 && std::find(cands.begin(), cands.end(), cached) != cands.end()) {
+        if (cached >= 0 && cached != missed && std::find(cands.begin(), cands.end(), cached) != cands.end()) {
             h->slab_variant = cached;
             h->tune_choice = cached;
             h->tune_source = 1;
@@ -1487,8 +1493,15 @@ static int solve_interface_body(mrcm_handle* h) {
             RefineOut run[3];
             bool ok[3] = {false, false, false};
             int steps[3] = {0, 0, 0};
+            int last = -1;   // the variant whose run the handle's state is
             for (int c : cands) {
-                h->slab_variant = c;
+                if (c == missed) {   // run above
+                    run[c] = missed_run;
+                    h->tune_ms[c] = run[c].ms;
+                    steps[c] = run[c].it;
+                    continue;
+                }
+                h->slab_variant = last = c;
                 hist += std::string(" [") + kSlabNames[c] + "]";
                 if ((rc = factor_refine(h, &run[c], &hist))) {
                     if (rc != MRCM_ERR_SINGULAR) return rc;
@@ -1505,7 +1518,6 @@ static int solve_interface_body(mrcm_handle* h) {
             // the variants differ (a 64x64 problem: 178 and 199 us), and results
             // depend on the choice in the last bits: where the two fastest are
             // within a quarter of each other, both once more, the lower time counts
-            int last = cands.back();   // the variant whose run the handle's state is
             int f1 = -1, f2 = -1;
             for (int c : cands) {
                 if (!ok[c]) continue;
