@@ -290,14 +290,18 @@ int mrcm_backward(mrcm_handle* h, const double* dL_du, const double* dL_dp, doub
  * most 256 unknowns); an LU factorisation followed by the inverse columns
  * (any size).  The first mrcm_solve_interface of a handle times every
  * admissible variant -- device time of the factorisation and of the
- * refinement steps it needs -- and keeps the fastest one that reaches ir_tol
- * (the LU when none does); a later refinement that stalls with a Gauss-Jordan
- * variant switches the handle to the LU.  mrcm_set_permeability keeps the
- * choice (it is one of shapes): the next solve uses it, and measures again
- * only if it does not reach ir_tol on the new operator.  With the environment variable MRCM_TUNE_CACHE naming a JSON file,
- * the choice is read from it by shape class (dimension, slab size, slab and
- * level counts, members, precision, space, ir_tol) when present and written to
- * it after a measurement.
+ * refinement steps it needs -- and keeps one that reaches ir_tol (the one that
+ * got closest when none does): the first of them in that order that takes at
+ * most 5/4 of the fastest one's time (in slabs of at most 24 unknowns the
+ * blocked elimination before the register-resident one where it needs fewer
+ * refinement steps), so that handles of one problem agree.  A later
+ * refinement that stalls with a Gauss-Jordan variant switches the handle to
+ * the LU.  mrcm_set_permeability keeps the choice (it is one of shapes): the
+ * next solve uses it, and measures again only if it does not reach ir_tol on
+ * the new operator.  With the environment variable MRCM_TUNE_CACHE naming a
+ * JSON file, the choice is read from it by shape class (dimension, slab size,
+ * slab and level counts, members, precision, space, ir_tol) when present and
+ * written to it after a measurement.
  *
  * Per-call metrics.  With the environment variable MRCM_METRICS naming a file
  * (or "stderr"), every outermost call among mrcm_build_basis,

@@ -1438,6 +1438,19 @@ static void tune_cache_store(const std::string& key, int variant, const double* 
     std::rename(tmp.c_str(), path);
 }
 
+// The choice among measured variants.  Results depend on it in the last bits,
+// and one timing of a few hundred microseconds is off by up to a tenth, so it
+// does not follow the stopwatch alone: the register-resident Gauss-Jordan is
+// preferred, then the blocked one, then the LU; in slabs of at most TUNE_SMALL
+// unknowns the blocked one first where it needs fewer refinement steps (a number
+// that does not vary).  A preferred variant loses only to one that is faster by
+// more than the factor TUNE_SLACK.  On 216 problems of 2 x 2 to 32 x 32
+// subdomains it was the fastest or within 2 %; register against blocked in slabs
+// of 14 unknowns: 338 us in three steps against 300 us in two, 337 us against 364
+// us in three each; in slabs of 62 unknowns 387 us in three against 437 us in two.
+constexpr double TUNE_SLACK = 1.25;
+constexpr int TUNE_SMALL = 24;
+
 static int solve_interface_body(mrcm_handle* h) {
     if (!h) return MRCM_ERR_BAD_INPUT;
     if (h->stage != ST_BASIS) return fail(h, MRCM_ERR_STATE, "mrcm_solve_interface must follow mrcm_build_basis");
@@ -1480,8 +1493,7 @@ static int solve_interface_body(mrcm_handle* h) {
         // autotuner: the cached choice for this shape class (unless it is the
         // one that has just missed ir_tol), else every admissible slab inverse
         // timed on this solve (device time of the factorisation and the
-        // refinement steps) and the fastest one that converges kept (the LU
-        // when none does)
+        // refinement steps) and one of those that converge kept
         const std::string key = tune_key(h);
         const int cached = tune_cache_lookup(key);
         if (cached >= 0 && cached != missed && std::find(cands.begin(), cands.end(), cached) != cands.end()) {
@@ -1494,7 +1506,10 @@ static int solve_interface_body(mrcm_handle* h) {
             bool ok[3] = {false, false, false};
             int steps[3] = {0, 0, 0};
             int last = -1;   // the variant whose run the handle's state is
-            for (int c : cands) {
+            // (in reverse order of preference: no run is repeated when the
+            // preferred one, run last, is taken)
+            for (auto it = cands.rbegin(); it != cands.rend(); ++it) {
+                const int c = *it;
                 if (c == missed) {   // run above
                     run[c] = missed_run;
                     h->tune_ms[c] = run[c].ms;
@@ -1514,34 +1529,22 @@ static int solve_interface_body(mrcm_handle* h) {
                 h->tune_ms[c] = run[c].ms;
                 steps[c] = run[c].it;
             }
-            // one timing of a few hundred microseconds can be off by more than
-            // the variants differ (a 64x64 problem: 178 and 199 us), and results
-            // depend on the choice in the last bits: where the two fastest are
-            // within a quarter of each other, both once more, the lower time counts
-            int f1 = -1, f2 = -1;
-            for (int c : cands) {
-                if (!ok[c]) continue;
-                if (f1 < 0 || run[c].ms < run[f1].ms) f2 = f1, f1 = c;
-                else if (f2 < 0 || run[c].ms < run[f2].ms) f2 = c;
-            }
-            if (f2 >= 0 && run[f2].ms <= 1.25 * run[f1].ms)
-                for (int c : {f2, f1}) {
-                    RefineOut again;
-                    h->slab_variant = last = c;
-                    hist += std::string(" [") + kSlabNames[c] + "]";
-                    if ((rc = factor_refine(h, &again, &hist))) return rc;
-                    again.ms = std::min(again.ms, run[c].ms);
-                    run[c] = again;
-                    h->tune_ms[c] = again.ms;
-                }
-            // the fastest that converges; when none does, the one that got
-            // closest (the GMRES fallback continues from its iterate)
-            int choice = 1;
+            // the preferred one of those that converge in at most 5/4 of the
+            // fastest one's time; when none converges, the one that got closest
+            // (the GMRES fallback continues from its iterate)
+            int fastest = -1, choice = 1;
             for (int c : cands)
-                if (ok[c] && (!ok[choice] || run[c].ms < run[choice].ms)) choice = c;
-            if (!ok[choice])
+                if (ok[c] && (fastest < 0 || run[c].ms < run[fastest].ms)) fastest = c;
+            if (fastest >= 0) {
+                const bool blocked_first = ok[0] && h->npad <= TUNE_SMALL && steps[0] < steps[2];
+                const int order[3] = {blocked_first ? 0 : 2, blocked_first ? 2 : 0, 1};
+                choice = fastest;
+                for (int k = 2; k >= 0; --k)
+                    if (ok[order[k]] && run[order[k]].ms <= TUNE_SLACK * run[fastest].ms) choice = order[k];
+            } else {
                 for (int c : cands)
                     if (std::isfinite(run[c].worst) && !(run[c].worst >= run[choice].worst)) choice = c;
+            }
             h->tune_source = 2;
             lu_measured = run[1].worst;
             tune_cache_store(key, choice, h->tune_ms, steps);
