@@ -409,14 +409,16 @@ __device__ __forceinline__ void store_line(const T (&a)[BW], T* S, int b, int ld
 // 1 / v for the pivots.  FP32: the hardware approximation and one
 // Newton-Raphson step.  FP64: from the FP32 seed r one third-order step,
 // r + r (e + e^2) with e = 1 - v r (e is about 2^-22, the error left e^3); the
-// conversions on the integer pipe.  Outside the FP32 normal range the division.
+// conversions on the integer pipe.  The division outside the FP32 normal range,
+// and from 2^126 on, where the seed would be subnormal and flushed to zero.
 __device__ __forceinline__ float rcp_piv(float v) {
     float r;
     asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
     return fmaf(r, fmaf(-v, r, 1.f), r);
 }
 __device__ __forceinline__ double rcp_piv(double v) {
-    if (!in_f32_range(v)) return 1.0 / v;
+    const unsigned e11 = ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
+    if (e11 < 1023u - 126u || e11 > 1023u + 125u) return 1.0 / v;
     const double r = f2d_bits(__frcp_rn(d2f_bits(v)));
     const double e = fma(-v, r, 1.0);
     return fma(r, fma(e, e, e), r);
