@@ -477,14 +477,14 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
     h->mth.pad = 0;
     for (int s = 0; s < nitems && d == 2 && prec != MRCM_FP64; ++s) {
         const SubDev& sd = h->sub[s];
-        const size_t lim = 227 * 1024;
+        const size_t lim = SMEM_LOCAL2D;
         const int bx = sd.hih[0] - sd.loh[0], by = sd.hih[1] - sd.loh[1];
         const int ix = sd.hi[0] - sd.lo[0], iy = sd.hi[1] - sd.lo[1];
         h->mth.pad = std::max(h->mth.pad, (bx + 3) & ~3);
         if (bx > 32) break;   // refused below
         const int nb = std::max(std::min(sd.nbasis + (h->mth.part_hat ? 1 : 0), 4), 1);
         if (local2d_smem(prec, bx, by, nb, false, 1) > lim || local2d_smem(prec, ix, iy, 1, true, 1) > lim ||
-            smooth2d_smem(prec, bx, by, 1) > lim || adj_smooth2d_smem(prec, bx, by, 1) > lim) {
+            smooth2d_smem(prec, bx, by, 1) > SMEM_SMOOTH2D || adj_smooth2d_smem(prec, bx, by, 1) > lim) {
             h->mth.pad = 0;
             break;
         }
@@ -531,11 +531,11 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
         if (!h->mth.same_alpha) add(JOB_SFACT, bx, by, 0, false);
         h->smooth_smem = std::max(h->smooth_smem, smooth2d_smem(prec, bx, by, pad));
     }
-    if (h->smooth_smem > 227 * 1024) return fail(h, MRCM_ERR_UNSUPPORTED, "subdomain box too large for shared memory");
+    if (h->smooth_smem > (d == 3 ? SMEM_SMOOTH3D : SMEM_SMOOTH2D)) return fail(h, MRCM_ERR_UNSUPPORTED, "subdomain box too large for shared memory");
     std::vector<Job> jobs;
     for (auto& kv : byw) {
         JobClass jc{kv.first, smem_w[kv.first], (int)jobs.size(), (int)kv.second.size()};
-        if (jc.smem > 227 * 1024) return fail(h, MRCM_ERR_UNSUPPORTED, "subdomain box too large for shared memory");
+        if (jc.smem > (d == 3 ? SMEM_LOCAL3D : SMEM_LOCAL2D)) return fail(h, MRCM_ERR_UNSUPPORTED, "subdomain box too large for shared memory");
         h->jclasses.push_back(jc);
         jobs.insert(jobs.end(), kv.second.begin(), kv.second.end());
     }
@@ -688,9 +688,9 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
     {
         size_t nmv = 0;
         for (auto& sl : h->slabs) nmv = std::max(nmv, (size_t)std::max(sl.nm, sl.nv));
-        while (elim_cw > 32 && elim_smem_bytes((int)nmv, elim_cw) > 227 * 1024) elim_cw = (elim_cw + 1) / 2;
+        while (elim_cw > 32 && elim_smem_bytes((int)nmv, elim_cw) > SMEM_CTA) elim_cw = (elim_cw + 1) / 2;
         h->elim_smem = elim_smem_bytes((int)nmv, elim_cw);
-        if (h->elim_smem > 227 * 1024) return fail(h, MRCM_ERR_UNSUPPORTED, "interface coupling blocks too large");
+        if (h->elim_smem > SMEM_CTA) return fail(h, MRCM_ERR_UNSUPPORTED, "interface coupling blocks too large");
         // 1 KB of the 227 KB per block is left to the slab LU's static shared memory
         while (xch > 4 && lu_smem(npad, xch) > 226 * 1024) xch /= 2;
         if (lu_smem(npad, xch) > 226 * 1024) return fail(h, MRCM_ERR_UNSUPPORTED, "interface slabs too large");
@@ -960,7 +960,7 @@ static int prepare_adjoint(mrcm_handle* h) {
     const int prec = h->prm.precision;
     const int nitems = (int)h->sub.size();
     const int nmem = (int)h->mem.size();
-    const size_t lim = 227 * 1024;
+    const size_t lim = SMEM_LOCAL2D;
     // jobs: basis problem on hat-Omega_i and particular problem on Omega_i,
     // grouped by band width and the number of warps that fit in shared memory
     std::map<std::pair<int, int>, std::vector<Job>> by;

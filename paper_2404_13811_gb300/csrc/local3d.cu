@@ -1033,7 +1033,7 @@ __host__ __device__ inline Lay3 lay3(int tsz, int nx, int ny, int nz, int nr, bo
     L.stage = tsz * rows * ld;
     const size_t tail = 64 + 32 + 2 * sizeof(uint64_t) * ST3;
     L.st = ST3;
-    while (L.st > 2 && L.fixed + L.work + L.st * L.stage + tail > 226 * 1024) --L.st;   // (1 KB for static shared memory)
+    while (L.st > 2 && L.fixed + L.work + L.st * L.stage + tail > 226 * 1024) --L.st;
     const size_t sol = L.work + L.st * L.stage;
     L.total = L.fixed + (L.fac > sol ? L.fac : sol) + tail;
     return L;
@@ -1041,10 +1041,10 @@ __host__ __device__ inline Lay3 lay3(int tsz, int nx, int ny, int nz, int nr, bo
 
 // Right-hand sides of a basis round: NR3, fewer where the work vectors of so
 // many do not fit (mixed form, boxes that nearly fill shared memory with their
-// operator: 3 x 22 x 34 cells take three).
+// operator: 3 x 22 x 34 cells take three, 7 x 15 x 22 two).
 __host__ __device__ inline int round3(int tsz, int nx, int ny, int nz) {
     int nr = NR3;
-    while (nr > 1 && lay3(tsz, nx, ny, nz, nr, false, false).total > 227 * 1024) --nr;
+    while (nr > 1 && lay3(tsz, nx, ny, nz, nr, false, false).total > SMEM_LOCAL3D) --nr;
     return nr;
 }
 

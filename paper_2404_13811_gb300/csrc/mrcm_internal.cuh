@@ -112,6 +112,15 @@ struct MethodDev {
 };
 
 
+// Dynamic shared memory the box kernels can have: the CTA's 227 KB less the
+// kernel's static shared memory (as the compiler reports it; the sizes of the
+// layouts are multiples of 16 bytes).
+constexpr size_t SMEM_CTA = 227 * 1024;
+constexpr size_t SMEM_LOCAL2D = SMEM_CTA - 128;    // k_local2d, k_adj_local2d, k_adj_smooth2d
+constexpr size_t SMEM_SMOOTH2D = SMEM_CTA - 144;
+constexpr size_t SMEM_LOCAL3D = SMEM_CTA - 480;
+constexpr size_t SMEM_SMOOTH3D = SMEM_CTA - 448;
+
 // Device pointers of the interface system.
 struct IfPtrs {
     double* Gv;    // [row][2][NB] FP64 row entries (owner block, neighbour block)
