@@ -820,9 +820,13 @@ __device__ void sweeps3(const Box3& B, const T* __restrict__ F, const T* c2s, T*
     }
 }
 
-__device__ __forceinline__ void warp_max_to(unsigned int* a, float v) {
-    for (int o = 16; o; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(a, __float_as_uint(v));
+// Maximum norms by the bits of |v|, whose order is that of the values, with NaN
+// above infinity: fmaxf would drop a NaN, and a solve whose every entry is one
+// would count as converged.
+__device__ __forceinline__ unsigned abs_bits(float v) { return __float_as_uint(v) & 0x7fffffffu; }
+__device__ __forceinline__ void warp_max_to(unsigned int* a, unsigned v) {
+    v = __reduce_max_sync(0xffffffffu, v);
+    if ((threadIdx.x & 31) == 0) atomicMax(a, v);
 }
 
 // Solves A x_q = rhs_q for NR right-hand sides with the whole CTA: sweeps
@@ -848,7 +852,7 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
     __syncthreads();
 #pragma unroll
     for (int q = 0; q < NR; ++q) {
-        float bn = 0.f, rn = 0.f;
+        unsigned bn = 0u, rn = 0u;
         for (int t = tid; t < nc; t += nt) {
             const double v = rhs(q, t);
             double r = v;
@@ -856,8 +860,8 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
             else X[q * nc + t] = 0.0;
             if constexpr (mixed) W[q * nc + t] = d2f_bits(r);
             else W[q * nc + t] = r;
-            bn = fmaxf(bn, fabsf((float)v));
-            rn = fmaxf(rn, fabsf((float)r));
+            bn = max(bn, abs_bits((float)v));
+            rn = max(rn, abs_bits((float)r));
         }
         warp_max_to(&nrm[q], bn);
         warp_max_to(&nrm[NR3 + q], rn);
@@ -901,16 +905,16 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
         __syncthreads();
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
-            float rn = 0.f;
+            unsigned rn = 0u;
             for (int t = tid; t < nc; t += nt) {
                 const double v = resid3(O, s1, s2, X + q * nc, rhs(q, t), t);
                 if constexpr (mixed) {
                     const float w = d2f_bits(v);
                     W[q * nc + t] = w;
-                    rn = fmaxf(rn, fabsf(w));
+                    rn = max(rn, abs_bits(w));
                 } else {
                     W[q * nc + t] = v;
-                    rn = fmaxf(rn, fabsf((float)v));
+                    rn = max(rn, abs_bits((float)v));
                 }
             }
             warp_max_to(&nrm[NR3 + q], rn);
