@@ -138,27 +138,35 @@ __device__ __forceinline__ double apply_A(const Box& B, const Ops& O, const doub
 // FP64 -> FP32 truncates the mantissa -- it serves only the right-hand side
 // of a correction solve, where an error below one FP32 ulp is immaterial --
 // flushes results below the FP32 normal range to zero and takes larger ones
-// to infinity (NaN stays NaN).
-__device__ __forceinline__ double f2d_bits(float f) {
+// to infinity (NaN stays NaN).  ex: the FP32 value stands for f 2^-ex.
+__device__ __forceinline__ double f2d_bits(float f, int ex = 0) {
     const unsigned u = __float_as_uint(f);
     const unsigned e = (u >> 23) & 0xffu;
     const unsigned hs = u & 0x80000000u;
-    const unsigned e11 = e == 0xffu ? 0x7ffu : e + 896u;
+    const unsigned e11 = e == 0xffu ? 0x7ffu : e + (unsigned)(896 - ex);
     const unsigned hi = e == 0u ? hs : (hs | (e11 << 20) | ((u & 0x7fffffu) >> 3));
     const unsigned lo = e == 0u ? 0u : (u << 29);
     return __hiloint2double((int)hi, (int)lo);
 }
-__device__ __forceinline__ float d2f_bits(double d) {
+__device__ __forceinline__ float d2f_bits(double d, int ex = 0) {
     const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
     const unsigned s = hi & 0x80000000u;
     const int e11 = (int)((hi >> 20) & 0x7ffu);
-    const int e = e11 - 896;
+    const int e = e11 - 896 + ex;
     const unsigned m = ((hi & 0xfffffu) << 3) | (lo >> 29);
     unsigned r = s | ((unsigned)e << 23) | m;
     if (e <= 0) r = s;
     if (e >= 255) r = s | 0x7f800000u | ((e11 == 0x7ff && ((hi & 0xfffffu) | lo)) ? 0x400000u : 0u);
     return __uint_as_float(r);
 }
+
+// The exponent ex that takes a vector of FP64 values to FP32 values of at most
+// 2 in magnitude, from the largest high word of the values (without signs).  A
+// refinement follows its right-hand side down by twelve or more digits, and
+// residuals below the FP32 normal range, flushed to zero, would count as
+// converged: with right-hand sides of 1e-30 the result is off by 1e-7.
+__device__ __forceinline__ unsigned abs_hi(double d) { return (unsigned)__double2hiint(d) & 0x7fffffffu; }
+__device__ __forceinline__ int norm_shift(unsigned hmax) { return max(-896, min(896, 1023 - (int)(hmax >> 20))); }
 
 // d2f_bits rounded to nearest (ties away from zero): for values that stay in the
 // factor, where truncation would shift every pivot the same way.
@@ -1245,8 +1253,10 @@ __device__ __forceinline__ void cell_ij(int c, int b, float rb, int& i, int& j) 
 // scaled norm).  Cells are visited 32 at a time by all lanes.  On exit x
 // holds x~ (the caller scales back with dsc).  Returns the number of sweeps.
 // SW: the line width where it is a template's (0: by column; -1: the row path
-// of the width b where there is one, chosen at run time).
-template <typename Rhs, int SW = 0>
+// of the width b where there is one, chosen at run time).  NORM: the FP32
+// vectors scaled by the right-hand side's exponent (the reverse pass, whose
+// seeds may be of any size).
+template <typename Rhs, int SW = 0, bool NORM = false>
 __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, const float* cys, double* x, float* w,
                              float* zbuf, const Rhs& rhs, double tol, int max_ir, int* noconv) {
     const int lane = threadIdx.x & 31;
@@ -1254,14 +1264,29 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
     const float rb = 1.f / (float)b;
     const int nit = (B.n + 31) >> 5;
     float bn = 0.f;
+    unsigned hm = 0u;
     for (int k = 0; k < nit; ++k) {
         const int c = k * 32 + lane;
         const bool ok = c < B.n;
         int i, j;
         cell_ij(ok ? c : 0, b, rb, i, j);
         const double bt = rhs(B, i, j);
-        if (ok) {
+        if (!ok) continue;
+        if constexpr (NORM) {
+            x[c] = bt;
+            hm = max(hm, abs_hi(bt));
+        } else {
             const float wc = d2f_bits(bt);
+            x[c] = 0.0;
+            w[c] = wc;
+            bn = fmaxf(bn, fabsf(wc));
+        }
+    }
+    int ex = 0;
+    if constexpr (NORM) {
+        ex = norm_shift(__reduce_max_sync(0xffffffffu, hm));
+        for (int c = lane; c < B.n; c += 32) {
+            const float wc = d2f_bits(x[c], ex);
             x[c] = 0.0;
             w[c] = wc;
             bn = fmaxf(bn, fabsf(wc));
@@ -1274,7 +1299,7 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
         if constexpr (SW > 0) tw_warp<float, SW>(Sinv, cys, w, zbuf, b, nb);
         else if constexpr (SW < 0) warp_sweeps<float>(Sinv, cys, w, zbuf, b, nb, b);
         else tw_warp<float, 0>(Sinv, cys, w, zbuf, b, nb);
-        for (int c = lane; c < B.n; c += 32) x[c] += f2d_bits(w[c]);
+        for (int c = lane; c < B.n; c += 32) x[c] += f2d_bits(w[c], ex);
         __syncwarp();
         float rn = 0.f;
         for (int k = 0; k < nit; ++k) {
@@ -1284,7 +1309,7 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
             cell_ij(ok ? c : 0, b, rb, i, j);
             const double bt = rhs(B, i, j);
             if (ok) {
-                const float wc = d2f_bits(resid_sc(B, O, x, bt, c, i, j));
+                const float wc = d2f_bits(resid_sc(B, O, x, bt, c, i, j), ex);
                 w[c] = wc;
                 rn = fmaxf(rn, fabsf(wc));
             }
@@ -1297,26 +1322,36 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
     return it;
 }
 
-// The same by the whole CTA (the smoothing solves): sweeps by warp 0 (both
-// chains), FP64 updates and residuals over all threads.  warm: x holds a
+// The same by the whole CTA (the smoothing solves): sweeps by two warps (a
+// chain each), FP64 updates and residuals over all threads.  warm: x holds a
 // starting x~ and the refinement starts from its residual (stopping rule
 // still relative to b~; no sweep when the start meets it).  b~ is stored.
 // BB > 0: lines of width at most BB; BB = 0: any width by a switch (bp).
-template <int BB = 0>
+// nrm: 3 entries.
+template <int BB = 0, bool NORM = false>
 __device__ int cta_solve_sc(const Box& B, const Ops& O, const float* Sinv, const float* cys, double* x, float* w,
                             float* zw, unsigned int* nrm, const double* bt, double tol, int max_ir, int* noconv,
                             bool warm, int bp) {
     const int tid = threadIdx.x, nt = blockDim.x;
     const int b = B.nx, nb = B.ny;
     const float rb = 1.f / (float)b;
-    if (tid < 2) nrm[tid] = 0u;
+    if (tid < 3) nrm[tid] = 0u;
     __syncthreads();
+    int ex = 0;
+    if constexpr (NORM) {
+        unsigned hm = 0u;
+        for (int c = tid; c < B.n; c += nt) hm = max(hm, abs_hi(bt[c]));
+        hm = __reduce_max_sync(0xffffffffu, hm);
+        if ((tid & 31) == 0) atomicMax(&nrm[2], hm);
+        __syncthreads();
+        ex = norm_shift(nrm[2]);
+    }
     float bn = 0.f, r0 = 0.f;
     for (int c = tid; c < B.n; c += nt) {
         int i, j;
         cell_ij(c, b, rb, i, j);
-        const float wb = d2f_bits(bt[c]);
-        const float wc = warm ? d2f_bits(resid_sc(B, O, x, bt[c], c, i, j)) : wb;
+        const float wb = d2f_bits(bt[c], ex);
+        const float wc = warm ? d2f_bits(resid_sc(B, O, x, bt[c], c, i, j), ex) : wb;
         w[c] = wc;
         bn = fmaxf(bn, fabsf(wb));
         r0 = fmaxf(r0, fabsf(wc));
@@ -1344,14 +1379,14 @@ __device__ int cta_solve_sc(const Box& B, const Ops& O, const float* Sinv, const
             if (tid < 64) warp2_sweeps(Sinv, cys, w, zw, b, nb, bp);
         }
         __syncthreads();
-        for (int c = tid; c < B.n; c += nt) x[c] += f2d_bits(w[c]);
+        for (int c = tid; c < B.n; c += nt) x[c] += f2d_bits(w[c], ex);
         if (tid == 0) nrm[1] = 0u;
         __syncthreads();
         float rn = 0.f;
         for (int c = tid; c < B.n; c += nt) {
             int i, j;
             cell_ij(c, b, rb, i, j);
-            const float wc = d2f_bits(resid_sc(B, O, x, bt[c], c, i, j));
+            const float wc = d2f_bits(resid_sc(B, O, x, bt[c], c, i, j), ex);
             w[c] = wc;
             rn = fmaxf(rn, fabsf(wc));
         }

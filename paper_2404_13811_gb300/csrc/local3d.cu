@@ -848,20 +848,43 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
     const int s1 = B.n[B.a0], s2 = B.b;
     const int mit = mixed ? max_ir : 4;
     if (*bad) return 0;   // a staged copy failed earlier: the buffers are not usable
-    if (tid < 3 * NR3) nrm[tid] = tid < 2 * NR3 ? 0u : 0x7f800000u;   // |b|, |r|, |r| of the previous step (inf)
+    // |b|, |r|, |r| of the previous step (inf), and (mixed form) the largest high word of b
+    if (tid < 4 * NR3) nrm[tid] = tid < 2 * NR3 || tid >= 3 * NR3 ? 0u : 0x7f800000u;
     __syncthreads();
+    // mixed form: the FP32 vectors of right-hand side q stand for their values times 2^-shift(q)
+    auto shift = [&](int q) { return norm_shift(nrm[3 * NR3 + q]); };
+    if constexpr (mixed) {
+#pragma unroll
+        for (int q = 0; q < NR; ++q) {
+            unsigned hm = 0u;
+            for (int t = tid; t < nc; t += nt) {
+                const double v = rhs(q, t);
+                if (!warm) X[q * nc + t] = v;   // kept for the next pass
+                hm = max(hm, abs_hi(v));
+            }
+            warp_max_to(&nrm[3 * NR3 + q], hm);
+        }
+        __syncthreads();
+    }
 #pragma unroll
     for (int q = 0; q < NR; ++q) {
         unsigned bn = 0u, rn = 0u;
+        const int ex = mixed ? shift(q) : 0;
         for (int t = tid; t < nc; t += nt) {
-            const double v = rhs(q, t);
+            const double v = mixed && !warm ? X[q * nc + t] : rhs(q, t);
             double r = v;
             if (warm) r = resid3(O, s1, s2, X + q * nc, v, t);
             else X[q * nc + t] = 0.0;
-            if constexpr (mixed) W[q * nc + t] = d2f_bits(r);
-            else W[q * nc + t] = r;
-            bn = max(bn, abs_bits((float)v));
-            rn = max(rn, abs_bits((float)r));
+            if constexpr (mixed) {
+                const float w = d2f_bits(r, ex);
+                W[q * nc + t] = w;
+                bn = max(bn, abs_bits(d2f_bits(v, ex)));
+                rn = max(rn, abs_bits(w));
+            } else {
+                W[q * nc + t] = r;
+                bn = max(bn, abs_bits((float)v));
+                rn = max(rn, abs_bits((float)r));
+            }
         }
         warp_max_to(&nrm[q], bn);
         warp_max_to(&nrm[NR3 + q], rn);
@@ -893,11 +916,13 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
         __syncthreads();
         if (*bad) break;
 #pragma unroll
-        for (int q = 0; q < NR; ++q)
+        for (int q = 0; q < NR; ++q) {
+            const int ex = mixed ? shift(q) : 0;
             for (int t = tid; t < nc; t += nt) {
-                if constexpr (mixed) X[q * nc + t] += f2d_bits(W[q * nc + t]);
+                if constexpr (mixed) X[q * nc + t] += f2d_bits(W[q * nc + t], ex);
                 else X[q * nc + t] += W[q * nc + t];
             }
+        }
         if (tid < NR3) {
             nrm[2 * NR3 + tid] = it == 0 && !warm ? 0x7f800000u : nrm[NR3 + tid];
             nrm[NR3 + tid] = 0u;
@@ -906,10 +931,11 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
             unsigned rn = 0u;
+            const int ex = mixed ? shift(q) : 0;
             for (int t = tid; t < nc; t += nt) {
                 const double v = resid3(O, s1, s2, X + q * nc, rhs(q, t), t);
                 if constexpr (mixed) {
-                    const float w = d2f_bits(v);
+                    const float w = d2f_bits(v, ex);
                     W[q * nc + t] = w;
                     rn = max(rn, abs_bits(w));
                 } else {
