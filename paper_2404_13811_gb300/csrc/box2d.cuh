@@ -170,9 +170,10 @@ __device__ __forceinline__ int norm_shift(unsigned hmax) { return max(-896, min(
 
 // d2f_bits rounded to nearest (ties away from zero): for values that stay in the
 // factor, where truncation would shift every pivot the same way.
-__device__ __forceinline__ float d2f_near(double d) {
-    const float t = d2f_bits(d);
-    return in_f32_range(d) ? __uint_as_float(__float_as_uint(t) + (((unsigned)__double2loint(d) >> 28) & 1u)) : t;
+__device__ __forceinline__ float d2f_near(double d, int ex = 0) {
+    const unsigned t = __float_as_uint(d2f_bits(d, ex));
+    const unsigned e = (t >> 23) & 0xffu;
+    return __uint_as_float(e - 1u < 254u ? t + (((unsigned)__double2loint(d) >> 28) & 1u) : t);
 }
 
 // The mixed form refines in Jacobi-scaled variables: O holds D A D (D =
@@ -414,16 +415,11 @@ __device__ __forceinline__ void store_line(const T (&a)[BW], T* S, int b, int ld
     }
 }
 
-// 1 / v for the pivots.  FP32: the hardware approximation and one
-// Newton-Raphson step.  FP64: from the FP32 seed r one third-order step,
+// 1 / v for the pivots.  FP32: correctly rounded.  FP64: from the FP32 seed r one third-order step,
 // r + r (e + e^2) with e = 1 - v r (e is about 2^-22, the error left e^3); the
 // conversions on the integer pipe.  The division outside the FP32 normal range,
 // and from 2^126 on, where the seed would be subnormal and flushed to zero.
-__device__ __forceinline__ float rcp_piv(float v) {
-    float r;
-    asm("rcp.approx.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return fmaf(r, fmaf(-v, r, 1.f), r);
-}
+__device__ __forceinline__ float rcp_piv(float v) { return __frcp_rn(v); }
 __device__ __forceinline__ double rcp_piv(double v) {
     const unsigned e11 = ((unsigned)__double2hiint(v) >> 20) & 0x7ffu;
     if (e11 < 1023u - 126u || e11 > 1023u + 125u) return 1.0 / v;

@@ -876,9 +876,9 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
             if (warm) r = resid3(O, s1, s2, X + q * nc, v, t);
             else X[q * nc + t] = 0.0;
             if constexpr (mixed) {
-                const float w = d2f_bits(r, ex);
+                const float w = d2f_near(r, ex);
                 W[q * nc + t] = w;
-                bn = max(bn, abs_bits(d2f_bits(v, ex)));
+                bn = max(bn, abs_bits(d2f_near(v, ex)));
                 rn = max(rn, abs_bits(w));
             } else {
                 W[q * nc + t] = r;
@@ -935,7 +935,7 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
             for (int t = tid; t < nc; t += nt) {
                 const double v = resid3(O, s1, s2, X + q * nc, rhs(q, t), t);
                 if constexpr (mixed) {
-                    const float w = d2f_bits(v, ex);
+                    const float w = d2f_near(v, ex);
                     W[q * nc + t] = w;
                     rn = max(rn, abs_bits(w));
                 } else {
@@ -1205,8 +1205,8 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
         if constexpr (mixed) {
             T* cs = C.fac + GJW3;   // in-plane couplings in T, in the factor phase's overlay
             for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
-                cs[t] = d2f_bits(C.O.c0[t]);
-                cs[B.nc + t] = d2f_bits(C.O.c1[t]);
+                cs[t] = d2f_near(C.O.c0[t]);
+                cs[B.nc + t] = d2f_near(C.O.c1[t]);
             }
             c0s = cs;
             c1s = cs + B.nc;
