@@ -831,9 +831,10 @@ __device__ __forceinline__ void warp_max_to(unsigned int* a, unsigned v) {
 
 // Solves A x_q = rhs_q for NR right-hand sides with the whole CTA: sweeps
 // with the kept factor (FP32 in the mixed form, FP64 in the FP64 form) and
-// refinement with FP64 residuals, the iterate X in FP64 (mixed form: the
-// scaled x~ = D^-1 x until the end, rhs scaled).  warm: X holds a starting x~.  High-contrast boxes reach a residual floor above what a
-// fixed tolerance can ask for, so the refinement runs to that floor: it stops
+// refinement with FP64 residuals from X = 0, the iterate X in FP64 (mixed form:
+// the scaled x~ = D^-1 x until the end, rhs scaled).  High-contrast boxes reach a
+// residual floor above what a fixed tolerance can ask for, so the refinement runs
+// to that floor: it stops
 // when every right-hand side has |r| <= 1e-3 ir_tol |b| (scaled max norms),
 // or has |r| <= ir_tol |b| and no longer halves its residual per step.  The
 // FP64 form (a direct solve, then refinement with the same rule, at most 4
@@ -841,8 +842,7 @@ __device__ __forceinline__ void warp_max_to(unsigned int* a, unsigned v) {
 // pairs.
 template <typename T, int NR, typename Rhs>
 __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, double* X, T* W, T* vb, T* red,
-                        Pipe3<T>& pp, unsigned int* nrm, const Rhs& rhs, double tol, int max_ir, int* noconv, int* bad,
-                        bool warm) {
+                        Pipe3<T>& pp, unsigned int* nrm, const Rhs& rhs, double tol, int max_ir, int* noconv, int* bad) {
     constexpr bool mixed = std::is_same<T, float>::value;
     const int nc = B.nc, tid = threadIdx.x, nt = blockDim.x;
     const int s1 = B.n[B.a0], s2 = B.b;
@@ -859,7 +859,7 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
             unsigned hm = 0u;
             for (int t = tid; t < nc; t += nt) {
                 const double v = rhs(q, t);
-                if (!warm) X[q * nc + t] = v;   // kept for the next pass
+                X[q * nc + t] = v;   // kept for the next pass
                 hm = max(hm, abs_hi(v));
             }
             warp_max_to(&nrm[3 * NR3 + q], hm);
@@ -868,26 +868,21 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
     }
 #pragma unroll
     for (int q = 0; q < NR; ++q) {
-        unsigned bn = 0u, rn = 0u;
+        unsigned bn = 0u;
         const int ex = mixed ? shift(q) : 0;
         for (int t = tid; t < nc; t += nt) {
-            const double v = mixed && !warm ? X[q * nc + t] : rhs(q, t);
-            double r = v;
-            if (warm) r = resid3(O, s1, s2, X + q * nc, v, t);
-            else X[q * nc + t] = 0.0;
+            const double v = mixed ? X[q * nc + t] : rhs(q, t);
+            X[q * nc + t] = 0.0;
             if constexpr (mixed) {
-                const float w = d2f_near(r, ex);
+                const float w = d2f_near(v, ex);
                 W[q * nc + t] = w;
-                bn = max(bn, abs_bits(d2f_near(v, ex)));
-                rn = max(rn, abs_bits(w));
+                bn = max(bn, abs_bits(w));
             } else {
-                W[q * nc + t] = r;
+                W[q * nc + t] = v;
                 bn = max(bn, abs_bits((float)v));
-                rn = max(rn, abs_bits((float)r));
             }
         }
         warp_max_to(&nrm[q], bn);
-        warp_max_to(&nrm[NR3 + q], rn);
     }
     __syncthreads();
     // done: every residual at its floor; reached: every residual within tol
@@ -902,15 +897,8 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
         }
         return done;
     };
-    bool reached = false;
+    bool reached = false, done = false;
     int it = 0;
-    bool done = warm && test(reached);
-    if (warm) {
-        // a zero right-hand side has the zero solution, whatever the start
-        for (int q = 0; q < NR; ++q)
-            if (nrm[q] == 0u)
-                for (int t = tid; t < nc; t += nt) X[q * nc + t] = 0.0;
-    }
     for (; !done && it < mit; ++it) {
         sweeps3<T, NR>(B, F, c2s, W, vb, red, pp, bad);
         __syncthreads();
@@ -924,7 +912,7 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
             }
         }
         if (tid < NR3) {
-            nrm[2 * NR3 + tid] = it == 0 && !warm ? 0x7f800000u : nrm[NR3 + tid];
+            nrm[2 * NR3 + tid] = it == 0 ? 0x7f800000u : nrm[NR3 + tid];
             nrm[NR3 + tid] = 0u;
         }
         __syncthreads();
@@ -963,10 +951,10 @@ template <typename T, typename Rhs>
 __device__ int solve3(int nr, const Box3& B, const Ops3& O, const T* F, const T* c2s, double* X, T* W, T* vb, T* red,
                       Pipe3<T>& pp, unsigned int* nrm, const Rhs& rhs, double tol, int max_ir, int* noconv, int* bad) {
     switch (nr) {   // the sweeps' work is that of the right-hand sides there are
-        case 1: return solve3_n<T, 1>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad, false);
-        case 2: return solve3_n<T, 2>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad, false);
-        case 3: return solve3_n<T, 3>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad, false);
-        default: return solve3_n<T, 4>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad, false);
+        case 1: return solve3_n<T, 1>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad);
+        case 2: return solve3_n<T, 2>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad);
+        case 3: return solve3_n<T, 3>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad);
+        default: return solve3_n<T, 4>(B, O, F, c2s, X, W, vb, red, pp, nrm, rhs, tol, max_ir, noconv, bad);
     }
 }
 
@@ -1283,7 +1271,7 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
         } else {
             RhsStored3 rs{C.bsrc};
             it = solve3_n<T, 1>(B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rs, Mth.ir_tol, Mth.max_ir,
-                                &C.flags[1], &C.flags[2], false);
+                                &C.flags[1], &C.flags[2]);
         }
         maxit = max(maxit, it);
         nsolve += it * nr;
@@ -1420,18 +1408,13 @@ __global__ void __launch_bounds__(T3, 1) k_smooth3d(DevPtrs P, MethodDev Mth, co
     }
     __syncthreads();
     const double* fm = P.f + md.cell_off;
-    for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
+    for (int t = threadIdx.x; t < B.nc; t += blockDim.x)
         C.bsrc[t] = (mixed ? C.O.dsc[t] : 1.0) * source_rhs3(B, C.O, md, fm, C.lam, t);
-        if constexpr (mixed) {
-            // the refinement starts from the current pressure, scaled (a start only: an FP32 reciprocal)
-            C.X[t] = pst[gidx(B, bcoord(B, t))] * f2d_bits(__frcp_rn(d2f_bits(C.O.dsc[t])));
-        }
-    }
     __syncthreads();
     const T* F = (const T*)P.fac + (size_t)item * P.fac_stride;
     RhsStored3 rs{C.bsrc};
     const int it = solve3_n<T, 1>(B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rs, Mth.ir_tol, Mth.max_ir,
-                                  &C.flags[0], &C.flags[2], mixed);
+                                  &C.flags[0], &C.flags[2]);
     if (C.flags[2]) drain3(C.pp);
     __syncthreads();
     // overwrite (u, p) on Omega_i with the restriction
