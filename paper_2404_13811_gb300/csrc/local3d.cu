@@ -14,8 +14,8 @@
 // round at once, so each plane inverse is read once per sweep.
 //
 // Precision: T = double is the FP64 form.  T = float is the mixed form:
-// Jacobi-scaled operator, Schur diagonals from FP64, FP32 sweeps, FP64
-// residual refinement to ir_tol in the scaled variables (as in 2D).
+// Jacobi-scaled factor, Schur diagonals from FP64, FP32 sweeps on scaled
+// residuals, FP64 residuals of the unscaled operator, refined to ir_tol.
 #include "box2d.cuh"
 
 namespace {
@@ -205,30 +205,45 @@ __device__ void build_ops3(const Box3& B, const MemberDev& md, const DevPtrs& P,
     __syncthreads();
 }
 
-// Mixed form: the operator in scaled variables, D A D (as scale_ops in 2D).
-__device__ void scale_ops3(const Box3& B, Ops3& O) {
-    const int s1 = B.n[B.a0], s2 = B.b;
+// Mixed form: the couplings of the scaled operator D A D in FP32, for the factor
+// and the sweeps (the operator itself stays unscaled).
+__device__ __forceinline__ float scaled3(const Ops3& O, const double* c, unsigned bit, int step, int t) {
+    return (O.nb[t] & bit) ? (float)(c[t] * O.dsc[t] * O.dsc[t + step]) : 0.f;
+}
+
+// Mixed form, after the factorisation: the diagonal's place takes its box-side
+// part, the rest of a row being differences (resid3).
+__device__ void side_diag3(const Box3& B, Ops3& O) {
     for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
         const unsigned char m = O.nb[t];
-        const double d = O.dsc[t];
-        O.cd[t] = O.cd[t] * d * d;
-        O.c0[t] = (m & 2) ? O.c0[t] * d * O.dsc[t + 1] : 0.0;
-        O.c1[t] = (m & 8) ? O.c1[t] * d * O.dsc[t + s1] : 0.0;
-        O.c2[t] = (m & 32) ? O.c2[t] * d * O.dsc[t + s2] : 0.0;
+        double d = 0.0;
+        if ((m & 63) != 63) {
+            const Ijk c = bcoord(B, t);
+            for (int sid = 0; sid < 6; ++sid)
+                if (!(m & B.bit[sid])) d += O.bT[B.soff[sid] + side_e(B, sid, c)];
+        }
+        O.cd[t] = d;
     }
     __syncthreads();
 }
 
-// b_t - (A x)_t in FP64 (both scaled in the mixed form)
+// b_t - (A x)_t in FP64.  DIFF (mixed form): in differences of neighbouring
+// values, so that its rounding is that of the fluxes and not of the pressures.
+// With entries of D A D, each rounded once more, the fluxes of 60 fields of 60 x
+// 110 x 40 cells came out 1.7 times further from the exact ones; with the rows
+// summed up by the unscaled diagonal they did not, but 4 of 60 layered fields of
+// 60 x 220 x 85 cells missed ir_tol (1 of 60 with DIFF and with D A D).
+template <bool DIFF>
 __device__ __forceinline__ double resid3(const Ops3& O, int s1, int s2, const double* x, double bt, int t) {
     const unsigned char m = O.nb[t];
-    double s = fma(-O.cd[t], x[t], bt);
-    if (m & 1) s = fma(O.c0[t - 1], x[t - 1], s);
-    if (m & 2) s = fma(O.c0[t], x[t + 1], s);
-    if (m & 4) s = fma(O.c1[t - s1], x[t - s1], s);
-    if (m & 8) s = fma(O.c1[t], x[t + s1], s);
-    if (m & 16) s = fma(O.c2[t - s2], x[t - s2], s);
-    if (m & 32) s = fma(O.c2[t], x[t + s2], s);
+    const double xt = x[t], x0 = DIFF ? xt : 0.0;
+    double s = fma(-O.cd[t], xt, bt);
+    if (m & 1) s = fma(O.c0[t - 1], DIFF ? x[t - 1] - x0 : x[t - 1], s);
+    if (m & 2) s = fma(O.c0[t], DIFF ? x[t + 1] - x0 : x[t + 1], s);
+    if (m & 4) s = fma(O.c1[t - s1], DIFF ? x[t - s1] - x0 : x[t - s1], s);
+    if (m & 8) s = fma(O.c1[t], DIFF ? x[t + s1] - x0 : x[t + s1], s);
+    if (m & 16) s = fma(O.c2[t - s2], DIFF ? x[t - s2] - x0 : x[t - s2], s);
+    if (m & 32) s = fma(O.c2[t], DIFF ? x[t + s2] - x0 : x[t + s2], s);
     return s;
 }
 
@@ -359,6 +374,7 @@ __device__ void factor3_reg(const Box3& B, const Ops3& O, const T* c0s, const T*
         // diagonal of S_j in FP64 (where the cancellation is)
         if (tid < b) {
             double s = O.cd[p0 + tid];
+            if constexpr (std::is_same<T, float>::value) s *= O.dsc[p0 + tid] * O.dsc[p0 + tid];
             if (j > 0) {
                 const double cc = (double)c2s[p0 - b + tid];
                 s -= cc * (cc * (double)dg[tid]);   // not cc^2 (range at tiny couplings)
@@ -579,6 +595,7 @@ __device__ void gj_cta(T* S, int b, int ld, T* rowbuf, T* colbuf, T* ipb, int* b
 template <typename T>
 __device__ void factor3_smem(const Box3& B, const Ops3& O, const T* c2s, T* F, T* Sb, T* rowbuf, T* colbuf, T* ipb,
                              int* bad) {
+    constexpr bool mixed = std::is_same<T, float>::value;
     const int b = B.b, ld = plane_ld(b), bb = b * b;
     const int tid = threadIdx.x, nt = blockDim.x;
     const int n0 = B.n[B.a0];
@@ -591,6 +608,7 @@ __device__ void factor3_smem(const Box3& B, const Ops3& O, const T* c2s, T* F, T
             const int sidx = i * ld + k;
             if (i == k) {
                 double s = O.cd[ci];
+                if constexpr (mixed) s *= O.dsc[ci] * O.dsc[ci];
                 if (j > 0) {
                     const double cc = (double)c2s[ci - b];
                     s -= cc * (cc * (double)Sb[sidx]);   // not cc^2 (range at tiny couplings)
@@ -598,10 +616,9 @@ __device__ void factor3_smem(const Box3& B, const Ops3& O, const T* c2s, T* F, T
                 Sb[sidx] = (T)s;
             } else {
                 T s = T(0);
-                if (k == i + 1) s -= (T)O.c0[ci];
-                if (k == i - 1) s -= (T)O.c0[ck];
-                if (k == i + n0) s -= (T)O.c1[ci];
-                if (k == i - n0) s -= (T)O.c1[ck];
+                const int dk = k > i ? k - i : i - k, cl = k > i ? ci : ck;   // the coupling of the lower cell
+                if (dk == 1) s -= mixed ? (T)scaled3(O, O.c0, 2u, 1, cl) : (T)O.c0[cl];
+                if (dk == n0) s -= mixed ? (T)scaled3(O, O.c1, 8u, n0, cl) : (T)O.c1[cl];
                 if (j > 0) s -= c2s[ci - b] * Sb[sidx] * c2s[ck - b];
                 Sb[sidx] = s;
             }
@@ -831,10 +848,10 @@ __device__ __forceinline__ void warp_max_to(unsigned int* a, unsigned v) {
 
 // Solves A x_q = rhs_q for NR right-hand sides with the whole CTA: sweeps
 // with the kept factor (FP32 in the mixed form, FP64 in the FP64 form) and
-// refinement with FP64 residuals from X = 0, the iterate X in FP64 (mixed form:
-// the scaled x~ = D^-1 x until the end, rhs scaled).  High-contrast boxes reach a
-// residual floor above what a fixed tolerance can ask for, so the refinement runs
-// to that floor: it stops
+// refinement with FP64 residuals from X = 0, the iterate X in FP64; in the mixed
+// form the sweeps take the scaled residual D r and X gets D times their result.
+// High-contrast boxes reach a residual floor above what a fixed tolerance can ask
+// for, so the refinement runs to that floor: it stops
 // when every right-hand side has |r| <= 1e-3 ir_tol |b| (scaled max norms),
 // or has |r| <= ir_tol |b| and no longer halves its residual per step.  The
 // FP64 form (a direct solve, then refinement with the same rule, at most 4
@@ -858,7 +875,7 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
         for (int q = 0; q < NR; ++q) {
             unsigned hm = 0u;
             for (int t = tid; t < nc; t += nt) {
-                const double v = rhs(q, t);
+                const double v = O.dsc[t] * rhs(q, t);
                 X[q * nc + t] = v;   // kept for the next pass
                 hm = max(hm, abs_hi(v));
             }
@@ -907,7 +924,7 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
         for (int q = 0; q < NR; ++q) {
             const int ex = mixed ? shift(q) : 0;
             for (int t = tid; t < nc; t += nt) {
-                if constexpr (mixed) X[q * nc + t] += f2d_bits(W[q * nc + t], ex);
+                if constexpr (mixed) X[q * nc + t] += O.dsc[t] * f2d_bits(W[q * nc + t], ex);
                 else X[q * nc + t] += W[q * nc + t];
             }
         }
@@ -921,9 +938,9 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
             unsigned rn = 0u;
             const int ex = mixed ? shift(q) : 0;
             for (int t = tid; t < nc; t += nt) {
-                const double v = resid3(O, s1, s2, X + q * nc, rhs(q, t), t);
+                const double v = resid3<mixed>(O, s1, s2, X + q * nc, rhs(q, t), t);
                 if constexpr (mixed) {
-                    const float w = d2f_near(v, ex);
+                    const float w = d2f_near(O.dsc[t] * v, ex);
                     W[q * nc + t] = w;
                     rn = max(rn, abs_bits(w));
                 } else {
@@ -937,11 +954,6 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
         done = test(reached);
         if (!done && it == mit - 1 && !reached && tid == 0 && mixed) *noconv = 1;
         __syncthreads();
-    }
-    if constexpr (mixed) {
-        // back from the scaled iterate
-        for (int q = 0; q < NR; ++q)
-            for (int t = tid; t < nc; t += nt) X[q * nc + t] *= O.dsc[t];
     }
     __syncthreads();
     return it;
@@ -983,7 +995,7 @@ __device__ double source_rhs3(const Box3& B, const Ops3& O, const MemberDev& md,
 struct RhsBasis3 {
     const Box3* B;
     const Ops3* O;
-    const double* bs;   // scaled in the mixed form
+    const double* bs;
     int sk[NR3], mk[NR3], bit[NR3];   // side, function, and the neighbour bit that cells of the side lack
     __device__ double operator()(int q, int t) const {
         if (sk[q] < 0) return bs[t];
@@ -991,8 +1003,7 @@ struct RhsBasis3 {
         const int sid = sk[q];
         const int ls = B->n[B->ts[sid]], lt = B->n[B->tt[sid]];
         const int e = side_e(*B, sid, bcoord(*B, t)), ct = e / ls;
-        const double v = O->bT[B->soff[sid] + e] * psi3(mk[q], e - ct * ls, ls, ct, lt);
-        return O->dsc ? O->dsc[t] * v : v;
+        return O->bT[B->soff[sid] + e] * psi3(mk[q], e - ct * ls, ls, ct, lt);
     }
 };
 
@@ -1180,8 +1191,7 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
     Carve3<T> C = carve3<T>(smem, B, round, part, false, P.xs + (size_t)blockIdx.x * P.xs_stride);
     build_ops3(B, md, P, C.O, mixed);
     if constexpr (mixed) {
-        scale_ops3(B, C.O);
-        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.c2s[t] = (T)C.O.c2[t];
+        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.c2s[t] = scaled3(C.O, C.O.c2, 32u, B.b, t);
         __syncthreads();
     }
     T* F;
@@ -1193,8 +1203,8 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
         if constexpr (mixed) {
             T* cs = C.fac + GJW3;   // in-plane couplings in T, in the factor phase's overlay
             for (int t = threadIdx.x; t < B.nc; t += blockDim.x) {
-                cs[t] = d2f_near(C.O.c0[t]);
-                cs[B.nc + t] = d2f_near(C.O.c1[t]);
+                cs[t] = scaled3(C.O, C.O.c0, 2u, 1, t);
+                cs[B.nc + t] = scaled3(C.O, C.O.c1, 8u, B.n[B.a0], t);
             }
             c0s = cs;
             c1s = cs + B.nc;
@@ -1211,6 +1221,7 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
         T* ipb = (T*)((unsigned char*)colbuf + align16(sizeof(T) * B.b));
         factor3_smem<T>(B, C.O, C.c2s, F, Sb, rowbuf, colbuf, ipb, &C.flags[0]);
     }
+    if constexpr (mixed) side_diag3(B, C.O);
     if (C.flags[0] && threadIdx.x == 0) {
         atomicOr(&P.status[0], ST_NOT_SPD);
         atomicExch(&P.status[2], job.item);
@@ -1227,8 +1238,7 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
     double* bsg = hat_part ? P.bsrc + (size_t)job.item * P.dsc_stride : nullptr;
     if (part || hat_part) {
         double* bs = part ? C.bsrc : bsg;
-        for (int t = threadIdx.x; t < B.nc; t += blockDim.x)
-            bs[t] = (mixed ? C.O.dsc[t] : 1.0) * source_rhs3(B, C.O, md, fm, nullptr, t);
+        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) bs[t] = source_rhs3(B, C.O, md, fm, nullptr, t);
         __syncthreads();
     }
     // Omega_i in the box (in shared memory: indexed by the axis at run time)
@@ -1393,8 +1403,8 @@ __global__ void __launch_bounds__(T3, 1) k_smooth3d(DevPtrs P, MethodDev Mth, co
     // (the Jacobi scale comes out as in the factorisation: the same faces, the same arithmetic)
     build_ops3(B, md, P, C.O, mixed);
     if constexpr (mixed) {
-        scale_ops3(B, C.O);
-        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.c2s[t] = (T)C.O.c2[t];
+        for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.c2s[t] = scaled3(C.O, C.O.c2, 32u, B.b, t);
+        side_diag3(B, C.O);
     }
     // Robin data from the current solution: lambda = -beta u.n + pi (n outward of hat-Omega_i)
     const double* pst = P.p + md.cell_off;
@@ -1408,8 +1418,7 @@ __global__ void __launch_bounds__(T3, 1) k_smooth3d(DevPtrs P, MethodDev Mth, co
     }
     __syncthreads();
     const double* fm = P.f + md.cell_off;
-    for (int t = threadIdx.x; t < B.nc; t += blockDim.x)
-        C.bsrc[t] = (mixed ? C.O.dsc[t] : 1.0) * source_rhs3(B, C.O, md, fm, C.lam, t);
+    for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.bsrc[t] = source_rhs3(B, C.O, md, fm, C.lam, t);
     __syncthreads();
     const T* F = (const T*)P.fac + (size_t)item * P.fac_stride;
     RhsStored3 rs{C.bsrc};
