@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
             warp_solve_sc<RhsScStored, -1, true>(B, O, Sinv, cys, xs, wv, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1]);
         } else {
             RhsStored rs{b};
-            warp_solve<T>(B, O, Sinv, cys, xs, (T*)xs, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1], B.nx);
+            warp_solve64(B, O, Sinv, cys, xs, zb, rs);
         }
     };
     for (int k = warp; k < nrhs; k += nw) {
@@ -539,10 +539,10 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
                 warp_solve_sc<RhsScSide, -1, true>(B, O, Sinv, cys, x, wv, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1]);
             } else {
                 RhsBasis rb{sk, mk};
-                warp_solve<T>(B, O, Sinv, cys, x, (T*)x, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1], B.nx);
+                warp_solve64(B, O, Sinv, cys, x, zb, rb);
             }
         } else {
-            double* bs = basis ? P.bsrc + (size_t)job.item * P.dsc_stride : bsrc;
+            double* bs = basis ? P.bsrc + (size_t)job.item * P.box_stride : bsrc;
             for (int c = lane; c < B.n; c += 32)
                 bs[c] = (mixed ? O.dsc[c] : 1.0) * source_rhs(B, O, fm, nxg, vol, ax, ay, nullptr, c % B.nx, c / B.nx);
             __syncwarp();

@@ -153,7 +153,6 @@ struct mrcm_handle {
     void* d_fac = nullptr;
     void* d_fac_aux = nullptr;
     void* d_fac_part = nullptr;
-    double* d_dsc = nullptr;
     double *d_Psi = nullptr, *d_Ug = nullptr, *d_pbar = nullptr, *d_ubg = nullptr, *d_mom = nullptr;
     int* d_status = nullptr;
     double* d_mean = nullptr;
@@ -469,7 +468,7 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
     // jobs: basis, particular, smoothing factor
     std::map<int, std::vector<Job>> byw;
     std::map<int, size_t> smem_w;
-    size_t fac_stride = 0, dsc_stride = 0, part_stride = 0;
+    size_t fac_stride = 0, box_stride = 0, part_stride = 0;
     const int nitems = (int)h->sub.size();
     // 2D FP32 lines widened to a multiple of 4, unless some box then does not
     // fit shared memory (tall boxes of a width that is no multiple of 4), be
@@ -499,7 +498,7 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
             const int pb = bx * by * bz / std::max({bx, by, bz});
             if (pb > 256) return fail(h, MRCM_ERR_UNSUPPORTED, "3D boxes with planes of more than 256 cells");
             fac_stride = std::max(fac_stride, (factor3_entries(bx, by, bz) + 3) & ~size_t(3));
-            dsc_stride = std::max(dsc_stride, (size_t)bx * by * bz);
+            box_stride = std::max(box_stride, (size_t)bx * by * bz);
             byw[0].push_back(Job{s, JOB_BASIS});
             smem_w[0] = std::max(smem_w[0], local3d_smem(prec, bx, by, bz, false));
             if (!h->mth.part_hat) {
@@ -516,7 +515,7 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
         if (bx > 32 || ix > 32)
             return fail(h, MRCM_ERR_UNSUPPORTED, "2D boxes wider than 32 cells along x are not supported");
         fac_stride = std::max(fac_stride, spack_bytes(prec, bx, by, pad) / tsz);   // smoothing packs, 16-byte multiples
-        dsc_stride = std::max(dsc_stride, (size_t)bx * by);
+        box_stride = std::max(box_stride, (size_t)bx * by);
         // with the particular problem on hat-Omega_i it is one more
         // right-hand side of the basis job (kept in global memory, so the
         // basis box needs no more shared memory)
@@ -571,11 +570,10 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
         if (!h->mth.same_alpha && (e = dalloc(h, (char**)&h->d_fac_aux, fac_stride * nitems * tsz))) return e;
         // FP64 iterates of the local solves: one slot of 4 right-hand sides per CTA of the largest launch
         const size_t slots = std::max(jobs.size(), (size_t)nitems);
-        if ((e = dalloc(h, &d_xs, slots * 4 * dsc_stride))) return e;
+        if ((e = dalloc(h, &d_xs, slots * 4 * box_stride))) return e;
     }
-    if ((e = dalloc(h, &h->d_dsc, dsc_stride * nitems))) return e;
     double* d_bsrc = nullptr;
-    if (h->mth.part_hat && (e = dalloc(h, &d_bsrc, dsc_stride * nitems))) return e;
+    if (h->mth.part_hat && (e = dalloc(h, &d_bsrc, box_stride * nitems))) return e;
     if ((e = dalloc(h, &h->d_Psi, (size_t)nitems * h->nbasis_max * h->ncell_i_max))) return e;
     if ((e = dalloc(h, &h->d_Ug, (size_t)nitems * h->nbasis_max * MRCM_MAXSIDE * h->side_max))) return e;
     if ((e = dalloc(h, &h->d_pbar, (size_t)nitems * h->ncell_i_max))) return e;
@@ -623,9 +621,8 @@ static int create_impl(int count, const mrcm_grid* grids, const double* const* K
     P.fac_part = h->d_fac_part;
     P.part_stride = (long long)part_stride;
     P.xs = d_xs;
-    P.xs_stride = (long long)(4 * dsc_stride);
-    P.dsc = h->d_dsc;
-    P.dsc_stride = (long long)dsc_stride;
+    P.xs_stride = (long long)(4 * box_stride);
+    P.box_stride = (long long)box_stride;
     P.bsrc = d_bsrc;
     P.Psi = h->d_Psi;
     P.Ug = h->d_Ug;

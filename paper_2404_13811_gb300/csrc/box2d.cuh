@@ -118,17 +118,6 @@ __device__ void build_ops(const Box& B, const MemberDev& md, const DevPtrs& P, O
     __syncthreads();
 }
 
-// (A x)_c for the unscaled FP64 operator.
-__device__ __forceinline__ double apply_A(const Box& B, const Ops& O, const double* x, int i, int j) {
-    const int c = j * B.nx + i;
-    double s = O.cd[c] * x[c];
-    if (i > 0) s -= O.cx[c - 1] * x[c - 1];
-    if (i < B.nx - 1) s -= O.cx[c] * x[c + 1];
-    if (j > 0) s -= O.cy[c - B.nx] * x[c - B.nx];
-    if (j < B.ny - 1) s -= O.cy[c] * x[c + B.nx];
-    return s;
-}
-
 // --- FP32 <-> FP64 conversions on the integer pipe ---------------------------
 // On GB300 every FP64-pipe warp instruction, conversions included, occupies
 // the sub-partition's FP64 unit for 64 cycles, and the refinement of the
@@ -1079,53 +1068,17 @@ __device__ double source_rhs(const Box& B, const Ops& O, const double* fm, int n
     return r;
 }
 
-// Solves A x = b for one right-hand side with one warp.  FP64 form: one
-// solve.  Mixed form: FP32 sweeps + FP64 residual refinement.  Returns the
-// number of sweeps (solves) performed.
-template <typename T, typename Rhs>
-__device__ int warp_solve(const Box& B, const Ops& O, const T* Sinv, const T* cys, double* x, T* w,
-                          T* zbuf, const Rhs& rhs, double tol, int max_ir, int* noconv, int bp) {
+// Solves A x = b for one right-hand side with one warp in the FP64 form: one
+// solve, in w.
+template <typename Rhs>
+__device__ int warp_solve64(const Box& B, const Ops& O, const double* Sinv, const double* cys, double* w, double* zbuf,
+                            const Rhs& rhs) {
     const int lane = threadIdx.x & 31;
-    const int b = B.nx, nb = B.ny;
-    if (std::is_same<T, double>::value) {
-        for (int j = 0; j < nb; ++j)
-            for (int i = lane; i < b; i += 32) w[j * b + i] = (T)rhs(B, O, i, j);
-        __syncwarp();
-        warp_sweeps<T>(Sinv, cys, w, zbuf, b, nb, bp);
-        return 1;
-    } else {
-        float bn = 0.f;
-        for (int j = 0; j < nb; ++j)
-            for (int i = lane; i < b; i += 32) {
-                const int c = j * b + i;
-                const T wc = (T)(O.dsc[c] * rhs(B, O, i, j));
-                x[c] = 0.0;
-                w[c] = wc;
-                bn = fmaxf(bn, fabsf((float)wc));
-            }
-        for (int o = 16; o; o >>= 1) bn = fmaxf(bn, __shfl_xor_sync(0xffffffffu, bn, o));
-        __syncwarp();
-        int it = 0;
-        for (; it < max_ir; ++it) {
-            warp_sweeps<T>(Sinv, cys, w, zbuf, b, nb, bp);
-            for (int c = lane; c < B.n; c += 32) x[c] += O.dsc[c] * (double)w[c];
-            __syncwarp();
-            // FP64 residual of the unscaled operator; the (scaled) norms are taken in FP32
-            float rn = 0.f;
-            for (int j = 0; j < nb; ++j)
-                for (int i = lane; i < b; i += 32) {
-                    const int c = j * b + i;
-                    const T wc = (T)(O.dsc[c] * (rhs(B, O, i, j) - apply_A(B, O, x, i, j)));
-                    w[c] = wc;
-                    rn = fmaxf(rn, fabsf((float)wc));
-                }
-            for (int o = 16; o; o >>= 1) rn = fmaxf(rn, __shfl_xor_sync(0xffffffffu, rn, o));
-            __syncwarp();
-            if ((double)rn <= tol * (double)bn || bn == 0.f) { ++it; break; }
-            if (it == max_ir - 1 && lane == 0) *noconv = 1;
-        }
-        return it;
-    }
+    for (int j = 0; j < B.ny; ++j)
+        for (int i = lane; i < B.nx; i += 32) w[j * B.nx + i] = rhs(B, O, i, j);
+    __syncwarp();
+    warp_sweeps<double>(Sinv, cys, w, zbuf, B.nx, B.ny, B.nx);
+    return 1;
 }
 
 // The twisted sweeps of an FP64 solve by four warps: two per chain, each with
@@ -1245,8 +1198,7 @@ __device__ __forceinline__ void cell_ij(int c, int b, float rb, int& i, int& j) 
 
 // One right-hand side by one warp in the mixed form: FP32 twisted sweeps of
 // the kept factor, FP64 residuals of the scaled operator, until
-// |r~|_inf <= tol |b~|_inf (the stopping rule of warp_solve, in the same
-// scaled norm).  Cells are visited 32 at a time by all lanes.  On exit x
+// |r~|_inf <= tol |b~|_inf.  Cells are visited 32 at a time by all lanes.  On exit x
 // holds x~ (the caller scales back with dsc).  Returns the number of sweeps.
 // SW: the line width where it is a template's (0: by column; -1: the row path
 // of the width b where there is one, chosen at run time).  NORM: the FP32

@@ -11,10 +11,10 @@
 // mat-vecs, one warp per right-hand side (Steps 2, 4, 7).
 //
 // Precision: T = double is the FP64 form.  T = float is the mixed form: the
-// operator is Jacobi scaled, the Schur diagonals and every Gauss-Jordan
-// pivot reciprocal are formed in FP64, the sweeps run in FP32, and each
-// right-hand side is refined with FP64 residuals of the unscaled operator
-// until |r|_inf <= ir_tol |b|_inf.
+// operator is Jacobi scaled, the Schur diagonals are formed in FP64, the
+// Gauss-Jordan elimination (correctly rounded FP32 pivot reciprocals) and the
+// sweeps run in FP32, and each right-hand side is refined with FP64 residuals
+// of the scaled operator until |r~|_inf <= ir_tol |b~|_inf.
 //
 // FP64 division and square root are avoided in the hot loops (GB300 has a
 // narrow FP64 pipe): face transmissibilities come precomputed per problem,
@@ -62,11 +62,9 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
         T* dst = (T*)pk;
         const size_t nS = sinv_len(B.nx, B.ny, sizeof(T), Mth.pad);
         for (size_t t = threadIdx.x; t < nS; t += blockDim.x) dst[t] = C.Sinv[t];
-        double* dd = P.dsc + (size_t)job.item * P.dsc_stride;
         const double* fk = P.f + md.cell_off;
         const double vk = md.h[0] * md.h[1];
         for (int c = threadIdx.x; c < B.n; c += blockDim.x) {
-            dd[c] = C.O.dsc[c];
             ((double*)(pk + L.cd))[c] = C.O.cd[c];
             ((double*)(pk + L.cx))[c] = C.O.cx[c];
             ((double*)(pk + L.cy))[c] = C.O.cy[c];
@@ -121,12 +119,11 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
                                                             Mth.max_ir, &C.flags[1]);
             } else {
                 RhsBasis rb{sk, mk};
-                it = warp_solve<T, RhsBasis>(B, C.O, C.Sinv, C.cys, x, w, zb, rb, Mth.ir_tol, Mth.max_ir,
-                                             &C.flags[1], B.nx);
+                it = warp_solve64(B, C.O, C.Sinv, C.cys, w, zb, rb);
             }
         } else {
             // the particular problem: fixed right-hand side staged once (b~ in the mixed form)
-            double* bs = hat_part ? P.bsrc + (size_t)job.item * P.dsc_stride : C.bsrc;
+            double* bs = hat_part ? P.bsrc + (size_t)job.item * P.box_stride : C.bsrc;
             for (int c = lane; c < B.n; c += 32) {
                 const int i = c % B.nx, j = c / B.nx;
                 bs[c] = C.O.dsc[c] * source_rhs(B, C.O, fm, md.n[0], vol, ax, ay, nullptr, i, j);
@@ -138,8 +135,7 @@ __global__ void __launch_bounds__(NWARP * 32, 1) k_local2d(DevPtrs P, MethodDev 
                                                               Mth.max_ir, &C.flags[1]);
             } else {
                 RhsStored rs{bs};
-                it = warp_solve<T, RhsStored>(B, C.O, C.Sinv, C.cys, x, w, zb, rs, Mth.ir_tol, Mth.max_ir,
-                                              &C.flags[1], B.nx);
+                it = warp_solve64(B, C.O, C.Sinv, C.cys, w, zb, rs);
             }
         }
         if constexpr (mixed) {

@@ -1235,7 +1235,7 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
     const int npsi = Mth.npsi;
     const double vol = md.h[0] * md.h[1] * md.h[2];
     const double* fm = P.f + md.cell_off;
-    double* bsg = hat_part ? P.bsrc + (size_t)job.item * P.dsc_stride : nullptr;
+    double* bsg = hat_part ? P.bsrc + (size_t)job.item * P.box_stride : nullptr;
     if (part || hat_part) {
         double* bs = part ? C.bsrc : bsg;
         for (int t = threadIdx.x; t < B.nc; t += blockDim.x) bs[t] = source_rhs3(B, C.O, md, fm, nullptr, t);

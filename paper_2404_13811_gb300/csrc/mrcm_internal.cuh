@@ -84,10 +84,9 @@ struct DevPtrs {
     long long part_stride;
     double* xs;          // 3D mixed form: FP64 iterates of the local solves, per CTA slot
     long long xs_stride;
-    double* dsc;         // Jacobi scaling of the smoothing operator (mixed form)
-    long long dsc_stride;
-    double* bsrc;        // particular problem on hat-Omega_i: scratch for its right-hand side [item][dsc_stride],
+    double* bsrc;        // particular problem on hat-Omega_i: scratch for its right-hand side [item][box_stride],
                          // written and read within one kernel (null otherwise)
+    long long box_stride;   // cells of the largest box
     // basis data
     double* Psi;         // [item][nbasis_max][ncell_i_max]
     double* Ug;          // [item][nbasis_max][2d][side_max]
