@@ -865,7 +865,7 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
     const int s1 = B.n[B.a0], s2 = B.b;
     const int mit = mixed ? max_ir : 4;
     if (*bad) return 0;   // a staged copy failed earlier: the buffers are not usable
-    // |b|, |r|, |r| of the previous step (inf), and (mixed form) the largest high word of b
+    // |b|, |r|, |r| of the previous step (inf), and (mixed form) the largest high word of b, or a bound of it
     if (tid < 4 * NR3) nrm[tid] = tid < 2 * NR3 || tid >= 3 * NR3 ? 0u : 0x7f800000u;
     __syncthreads();
     // mixed form: the FP32 vectors of right-hand side q stand for their values times 2^-shift(q)
@@ -873,13 +873,7 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
     if constexpr (mixed) {
 #pragma unroll
         for (int q = 0; q < NR; ++q) {
-            unsigned hm = 0u;
-            for (int t = tid; t < nc; t += nt) {
-                const double v = O.dsc[t] * rhs(q, t);
-                X[q * nc + t] = v;   // kept for the next pass
-                hm = max(hm, abs_hi(v));
-            }
-            warp_max_to(&nrm[3 * NR3 + q], hm);
+            warp_max_to(&nrm[3 * NR3 + q], rhs.top(q, tid, nt));
         }
         __syncthreads();
     }
@@ -888,10 +882,10 @@ __device__ int solve3_n(const Box3& B, const Ops3& O, const T* F, const T* c2s, 
         unsigned bn = 0u;
         const int ex = mixed ? shift(q) : 0;
         for (int t = tid; t < nc; t += nt) {
-            const double v = mixed ? X[q * nc + t] : rhs(q, t);
+            const double v = rhs(q, t);
             X[q * nc + t] = 0.0;
             if constexpr (mixed) {
-                const float w = d2f_near(v, ex);
+                const float w = d2f_near(O.dsc[t] * v, ex);
                 W[q * nc + t] = w;
                 bn = max(bn, abs_bits(w));
             } else {
@@ -1005,11 +999,33 @@ struct RhsBasis3 {
         const int e = side_e(*B, sid, bcoord(*B, t)), ct = e / ls;
         return O->bT[B->soff[sid] + e] * psi3(mk[q], e - ct * ls, ls, ct, lt);
     }
+    // this thread's part of the largest high word of D b: at most that of its side's face coefficients (|psi| <= 1)
+    __device__ unsigned top(int q, int tid, int nt) const {
+        unsigned h = 0u;
+        if (sk[q] < 0) {
+            for (int t = tid; t < B->nc; t += nt) h = max(h, abs_hi(O->dsc[t] * bs[t]));
+            return h;
+        }
+        const int sid = sk[q], a = sid >> 1, ls = B->n[B->ts[sid]];
+        for (int f = B->soff[sid] + tid; f < B->soff[sid + 1]; f += nt) {
+            const int e = f - B->soff[sid], ct = e / ls;
+            const int t = (e - ct * ls) * B->bs[B->ts[sid]] + ct * B->bs[B->tt[sid]] + ((sid & 1) ? (B->n[a] - 1) * B->bs[a] : 0);
+            h = max(h, abs_hi(O->dsc[t] * O->bT[f]));
+        }
+        return h;
+    }
 };
 
 struct RhsStored3 {
     const double* b;
+    const double* dsc;   // (mixed form)
+    int nc;
     __device__ double operator()(int, int t) const { return b[t]; }
+    __device__ unsigned top(int, int tid, int nt) const {
+        unsigned h = 0u;
+        for (int t = tid; t < nc; t += nt) h = max(h, abs_hi(dsc[t] * b[t]));
+        return h;
+    }
 };
 
 // Shared-memory layout.  Persistent: the operator, neighbour bits, scaled
@@ -1279,7 +1295,7 @@ __global__ void __launch_bounds__(T3, 1) k_local3d(DevPtrs P, MethodDev Mth, con
             it = solve3<T>(nr, B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rb, Mth.ir_tol, Mth.max_ir,
                            &C.flags[1], &C.flags[2]);
         } else {
-            RhsStored3 rs{C.bsrc};
+            RhsStored3 rs{C.bsrc, C.O.dsc, B.nc};
             it = solve3_n<T, 1>(B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rs, Mth.ir_tol, Mth.max_ir,
                                 &C.flags[1], &C.flags[2]);
         }
@@ -1421,7 +1437,7 @@ __global__ void __launch_bounds__(T3, 1) k_smooth3d(DevPtrs P, MethodDev Mth, co
     for (int t = threadIdx.x; t < B.nc; t += blockDim.x) C.bsrc[t] = source_rhs3(B, C.O, md, fm, C.lam, t);
     __syncthreads();
     const T* F = (const T*)P.fac + (size_t)item * P.fac_stride;
-    RhsStored3 rs{C.bsrc};
+    RhsStored3 rs{C.bsrc, C.O.dsc, B.nc};
     const int it = solve3_n<T, 1>(B, C.O, F, C.c2s, C.X, C.W, C.vb, C.red, C.pp, C.nrm, rs, Mth.ir_tol, Mth.max_ir,
                                   &C.flags[0], &C.flags[2]);
     if (C.flags[2]) drain3(C.pp);
