@@ -229,10 +229,11 @@ __device__ void side_diag3(const Box3& B, Ops3& O) {
 
 // b_t - (A x)_t in FP64.  DIFF (mixed form): in differences of neighbouring
 // values, so that its rounding is that of the fluxes and not of the pressures.
-// With entries of D A D, each rounded once more, the fluxes of 60 fields of 60 x
-// 110 x 40 cells came out 1.7 times further from the exact ones; with the rows
-// summed up by the unscaled diagonal they did not, but 4 of 60 layered fields of
-// 60 x 220 x 85 cells missed ir_tol (1 of 60 with DIFF and with D A D).
+// With entries of D A D, each rounded once more, the fluxes of 60 layered fields
+// of 60 x 110 x 40 cells came out 1.7 times further from the exact ones; with rows
+// summed up by the unscaled diagonal they did not, but 5 of 200 layered fields of
+// 60 x 220 x 85 cells missed ir_tol (a box's rounding floor above it) against 1
+// with DIFF.  It costs six FP64 instructions a cell: 45.2 against 42.8 ms a step.
 template <bool DIFF>
 __device__ __forceinline__ double resid3(const Ops3& O, int s1, int s2, const double* x, double bt, int t) {
     const unsigned char m = O.nb[t];

@@ -45,7 +45,8 @@
 // Records live in a ring of R slots.  A cluster barrier every G panels
 // bounds how far a producer can run ahead (R = 2 G: a slot is rewritten only
 // after every CTA has read it) and lets each CTA re-arm a slot right after
-// reading it.  Every wait on a record is bounded; a wait that runs out marks
+// reading it (a CTA that fetches its records arms the slot as it fetches).
+// Every wait on a record is bounded; a wait that runs out marks
 // the launch (ST_BAD) and the kernel runs to its end without further waits.
 #include "mrcm_internal.cuh"
 
