@@ -211,7 +211,7 @@ __global__ void __launch_bounds__((sizeof(T) == 4 ? 2 : 1) * AS_WARPS * 32) k_ad
     }
     __syncthreads();
     if constexpr (mixed) {
-        cta_solve_sc<0, true>(B, O, (const float*)Sinv, (const float*)cys, mu, (float*)w, (float*)zbuf, nrm, rt, Mth.ir_tol,
+        cta_solve_sc(B, O, (const float*)Sinv, (const float*)cys, mu, (float*)w, (float*)zbuf, nrm, rt, Mth.ir_tol,
                      Mth.max_ir, &flags[0], false, line_width(B.nx, sizeof(T), Mth.pad));
         for (int c = threadIdx.x; c < B.n; c += blockDim.x) mu[c] *= O.dsc[c];
         __syncthreads();
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
     auto stored = [&](double* xs, const double* b) {
         if constexpr (mixed) {
             RhsScStored rs{b};
-            warp_solve_sc<RhsScStored, -1, true>(B, O, Sinv, cys, xs, wv, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1]);
+            warp_solve_sc<RhsScStored, -1>(B, O, Sinv, cys, xs, wv, zb, rs, Mth.ir_tol, Mth.max_ir, &flags[1]);
         } else {
             RhsStored rs{b};
             warp_solve64(B, O, Sinv, cys, xs, zb, rs);
@@ -536,7 +536,7 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
                 const int len = (sk >> 1) == 0 ? B.ny : B.nx;
                 const double mine = lane < len ? RhsScSide::face(B, O.dsc, O.bT, sk, mk, lane) : 0.0;
                 RhsScSide rb{sk, mk, O.dsc, O.bT, mine};
-                warp_solve_sc<RhsScSide, -1, true>(B, O, Sinv, cys, x, wv, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1]);
+                warp_solve_sc<RhsScSide, -1>(B, O, Sinv, cys, x, wv, zb, rb, Mth.ir_tol, Mth.max_ir, &flags[1]);
             } else {
                 RhsBasis rb{sk, mk};
                 warp_solve64(B, O, Sinv, cys, x, zb, rb);

@@ -1183,10 +1183,22 @@ struct RhsScSide {
         if (on && pos >= 32) return face(B, dsc, bT, sk, m, pos);
         return on ? v : 0.0;
     }
+    // this lane's part of the largest high word of b~
+    __device__ unsigned top(const Box& B) const {
+        unsigned h = abs_hi(mine);
+        for (int pos = (threadIdx.x & 31) + 32; pos < ((sk >> 1) == 0 ? B.ny : B.nx); pos += 32)
+            h = max(h, abs_hi(face(B, dsc, bT, sk, m, pos)));
+        return h;
+    }
 };
 struct RhsScStored {
     const double* b;
     __device__ double operator()(const Box& B, int i, int j) const { return b[j * B.nx + i]; }
+    __device__ unsigned top(const Box& B) const {
+        unsigned h = 0u;
+        for (int c = threadIdx.x & 31; c < B.n; c += 32) h = max(h, abs_hi(b[c]));
+        return h;
+    }
 };
 
 // (i, j) of cell c of lines of b <= 32 cells, rb = 1.f / b: (c + 0.5) / b is
@@ -1201,10 +1213,9 @@ __device__ __forceinline__ void cell_ij(int c, int b, float rb, int& i, int& j) 
 // |r~|_inf <= tol |b~|_inf.  Cells are visited 32 at a time by all lanes.  On exit x
 // holds x~ (the caller scales back with dsc).  Returns the number of sweeps.
 // SW: the line width where it is a template's (0: by column; -1: the row path
-// of the width b where there is one, chosen at run time).  NORM: the FP32
-// vectors scaled by the right-hand side's exponent (the reverse pass, whose
-// seeds may be of any size).
-template <typename Rhs, int SW = 0, bool NORM = false>
+// of the width b where there is one, chosen at run time).  The FP32 vectors
+// are scaled by the right-hand side's exponent (norm_shift).
+template <typename Rhs, int SW = 0>
 __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, const float* cys, double* x, float* w,
                              float* zbuf, const Rhs& rhs, double tol, int max_ir, int* noconv) {
     const int lane = threadIdx.x & 31;
@@ -1212,29 +1223,15 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
     const float rb = 1.f / (float)b;
     const int nit = (B.n + 31) >> 5;
     float bn = 0.f;
-    unsigned hm = 0u;
+    const int ex = norm_shift(__reduce_max_sync(0xffffffffu, rhs.top(B)));
     for (int k = 0; k < nit; ++k) {
         const int c = k * 32 + lane;
         const bool ok = c < B.n;
         int i, j;
         cell_ij(ok ? c : 0, b, rb, i, j);
         const double bt = rhs(B, i, j);
-        if (!ok) continue;
-        if constexpr (NORM) {
-            x[c] = bt;
-            hm = max(hm, abs_hi(bt));
-        } else {
-            const float wc = d2f_bits(bt);
-            x[c] = 0.0;
-            w[c] = wc;
-            bn = fmaxf(bn, fabsf(wc));
-        }
-    }
-    int ex = 0;
-    if constexpr (NORM) {
-        ex = norm_shift(__reduce_max_sync(0xffffffffu, hm));
-        for (int c = lane; c < B.n; c += 32) {
-            const float wc = d2f_bits(x[c], ex);
+        if (ok) {
+            const float wc = d2f_bits(bt, ex);
             x[c] = 0.0;
             w[c] = wc;
             bn = fmaxf(bn, fabsf(wc));
@@ -1276,7 +1273,7 @@ __device__ int warp_solve_sc(const Box& B, const Ops& O, const float* Sinv, cons
 // still relative to b~; no sweep when the start meets it).  b~ is stored.
 // BB > 0: lines of width at most BB; BB = 0: any width by a switch (bp).
 // nrm: 3 entries.
-template <int BB = 0, bool NORM = false>
+template <int BB = 0>
 __device__ int cta_solve_sc(const Box& B, const Ops& O, const float* Sinv, const float* cys, double* x, float* w,
                             float* zw, unsigned int* nrm, const double* bt, double tol, int max_ir, int* noconv,
                             bool warm, int bp) {
@@ -1285,15 +1282,12 @@ __device__ int cta_solve_sc(const Box& B, const Ops& O, const float* Sinv, const
     const float rb = 1.f / (float)b;
     if (tid < 3) nrm[tid] = 0u;
     __syncthreads();
-    int ex = 0;
-    if constexpr (NORM) {
-        unsigned hm = 0u;
-        for (int c = tid; c < B.n; c += nt) hm = max(hm, abs_hi(bt[c]));
-        hm = __reduce_max_sync(0xffffffffu, hm);
-        if ((tid & 31) == 0) atomicMax(&nrm[2], hm);
-        __syncthreads();
-        ex = norm_shift(nrm[2]);
-    }
+    unsigned hm = 0u;
+    for (int c = tid; c < B.n; c += nt) hm = max(hm, abs_hi(bt[c]));
+    hm = __reduce_max_sync(0xffffffffu, hm);
+    if ((tid & 31) == 0) atomicMax(&nrm[2], hm);
+    __syncthreads();
+    const int ex = norm_shift(nrm[2]);
     float bn = 0.f, r0 = 0.f;
     for (int c = tid; c < B.n; c += nt) {
         int i, j;

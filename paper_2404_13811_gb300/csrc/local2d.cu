@@ -398,9 +398,9 @@ __global__ void __launch_bounds__(SMW<T> * 32, 2) k_smooth2d(DevPtrs P, MethodDe
             __syncthreads();
         }
         if constexpr (mixed) {
-            // the scaled start x~ = D^-1 x (an FP32 reciprocal of the FP32 scale: a start only)
+            // the scaled start x~ = D^-1 x (a start only: an FP32 reciprocal, the division where that is 0 or infinite)
             for (int c = threadIdx.x; c < B.n; c += blockDim.x)
-                x[c] *= f2d_bits(__frcp_rn(d2f_bits(O.dsc[c])));
+                x[c] = in_f32_range(O.dsc[c]) ? x[c] * f2d_bits(__frcp_rn(d2f_bits(O.dsc[c]))) : x[c] / O.dsc[c];
             __syncthreads();
             it = cta_solve_sc<BB>(B, O, (const float*)Sinv, (const float*)cys, x, (float*)w, (float*)zbuf, nrm, bsrc,
                               Mth.ir_tol, Mth.max_ir, &flags[0], true, line_width(B.nx, sizeof(T), Mth.pad));
