@@ -419,7 +419,8 @@ __global__ void k_adj_moments(DevPtrs P, MethodDev Mth, AdjPtrs A) {
 // ---------------------------------------------------------------------------
 // Basis problems (one adjoint solve per basis function on hat-Omega_i) and
 // particular problems (one on Omega_i) backwards.  One CTA per job, one
-// warp per right-hand side: recompute the forward solution x_k with the
+// warp per right-hand side (nw of them at a time, as many as fit shared memory
+// with their vectors; the CTA has two warps at least): recompute the forward solution x_k with the
 // box factor, form the adjoint right-hand side from dL/d(pressure on
 // Omega_i), dL/d(Gamma velocities) and dL/d(moments), solve for mu_k and
 // accumulate the face-coefficient adjoints of all k in shared memory; the
@@ -440,10 +441,10 @@ __host__ __device__ inline size_t adj_carve_bytes(int nx, int ny, int nw, bool p
 }
 
 template <typename T, int BW>
-__global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth, AdjPtrs A, const Job* jobs) {
+__global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth, AdjPtrs A, const Job* jobs,
+                                                                     int nw) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr bool mixed = std::is_same<T, float>::value;
-    const int nw = blockDim.x >> 5;
     const Job job = jobs[blockIdx.x];
     const SubDev sd = P.sub[job.item];
     const MemberDev& md = P.mem[sd.member];
@@ -520,7 +521,7 @@ __global__ void __launch_bounds__(128, 1) k_adj_local2d(DevPtrs P, MethodDev Mth
             warp_solve64(B, O, Sinv, cys, xs, zb, rs);
         }
     };
-    for (int k = warp; k < nrhs; k += nw) {
+    for (int k = warp < nw ? warp : nrhs; k < nrhs; k += nw) {
         // forward solution x_k
         int sk = -1, mk = 0;
         const bool pk = !basis || k >= sd.nbasis;   // the particular problem
@@ -799,7 +800,8 @@ static cudaError_t launch_adj_local_t(const DevPtrs& P, const MethodDev& M, cons
     static size_t cur = 0;
     cudaError_t e = set_smem_attr(k_adj_local2d<T, BW>, smem, &cur);
     if (e != cudaSuccess) return e;
-    k_adj_local2d<T, BW><<<njobs, nw * 32, smem, s>>>(P, M, A, jobs);
+    // two warps at least: the factorisation runs a chain on each
+    k_adj_local2d<T, BW><<<njobs, (nw > 2 ? nw : 2) * 32, smem, s>>>(P, M, A, jobs, nw);
     return cudaGetLastError();
 }
 
