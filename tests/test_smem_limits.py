@@ -42,3 +42,18 @@ def test_box_between_the_limits_matches_oracle(precision, tol):
     s.close()
     ep, eu = O.rel_errors(prob, p, u, ref.p, ref.u)
     assert ep <= tol and eu <= tol, (ep, eu)
+
+
+def test_no_box_of_the_shapes_test_is_refused():
+    """The 3D shapes test skips a box that is refused; none of its boxes may be."""
+    from paper_2404_13811_gb300 import build
+    from tests.test_gpu_local3d import CASES
+    lib = ctypes.CDLL(build.build())
+    basis, smooth = lib._Z12local3d_smemiiiib, lib._Z13smooth3d_smemiiii
+    basis.restype = smooth.restype = ctypes.c_size_t
+    for n, sub, ov, _ in CASES:
+        # the largest box: inner subdomains grow on both sides, of two on one
+        box = [min(n[a], sub[a] + ov * min(2, n[a] // sub[a] - 1)) for a in range(3)]
+        for prec in (0, 1):
+            assert max(basis(prec, *box, False), basis(prec, *sub, True)) <= CTA - STATIC_LOCAL3D, (box, prec)
+            assert smooth(prec, *box) <= CTA - 448, (box, prec)
